@@ -10,7 +10,11 @@
  *     its ordered dendrogram for a start point s and the reachability plot from s (Sec. 4).
  * Both follow the method of Sec. 3: a spatial-median k-d tree, the well-separated pair
  * decomposition traversed lazily by MemoGFK rounds (Algorithm 3) with batched BCCP / BCCP*
- * computations, and batched Kruskal over a union-find shared across rounds; the dendrogram and
+ * computations, and batched Kruskal over a union-find shared across rounds.  By default the forest
+ * is first built by nearest-component rounds on the same tree (Boruvka's algorithm, the single-tree
+ * form of the dual-tree method that Sec. 5 compares with), which return the same tree faster; MemoGFK
+ * rounds build what they leave, and everything in the FP64 form, under wm_set_tuning, for EMSTs above
+ * 8 dimensions, and for HDBSCAN* under the geometric separation or with overflowing ties.  The dendrogram and
  * plot come from a top-down heavy/light construction after Sec. 4.2 (the heavy set of a
  * subproblem is the upper half of its rank interval, light components come from a union-find,
  * and the output equals the sequential definition exactly).
@@ -71,7 +75,8 @@ extern "C" {
 
 /* Methods (wm_opts.method): an algorithm, optionally OR'ed with WM_SEPARATION_GEOMETRIC; all
  * compute the same tree. */
-#define WM_METHOD_MEMOGFK 0   /* MemoGFK rounds (Sec. 3.2.3, Algorithm 3), the default */
+#define WM_METHOD_MEMOGFK 0   /* the default: nearest-component rounds where they apply (see the top),
+                                 MemoGFK rounds (Sec. 3.2.3, Algorithm 3) otherwise */
 #define WM_METHOD_GFK 1       /* GFK (Sec. 3.2.2, Algorithm 2): the full WSPD is materialised and each
                                  pair's BCCP computed once and kept until its round */
 #define WM_METHOD_NAIVE 2     /* EMST-Naive (Sec. 5): the BCCP of every pair of the full WSPD, then
@@ -107,10 +112,11 @@ typedef struct {
     double ms_build_tree;
     double ms_core_dist;
     double ms_wspd;       /* GetRho + GetPairs traversals (including inline BCCP)   */
-    double ms_bccp;       /* BCCP flushes (all size classes and their readbacks)    */
+    double ms_bccp;       /* nearest-component rounds; BCCP flushes (all size classes
+                             and their readbacks)                                   */
     double ms_kruskal;    /* batched Kruskal of every round + final sort of the tree */
     double ms_dendrogram;
-    int64_t rounds;       /* MemoGFK rounds                                         */
+    int64_t rounds;       /* nearest-component and MemoGFK rounds                   */
     int64_t pairs_retrieved;   /* well-separated pairs whose BCCP was evaluated     */
     int64_t bccp_evals;        /* point-pair distance evaluations in BCCP / BCCP*   */
     int64_t bccp_tile_evals;   /* of which in the tile kernel                        */
@@ -144,7 +150,8 @@ typedef struct {
     int64_t getpairs_launches;     /* number of GetPairs step launches                  */
     int64_t getpairs_visits;       /* node pairs examined by the GetPairs traversals     */
     int64_t getrho_visits;         /* node pairs examined by the GetRho traversals       */
-    int64_t bccp_dual_evals;       /* distance evaluations in the pruned dual-tree BCCP */
+    int64_t bccp_dual_evals;       /* distance evaluations in the nearest-component search and
+                                      in the pruned dual-tree BCCP                        */
     int64_t rho_shrinks;           /* times a round lowered rho_hi to fit its edge batch  */
     int64_t max_pending_pairs;     /* peak node pairs pending in a WSPD traversal         */
     int64_t bccp_pairs_below;      /* retrieved pairs whose BCCP lay below the round's
@@ -157,7 +164,8 @@ typedef struct {
                                         chunk's bounding box ruled out                   */
     double ms_getrho;              /* CUDA-event time of the GetRho traversals           */
     double ms_bccp_group;          /* ... of the group BCCP kernels (tiny, small pairs)  */
-    double ms_bccp_dual;           /* ... of the dual-tree BCCP kernel (huge pairs)      */
+    double ms_bccp_dual;           /* ... of the nearest-component search and of the dual-tree
+                                      BCCP kernel (huge pairs)                           */
     int64_t wspd_pairs;            /* GFK / EMST-Naive: pairs of the materialised WSPD     */
 } wm_stats;
 

@@ -8,6 +8,7 @@
 #include <cstring>
 #include <condition_variable>
 #include <deque>
+#include <functional>
 #include <mutex>
 #include <thread>
 #include <unordered_map>
@@ -16,6 +17,7 @@
 
 #include "wm_internal.cuh"
 #include "wspd.cuh"
+#include "boruvka.cuh"
 #include "batch.cuh"
 #include "hdb.cuh"
 
@@ -223,10 +225,11 @@ static bool tuning_valid(const wm_tuning &t)
            t.range_gate <= 1 << 20;
 }
 
-static wm_tuning tuning_for(long long n, int d, int min_pts)
+static wm_tuning tuning_for(long long n, int d, int min_pts, bool *overridden = nullptr)
 {
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
+        if (overridden) *overridden = g_tune_set;
         if (g_tune_set) return g_tune_override;
     }
     wm_tuning t{};
@@ -358,6 +361,7 @@ struct Call {
     int *pin = nullptr;
     wm_stats stats{};
     wm_tuning tune{};
+    bool tune_override = false;       // tune comes from wm_set_tuning
     int method = WM_METHOD_MEMOGFK;   // wm_opts.method
     int disjunctive = 1;              // HDBSCAN*: the separation of Sec. 3.1.2 (0: GanTao's)
     int precision = WM_PREC_FP32_SCREEN;
@@ -432,7 +436,27 @@ static void set_rho(TravArgs &a, double lo, double hi)
     a.above_f = above_threshold(hi, a);
 }
 
-// MemoGFK rounds (Algorithm 3).  On return E_out holds the tree edges in K order: n-1 of them, or
+// Whether the forest is built by nearest-component rounds (boruvka.cu) rather than MemoGFK rounds.  Both
+// give the K-minimum tree; the nearest-component rounds answer one question per component and round
+// instead of visiting every well-separated pair, and are the faster of the two on every generator and
+// size measured up to 8 dimensions (GB300, ms: EMST uniform 3-D / 5-D and variable-density 7-D points at
+// 10^7: 35 / 72 / 212 against 58 / 130 / 890; uniform 2-D at 3x10^6, FP64: 10.3 against 11.3; 10^3
+// points in 3-D: 1.6 against 3.5; HDBSCAN* of 10^6 points in 3-D: 14 against 31).  MemoGFK keeps
+//   - the plain FP64 form, whose distances are all FP64 (the lists here are screened in FP32);
+//   - calls under wm_set_tuning, whose parameters are those of the traversals, and the geometric
+//     separation of the GanTao baseline, which is a property of the WSPD;
+//   - HDBSCAN* inputs whose repair list overflowed: the rounds here need it complete;
+//   - EMSTs above 8 dimensions: on uniform points every search visits much of the tree (10^5 points in
+//     10-D: 71 against 57 ms; 3x10^4 in 16-D: 178 against 96), which the pair traversal shares better;
+//   - 2^28 points and more (references hold 28-bit positions).
+static bool nearest_rounds_apply(const Call &C, int n, int d, const HdbState *hdb)
+{
+    if (C.precision == WM_PREC_FP64 || C.tune_override || n >= 1 << 28) return false;
+    return hdb ? C.disjunctive && !C.stats.tie_overflow : d <= 8;
+}
+
+// The spanning tree: nearest-component rounds where they apply, else (or for what they leave) MemoGFK
+// rounds (Algorithm 3).  On return E_out holds the tree edges in K order: n-1 of them, or
 // `target` when the points form several instances that must not be joined (a batch): then every
 // edge weight is below rho_cap, rho_hi never exceeds it, and no pair at or above it is retrieved.
 // hdb: optional HDBSCAN* state (node cd bounds, per-position cd2, repair edges).
@@ -446,49 +470,16 @@ static int memogfk(Call &C, Points &P, Tree &T, const HdbState *hdb, const Caps 
     *overflow_bits = 0;
     if (n <= 1) return 0;
     size_t mark = ar.off;
-    const int chunk = (int)caps.chunk;
-    const long long fcap = ((long long)T.N / 2 + 2 + (2LL * T.depth + 4) * 2 * chunk) * caps.frontier_scale;
-    if (fcap > 0x7fffffffLL) { set_detail("WSPD stack capacity exceeds 2^31 pairs%s", ""); return WM_ENOMEM; }
-    int2 *stack = ar.get<int2>(fcap);
-    int2 *const xbuf[2] = {ar.get<int2>(4LL * chunk), ar.get<int2>(4LL * chunk)};   // step outputs
-    // pair lists hold kListChunks chunks' worth of retrieved pairs; they are flushed (BCCP) when
-    // one of them could overflow within the next poll interval, and when the traversal ends
-    const int kPoll = 3, kListChunks = 8;
-    const long long lcap = (long long)kListChunks * chunk;
-    int2 *lists[5];
-    float *list_lbs[5];
-    for (int c = 0; c < 5; ++c) {
-        lists[c] = ar.get<int2>(lcap);
-        list_lbs[c] = ar.get<float>(lcap);
-    }
-    EdgeK *huge_best = ar.get<EdgeK>(lcap + 1);
-    unsigned *huge_sbest = ar.get<unsigned>(lcap + 1);
-    long long *huge_items = ar.get<long long>(lcap + 1);
-    const int stack_warps = num_sms() * 8 * 8;   // warps of the dual-tree kernel (grid-stride)
-    int *dual_stack = ar.get<int>((size_t)stack_warps * (T.depth + 4));
     const int dp = P.d <= 4 ? 4 : P.d <= 8 ? 8 : 16;
-    NodeRec *rec = ar.get<NodeRec>(T.N);
-    float *box = ar.get<float>((size_t)T.N * 2 * dp);
-    float4 *x4 = ar.get<float4>((size_t)n * (dp / 4));
-    EdgeK *batch = ar.get<EdgeK>(caps.edges), *filt = ar.get<EdgeK>(caps.edges), *tmp = ar.get<EdgeK>(caps.edges);
     int *cnts = ar.get<int>(64);
     unsigned *rho = ar.get<unsigned>(2);
-    int *split_hist = ar.get<int>(kSplitBins);
-    unsigned long long *split_max = ar.get<unsigned long long>(1);
     unsigned *ovf = ar.get<unsigned>(2);
     unsigned long long *stat = ar.get<unsigned long long>(16);
-    int *comp_scratch = ar.get<int>(2LL * n + 1);
     if (ar.failed) return WM_ENOMEM;
     // counters: [2..6] pair-list counts, [7] edge count, [10..11] counts of the two node lists,
     // [12..13] 64-bit huge-pair item total, [16..17] tile-kernel pair dispensers,
     // [32..32+kTravCounters) traversal state
     int *lcount = cnts + 2, *ecount = cnts + 7, *tcnt = cnts + 32;
-    {
-        Tree T2 = T;
-        if (hdb) { T2.cdmin = hdb->cdmin; T2.cdmax = hdb->cdmax; }
-        pack_nodes(T2, P.d, dp, rec, box, st);
-        point_major(P.x32, n, P.d, dp, x4, st);
-    }
     WM_CK(cudaMemsetAsync(stat, 0, 16 * sizeof(unsigned long long), st));
     WM_CK(cudaMemsetAsync(ovf, 0, 2 * sizeof(unsigned), st));
     WM_CK(cudaMemsetAsync(cnts, 0, 64 * sizeof(int), st));
@@ -497,9 +488,10 @@ static int memogfk(Call &C, Points &P, Tree &T, const HdbState *hdb, const Caps 
     a.N = T.N; a.n = n; a.d = P.d;
     a.lo = T.lo; a.hi = T.hi; a.diam2 = T.diam2;
     a.begin = T.begin; a.end = T.end; a.left = T.left; a.right = T.right; a.comp = T.comp;
-    a.x32 = P.x32; a.x4 = x4; a.x64 = P.x64; a.pid = P.pid;
+    a.x32 = P.x32; a.x64 = P.x64; a.pid = P.pid;
     a.fp64 = C.precision == WM_PREC_FP64;
     a.eta = a.fp64 ? 0.0 : 2.0 * (double)P.delta * std::sqrt((double)P.d) * (1.0 + 1e-6);
+    a.eta2_f = float_ru(2.0 * a.eta);
     a.exact32 = a.eta == 0.0;
     a.delta32 = P.delta;
     a.dfs_budget = C.tune.dfs_budget;
@@ -510,25 +502,9 @@ static int memogfk(Call &C, Points &P, Tree &T, const HdbState *hdb, const Caps 
     if (hdb) {
         a.cdmin = hdb->cdmin; a.cdmax = hdb->cdmax; a.cd32 = hdb->cd32; a.cd64 = hdb->cd64;
     }
-    a.frontier_cap = (int)fcap;
-    a.rec = rec; a.box = box; a.dp = dp;
-    for (int c = 0; c < 5; ++c) { a.list[c] = lists[c]; a.list_lb[c] = list_lbs[c]; a.list_cap[c] = (int)lcap; }
-    a.list_count = lcount;
-    a.big = lists[3]; a.big_count = lcount + 3;
-    a.huge_best = huge_best; a.huge_sbest = huge_sbest;
-    a.stack = dual_stack; a.stack_cap = T.depth + 4;
-    a.edges = batch; a.edge_count = ecount;
-    a.edge_cap = (int)(caps.edges_soft > 0 && caps.edges_soft < caps.edges ? caps.edges_soft : caps.edges);
+    a.dp = dp;
     a.overflow = ovf;
     a.stat = stat;
-    a.rho_bits = rho;
-    EdgeK *spare = filt;   // second edge buffer for compaction when rho_hi shrinks
-    int *nodes[2] = {ar.get<int>(T.N / 2 + 1), ar.get<int>(T.N / 2 + 1)};
-    if (ar.failed) return WM_ENOMEM;
-    a.node_in = nullptr;
-    a.node_in_n = nullptr;
-    a.node_out = nodes[0];
-    a.node_out_n = cnts + 10;
 
     // CUDA-event intervals of the round's kernels (when C.timing), summed into the stats per kind
     enum { kSpanGetPairs, kSpanGetRho, kSpanFlush, kSpanGroup, kSpanTile, kSpanDual };
@@ -570,7 +546,97 @@ static int memogfk(Call &C, Points &P, Tree &T, const HdbState *hdb, const Caps 
         spans.clear();
         return 0;
     };
-    int nE = 0;
+    int nE = 0, rounds = 0;
+    if (nearest_rounds_apply(C, n, P.d, hdb)) {
+        Timer tn;
+        struct Hooks {
+            std::function<int()> mark;
+            std::function<void(int, int)> span;
+        } hooks{[&] { return mark_event(); }, [&](int i, int j) { add_span(i, j, kSpanDual); }};
+        NcCall N;
+        N.st = st;
+        N.ar = &ar;
+        N.pin = C.pin;
+        N.depth = T.depth;
+        N.T = &T;
+        N.pos = P.pos;
+        N.uf = uf;
+        N.out = E_out;
+        N.target = target;
+        N.cap = rho_cap;
+        N.cap_f = float_ru(rho_cap);
+        N.rep = hdb ? hdb->rep : nullptr;
+        N.nrep = hdb ? hdb->nrep : 0;
+        N.ctx = &hooks;
+        N.mark = [](void *h) { return ((Hooks *)h)->mark(); };
+        N.span = [](void *h, int i, int j) { ((Hooks *)h)->span(i, j); };
+        WM_TRY(nearest_component_rounds(N, a));
+        WM_TRY(collect_spans());
+        nE = (int)N.done;
+        rounds = N.rounds;
+        C.stats.candidate_edges += N.candidates;
+        C.stats.ms_bccp += tn.ms();
+    }
+    // ---- MemoGFK state
+    const int chunk = (int)caps.chunk;
+    const int kPoll = 3, kListChunks = 8;
+    const long long lcap = (long long)kListChunks * chunk;
+    int2 *stack = nullptr, *xbuf[2] = {nullptr, nullptr}, *lists[5] = {};
+    float *list_lbs[5] = {};
+    long long *huge_items = nullptr;
+    const int stack_warps = num_sms() * 8 * 8;   // warps of the dual-tree kernel (grid-stride)
+    EdgeK *batch = nullptr, *filt = nullptr, *tmp = nullptr;
+    int *split_hist = nullptr, *comp_scratch = nullptr, *nodes[2] = {nullptr, nullptr};
+    unsigned long long *split_max = nullptr;
+    NodeRec *rec = nullptr;
+    if (nE < target) {
+        Tree T2 = T;
+        if (hdb) { T2.cdmin = hdb->cdmin; T2.cdmax = hdb->cdmax; }
+        rec = ar.get<NodeRec>(T.N);
+        float *box = ar.get<float>((size_t)T.N * 2 * dp);
+        float4 *x4 = ar.get<float4>((size_t)n * (dp / 4));
+        if (ar.failed) return WM_ENOMEM;
+        pack_nodes(T2, P.d, dp, rec, box, st);
+        point_major(P.x32, n, P.d, dp, x4, st);
+        a.rec = rec; a.box = box; a.x4 = x4;
+        const long long fcap = ((long long)T.N / 2 + 2 + (2LL * T.depth + 4) * 2 * chunk) * caps.frontier_scale;
+        if (fcap > 0x7fffffffLL) { set_detail("WSPD stack capacity exceeds 2^31 pairs%s", ""); return WM_ENOMEM; }
+        stack = ar.get<int2>(fcap);
+        for (int i = 0; i < 2; ++i) xbuf[i] = ar.get<int2>(4LL * chunk);   // step outputs
+        // pair lists hold kListChunks chunks' worth of retrieved pairs; they are flushed (BCCP) when
+        // one of them could overflow within the next poll interval, and when the traversal ends
+        for (int c = 0; c < 5; ++c) {
+            lists[c] = ar.get<int2>(lcap);
+            list_lbs[c] = ar.get<float>(lcap);
+        }
+        a.huge_best = ar.get<EdgeK>(lcap + 1);
+        a.huge_sbest = ar.get<unsigned>(lcap + 1);
+        huge_items = ar.get<long long>(lcap + 1);
+        a.stack = ar.get<int>((size_t)stack_warps * (T.depth + 4));
+        batch = ar.get<EdgeK>(caps.edges);
+        filt = ar.get<EdgeK>(caps.edges);
+        tmp = ar.get<EdgeK>(caps.edges);
+        split_hist = ar.get<int>(kSplitBins);
+        split_max = ar.get<unsigned long long>(1);
+        comp_scratch = ar.get<int>(2LL * n + 1);
+        for (int i = 0; i < 2; ++i) nodes[i] = ar.get<int>(T.N / 2 + 1);
+        a.frontier_cap = (int)fcap;
+    } else {
+        tmp = ar.get<EdgeK>(n);   // the final sort's second buffer
+    }
+    if (ar.failed) return WM_ENOMEM;
+    for (int c = 0; c < 5; ++c) { a.list[c] = lists[c]; a.list_lb[c] = list_lbs[c]; a.list_cap[c] = (int)lcap; }
+    a.list_count = lcount;
+    a.big = lists[3]; a.big_count = lcount + 3;
+    a.stack_cap = T.depth + 4;
+    a.edges = batch; a.edge_count = ecount;
+    a.edge_cap = (int)(caps.edges_soft > 0 && caps.edges_soft < caps.edges ? caps.edges_soft : caps.edges);
+    a.rho_bits = rho;
+    EdgeK *spare = filt;   // second edge buffer for compaction when rho_hi shrinks
+    a.node_in = nullptr;
+    a.node_in_n = nullptr;
+    a.node_out = nodes[0];
+    a.node_out_n = cnts + 10;
     double rho_lo = 0.0;
     long long beta = 2;
     // tuning combined = 2: rounds start as two passes; once, after two rounds or more, the GetRho
@@ -580,7 +646,6 @@ static int memogfk(Call &C, Points &P, Tree &T, const HdbState *hdb, const Caps 
     constexpr double kOnePassRatio = 0.5;
     bool adaptive_one_pass = false;
     const double inf = INFINITY;
-    int rounds = 0;
     while (nE < target) {
         if (++rounds > 4096) { set_detail("MemoGFK made no progress%s (%lld rounds)", "", rounds); return WM_EINTERNAL; }
         Timer tw;
@@ -917,6 +982,7 @@ static int gfk_rounds(Call &C, Points &P, Tree &T, const HdbState *hdb, const Ca
     a.x32 = P.x32; a.x4 = x4; a.x64 = P.x64; a.pid = P.pid;
     a.fp64 = C.precision == WM_PREC_FP64;
     a.eta = a.fp64 ? 0.0 : 2.0 * (double)P.delta * std::sqrt((double)P.d) * (1.0 + 1e-6);
+    a.eta2_f = float_ru(2.0 * a.eta);
     a.exact32 = a.eta == 0.0;
     a.delta32 = P.delta;
     a.dfs_budget = C.tune.dfs_budget;
@@ -1159,7 +1225,7 @@ static int run_call(const wm_opts *opts, long long n, int d, int min_pts, Body b
     Caps caps = caps_for(n, d, min_pts);
     caps.extra_bytes = extra_bytes;
     if (C.method == WM_METHOD_GFK || C.method == WM_METHOD_NAIVE) caps.wspd_pairs = wspd_pairs_guess(n, d);
-    C.tune = tuning_for(n, d, min_pts);
+    C.tune = tuning_for(n, d, min_pts, &C.tune_override);
     const bool user_ws = opts && opts->workspace;
     int rc = 0;
     unsigned ovf_seen = 0;   // capacities that overflowed in earlier attempts
@@ -1922,7 +1988,7 @@ extern "C" int wm_emst_noalloc(const void *pts, int64_t n, int32_t d, int32_t dt
     C.precision = precision;
     C.timing = false;
     C.pin = g_noalloc_host;
-    C.tune = tuning_for(n, d, 0);
+    C.tune = tuning_for(n, d, 0, &C.tune_override);
     C.ar.base = (char *)nd.scratch;
     C.ar.cap = WM_NOALLOC_SCRATCH_BYTES;
     // Capacities sized for WM_NOALLOC_MAX_POINTS: traversal chunks of 4096 pairs and edge batches of

@@ -1,0 +1,40 @@
+// boruvka.cuh -- the nearest-component rounds (boruvka.cu).
+#pragma once
+
+#include <cmath>
+
+#include "wspd.cuh"
+
+namespace wm {
+
+struct NcCall {
+    cudaStream_t st = nullptr;
+    Arena *ar = nullptr;
+    int *pin = nullptr;             // pinned host scratch
+    int depth = 0;                  // tree levels
+    const Tree *T = nullptr;
+    const int *pos = nullptr;       // input id -> tree position
+    int *uf = nullptr;              // union-find over input ids, left flat on return
+    EdgeK *out = nullptr;           // tree edges, in no particular order
+    long long target = 0;           // edges to find
+    double cap = INFINITY;          // no edge at or above this weight is taken (batches)
+    float cap_f = INFINITY;         // the smallest float >= cap
+    const EdgeK *rep = nullptr;     // HDBSCAN*: the complete list of edges with D <= max(cd2, cd2)
+    int nrep = 0;
+    EdgeK *rep_tmp0 = nullptr, *rep_tmp1 = nullptr;
+    int *E = nullptr;
+    // results
+    long long done = 0;             // tree edges found (< target: the caller finishes the forest)
+    int rounds = 0;
+    long long candidates = 0;
+    // timing hooks around the search kernel
+    void *ctx = nullptr;
+    int (*mark)(void *ctx) = nullptr;
+    void (*span)(void *ctx, int from, int to) = nullptr;
+};
+
+// Boruvka rounds on the tree packed in a.rec / a.box / a.x4.  Returns 0 or an error code; C.done tells
+// how far the forest got.
+int nearest_component_rounds(NcCall &C, TravArgs &a);
+
+}  // namespace wm

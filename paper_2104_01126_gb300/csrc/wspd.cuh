@@ -19,6 +19,7 @@ struct TravArgs {
     const float *cd32 = nullptr;                       // HDBSCAN* cd2 per tree position
     const double *cd64 = nullptr;
     double eta = 0.0;          // absolute distance error of the FP32 copy (FP64 input), else 0
+    float eta2_f = 0.f;        // the smallest float >= 2 eta
     float delta32 = 0.f;       // largest |x64 - x32| of a coordinate (0 for FP32 input)
     int exact32 = 1;           // eta == 0: the FP32 copy is exact
     int fp64 = 0;              // plain FP64 form
