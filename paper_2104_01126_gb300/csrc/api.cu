@@ -460,7 +460,7 @@ static bool nearest_rounds_apply(const Call &C, int n, int d, const HdbState *hd
 // `target` when the points form several instances that must not be joined (a batch): then every
 // edge weight is below rho_cap, rho_hi never exceeds it, and no pair at or above it is retrieved.
 // hdb: optional HDBSCAN* state (node cd bounds, per-position cd2, repair edges).
-static int memogfk(Call &C, Points &P, Tree &T, const HdbState *hdb, const Caps &caps, EdgeK *E_out, int *uf,
+static int memogfk(Call &C, Points &P, Tree &T, SearchTree &X, const HdbState *hdb, const Caps &caps, EdgeK *E_out, int *uf,
                    unsigned long long *R, unsigned *overflow_bits, long long target = -1, double rho_cap = INFINITY)
 {
     const int n = P.n;
@@ -499,9 +499,7 @@ static int memogfk(Call &C, Points &P, Tree &T, const HdbState *hdb, const Caps 
     a.big_max = C.tune.big_max;
     a.disjunctive = C.disjunctive;
     a.rho_sample = C.tune.getrho_sample > 0 ? C.tune.getrho_sample : 1;
-    if (hdb) {
-        a.cdmin = hdb->cdmin; a.cdmax = hdb->cdmax; a.cd32 = hdb->cd32; a.cd64 = hdb->cd64;
-    }
+    if (hdb) { a.cd32 = hdb->cd32; a.cd64 = hdb->cd64; }
     a.dp = dp;
     a.overflow = ovf;
     a.stat = stat;
@@ -549,6 +547,8 @@ static int memogfk(Call &C, Points &P, Tree &T, const HdbState *hdb, const Caps 
     int nE = 0, rounds = 0;
     if (nearest_rounds_apply(C, n, P.d, hdb)) {
         Timer tn;
+        const size_t xmark = ar.off;
+        if (!X.rows) WM_TRY(build_search_tree(P, T, X, ar, st, C.pin));
         struct Hooks {
             std::function<int()> mark;
             std::function<void(int, int)> span;
@@ -557,8 +557,7 @@ static int memogfk(Call &C, Points &P, Tree &T, const HdbState *hdb, const Caps 
         N.st = st;
         N.ar = &ar;
         N.pin = C.pin;
-        N.depth = T.depth;
-        N.T = &T;
+        N.X = &X;
         N.pos = P.pos;
         N.uf = uf;
         N.out = E_out;
@@ -576,6 +575,8 @@ static int memogfk(Call &C, Points &P, Tree &T, const HdbState *hdb, const Caps 
         rounds = N.rounds;
         C.stats.candidate_edges += N.candidates;
         C.stats.ms_bccp += tn.ms();
+        ar.off = xmark;
+        X.rows = nullptr;   // its memory is released, or its labels are used up
     }
     // ---- MemoGFK state
     const int chunk = (int)caps.chunk;
@@ -591,7 +592,14 @@ static int memogfk(Call &C, Points &P, Tree &T, const HdbState *hdb, const Caps 
     NodeRec *rec = nullptr;
     if (nE < target) {
         Tree T2 = T;
-        if (hdb) { T2.cdmin = hdb->cdmin; T2.cdmax = hdb->cdmax; }
+        if (hdb) {
+            T2.cdmin = ar.get<float>(T.N);
+            T2.cdmax = ar.get<float>(T.N);
+            if (ar.failed) return WM_ENOMEM;
+            WM_TRY(node_core_bounds(T, *hdb, T2.cdmin, T2.cdmax, ar, st));
+            a.cdmin = T2.cdmin;
+            a.cdmax = T2.cdmax;
+        }
         rec = ar.get<NodeRec>(T.N);
         float *box = ar.get<float>((size_t)T.N * 2 * dp);
         float4 *x4 = ar.get<float4>((size_t)n * (dp / 4));
@@ -966,12 +974,15 @@ static int gfk_rounds(Call &C, Points &P, Tree &T, const HdbState *hdb, const Ca
     // counters: [2..6] class-list counts, [7] pool count, [8] kept pairs, [9] batch count,
     // [10..11] node lists, [12..13] huge items, [16..17] tile dispensers, [32..] traversal state
     int *lcount = cnts + 2, *pcount = cnts + 7, *kcount = cnts + 8, *bcount = cnts + 9, *tcnt = cnts + 32;
-    {
-        Tree T2 = T;
-        if (hdb) { T2.cdmin = hdb->cdmin; T2.cdmax = hdb->cdmax; }
-        pack_nodes(T2, P.d, dp, rec, box, st);
-        point_major(P.x32, n, P.d, dp, x4, st);
+    Tree T2 = T;
+    if (hdb) {
+        T2.cdmin = ar.get<float>(T.N);
+        T2.cdmax = ar.get<float>(T.N);
+        if (ar.failed) return WM_ENOMEM;
+        WM_TRY(node_core_bounds(T, *hdb, T2.cdmin, T2.cdmax, ar, st));
     }
+    pack_nodes(T2, P.d, dp, rec, box, st);
+    point_major(P.x32, n, P.d, dp, x4, st);
     WM_CK(cudaMemsetAsync(stat, 0, 16 * sizeof(unsigned long long), st));
     WM_CK(cudaMemsetAsync(ovf, 0, 2 * sizeof(unsigned), st));
     WM_CK(cudaMemsetAsync(cnts, 0, 64 * sizeof(int), st));
@@ -990,7 +1001,7 @@ static int gfk_rounds(Call &C, Points &P, Tree &T, const HdbState *hdb, const Ca
     a.big_max = C.tune.big_max;
     a.disjunctive = C.disjunctive;
     a.rho_sample = C.tune.getrho_sample > 0 ? C.tune.getrho_sample : 1;
-    if (hdb) { a.cdmin = hdb->cdmin; a.cdmax = hdb->cdmax; a.cd32 = hdb->cd32; a.cd64 = hdb->cd64; }
+    if (hdb) { a.cdmin = T2.cdmin; a.cdmax = T2.cdmax; a.cd32 = hdb->cd32; a.cd64 = hdb->cd64; }
     a.frontier_cap = (int)fcap;
     a.rec = rec; a.box = box; a.dp = dp;
     a.list_count = lcount;
@@ -1137,6 +1148,7 @@ static int gfk_rounds(Call &C, Points &P, Tree &T, const HdbState *hdb, const Ca
 struct Prepared {
     Points P;
     Tree T;
+    SearchTree X;   // built where the FP32-screened walks need it (rows is null otherwise)
 };
 
 static int prepare(Call &C, const void *pts, int64_t n, int32_t d, int32_t dtype, int32_t layout, Prepared &S)
@@ -1161,6 +1173,13 @@ static int prepare(Call &C, const void *pts, int64_t n, int32_t d, int32_t dtype
     C.stats.tree_nodes = S.T.N;
     C.stats.tree_depth = S.T.depth;
     return 0;
+}
+
+// the k-NN pass of the FP32 screen walks the search tree (positions of 28 bits)
+static int search_tree_for_knn(Call &C, Prepared &S)
+{
+    if (C.precision == WM_PREC_FP64 || S.P.n >= 1 << 28) return 0;
+    return build_search_tree(S.P, S.T, S.X, C.ar, C.st, C.pin);
 }
 
 static int write_edges(Call &C, const EdgeK *E, int m, wm_edge *out, double *total)
@@ -1325,7 +1344,7 @@ static int emst_body(Call &C, void *vctx, const Caps &caps, unsigned *ovf)
     if (C.method == WM_METHOD_GFK || C.method == WM_METHOD_NAIVE)
         WM_TRY(gfk_rounds(C, S.P, S.T, nullptr, caps, E, uf, R, ovf, C.method == WM_METHOD_NAIVE));
     else
-        WM_TRY(memogfk(C, S.P, S.T, nullptr, caps, E, uf, R, ovf));
+        WM_TRY(memogfk(C, S.P, S.T, S.X, nullptr, caps, E, uf, R, ovf));
     if (*ovf) return 0;
     return write_edges(C, E, n - 1, x.out, x.total);
 }
@@ -1349,7 +1368,8 @@ static int hdbscan_body(Call &C, void *vctx, const Caps &caps, unsigned *ovf)
     const int n = (int)x.n;
     HdbState H;
     Timer tc;
-    WM_TRY(core_distances(S.P, S.T, x.min_pts, C.precision == WM_PREC_FP64, H, C.ar, C.st, C.pin, &C.stats));
+    WM_TRY(search_tree_for_knn(C, S));
+    WM_TRY(core_distances(S.P, S.T, &S.X, x.min_pts, C.precision == WM_PREC_FP64, H, C.ar, C.st, C.pin, &C.stats));
     C.stats.ms_core_dist = tc.ms();
     int *uf = C.ar.get<int>(n);
     unsigned long long *R = C.ar.get<unsigned long long>(4LL * n);
@@ -1359,7 +1379,7 @@ static int hdbscan_body(Call &C, void *vctx, const Caps &caps, unsigned *ovf)
     if (C.method == WM_METHOD_GFK || C.method == WM_METHOD_NAIVE)
         WM_TRY(gfk_rounds(C, S.P, S.T, &H, caps, E, uf, R, ovf, C.method == WM_METHOD_NAIVE));
     else
-        WM_TRY(memogfk(C, S.P, S.T, &H, caps, E, uf, R, ovf));
+        WM_TRY(memogfk(C, S.P, S.T, S.X, &H, caps, E, uf, R, ovf));
     if (*ovf) return 0;
     WM_TRY(write_core_distances(S.P, H, x.cd, C.ar, C.st));
     WM_TRY(write_edges(C, E, n - 1, x.mst, nullptr));
@@ -1525,7 +1545,8 @@ static int batch_body(Call &C, void *vctx, const Caps &caps, unsigned *ovf)
     HdbState H;
     if (hdb) {
         Timer tc;
-        WM_TRY(core_distances(S.P, S.T, x.min_pts, C.precision == WM_PREC_FP64, H, ar, st, C.pin, &C.stats));
+        WM_TRY(search_tree_for_knn(C, S));
+        WM_TRY(core_distances(S.P, S.T, &S.X, x.min_pts, C.precision == WM_PREC_FP64, H, ar, st, C.pin, &C.stats));
         C.stats.ms_core_dist = tc.ms();
     }
     int *uf = ar.get<int>(n);
@@ -1533,7 +1554,7 @@ static int batch_body(Call &C, void *vctx, const Caps &caps, unsigned *ovf)
     EdgeK *E = ar.get<EdgeK>(n);
     if (ar.failed) return WM_ENOMEM;
     launch(init_uf_kernel, grid_for(n, 256), 256, 0, st, uf, R, n);
-    WM_TRY(memogfk(C, S.P, S.T, hdb ? &H : nullptr, caps, E, uf, R, ovf, m, L * L / 4));
+    WM_TRY(memogfk(C, S.P, S.T, S.X, hdb ? &H : nullptr, caps, E, uf, R, ovf, m, L * L / 4));
     if (*ovf) return 0;
     // ---- tree edges grouped by instance, K order inside each
     EdgeK *keys = ar.get<EdgeK>(m + 1), *ktmp = ar.get<EdgeK>(m + 1);

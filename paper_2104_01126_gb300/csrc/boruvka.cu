@@ -33,25 +33,25 @@
 
 #include "boruvka.cuh"
 #include "screen.cuh"
+#include "stree.cuh"
 #include "wspd.cuh"
 
 namespace wm {
 
 namespace {
 
-constexpr int kNcK = 4;         // list entries per point
-constexpr int kNcBucket = 8;    // a subtree of at most this many points is scanned directly
-constexpr int kNcThreads = 128; // threads per block of the search
-constexpr int kNcStack = 16;    // stack entries of a thread in shared memory (the rest in global memory)
-constexpr unsigned kBucketBit = 0x80000000u, kDone = 0xffffffffu;
+// List entries per point, by dimension.  A longer list serves more rounds, a shorter one has the smaller
+// radius to search first: at 10^7 points 4 -> 6 entries took the search from 9.3 to 7.7 ms in 3-D and
+// from 8.0 to 7.7 in 2-D, left it in 5-D (31 ms) and cost 13 % in 7-D; 2 entries were slower everywhere.
+__host__ __device__ constexpr int list_len(int D) { return D <= 3 ? 6 : 4; }
 
 struct NcArgs {
     int *lab;                  // component of a tree position (a tree position: the root)
     int *par;                  // links between roots
     unsigned *S;               // per root: smallest screened weight seen this round (float bits)
     unsigned long long *bhi, *blo;   // per root: K-minimum outgoing edge
-    float *ls;                 // [kNcK][n] list weights, ascending
-    int *lj;                   // [kNcK][n] list positions (-1: none)
+    float *ls;                 // [list_len][n] list weights, ascending
+    int *lj;                   // [list_len][n] list positions (-1: none)
     float *R;                  // every point outside the component and the list screens at >= R
     unsigned char *hd;         // first list entry that may lie outside the component
     int *act, *amb;            // active points; points that need the exact scan
@@ -59,43 +59,14 @@ struct NcArgs {
     int *cand_c;
     int *cnt;                  // [0] active, [1] search dispenser, [2] candidates, [3] exact scans,
                                // [4] their dispenser, [5] tree edges, [6] repair edges left
+    int K;                     // list_len
     const int *pos;            // input id -> tree position
     unsigned cap_bits;         // no edge at or above this weight (float bits; +inf: none)
     unsigned long long cap64;  // the same in FP64 bits
-    const float4 *rows;        // point rows: coordinates, label in the last slot
-    const float4 *nodes;       // search tree rows
-    const int2 *range;         // their point ranges
-    const float *ncd;          // HDBSCAN*: their smallest core distance (rounded down)
-    unsigned root;             // reference of the root
-    int Ns;                    // nodes of the search tree
-    uint2 *deep;               // stack entries beyond kNcStack, [stack_cap - kNcStack][threads]
+    float *rows;               // the search tree's point rows
+    const float *ncd;          // HDBSCAN*: smallest core distance of a node (rounded down)
     int first;                 // first search: components are single points, nothing is pruned by S
-    int stack_cap;
 };
-
-__device__ __forceinline__ float next_up(float x) { return x < INFINITY ? __uint_as_float(__float_as_uint(x) + 1u) : x; }
-
-// one point of the point-major copy into registers (rows of 4, 8 or 16 floats)
-template <int S>
-__device__ __forceinline__ void load_row(const float4 *__restrict__ x4, int i, float (&v)[S])
-{
-    if (S == 4) {
-        const float4 p = x4[i];
-        v[0] = p.x; v[1] = p.y; v[2] = p.z; v[3] = p.w;
-    } else {
-#pragma unroll
-        for (int c = 0; c < S / 8; ++c) {
-            float4 p, q;
-            ldg256((const float *)x4 + (size_t)i * S + 8 * c, p, q);
-            v[8 * c] = p.x; v[8 * c + 1] = p.y; v[8 * c + 2] = p.z; v[8 * c + 3] = p.w;
-            v[8 * c + 4] = q.x; v[8 * c + 5] = q.y; v[8 * c + 6] = q.z; v[8 * c + 7] = q.w;
-        }
-    }
-}
-
-// floats per point row: the coordinates and, in the last slot, the component label
-template <int D>
-__device__ __host__ __forceinline__ constexpr int row_floats() { return D <= 3 ? 4 : D <= 7 ? 8 : D <= 15 ? 16 : 24; }
 
 // HDBSCAN*: true when the FP32 squared distance d32 proves D <= c for a core distance c (FP32 copy)
 __device__ inline bool proven_repair(const TravArgs &a, float d32, float c)
@@ -112,185 +83,135 @@ __device__ inline void note_err(float s, double w, float &err)
 }
 
 // ---------------------------------------------------------------------------------- search
-// The search tree: the nodes of the k-d tree down to the subtrees of at most kNcBucket points, siblings
-// adjacent.  A node row holds its box in groups of four dimensions (lo then hi, as the traversals'
-// packed boxes) and, in the last padded dimension, a reference (lo slot) and the component label or -1
-// (hi slot).  A reference is the row of the left child, or for a bucket
-// kBucketBit | (size - 1) << 28 | first point.
-//
+// A thread per query on the search tree (stree.cuh).
 // EXACT = false rebuilds the lists of the active points.  EXACT = true answers the points whose list may
 // have dropped a tie: every point within T(S[c]) is evaluated in FP64 and the K-minimum becomes the
 // point's candidate edge.
 template <int D, bool HDB, bool EXACT>
-__global__ void __launch_bounds__(kNcThreads) nc_search_kernel(TravArgs a, NcArgs b, int m_all)
+__global__ void __launch_bounds__(kWalkThreads) nc_search_kernel(TravArgs a, NcArgs b, SearchTree X, int m_all)
 {
-    __shared__ uint2 sst[kNcStack][kNcThreads];
-    constexpr int S = row_floats<D>(), G = S / 4, K = kNcK;
+    __shared__ uint2 sst[kWalkStack][kWalkThreads];
+    constexpr int S = row_floats(D), K = list_len(D);
+    constexpr bool kStream = S > 4 && !HDB;
     const int lane = threadIdx.x & 31;
     const int n = a.n;
     const int m = EXACT ? b.cnt[3] : b.first ? m_all : b.cnt[0];
-    const size_t nthr = (size_t)gridDim.x * kNcThreads;
-    uint2 *deep = b.deep + (size_t)blockIdx.x * kNcThreads + threadIdx.x;
     unsigned long long n_ev = 0, n_re = 0;
     float err = 0.f;
-    while (true) {
-        int base = 0;
-        if (lane == 0) base = atomicAdd(b.cnt + (EXACT ? 4 : 1), 32);
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (base >= m) break;
-        const bool valid = base + lane < m;
-        const int t = valid ? base + lane : base;
-        const int i = EXACT ? b.amb[t] : b.first ? t : b.act[t];
-        float q[S];
-        load_row<S>(b.rows, i, q);
-        const int c = b.lab[i];
-        const float qcd = HDB ? a.cd32[i] : 0.f;
-        const float qcd_lo = HDB ? qcd * (1.0f - 1.0f / 4194304.0f) : 0.f;
-        float Sc = __uint_as_float(*(volatile unsigned *)(b.S + c));
-        float sl[K];
-        int sj[K];
+    // the lane's query
+    float q[S];
+    int i = 0, c = 0;
+    float qcd = 0.f, qcd_lo = 0.f, Sc = 0.f;
+    float sl[K];
+    int sj[K];
+    KMin best{~0ull, ~0ull};
+    float lim = 0.f, pb = 0.f;   // a candidate screens below lim; a node is skipped when its lower bound
+                                 // exceeds pb (it bounds the exact weight, within 2^-19 of the screened one)
+    unsigned ev = 0;
+    auto begin = [&](int t) {
+        i = EXACT ? b.amb[t] : b.first ? t : b.act[t];
+        load_row<S>(X.rows, i, q);
+        c = b.lab[i];
+        if (HDB) {
+            qcd = a.cd32[i];
+            qcd_lo = qcd * (1.0f - 1.0f / 4194304.0f);
+        }
+        Sc = __uint_as_float(*(volatile unsigned *)(b.S + c));
 #pragma unroll
         for (int k = 0; k < K; ++k) { sl[k] = INFINITY; sj[k] = -1; }
-        KMin best{~0ull, ~0ull};
-        // a candidate screens below lim; a node is skipped when its lower bound exceeds pb (the
-        // bound is on the exact weight, which is within 2^-19 of the screened one)
-        float lim = next_up(screen_threshold(Sc, a));
-        float pb = lim * (1.0f + 1.0f / 131072.0f);
-        int sp = 0, since = 0;
-        unsigned cur = valid ? b.root : kDone;
-        unsigned ev = 0;
-        for (unsigned guard = 0; guard < 2u * (unsigned)a.N + 2u; ++guard) {
-            // ---- down to the next bucket within the bound
-            while (!(cur & kBucketBit)) {
-                const float *bx = (const float *)b.nodes + (size_t)cur * 2 * S;
-                float g0 = 0.f, g1 = 0.f;
-                unsigned r0 = 0, r1 = 0;
-                int l0 = 0, l1 = 0;
+        best = KMin{~0ull, ~0ull};
+        lim = next_up(screen_threshold(Sc, a));
+        pb = lim * (1.0f + 1.0f / 131072.0f);
+        ev = 0;
+    };
+    auto bound = [&](unsigned node, float &g0, float &g1) {
+        if (HDB) {
+            g0 = fmaxf(g0, fmaxf(qcd_lo, b.ncd[node]));
+            g1 = fmaxf(g1, fmaxf(qcd_lo, b.ncd[node + 1]));
+        }
+    };
+    auto need = [&](float g, int l) { return g <= pb && l != c; };
+    auto pending = [&](float g) { return g <= pb; };
+    auto scan = [&](int j0, int sz) {
+        // screened values first, then the ones below the limit one by one: few lanes have any, and
+        // they run their insertions together
+        float w[kBucket];
+        unsigned todo = 0;
 #pragma unroll
-                for (int g = 0; g < G; ++g) {
-                    float4 lo0, hi0, lo1, hi1;
-                    ldg256(bx + 8 * g, lo0, hi0);
-                    ldg256(bx + 2 * S + 8 * g, lo1, hi1);
-                    const float a0[4] = {lo0.x, lo0.y, lo0.z, lo0.w}, z0[4] = {hi0.x, hi0.y, hi0.z, hi0.w};
-                    const float a1[4] = {lo1.x, lo1.y, lo1.z, lo1.w}, z1[4] = {hi1.x, hi1.y, hi1.z, hi1.w};
+        for (int h = 0; h < kBucket; h += 4) {
+            if (h && h >= sz) break;
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        if (4 * g + k < D) {
-                            const float u = fmaxf(fmaxf(a0[k] - q[4 * g + k], q[4 * g + k] - z0[k]), 0.f);
-                            const float v = fmaxf(fmaxf(a1[k] - q[4 * g + k], q[4 * g + k] - z1[k]), 0.f);
-                            g0 = fmaf(u, u, g0);
-                            g1 = fmaf(v, v, g1);
-                        }
-                    }
-                    if (g == G - 1) {
-                        r0 = __float_as_uint(lo0.w);
-                        r1 = __float_as_uint(lo1.w);
-                        l0 = __float_as_int(hi0.w);
-                        l1 = __float_as_int(hi1.w);
-                    }
-                }
-                g0 = lower_w2(g0);
-                g1 = lower_w2(g1);
-                if (HDB) {
-                    g0 = fmaxf(g0, fmaxf(qcd_lo, b.ncd[cur]));
-                    g1 = fmaxf(g1, fmaxf(qcd_lo, b.ncd[cur + 1]));
-                }
-                const bool n0 = g0 <= pb && l0 != c, n1 = g1 <= pb && l1 != c;
-                if (n0 && n1) {
-                    const bool sw = g1 < g0;
-                    const uint2 far = sw ? make_uint2(r0, __float_as_uint(g0)) : make_uint2(r1, __float_as_uint(g1));
-                    if (sp < kNcStack) sst[sp][threadIdx.x] = far;
-                    else if (sp < b.stack_cap) deep[(size_t)(sp - kNcStack) * nthr] = far;
-                    else { atomicOr(a.overflow, 8u); cur = kDone; break; }   // cannot happen: one entry per level
-                    ++sp;
-                    cur = sw ? r1 : r0;
-                } else if (n0 || n1) {
-                    cur = n0 ? r0 : r1;
-                } else {
-                    cur = kDone;
-                    while (sp > 0) {
-                        --sp;
-                        const uint2 e = sp < kNcStack ? sst[sp][threadIdx.x] : deep[(size_t)(sp - kNcStack) * nthr];
-                        if (__uint_as_float(e.y) <= pb) { cur = e.x; break; }
-                    }
-                }
-            }
-            if (cur == kDone) break;
-            // ---- scan the bucket
-            const int j0 = (int)(cur & 0x0fffffffu), sz = (int)((cur >> 28) & 7u) + 1;
-            const float was = sl[0];
-            for (int p = 0; p < sz; ++p) {
+            for (int p = h; p < h + 4; ++p) {
+                const int j = j0 + min(p, sz - 1);
                 float x[S];
-                load_row<S>(b.rows, j0 + p, x);
-                float s = 0.f;
-#pragma unroll
-                for (int k = 0; k < D; ++k) {
-                    const float dx = q[k] - x[k];
-                    s = fmaf(dx, dx, s);
-                }
-                float w = s, cdm = 0.f;
+                load_row<S, kStream>(X.rows, j, x);
+                const float s = row_dist<D>(q, x);
+                bool take = p < sz && __float_as_int(x[S - 1]) != c;
+                w[p] = s;
                 if (HDB) {
-                    cdm = fmaxf(qcd, a.cd32[j0 + p]);
-                    w = fmaxf(s, cdm);
+                    const float cdm = fmaxf(qcd, a.cd32[j]);
+                    w[p] = fmaxf(s, cdm);
+                    take = take && w[p] < lim && !proven_repair(a, s, cdm);
                 }
-                if (w < lim && __float_as_int(x[S - 1]) != c && (!HDB || !proven_repair(a, s, cdm))) {
-                    if (EXACT) {
-                        const int j = j0 + p;
-                        double x2 = dist64(a.x64, n, a.d, i, j);
-                        if (HDB) x2 = pos_dmax(x2, pos_dmax(a.cd64[i], a.cd64[j]));
-                        note_err(w, x2, err);
-                        kmin_update(best, x2, a.pid[i], a.pid[j]);
-                        ++n_re;
-                        continue;
-                    }
+                if (take && w[p] < lim) todo |= 1u << p;
+            }
+        }
+        ev += (unsigned)sz;
+        const float was = sl[0];
+        while (todo) {
+            const int p = __ffs(todo) - 1;
+            todo &= todo - 1;
+            float v = w[0];
 #pragma unroll
-                    for (int k = K - 1; k >= 0; --k) {
-                        if (k > 0 && w < sl[k - 1]) {
-                            sl[k] = sl[k - 1];
-                            sj[k] = sj[k - 1];
-                        } else if (w < sl[k]) {
-                            sl[k] = w;
-                            sj[k] = j0 + p;
-                        }
+            for (int r = 1; r < kBucket; ++r) v = r == p ? w[r] : v;
+            if (EXACT) {
+                const int j = j0 + p;
+                double x2 = dist64(a.x64, n, a.d, i, j);
+                if (HDB) x2 = pos_dmax(x2, pos_dmax(a.cd64[i], a.cd64[j]));
+                note_err(v, x2, err);
+                kmin_update(best, x2, a.pid[i], a.pid[j]);
+                ++n_re;
+            } else if (v < lim) {
+#pragma unroll
+                for (int k = K - 1; k >= 0; --k) {
+                    if (k > 0 && v < sl[k - 1]) {
+                        sl[k] = sl[k - 1];
+                        sj[k] = sj[k - 1];
+                    } else if (v < sl[k]) {
+                        sl[k] = v;
+                        sj[k] = j0 + p;
                     }
-                    lim = fminf(lim, sl[K - 1]);
                 }
+                lim = fminf(lim, sl[K - 1]);
             }
-            ev += (unsigned)sz;
-            if (!EXACT && !b.first) {
-                // the component's minimum: lowered by this point, else re-read now and then
-                ++since;
-                float now = Sc;
-                if (sl[0] < was && sl[0] < Sc)
-                    now = fminf(sl[0], __uint_as_float(atomicMin(b.S + c, __float_as_uint(sl[0]))));
-                else if ((since & 3) == 0)
-                    now = __uint_as_float(*(volatile unsigned *)(b.S + c));
-                if (now < Sc) {
-                    Sc = now;
-                    lim = fminf(lim, next_up(screen_threshold(Sc, a)));
-                }
-            }
-            pb = lim * (1.0f + 1.0f / 131072.0f);
-            // ---- next pending node within the bound
-            cur = kDone;
-            while (sp > 0) {
-                --sp;
-                const uint2 e = sp < kNcStack ? sst[sp][threadIdx.x] : deep[(size_t)(sp - kNcStack) * nthr];
-                if (__uint_as_float(e.y) <= pb) { cur = e.x; break; }
-            }
-            if (cur == kDone) break;
         }
+        if (!EXACT && !b.first) {
+            // the component's minimum: lowered by this point, else re-read
+            float now = Sc;
+            if (sl[0] < was && sl[0] < Sc)
+                now = fminf(sl[0], __uint_as_float(atomicMin(b.S + c, __float_as_uint(sl[0]))));
+            else if ((ev & 31u) < 8u)   // now and then
+                now = __uint_as_float(*(volatile unsigned *)(b.S + c));
+            if (now < Sc) {
+                Sc = now;
+                lim = fminf(lim, next_up(screen_threshold(Sc, a)));
+            }
+        }
+        pb = lim * (1.0f + 1.0f / 131072.0f);
+    };
+    auto finish = [&] {
         n_ev += ev;
-        if (EXACT && valid && best.hi < b.cap64) {
-            const int slot = atomicAdd(b.cnt + 2, 1);   // at most one candidate per point: within n
-            EdgeK e;
-            e.hi = best.hi;
-            e.lo = best.lo;
-            b.cand[slot] = e;
-            b.cand_c[slot] = c;
-            if (best.hi < *(volatile unsigned long long *)(b.bhi + c)) atomicMin(b.bhi + c, best.hi);
-        }
-        if (!EXACT && valid) {
+        if (EXACT) {
+            if (best.hi < b.cap64) {
+                const int slot = atomicAdd(b.cnt + 2, 1);   // at most one candidate per point: within n
+                EdgeK e;
+                e.hi = best.hi;
+                e.lo = best.lo;
+                b.cand[slot] = e;
+                b.cand_c[slot] = c;
+                if (best.hi < *(volatile unsigned long long *)(b.bhi + c)) atomicMin(b.bhi + c, best.hi);
+            }
+        } else {
 #pragma unroll
             for (int k = 0; k < K; ++k) {
                 b.ls[(size_t)k * n + i] = sl[k];
@@ -299,8 +220,11 @@ __global__ void __launch_bounds__(kNcThreads) nc_search_kernel(TravArgs a, NcArg
             b.R[i] = lim;
             b.hd[i] = 0;
         }
-        __syncwarp();
-    }
+    };
+    walk_queries<D, S, kStream>(X, m, b.cnt + (EXACT ? 4 : 1), &sst[0][threadIdx.x], kWalkThreads,
+                                X.deep + (size_t)blockIdx.x * kWalkThreads + threadIdx.x,
+                                (size_t)gridDim.x * kWalkThreads, (int *)a.overflow, 8, q, begin, bound, need, pending,
+                                scan, finish);
     n_ev = warp_sum_u64(n_ev);
     if (lane == 0 && n_ev) {
         atomicAdd(a.stat + 1, n_ev);
@@ -313,53 +237,29 @@ __global__ void __launch_bounds__(kNcThreads) nc_search_kernel(TravArgs a, NcArg
     }
 }
 
-// ---------------------------------------------------------------------------- search tree
-// flag of the nodes the search tree keeps: the root and every child of a node above kNcBucket points
-__global__ void nc_flag_kernel(int N, const int *__restrict__ begin, const int *__restrict__ end,
-                               const int *__restrict__ parent, int *__restrict__ flag)
+// HDBSCAN*: smallest core distance (rounded down) of every search tree node: buckets from their
+// points, the rest bottom-up, the second child to arrive composing the parent
+__global__ void nc_core_min_kernel(int Ns, const int2 *__restrict__ range, const int *__restrict__ parent,
+                                   const double *__restrict__ cd64, float *ncd, int *arrive)
 {
-    for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < N; x += gridDim.x * blockDim.x) {
-        const int p = parent[x];
-        flag[x] = p < 0 || end[p] - begin[p] > kNcBucket;
-    }
-}
-
-// rows of the kept nodes (idx: exclusive prefix of the flags)
-template <int S>
-__global__ void nc_nodes_kernel(int N, int d, const int *__restrict__ begin, const int *__restrict__ end,
-                                const int *__restrict__ left, const int *__restrict__ parent,
-                                const float *__restrict__ lo, const float *__restrict__ hi,
-                                const float *__restrict__ cdmin, const int *__restrict__ idx, float *__restrict__ rows,
-                                int2 *__restrict__ range, float *__restrict__ ncd)
-{
-    for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < N; x += gridDim.x * blockDim.x) {
-        const int p = parent[x];
-        if (p >= 0 && end[p] - begin[p] <= kNcBucket) continue;
-        const int t = idx[x], bb = begin[x], sz = end[x] - bb;
-        float *r = rows + (size_t)t * 2 * S;
-        const unsigned ref = sz > kNcBucket ? (unsigned)idx[left[x]] : kBucketBit | (unsigned)(sz - 1) << 28 | (unsigned)bb;
-#pragma unroll
-        for (int k = 0; k < S; ++k) {
-            r[box_lo(k)] = k < d ? lo[(size_t)k * N + x] : k == S - 1 ? __uint_as_float(ref) : 0.f;
-            r[box_hi(k)] = k < d ? hi[(size_t)k * N + x] : k == S - 1 ? __int_as_float(-1) : 0.f;
-        }
-        range[t] = make_int2(bb, bb + sz);
-        if (ncd) ncd[t] = cdmin[x];
-    }
-}
-
-template <int S>
-__global__ void nc_rows_kernel(int n, int d, const float *__restrict__ x32, float *__restrict__ rows)
-{
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        float4 *r = (float4 *)(rows + (size_t)i * S);
-#pragma unroll
-        for (int c = 0; c < S / 4; ++c) {
-            float v[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                v[k] = 4 * c + k < d ? x32[(size_t)(4 * c + k) * n + i] : 4 * c + k == S - 1 ? __int_as_float(i) : 0.f;
-            r[c] = make_float4(v[0], v[1], v[2], v[3]);
+    for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < Ns; x += gridDim.x * blockDim.x) {
+        const int2 r = range[x];
+        if (r.y - r.x > kBucket) continue;
+        double m = cd64[r.x];
+        for (int i = r.x + 1; i < r.y; ++i) m = fmin(m, cd64[i]);
+        float f = __double2float_rd(m);
+        *(volatile float *)(ncd + x) = f;
+        int cur = x;
+        for (int it = 0; it < Ns; ++it) {
+            const int p = parent[cur];
+            if (p < 0) break;
+            __threadfence();
+            if (atomicAdd(arrive + p, 1) == 0) break;   // the sibling composes the parent
+            __threadfence();
+            // the sibling shares the pair that starts at an odd row (the root is row 0)
+            f = fminf(f, *(volatile float *)(ncd + (((cur - 1) ^ 1) + 1)));
+            *(volatile float *)(ncd + p) = f;
+            cur = p;
         }
     }
 }
@@ -374,7 +274,7 @@ __global__ void nc_init_kernel(TravArgs a, NcArgs b, bool hdb)
         b.bhi[i] = ~0ull;
         b.blo[i] = ~0ull;
         if (hdb) {   // no list yet: an edge outside the repair list is longer than the core distance
-            b.hd[i] = (unsigned char)kNcK;
+            b.hd[i] = (unsigned char)b.K;
             b.R[i] = __double2float_rd(a.cd64[i]);
         }
     }
@@ -392,22 +292,22 @@ __device__ __forceinline__ void s_min(unsigned *S, int c, float v)
 template <int D, bool HDB>
 __global__ void nc_refresh_kernel(TravArgs a, NcArgs b)
 {
-    constexpr int S = row_floats<D>();
+    constexpr int S = row_floats(D);
     const int n = a.n;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int c = b.lab[i];
         int h = b.hd[i];
-        if (h < kNcK) {
+        if (h < b.K) {
             const int h0 = h;
             int j = -1;
-            for (; h < kNcK; ++h) {
+            for (; h < b.K; ++h) {
                 j = b.lj[(size_t)h * n + i];
                 if (j >= 0 && b.lab[j] != c) break;
             }
             if (h != h0) b.hd[i] = (unsigned char)h;
-            if (h < kNcK) s_min(b.S, c, b.ls[(size_t)h * n + i]);
+            if (h < b.K) s_min(b.S, c, b.ls[(size_t)h * n + i]);
         }
-        if (h >= kNcK) {
+        if (h >= b.K) {
 #pragma unroll
             for (int o = -1; o <= 1; o += 2) {
                 const int j = i + o;
@@ -415,12 +315,7 @@ __global__ void nc_refresh_kernel(TravArgs a, NcArgs b)
                 float x[S], y[S];
                 load_row<S>(b.rows, i, x);
                 load_row<S>(b.rows, j, y);
-                float acc = 0.f;
-#pragma unroll
-                for (int k = 0; k < D; ++k) {
-                    const float dx = x[k] - y[k];
-                    acc = fmaf(dx, dx, acc);
-                }
+                float acc = row_dist<D>(x, y);
                 if (HDB) acc = fmaxf(acc, fmaxf(a.cd32[i], a.cd32[j]));
                 s_min(b.S, c, acc);
             }
@@ -501,7 +396,7 @@ __global__ void nc_pick_kernel(TravArgs a, NcArgs b)
             exact = b.R[i] <= T;
             if (HDB && exact) exact = !settled(a, b, i, c);
             if (!exact) {
-                for (int h = b.hd[i]; h < kNcK; ++h) {
+                for (int h = b.hd[i]; h < b.K; ++h) {
                     const float s = b.ls[(size_t)h * n + i];
                     if (s > T) break;
                     const int j = b.lj[(size_t)h * n + i];
@@ -606,7 +501,7 @@ __global__ void nc_relabel_kernel(NcArgs b, int n, int S)
         }
         if (x != c) {
             b.lab[i] = x;
-            const_cast<float *>((const float *)b.rows)[(size_t)i * S + S - 1] = __int_as_float(x);
+            b.rows[(size_t)i * S + S - 1] = __int_as_float(x);
         }
         if (x == i) {   // only roots' slots are read
             b.S[i] = b.cap_bits;
@@ -644,39 +539,23 @@ int rounds(NcCall &C, TravArgs &a, NcArgs &b)
     cudaStream_t st = C.st;
     const int n = a.n;
     const int g = grid_for(n, 256);
-    constexpr int S = row_floats<D>();
+    constexpr int S = row_floats(D);
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, nc_search_kernel<D, HDB, false>, kNcThreads, 0) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, nc_search_kernel<D, HDB, false>, kWalkThreads, 0) != cudaSuccess ||
         per_sm < 1) {
         cudaGetLastError();
         return 0;
     }
-    const int gs = (int)std::min<long long>((long long)num_sms() * per_sm, ((long long)n + kNcThreads - 1) / kNcThreads);
-    // ---- the search tree and the point rows
-    const Tree &T = *C.T;
-    float *rows = C.ar->get<float>((size_t)n * S);
-    b.deep = C.ar->get<uint2>((size_t)gs * kNcThreads * std::max(1, b.stack_cap - kNcStack));
-    int *idx = C.ar->get<int>((size_t)a.N + 1);
-    if (C.ar->failed) return WM_ENOMEM;
-    const int gN = grid_for(a.N, 256);
-    launch(nc_flag_kernel, gN, 256, 0, st, a.N, T.begin, T.end, T.parent, idx);
-    int rc0 = scan_exclusive_i32(idx, idx, a.N, idx + a.N, st, *C.ar);
-    if (rc0) return rc0;
-    cudaMemcpyAsync(C.pin, idx + a.N, sizeof(int), cudaMemcpyDeviceToHost, st);
-    if (cudaStreamSynchronize(st) != cudaSuccess) return WM_ECUDA;
-    b.Ns = C.pin[0];
-    float *nodes = C.ar->get<float>((size_t)b.Ns * 2 * S);
-    int2 *range = C.ar->get<int2>(b.Ns);
-    float *ncd = HDB ? C.ar->get<float>(b.Ns) : nullptr;
-    if (C.ar->failed) return WM_ENOMEM;
-    launch(nc_nodes_kernel<S>, gN, 256, 0, st, a.N, a.d, T.begin, T.end, T.left, T.parent, T.lo, T.hi, a.cdmin, idx, nodes,
-           range, ncd);
-    launch(nc_rows_kernel<S>, g, 256, 0, st, n, a.d, a.x32, rows);
-    b.rows = (const float4 *)rows;
-    b.nodes = (const float4 *)nodes;
-    b.range = range;
-    b.ncd = ncd;
-    b.root = n > kNcBucket ? 1u : kBucketBit | (unsigned)(n - 1) << 28;
+    const int gs = std::min(num_sms() * per_sm, C.X->walk_blocks);
+    const SearchTree &X = *C.X;
+    if (HDB) {
+        float *ncd = C.ar->get<float>(X.Ns);
+        int *arrive = C.ar->get<int>(X.Ns);
+        if (C.ar->failed) return WM_ENOMEM;
+        cudaMemsetAsync(arrive, 0, sizeof(int) * X.Ns, st);
+        launch(nc_core_min_kernel, grid_for(X.Ns, 256), 256, 0, st, X.Ns, X.range, X.parent, a.cd64, ncd, arrive);
+        b.ncd = ncd;
+    }
     launch(nc_init_kernel, g, 256, 0, st, a, b, HDB);
     const EdgeK *rin = C.rep;
     EdgeK *rbuf[2] = {C.rep_tmp0, C.rep_tmp1};
@@ -698,12 +577,12 @@ int rounds(NcCall &C, TravArgs &a, NcArgs &b)
             launch(nc_active_kernel<HDB>, g, 256, 0, st, a, b);
         }
         const int e0 = C.mark(C.ctx);
-        launch(nc_search_kernel<D, HDB, false>, gs, kNcThreads, 0, st, a, b, n);
+        launch(nc_search_kernel<D, HDB, false>, gs, kWalkThreads, 0, st, a, b, X, n);
         const int e1 = C.mark(C.ctx);
         C.span(C.ctx, e0, e1);
         if (b.first) launch(nc_refresh_kernel<D, HDB>, g, 256, 0, st, a, b);   // the lists' minima into S
         launch(nc_pick_kernel<HDB>, g, 256, 0, st, a, b);
-        launch(nc_search_kernel<D, HDB, true>, gs, kNcThreads, 0, st, a, b, n);
+        launch(nc_search_kernel<D, HDB, true>, gs, kWalkThreads, 0, st, a, b, X, n);
         launch(nc_low_kernel, g, 256, 0, st, b);
         if (HDB) launch(nc_low_repair_kernel, grid_for(C.nrep, 256), 256, 0, st, b, rnow, rn);
         launch(nc_merge_kernel, g, 256, 0, st, a, b, C.out, n - 1);
@@ -711,7 +590,7 @@ int rounds(NcCall &C, TravArgs &a, NcArgs &b)
         launch(nc_change_kernel, g, 256, 0, st, b.lab, n, C.E);
         int rc = scan_exclusive_i32(C.E, C.E, n, C.E + n, st, *C.ar);
         if (rc) return rc;
-        launch(nc_node_labels_kernel, grid_for(b.Ns, 256), 256, 0, st, b.Ns, S, range, nodes, b.lab, C.E);
+        launch(nc_node_labels_kernel, grid_for(X.Ns, 256), 256, 0, st, X.Ns, S, X.range, X.nodes, b.lab, C.E);
         cudaMemcpyAsync(C.pin, b.cnt, 8 * sizeof(int), cudaMemcpyDeviceToHost, st);
         cudaMemcpyAsync(C.pin + 8, a.overflow, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
         if (cudaStreamSynchronize(st) != cudaSuccess) return WM_ECUDA;
@@ -743,8 +622,9 @@ int nearest_component_rounds(NcCall &C, TravArgs &a)
     b.S = ar.get<unsigned>(n);
     b.bhi = ar.get<unsigned long long>(n);
     b.blo = ar.get<unsigned long long>(n);
-    b.ls = ar.get<float>((size_t)kNcK * n);
-    b.lj = ar.get<int>((size_t)kNcK * n);
+    b.K = list_len(walk_dim(a.d));
+    b.ls = ar.get<float>((size_t)b.K * n);
+    b.lj = ar.get<int>((size_t)b.K * n);
     b.R = ar.get<float>(n);
     b.hd = ar.get<unsigned char>(n);
     b.act = ar.get<int>(n);
@@ -760,7 +640,7 @@ int nearest_component_rounds(NcCall &C, TravArgs &a)
     if (ar.failed) return WM_ENOMEM;
     cudaMemsetAsync(b.cnt, 0, 16 * sizeof(int), C.st);
     b.pos = C.pos;
-    b.stack_cap = C.depth + 4;
+    b.rows = C.X->rows;
     const float cf = C.cap < INFINITY ? C.cap_f : INFINITY;
     memcpy(&b.cap_bits, &cf, sizeof cf);
     memcpy(&b.cap64, &C.cap, sizeof C.cap);
@@ -768,14 +648,19 @@ int nearest_component_rounds(NcCall &C, TravArgs &a)
     int rc;
     const bool hdb = a.cd64 != nullptr;
 #define WM_NC(DV) rc = hdb ? rounds<DV, true>(C, a, b) : rounds<DV, false>(C, a, b)
-    if (a.d == 2) WM_NC(2);
-    else if (a.d == 3) WM_NC(3);
-    else if (a.d <= 4) WM_NC(4);
-    else if (a.d == 5) WM_NC(5);
-    else if (a.d == 6) WM_NC(6);
-    else if (a.d == 7) WM_NC(7);
-    else if (a.d <= 8) WM_NC(8);
-    else WM_NC(16);
+    const int wd = walk_dim(a.d);
+    if (row_floats(wd) != C.X->S) { ar.off = mark; return WM_EINTERNAL; }
+    switch (wd) {
+    case 2: WM_NC(2); break;
+    case 3: WM_NC(3); break;
+    case 4: WM_NC(4); break;
+    case 5: WM_NC(5); break;
+    case 6: WM_NC(6); break;
+    case 7: WM_NC(7); break;
+    case 8: WM_NC(8); break;
+    case 15: WM_NC(15); break;
+    default: WM_NC(16); break;
+    }
 #undef WM_NC
     ar.off = mark;
     return rc;

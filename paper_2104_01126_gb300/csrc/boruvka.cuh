@@ -3,6 +3,7 @@
 
 #include <cmath>
 
+#include "stree.cuh"
 #include "wspd.cuh"
 
 namespace wm {
@@ -11,8 +12,7 @@ struct NcCall {
     cudaStream_t st = nullptr;
     Arena *ar = nullptr;
     int *pin = nullptr;             // pinned host scratch
-    int depth = 0;                  // tree levels
-    const Tree *T = nullptr;
+    const SearchTree *X = nullptr;
     const int *pos = nullptr;       // input id -> tree position
     int *uf = nullptr;              // union-find over input ids, left flat on return
     EdgeK *out = nullptr;           // tree edges, in no particular order
@@ -33,7 +33,7 @@ struct NcCall {
     void (*span)(void *ctx, int from, int to) = nullptr;
 };
 
-// Boruvka rounds on the tree packed in a.rec / a.box / a.x4.  Returns 0 or an error code; C.done tells
+// Boruvka rounds on the search tree (whose labels they overwrite).  Returns 0 or an error code; C.done tells
 // how far the forest got.
 int nearest_component_rounds(NcCall &C, TravArgs &a);
 

@@ -3,15 +3,18 @@
 // per-node cd_min / cd_max bounds (Table 1) and the repair edges that make the returned MST the
 // canonical one under the key K.
 //
-// k-NN: one warp answers 32 consecutive tree positions (spatially close queries) with a shared
-// depth-first traversal of the k-d tree.  A subtree of at most 32 points is scanned directly:
-// its points are loaded once and broadcast with shuffles.  Each lane keeps the KL = minPts + 8
-// smallest screened values in a sorted list in shared memory (slot-major, one bank per lane).
-// A node is skipped for a lane when its box is provably farther than the lane's KL-th value.
-// FP32 screen: the k-th screened value s_k gives the band threshold T(s_k); when the list
-// provably holds every point with screened value <= T (its KL-th value exceeds T), those
-// candidates are re-evaluated in FP64 and sorted, giving the exact k-th squared distance.  A
-// query whose band overflows the list (ties, duplicates) is answered by an exact FP64 scan.
+// k-NN, FP32 screen: one thread per query walks the search tree (stree.cuh), the nearer child first, and
+// keeps the minPts smallest screened values in a max-heap in shared memory (slot-major, one bank per
+// lane).  A node is skipped when its box is provably beyond the band threshold T of the heap's top, so
+// every point that the walk does not evaluate screens above T.  The smallest value that the heap
+// turned away or gave up (out) then tells whether the heap holds exactly the points screened within
+// T(s_k): if out > T(s_k), the k-th squared distance is the largest FP64 distance of the heap's points
+// and all of them (but the point itself) are its repair edges.  Otherwise (ties within the band) a warp
+// collects every point within T(s_k), evaluates them in FP64 and selects the k-th; a band of more than
+// kTieCap points (heavy duplicates) is answered by an exact FP64 scan of all points.
+//
+// k-NN, plain FP64 form: one warp answers 32 consecutive tree positions with a shared depth-first
+// traversal of the k-d tree; each lane keeps the KL = minPts + 8 smallest values in a sorted list.
 //
 // Repair edges: R = {(p,q), q != p : w2(p,q) <= cd2(p)}, weighted by the mutual reachability
 // distance.  Under general position every edge of the K-minimum spanning tree of G_MR either has
@@ -19,10 +22,12 @@
 // d(p,q) <= max(cd(p), cd(q)) (then it is in R); adding R to the MemoGFK batches of their weight
 // range therefore yields the K-minimum tree itself.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
-#include <type_traits>
 
 #include "hdb.cuh"
+#include "screen.cuh"
+#include "stree.cuh"
 #include "wspd.cuh"
 
 namespace wm {
@@ -31,22 +36,20 @@ namespace {
 
 struct KnnArgs {
     int N, n, d, k, KL;
-    const float *lo, *hi;
-    const int *begin, *end, *left, *right;
-    const NodeRec *rec;  // packed node records (right child = left + 1)
+    const NodeRec *rec;  // FP64 form: packed node records (right child = left + 1)
     const float *box;    // packed boxes, 2 DMP floats per node (DMP = d rounded up to 4, 8, 16) in groups of
                          // four dimensions: lo[4c..4c+3], hi[4c..4c+3]
     const float *x32;
     const double *x64;
-    double eta;
-    int stack_cap;       // entries of a warp's traversal stack (in shared memory): depth + 4
-    double *wscratch;    // [warps][KL][32] FP64 candidate values
+    int stack_cap;       // FP64 form: entries of a warp's traversal stack (in shared memory): depth + 4
     double *cd64;
     float *cd32;
-    int *rep_q;          // [n][KL-1] tree positions
-    double *rep_d;       // [n][KL-1] FP64 squared distances
+    int rq;              // slots of a repair row
+    int *rep_q;          // [rq][n] tree positions
+    double *rep_d;       // [rq][n] FP64 squared distances
     int *rep_cnt;        // [n]
-    int *slow;           // slow query list
+    int *slow;           // queries with ties around the k-th value
+    float *slow_s;       // their screened k-th values
     int *slow_cnt;
     int *next_group;     // dispenser of 32-query groups
     int *err;            // set when a traversal stack would overflow (an internal error)
@@ -54,75 +57,32 @@ struct KnnArgs {
                                 //     error of a screened k-th value against the exact one
 };
 
-__device__ inline double d64(const double *__restrict__ x64, int n, int d, int i, int j)
-{
-    double s = 0.0;
-    for (int k = 0; k < d; ++k) {
-        double t = __dsub_rn(x64[(size_t)k * n + i], x64[(size_t)k * n + j]);
-        s = __dadd_rn(s, __dmul_rn(t, t));
-    }
-    return s;
-}
-
-__device__ inline float knn_threshold(float s, double eta)
-{
-    double t;
-    if (eta == 0.0) {
-        t = (double)s * (1.0 + 4.0 * kEps32) + 1.5e-42;
-    } else {
-        double r = sqrt((double)s * (1.0 + 2.0 * kEps32)) + eta;
-        double U = r * r * (1.0 + 2.0 * kGam64);
-        double q = sqrt(U * (1.0 + 2.0 * kGam64)) + eta;
-        t = q * q * (1.0 + 2.0 * kEps32) + 1.5e-42;
-    }
-    return __double2float_ru(t);
-}
-
-// Upper bound of knn_threshold(s, 0) in FP32 with directed rounding: s (1 + 2^-17) + 1.6e-42, both
-// steps rounded up (1.6e-42 as a float exceeds 1.5e-42).  Any float >= the exact threshold is
-// >= its rounded-up value as well, so it can stand in for it as a pruning bound.
-__device__ inline float knn_threshold_fast(float s)
-{
-    return __fadd_ru(__fmul_ru(s, 1.0f + 4.0f / 524288.0f), 1.6e-42f);
-}
-
-// coordinates per leaf point in the shared-memory broadcast buffer (d rounded up to 4, 8 or 16:
-// the stride of the packed boxes as well)
+// stride of the packed boxes: d rounded up to 4, 8 or 16
 template <int DM> constexpr int knn_dmp() { return DM <= 4 ? 4 : DM <= 8 ? 8 : 16; }
 
-// shared memory of one warp of the k-NN kernel: leaf points, screened lists, indices, stack,
-// rounded up to 16 bytes so that the next warp's region starts float4-aligned
-__host__ __device__ inline size_t knn_warp_smem(int dmp, int KL, size_t vsize, int stack_cap)
+// shared memory of one warp of the FP64 kernel: values, indices, stack
+__host__ __device__ inline size_t knn_warp_smem(int KL, int stack_cap)
 {
-    const size_t b = (size_t)32 * dmp * sizeof(float) + (size_t)KL * 32 * (vsize + sizeof(int)) +
-                     (size_t)stack_cap * sizeof(int);
+    const size_t b = (size_t)KL * 32 * (sizeof(double) + sizeof(int)) + (size_t)stack_cap * sizeof(int);
     return (b + 15) & ~(size_t)15;
 }
 
-template <int DM, bool FP64>
-__global__ void __launch_bounds__(256) knn_fast_kernel(KnnArgs a)
+template <int DM>
+__global__ void __launch_bounds__(256) knn64_kernel(KnnArgs a)
 {
-    using V = typename std::conditional<FP64, double, float>::type;
     extern __shared__ unsigned char smem_raw[];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, nwb = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int KL = a.KL;
-    // per-warp shared region: float4 leaf[32][DMP/4] (the scanned subtree's points, read as
-    // broadcasts); V sv[KL][32]; int sj[KL][32] (slot-major, one bank per lane); int stk[stack_cap]
-    // (the warp's traversal stack); the FP64 candidate values of the epilogue live in global
-    // scratch: double sw[KL][32]
+    // per-warp shared region: double sv[KL][32]; int sj[KL][32] (slot-major, one bank per lane);
+    // int stk[stack_cap] (the warp's traversal stack)
     constexpr int DMP = knn_dmp<DM>(), DQ = DMP / 4;
-    size_t per_warp = knn_warp_smem(DMP, KL, sizeof(V), a.stack_cap);
+    size_t per_warp = knn_warp_smem(KL, a.stack_cap);
     unsigned char *base = smem_raw + per_warp * wib;
-    float4 *leaf = (float4 *)base;
-    V *sv = (V *)(base + (size_t)32 * DMP * sizeof(float));
-    int *sj = (int *)((unsigned char *)sv + (size_t)KL * 32 * sizeof(V));
+    double *sv = (double *)base;
+    int *sj = (int *)(sv + (size_t)KL * 32);
     int *stk = sj + (size_t)KL * 32;
-    const int gw = blockIdx.x * nwb + wib;
-    double *sw = a.wscratch + (size_t)gw * KL * 32;
     const int n = a.n, d = a.d;
-    const bool exact32 = a.eta == 0.0;   // FP32 copy is exact: threshold in FP32
-    unsigned long long n_ev = 0, n_re = 0;
-    float kerr = 0.f;   // largest relative error of a screened k-th value (FP32 screen)
+    unsigned long long n_ev = 0;
     // 32-query groups handed out dynamically: their costs differ too much for a static deal
     while (true) {
         int q0 = 0;
@@ -136,11 +96,8 @@ __global__ void __launch_bounds__(256) knn_fast_kernel(KnnArgs a)
 #pragma unroll
         for (int k = 0; k < DMP; ++k) qx[k] = k < d && valid ? a.x32[(size_t)k * n + i] : 0.f;
 #pragma unroll
-        for (int k = 0; k < DM; ++k) {
-            if (k < d) {
-                if (FP64) qx64[k] = valid ? a.x64[(size_t)k * n + i] : 0.0;
-            }
-        }
+        for (int k = 0; k < DM; ++k)
+            if (k < d) qx64[k] = valid ? a.x64[(size_t)k * n + i] : 0.0;
         // the group's centroid orders the children of a visited node (nearer first) without a
         // reduction over the lanes at every node
         float cent[DMP];
@@ -154,13 +111,8 @@ __global__ void __launch_bounds__(256) knn_fast_kernel(KnnArgs a)
             }
         }
         int cnt = 0;
-        V thr = (V)INFINITY;   // KL-th kept value (list full) or +inf
-        // cut: the band threshold of the current k-th value; a point screened above it can never
-        // be a candidate, and a node is skipped when its box bound exceeds cut (1 + 2^-17)
-        // (the bound is a rigorous lower bound of the true distance and a screened value is
-        // within 2^-19 of the true one, so every skipped point screens above cut as well).
-        // cut only decreases, so the final threshold T(s_k) is below every cut used.
-        V cut = (V)INFINITY;
+        double thr = INFINITY;   // KL-th kept value (list full) or +inf
+        double cut = INFINITY;   // the current k-th value: a point above it can never be a candidate
         int sp = 0;
         if (lane == 0) stk[0] = 0;
         sp = 1;
@@ -186,56 +138,24 @@ __global__ void __launch_bounds__(256) knn_fast_kernel(KnnArgs a)
                     }
                 }
             }
-            bool need = valid && (V)lower_w2(lb) <= cut * (V)(1.0f + 1.0f / 131072.0f) &&
-                        (cnt < KL || (V)lower_w2(lb) <= thr);
+            const double lw = lower_w2(lb);
+            const bool need = valid && lw <= cut * (1.0 + 1.0 / 131072.0) && (cnt < KL || lw <= thr);
             if (!__any_sync(0xffffffffu, need)) continue;
             if (e - b <= 32) {
                 // scan the subtree's points
                 const int m = e - b;
                 double px64[DM];
-                if (FP64) {
 #pragma unroll
-                    for (int k = 0; k < DM; ++k)
-                        if (k < d) px64[k] = lane < m ? a.x64[(size_t)k * n + b + lane] : 0.0;
-                } else {
-                    if (lane < m) {
-#pragma unroll
-                        for (int c = 0; c < DQ; ++c) {
-                            float v[4];
-#pragma unroll
-                            for (int r = 0; r < 4; ++r)
-                                v[r] = 4 * c + r < d ? a.x32[(size_t)(4 * c + r) * n + b + lane] : 0.f;
-                            leaf[lane * DQ + c] = make_float4(v[0], v[1], v[2], v[3]);
-                        }
-                    }
-                    __syncwarp();
-                }
+                for (int k = 0; k < DM; ++k)
+                    if (k < d) px64[k] = lane < m ? a.x64[(size_t)k * n + b + lane] : 0.0;
                 for (int p = 0; p < m; ++p) {
-                    V s;
-                    if (FP64) {
-                        double acc = 0.0;
+                    double s = 0.0;
 #pragma unroll
-                        for (int k = 0; k < DM; ++k) {
-                            if (k < d) {
-                                double t = __dsub_rn(qx64[k], __shfl_sync(0xffffffffu, px64[k], p));
-                                acc = __dadd_rn(acc, __dmul_rn(t, t));
-                            }
+                    for (int k = 0; k < DM; ++k) {
+                        if (k < d) {
+                            double t = __dsub_rn(qx64[k], __shfl_sync(0xffffffffu, px64[k], p));
+                            s = __dadd_rn(s, __dmul_rn(t, t));
                         }
-                        s = (V)acc;
-                    } else {
-                        // padded coordinates are 0 on both sides and add nothing
-                        float acc = 0.f;
-#pragma unroll
-                        for (int c = 0; c < DQ; ++c) {
-                            const float4 v = leaf[p * DQ + c];
-                            const float pv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                            for (int r = 0; r < 4; ++r) {
-                                float t = qx[4 * c + r] - pv[r];
-                                acc = fmaf(t, t, acc);
-                            }
-                        }
-                        s = (V)acc;
                     }
                     if (valid && s <= cut && (cnt < KL || s < thr)) {
                         int pos = cnt < KL ? cnt : KL - 1;
@@ -248,15 +168,13 @@ __global__ void __launch_bounds__(256) knn_fast_kernel(KnnArgs a)
                         sj[pos * 32 + lane] = b + p;
                         if (cnt < KL) ++cnt;
                         if (cnt >= a.k && pos < a.k) {
-                            V sk = sv[(a.k - 1) * 32 + lane];
-                            cut = FP64 ? sk : exact32 ? (V)knn_threshold_fast((float)sk) : (V)knn_threshold((float)sk, a.eta);
+                            cut = sv[(a.k - 1) * 32 + lane];
                             // entries above the cut can never be candidates again: drop them
                             while (cnt > a.k && sv[(cnt - 1) * 32 + lane] > cut) --cnt;
                         }
-                        thr = cnt == KL ? sv[(KL - 1) * 32 + lane] : (V)INFINITY;
+                        thr = cnt == KL ? sv[(KL - 1) * 32 + lane] : INFINITY;
                     }
                 }
-                if (!FP64) __syncwarp();   // the leaf buffer is reused by the next scan
                 n_ev += (unsigned long long)m;
             } else {
                 // push the farther child (from the group's centroid) first so the nearer one is
@@ -290,76 +208,293 @@ __global__ void __launch_bounds__(256) knn_fast_kernel(KnnArgs a)
             }
         }
         if (!valid) continue;
-        // ---- exact k-th value and repair candidates
-        const int k = a.k;
-        double cd2;
-        int ncand;
-        bool complete;
-        if (FP64) {
-            cd2 = (double)sv[(k - 1) * 32 + lane];
-            complete = cnt < KL || (double)sv[(KL - 1) * 32 + lane] > cd2;
-            ncand = 0;
-            while (ncand < cnt && (double)sv[ncand * 32 + lane] <= cd2) {
-                sw[ncand * 32 + lane] = (double)sv[ncand * 32 + lane];
-                ++ncand;
-            }
-        } else {
-            const float sk = (float)sv[(k - 1) * 32 + lane];
-            const float T = exact32 ? knn_threshold_fast(sk) : knn_threshold(sk, a.eta);
-            complete = cnt < KL || (float)sv[(KL - 1) * 32 + lane] > T;
-            ncand = 0;
-            while (ncand < cnt && (float)sv[ncand * 32 + lane] <= T) ++ncand;
-            if (complete) {
-                for (int c = 0; c < ncand; ++c) {
-                    int j = sj[c * 32 + lane];
-                    double w = j == i ? 0.0 : d64(a.x64, n, d, i, j);
-                    // insertion sort by w (non-negative doubles compared through their bit patterns)
-                    int pos = c;
-                    while (pos > 0 && __double_as_longlong(sw[(pos - 1) * 32 + lane]) > __double_as_longlong(w)) {
-                        sw[pos * 32 + lane] = sw[(pos - 1) * 32 + lane];
-                        sj[pos * 32 + lane] = sj[(pos - 1) * 32 + lane];
-                        --pos;
-                    }
-                    sw[pos * 32 + lane] = w;
-                    sj[pos * 32 + lane] = j;
-                }
-                n_re += (unsigned long long)ncand;
-            }
-            cd2 = complete ? sw[(k - 1) * 32 + lane] : 0.0;
-        }
-        if (!complete) {
-            int s = atomicAdd(a.slow_cnt, 1);
-            a.slow[s] = i;
+        const double cd2 = sv[(a.k - 1) * 32 + lane];
+        if (cnt == KL && !(sv[(KL - 1) * 32 + lane] > cd2)) {   // ties may have been dropped
+            a.slow[atomicAdd(a.slow_cnt, 1)] = i;
             continue;
-        }
-        if (!FP64 && cd2 > 0.0) {   // the ratio in FP32 with outward rounding
-            const double sk = (double)sv[(k - 1) * 32 + lane];
-            kerr = fmaxf(kerr, __fdiv_ru(__double2float_ru(fabs(sk - cd2)), __double2float_rd(cd2)));
         }
         a.cd64[i] = cd2;
         a.cd32[i] = __double2float_rn(cd2);
         int r = 0;
-        for (int c = 0; c < ncand && r < KL - 1; ++c) {
-            int j = sj[c * 32 + lane];
-            double w = sw[c * 32 + lane];
-            if (j != i && __double_as_longlong(w) <= __double_as_longlong(cd2)) {
-                a.rep_q[(size_t)i * (KL - 1) + r] = j;
-                a.rep_d[(size_t)i * (KL - 1) + r] = w;
-                ++r;
-            }
+        for (int c = 0; c < cnt && r < a.rq; ++c) {
+            const double w = sv[c * 32 + lane];
+            if (!(w <= cd2)) break;
+            const int j = sj[c * 32 + lane];
+            if (j == i) continue;
+            a.rep_q[(size_t)r * n + i] = j;
+            a.rep_d[(size_t)r * n + i] = w;
+            ++r;
         }
         a.rep_cnt[i] = r;
     }
-    for (int o = 16; o; o >>= 1) {
-        n_ev += __shfl_xor_sync(0xffffffffu, n_ev, o);
-        n_re += __shfl_xor_sync(0xffffffffu, n_re, o);
-        kerr = fmaxf(kerr, __shfl_xor_sync(0xffffffffu, kerr, o));
-    }
+    for (int o = 16; o; o >>= 1) n_ev += __shfl_xor_sync(0xffffffffu, n_ev, o);
+    if (lane == 0) atomicAdd(a.stat + 0, n_ev);
+}
+
+// ------------------------------------------------------------------- FP32 screen, thread per query
+// Shared memory of a block of T threads: uint2 stk[kWalkStack][T], uint2 heap[k][T] (value bits,
+// position), both slot-major: a lane's slots lie in its own banks, whatever slots its neighbours use.
+template <int D>
+__global__ void __launch_bounds__(kWalkThreads) knn_walk_kernel(KnnArgs a, SearchTree X, TravArgs band)
+{
+    extern __shared__ uint2 walk_smem[];
+    constexpr int S = row_floats(D);
+    constexpr bool kStream = S > 4;
+    const int lane = threadIdx.x & 31, T = blockDim.x;
+    uint2 *heap = walk_smem + (size_t)kWalkStack * T + threadIdx.x;
+    const int n = a.n, k = a.k;
+    unsigned long long n_ev = 0, n_re = 0;
+    float kerr = 0.f;   // largest relative error of a screened k-th value
+    // the lane's query
+    float q[S];
+    int i = 0, cnt = 0;
+    float top = 0.f;   // the heap's largest value once it is full
+    float out = 0.f;   // the smallest value that is not in the heap
+    float pb = 0.f;    // a node whose lower bound exceeds pb holds no point within T(top)
+    unsigned ev = 0;
+    auto begin = [&](int t) {
+        i = t;
+        load_row<S>(X.rows, i, q);
+        cnt = 0;
+        top = out = pb = INFINITY;
+        ev = 0;
+    };
+    auto bound = [](unsigned, float &, float &) {};
+    auto need = [&](float g, int) { return g <= pb; };
+    auto pending = [&](float g) { return g <= pb; };
+    auto scan = [&](int j0, int sz) {
+        // screened values first, then the ones below the top enter the heap, so that the lanes of a
+        // warp run their insertions together
+        float s[kBucket];
+        unsigned todo = 0;
+#pragma unroll
+        for (int h = 0; h < kBucket; h += 4) {
+            if (h && h >= sz) break;
+#pragma unroll
+            for (int p = h; p < h + 4; ++p) {
+                float x[S];
+                load_row<S, kStream>(X.rows, j0 + min(p, sz - 1), x);
+                s[p] = row_dist<D>(q, x);
+                if (p < sz) {
+                    if (s[p] < top) todo |= 1u << p;
+                    else out = fminf(out, s[p]);
+                }
+            }
+        }
+        ev += (unsigned)sz;
+        while (todo) {
+            const int p = __ffs(todo) - 1;
+            todo &= todo - 1;
+            float v = s[0];
+#pragma unroll
+            for (int r = 1; r < kBucket; ++r) v = r == p ? s[r] : v;
+            const uint2 mine = make_uint2(__float_as_uint(v), (unsigned)(j0 + p));
+            if (cnt < k) {   // fill: sift up
+                int h = cnt++;
+                while (h > 0) {
+                    const int u = (h - 1) >> 1;
+                    const uint2 e = heap[u * T];
+                    if (__uint_as_float(e.x) >= v) break;
+                    heap[h * T] = e;
+                    h = u;
+                }
+                heap[h * T] = mine;
+                if (cnt == k) top = __uint_as_float(heap[0].x);
+            } else if (v < top) {   // replace the top: sift down
+                out = fminf(out, top);
+                int h = 0;
+                while (true) {
+                    int u = 2 * h + 1;
+                    if (u >= k) break;
+                    uint2 e = heap[u * T];
+                    if (u + 1 < k) {
+                        const uint2 f = heap[(u + 1) * T];
+                        if (__uint_as_float(f.x) > __uint_as_float(e.x)) { e = f; ++u; }
+                    }
+                    if (__uint_as_float(e.x) <= v) break;
+                    heap[h * T] = e;
+                    h = u;
+                }
+                heap[h * T] = mine;
+                top = __uint_as_float(heap[0].x);
+            } else {
+                out = fminf(out, v);
+            }
+        }
+        pb = screen_threshold(top, band) * (1.0f + 1.0f / 131072.0f);
+    };
+    auto finish = [&] {
+        n_ev += ev;
+        if (cnt < k || !(out > screen_threshold(top, band))) {
+            const int t = atomicAdd(a.slow_cnt, 1);
+            a.slow[t] = i;
+            a.slow_s[t] = top;
+            return;
+        }
+        // the k points of the heap are the k nearest; all but the point itself are repair edges
+        unsigned long long cd = 0;
+        int r = 0;
+        for (int h = 0; h < k; ++h) {
+            const int j = (int)heap[h * T].y;
+            if (j == i) continue;
+            const double w = dist64(a.x64, n, a.d, i, j);
+            cd = max(cd, (unsigned long long)__double_as_longlong(w));
+            if (r < a.rq) {
+                a.rep_q[(size_t)r * n + i] = j;
+                a.rep_d[(size_t)r * n + i] = w;
+                ++r;
+            }
+        }
+        n_re += (unsigned long long)k;
+        const double cd2 = __longlong_as_double((long long)cd);
+        a.cd64[i] = cd2;
+        a.cd32[i] = __double2float_rn(cd2);
+        a.rep_cnt[i] = r;
+        if (cd2 > 0.0)
+            kerr = fmaxf(kerr, __fdiv_ru(__double2float_ru(fabs((double)top - cd2)), __double2float_rd(cd2)));
+    };
+    walk_queries<D, S, kStream>(X, n, a.next_group, walk_smem + threadIdx.x, T, X.deep + (size_t)blockIdx.x * T + threadIdx.x,
+                                (size_t)gridDim.x * T, a.err, 1, q, begin, bound, need, pending, scan, finish);
+    n_ev = warp_sum_u64(n_ev);
+    n_re = warp_sum_u64(n_re);
+    for (int o = 16; o; o >>= 1) kerr = fmaxf(kerr, __shfl_xor_sync(0xffffffffu, kerr, o));
     if (lane == 0) {
         atomicAdd(a.stat + 0, n_ev);
         atomicAdd(a.stat + 1, n_re);
         if (kerr > 0.f) atomicMax(a.stat + 2, (unsigned long long)__float_as_uint(kerr));
     }
+}
+
+// Ties around the k-th value: a warp per query collects every point within the band of the screened
+// k-th value, evaluates them in FP64 and takes the k-th smallest.
+constexpr int kTieCap = 512, kTieWarps = 4;
+
+template <int D>
+__global__ void __launch_bounds__(32 * kTieWarps) knn_tie_kernel(KnnArgs a, SearchTree X, TravArgs band,
+                                                                 const int *__restrict__ m_dev, int *next, int *slow2,
+                                                                 int *slow2_cnt, int *extra_q, int *extra_p,
+                                                                 double *extra_d, int *extra_cnt, int extra_cap,
+                                                                 int *tie_overflow)
+{
+    __shared__ int cj_[kTieWarps][kTieCap];
+    __shared__ double cw_[kTieWarps][kTieCap];
+    extern __shared__ uint2 walk_smem[];
+    constexpr int S = row_floats(D);
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    int *cj = cj_[wib];
+    double *cw = cw_[wib];
+    unsigned *stk = (unsigned *)walk_smem + (size_t)wib * (X.stack_cap + 2);
+    const int n = a.n, k = a.k, m = *m_dev;
+    unsigned long long n_re = 0;
+    while (true) {
+        int t = 0;
+        if (lane == 0) t = atomicAdd(next, 1);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (t >= m) break;
+        const int i = a.slow[t];
+        const float Tk = screen_threshold(a.slow_s[t], band);
+        const float pb = Tk * (1.0f + 1.0f / 131072.0f);
+        float q[S];
+        load_row<S>(X.rows, i, q);
+        int c = 0, sp = 1;
+        __syncwarp();
+        if (lane == 0) stk[0] = X.root;
+        __syncwarp();
+        while (sp > 0 && c <= kTieCap) {
+            const unsigned ref = stk[sp - 1];
+            __syncwarp();
+            --sp;
+            bool take = false;
+            int j = 0;
+            if (ref & kBucketBit) {
+                const int sz = (int)((ref >> 28) & 7u) + 1;
+                if (lane < sz) {
+                    j = (int)(ref & 0x0fffffffu) + lane;
+                    float x[S];
+                    load_row<S>(X.rows, j, x);
+                    take = row_dist<D>(q, x) <= Tk;
+                }
+                const unsigned b = __ballot_sync(0xffffffffu, take);
+                const int slot = c + __popc(b & lanemask_lt());
+                if (take && slot < kTieCap) cj[slot] = j;
+                c += __popc(b);
+            } else {
+                float g0, g1;
+                unsigned r0, r1;
+                int l0, l1;
+                visit_children<D, S, false>(X.nodes, ref, q, g0, g1, r0, r1, l0, l1);
+                if (sp + 2 > X.stack_cap + 2) {   // cannot happen: one entry per level and one more
+                    if (lane == 0) atomicOr(a.err, 1);
+                    break;
+                }
+                if (lane == 0) {
+                    int u = sp;
+                    if (g0 <= pb) stk[u++] = r0;
+                    if (g1 <= pb) stk[u++] = r1;
+                }
+                __syncwarp();
+                sp += (g0 <= pb) + (g1 <= pb);
+            }
+        }
+        __syncwarp();
+        if (c > kTieCap || c < k) {
+            if (lane == 0) slow2[atomicAdd(slow2_cnt, 1)] = i;
+            continue;
+        }
+        for (int e = lane; e < c; e += 32) cw[e] = cj[e] == i ? 0.0 : dist64(a.x64, n, a.d, i, cj[e]);
+        n_re += (unsigned long long)(lane == 0 ? c : 0);
+        __syncwarp();
+        // the k-th smallest: the value with fewer than k values below it and at least k at or below it
+        unsigned long long kth = 0;
+        for (int e = lane; e < c; e += 32) {
+            const unsigned long long v = (unsigned long long)__double_as_longlong(cw[e]);
+            int lt = 0, le = 0;
+            for (int f = 0; f < c; ++f) {
+                const unsigned long long u = (unsigned long long)__double_as_longlong(cw[f]);
+                lt += u < v;
+                le += u <= v;
+            }
+            if (lt < k && le >= k) kth = v;
+        }
+        for (int o = 16; o; o >>= 1) kth = max(kth, __shfl_xor_sync(0xffffffffu, kth, o));
+        const double cd2 = __longlong_as_double((long long)kth);
+        // its repair edges: into the row when they fit, else all into the overflow list
+        int total = 0;
+        for (int e = lane; e < c; e += 32)
+            total += cj[e] != i && (unsigned long long)__double_as_longlong(cw[e]) <= kth;
+        total = __reduce_add_sync(0xffffffffu, total);
+        int xbase = 0, r = 0;
+        if (total > a.rq) {
+            if (lane == 0) xbase = atomicAdd(extra_cnt, total);
+            xbase = __shfl_sync(0xffffffffu, xbase, 0);
+        }
+        for (int e0 = 0; e0 < c; e0 += 32) {
+            const int e = e0 + lane;
+            const bool keep = e < c && cj[e] != i && (unsigned long long)__double_as_longlong(cw[e]) <= kth;
+            const unsigned b = __ballot_sync(0xffffffffu, keep);
+            const int slot = r + __popc(b & lanemask_lt());
+            if (keep) {
+                if (total <= a.rq) {
+                    a.rep_q[(size_t)slot * n + i] = cj[e];
+                    a.rep_d[(size_t)slot * n + i] = cw[e];
+                } else if (xbase + slot < extra_cap) {
+                    extra_p[xbase + slot] = i;
+                    extra_q[xbase + slot] = cj[e];
+                    extra_d[xbase + slot] = cw[e];
+                } else {
+                    atomicOr(tie_overflow, 1);
+                }
+            }
+            r += __popc(b);
+        }
+        if (lane == 0) {
+            a.cd64[i] = cd2;
+            a.cd32[i] = __double2float_rn(cd2);
+            a.rep_cnt[i] = total <= a.rq ? total : 0;
+        }
+        __syncwarp();
+    }
+    if (lane == 0 && n_re) atomicAdd(a.stat + 1, n_re);
 }
 
 // Exact FP64 answer for one query per warp (ties or duplicates overflowed the list): each lane
@@ -375,10 +510,11 @@ __global__ void __launch_bounds__(32) knn_slow_kernel(KnnArgs a, const int *__re
     double *lw = (double *)smem_raw;            // [k][32]
     int *head = (int *)(lw + (size_t)k * 32);   // [32]
     for (int t = blockIdx.x; t < nslow; t += gridDim.x) {
+        __syncwarp();
         const int i = slow[t];
         int cnt = 0;
         for (int j = lane; j < n; j += 32) {
-            double w = j == i ? 0.0 : d64(a.x64, n, d, i, j);
+            double w = j == i ? 0.0 : dist64(a.x64, n, d, i, j);
             if (cnt < k || w < lw[(k - 1) * 32 + lane]) {
                 int pos = cnt < k ? cnt : k - 1;
                 while (pos > 0 && lw[(pos - 1) * 32 + lane] > w) { lw[pos * 32 + lane] = lw[(pos - 1) * 32 + lane]; --pos; }
@@ -405,7 +541,7 @@ __global__ void __launch_bounds__(32) knn_slow_kernel(KnnArgs a, const int *__re
         }
         for (int j = lane; j < n; j += 32) {
             if (j == i) continue;
-            double w = d64(a.x64, n, d, i, j);
+            double w = dist64(a.x64, n, d, i, j);
             if (w <= kth) {
                 int s = atomicAdd(extra_cnt, 1);
                 if (s < extra_cap) { extra_p[s] = i; extra_q[s] = j; extra_d[s] = w; }
@@ -453,28 +589,22 @@ __device__ inline bool rep_keep(int i, int j, double D, const double *__restrict
     return !(__double_as_longlong(D) <= __double_as_longlong(cd64[j]) && pid[j] < pid[i]);
 }
 
-__global__ void rep_flags_kernel(const int *__restrict__ rep_q, const double *__restrict__ rep_d,
-                                 const int *__restrict__ rep_cnt, int n, int KL, const double *__restrict__ cd64,
-                                 const int *__restrict__ pid, int *__restrict__ out)
-{
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        int k = 0;
-        for (int r = 0; r < rep_cnt[i]; ++r)
-            k += rep_keep(i, rep_q[(size_t)i * (KL - 1) + r], rep_d[(size_t)i * (KL - 1) + r], cd64, pid);
-        out[i] = k;
-    }
-}
-
-// repair edge of positions (i, j) with FP64 squared distance D: weight max(cd2 i, cd2 j, D)
+// repair edge of positions (i, j) with FP64 squared distance D: weight max(cd2 i, cd2 j, D); appended in
+// no particular order
 __global__ void rep_emit_kernel(const int *__restrict__ rep_q, const double *__restrict__ rep_d,
-                                const int *__restrict__ rep_cnt, const int *__restrict__ off, int n, int KL,
-                                const double *__restrict__ cd64, const int *__restrict__ pid, EdgeK *__restrict__ out)
+                                const int *__restrict__ rep_cnt, int n, const double *__restrict__ cd64,
+                                const int *__restrict__ pid, EdgeK *__restrict__ out, int *count)
 {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        int o = off[i];
-        for (int r = 0; r < rep_cnt[i]; ++r) {
-            const int j = rep_q[(size_t)i * (KL - 1) + r];
-            const double D = rep_d[(size_t)i * (KL - 1) + r];
+    __shared__ int sh[32];
+    for (int b0 = blockIdx.x * blockDim.x; b0 < n; b0 += gridDim.x * blockDim.x) {
+        const int i = b0 + threadIdx.x;
+        const int m = i < n ? rep_cnt[i] : 0;
+        int k = 0;
+        for (int r = 0; r < m; ++r) k += rep_keep(i, rep_q[(size_t)r * n + i], rep_d[(size_t)r * n + i], cd64, pid);
+        int o = block_append(count, k, sh);
+        for (int r = 0; r < m; ++r) {
+            const int j = rep_q[(size_t)r * n + i];
+            const double D = rep_d[(size_t)r * n + i];
             if (!rep_keep(i, j, D, cd64, pid)) continue;
             const double c = __double_as_longlong(cd64[i]) >= __double_as_longlong(cd64[j]) ? cd64[i] : cd64[j];
             out[o++] = make_edge(__double_as_longlong(c) >= __double_as_longlong(D) ? c : D, pid[i], pid[j]);
@@ -516,16 +646,25 @@ __global__ void core_out_kernel(const double *__restrict__ cd64, const int *__re
 
 }  // namespace
 
-int core_distances(Points &P, Tree &T, int min_pts, bool fp64, HdbState &H, Arena &ar, cudaStream_t st, int *pin,
-                   wm_stats *stats)
+// Shared memory limits of the kernels above.  They are set to the same value by every call: a limit that
+// followed the call's own size could be lowered by a concurrent call (batch groups, server workers)
+// between another call's setting and its launch.
+constexpr int kWalkSmemMax = 100 << 10;    // (kWalkStack + minPts) entries for at least 32 threads
+constexpr int kTieSmemMax = 64 << 10;      // stacks of kTieWarps warps in the deepest tree (FP32 exponents
+                                           // and mantissas allow about 3800 levels in 16 dimensions)
+constexpr int kKnn64SmemMax = 128 << 10;   // lists of minPts + 8 entries and a stack for one warp
+static_assert((kWalkStack + kMaxMinPts) * 32 * 8 <= kWalkSmemMax && (kMaxMinPts + 8) * 32 * 12 + 3800 * 4 <= kKnn64SmemMax,
+              "shared memory limits of the k-NN kernels");
+
+// core distances and repair edges; X: the search tree (without it, or in the FP64 form, all in FP64)
+int core_distances(Points &P, Tree &T, const SearchTree *X, int min_pts, bool fp64, HdbState &H, Arena &ar,
+                   cudaStream_t st, int *pin, wm_stats *stats)
 {
     const int n = P.n, d = P.d, N = T.N;
     if (min_pts > kMaxMinPts) return WM_EINVAL;
     const int KL = std::min(min_pts + 8, n);
     H.cd64 = ar.get<double>(n);
     H.cd32 = ar.get<float>(n);
-    H.cdmin = ar.get<float>(N);
-    H.cdmax = ar.get<float>(N);
     if (ar.failed) return WM_ENOMEM;
     // persistent output of this function: repair edges (allocated before the scratch)
     const int RQ = KL > 1 ? KL - 1 : 1;
@@ -534,66 +673,118 @@ int core_distances(Points &P, Tree &T, int min_pts, bool fp64, HdbState &H, Aren
     if (!rep) return WM_ENOMEM;
     size_t mark = ar.off;
     KnnArgs a;
+    memset(&a, 0, sizeof a);
     a.N = N; a.n = n; a.d = d; a.k = min_pts; a.KL = KL;
-    a.lo = T.lo; a.hi = T.hi; a.begin = T.begin; a.end = T.end; a.left = T.left; a.right = T.right;
     a.x32 = P.x32; a.x64 = P.x64;
-    a.eta = fp64 ? 0.0 : 2.0 * (double)P.delta * sqrt((double)d) * (1.0 + 1e-6);
     a.stack_cap = T.depth + 4;
     a.cd64 = H.cd64; a.cd32 = H.cd32;
+    a.rq = RQ;
     a.rep_q = ar.get<int>((size_t)n * RQ);
     a.rep_d = ar.get<double>((size_t)n * RQ);
     a.rep_cnt = ar.get<int>(n + 1);
     a.slow = ar.get<int>(n);
+    a.slow_s = ar.get<float>(n);
+    int *slow2 = ar.get<int>(n);
+    // [0] queries with ties, [1] overflow edges, [2] overflow flag, [3] repair edges, [4] dispenser of
+    // the tie kernel, [5] error, [6] dispenser of the walk, [7] queries left for the full scan
     int *cnts = ar.get<int>(8);
     a.slow_cnt = cnts;
     a.stat = ar.get<unsigned long long>(4);
     int *ex_p = ar.get<int>(extra_cap), *ex_q = ar.get<int>(extra_cap);
     double *ex_d = ar.get<double>(extra_cap);
-    double *nmin = ar.get<double>(N), *nmax = ar.get<double>(N);
-    int *off = ar.get<int>(n + 1);
     if (ar.failed) return WM_ENOMEM;
     cudaMemsetAsync(cnts, 0, 8 * sizeof(int), st);
     cudaMemsetAsync(a.stat, 0, 4 * sizeof(unsigned long long), st);
-    // launch shape: warps per block limited by shared memory; the grid fills the SMs
-    const int dmp = d <= 3 ? 4 : d <= 7 ? 8 : 16;   // = knn_dmp<DM> of the instantiation used
-    size_t per_warp = knn_warp_smem(dmp, KL, fp64 ? 8 : 4, a.stack_cap);
-    int wpb = (int)std::min<size_t>(8, std::max<size_t>(1, (48u << 10) / per_warp));
-    size_t smem = per_warp * wpb;
-    int blocks = num_sms() * std::max(1, 32 / wpb);
-    int total_warps = blocks * wpb;
     a.next_group = cnts + 6;
     a.err = cnts + 5;
-    a.wscratch = ar.get<double>((size_t)total_warps * KL * 32);
-    // packed node records and boxes (the traversal reads a node with two or three vector loads)
-    NodeRec *rec = ar.get<NodeRec>(N);
-    float *box = ar.get<float>((size_t)N * 2 * dmp);
-    if (!a.wscratch || !rec || !box) return WM_ENOMEM;
-    pack_nodes(T, d, dmp, rec, box, st);
-    a.rec = rec;
-    a.box = box;
-#define WM_KNN(DM)                                                                                           \
-    do {                                                                                                     \
-        if (fp64) {                                                                                          \
-            cudaFuncSetAttribute(knn_fast_kernel<DM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
-            launch(knn_fast_kernel<DM, true>, blocks, 32 * wpb, smem, st, a);                                    \
-        } else {                                                                                             \
-            cudaFuncSetAttribute(knn_fast_kernel<DM, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
-            launch(knn_fast_kernel<DM, false>, blocks, 32 * wpb, smem, st, a);                                   \
-        }                                                                                                    \
-    } while (0)
     cudaEvent_t k0, k1;
     cudaEventCreate(&k0);
     cudaEventCreate(&k1);
-    cudaEventRecord(k0, st);
-    if (d <= 2) WM_KNN(2);
-    else if (d <= 3) WM_KNN(3);
-    else if (d <= 5) WM_KNN(5);
-    else if (d <= 7) WM_KNN(7);
-    else WM_KNN(16);
+    if (fp64 || !X->rows) {
+        // launch shape: warps per block limited by shared memory; the grid fills the SMs
+        const int dmp = d <= 3 ? 4 : d <= 7 ? 8 : 16;   // = knn_dmp<DM> of the instantiation used
+        const size_t per_warp = knn_warp_smem(KL, a.stack_cap);
+        const int wpb = (int)std::min<size_t>(8, std::max<size_t>(1, (48u << 10) / per_warp));
+        const size_t smem = per_warp * wpb;
+        const int blocks = num_sms() * std::max(1, 32 / wpb);
+        // packed node records and boxes (the traversal reads a node with two or three vector loads)
+        NodeRec *rec = ar.get<NodeRec>(N);
+        float *box = ar.get<float>((size_t)N * 2 * dmp);
+        if (!rec || !box) { cudaEventDestroy(k0); cudaEventDestroy(k1); return WM_ENOMEM; }
+        pack_nodes(T, d, dmp, rec, box, st);
+        a.rec = rec;
+        a.box = box;
+        cudaEventRecord(k0, st);
+#define WM_KNN(DM)                                                                                            \
+    do {                                                                                                      \
+        cudaFuncSetAttribute(knn64_kernel<DM>, cudaFuncAttributeMaxDynamicSharedMemorySize, kKnn64SmemMax);   \
+        launch(knn64_kernel<DM>, blocks, 32 * wpb, smem, st, a);                                              \
+    } while (0)
+        if (d <= 2) WM_KNN(2);
+        else if (d <= 3) WM_KNN(3);
+        else if (d <= 5) WM_KNN(5);
+        else if (d <= 7) WM_KNN(7);
+        else WM_KNN(16);
 #undef WM_KNN
-    cudaEventRecord(k1, st);
-    cudaMemcpyAsync(pin, cnts, sizeof(int), cudaMemcpyDeviceToHost, st);
-    if (cudaStreamSynchronize(st) != cudaSuccess) {
+        cudaEventRecord(k1, st);
+        cudaMemcpyAsync(cnts + 7, cnts, sizeof(int), cudaMemcpyDeviceToDevice, st);   // all ties: the full scan
+        slow2 = a.slow;
+    } else {
+        TravArgs band;
+        band.eta = 2.0 * (double)P.delta * sqrt((double)d) * (1.0 + 1e-6);
+        band.exact32 = band.eta == 0.0;
+        band.eta2_f = (float)(2.0 * band.eta);
+        if ((double)band.eta2_f < 2.0 * band.eta) band.eta2_f = std::nextafter(band.eta2_f, INFINITY);
+        // threads per block: four warps while two blocks of them fit an SM's shared memory
+        const size_t per_thread = (size_t)(kWalkStack + min_pts) * sizeof(uint2);
+        int threads = kWalkThreads;
+        while (threads > 32 && per_thread * threads > (size_t)kWalkSmemMax) threads >>= 1;
+        const size_t smem = per_thread * threads;
+        const size_t smem_tie = (size_t)kTieWarps * (X->stack_cap + 2) * sizeof(unsigned);
+        int rc = 0;
+#define WM_KNN(DM)                                                                                            \
+    do {                                                                                                      \
+        int per_sm = 0;                                                                                       \
+        if (cudaFuncSetAttribute(knn_walk_kernel<DM>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWalkSmemMax) != cudaSuccess || \
+            cudaFuncSetAttribute(knn_tie_kernel<DM>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTieSmemMax) != cudaSuccess || \
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, knn_walk_kernel<DM>, threads, smem) != cudaSuccess || \
+            per_sm < 1) {                                                                                     \
+            rc = WM_ECUDA;                                                                                    \
+            break;                                                                                            \
+        }                                                                                                     \
+        const int blocks = (int)std::min<long long>(std::min<long long>((long long)num_sms() * per_sm,        \
+                                                    (long long)X->walk_blocks * (kWalkThreads / threads)),    \
+                                                    ((long long)n + threads - 1) / threads);                  \
+        cudaEventRecord(k0, st);                                                                              \
+        launch(knn_walk_kernel<DM>, blocks, threads, smem, st, a, *X, band);                                  \
+        launch(knn_tie_kernel<DM>, num_sms() * 4, 32 * kTieWarps, smem_tie, st, a, *X, band, cnts, cnts + 4, slow2,   \
+               cnts + 7, ex_q, ex_p, ex_d, cnts + 1, extra_cap, cnts + 2);                                    \
+        cudaEventRecord(k1, st);                                                                              \
+    } while (0)
+        const int wd = walk_dim(d);
+        if (row_floats(wd) != X->S) rc = WM_EINTERNAL;
+        else switch (wd) {
+            case 2: WM_KNN(2); break;
+            case 3: WM_KNN(3); break;
+            case 4: WM_KNN(4); break;
+            case 5: WM_KNN(5); break;
+            case 6: WM_KNN(6); break;
+            case 7: WM_KNN(7); break;
+            case 8: WM_KNN(8); break;
+            case 15: WM_KNN(15); break;
+            default: WM_KNN(16); break;
+            }
+#undef WM_KNN
+        if (rc) {
+            cudaGetLastError();
+            cudaEventDestroy(k0);
+            cudaEventDestroy(k1);
+            set_error_detail("k-NN: the launch configuration was refused");
+            return rc;
+        }
+    }
+    cudaMemcpyAsync(pin, cnts, 8 * sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (cudaPeekAtLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) {
         cudaEventDestroy(k0);
         cudaEventDestroy(k1);
         return WM_ECUDA;
@@ -605,23 +796,15 @@ int core_distances(Points &P, Tree &T, int min_pts, bool fp64, HdbState &H, Aren
     }
     cudaEventDestroy(k0);
     cudaEventDestroy(k1);
-    const int nslow = pin[0];
+    const int nslow = pin[7];
     if (nslow > 0) {
         size_t sm2 = (size_t)min_pts * 32 * 8 + 32 * 4;
-        cudaFuncSetAttribute(knn_slow_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
-        launch(knn_slow_kernel, std::min(nslow, num_sms() * 8), 32, sm2, st, a, a.slow, nslow, ex_q, ex_p, ex_d, cnts + 1,
+        cudaFuncSetAttribute(knn_slow_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxMinPts * 32 * 8 + 32 * 4);
+        launch(knn_slow_kernel, std::min(nslow, num_sms() * 8), 32, sm2, st, a, slow2, nslow, ex_q, ex_p, ex_d, cnts + 1,
                                                                      extra_cap, cnts + 2);
     }
-    // node bounds
-    cudaMemsetAsync(T.arrive, 0, sizeof(int) * N, st);
-    launch(cd_bounds_kernel, grid_for(N, 256), 256, 0, st, N, T.left, T.right, T.parent, T.begin, H.cd64, nmin, nmax,
-                                                       H.cdmin, H.cdmax, T.arrive);
-    // repair edges: one copy of each, weighted, in no particular order (each MemoGFK round takes
-    // those of its weight range)
-    launch(rep_flags_kernel, grid_for(n, 256), 256, 0, st, a.rep_q, a.rep_d, a.rep_cnt, n, KL, H.cd64, P.pid, off);
-    int rc = scan_exclusive_i32(off, off, n, cnts + 3, st, ar);
-    if (rc) return rc;
-    launch(rep_emit_kernel, grid_for(n, 256), 256, 0, st, a.rep_q, a.rep_d, a.rep_cnt, off, n, KL, H.cd64, P.pid, rep);
+    // repair edges: one copy of each, weighted, in no particular order (each round takes those it needs)
+    launch(rep_emit_kernel, grid_for(n, 256), 256, 0, st, a.rep_q, a.rep_d, a.rep_cnt, n, H.cd64, P.pid, rep, cnts + 3);
     launch(rep_emit_extra_kernel, grid_for(extra_cap, 256), 256, 0, st, ex_p, ex_q, ex_d, cnts + 1, extra_cap, H.cd64,
            P.pid, rep, cnts + 3);
     cudaMemcpyAsync(pin, cnts, 8 * sizeof(int), cudaMemcpyDeviceToHost, st);
@@ -646,7 +829,21 @@ int core_distances(Points &P, Tree &T, int min_pts, bool fp64, HdbState &H, Aren
     H.rep = rep;
     H.nrep = nrep;
     ar.off = mark;
-    // keep the cd arrays and node bounds (allocated before mark); drop the scratch
+    // keep the cd arrays (allocated before mark); drop the scratch
+    return 0;
+}
+
+// node bounds of the core distances for the WSPD traversals (T.arrive is scratch)
+int node_core_bounds(const Tree &T, const HdbState &H, float *cdmin, float *cdmax, Arena &ar, cudaStream_t st)
+{
+    const int N = T.N;
+    size_t mark = ar.off;
+    double *nmin = ar.get<double>(N), *nmax = ar.get<double>(N);
+    if (ar.failed) return WM_ENOMEM;
+    cudaMemsetAsync(T.arrive, 0, sizeof(int) * N, st);
+    launch(cd_bounds_kernel, grid_for(N, 256), 256, 0, st, N, T.left, T.right, T.parent, T.begin, H.cd64, nmin, nmax, cdmin,
+           cdmax, T.arrive);
+    ar.off = mark;
     return 0;
 }
 
