@@ -123,7 +123,8 @@ typedef struct {
     int64_t knn_evals;         /* point-pair distance evaluations in the k-NN pass   */
     int64_t fp64_rechecks;     /* FP64 re-evaluations of screened candidates         */
     int64_t candidate_edges;   /* edges handed to Kruskal over all rounds            */
-    int64_t tree_nodes;
+    int64_t tree_nodes;        /* nodes of the k-d tree down to single points, 2 n - 1 (the
+                                  search tree stores those above its buckets of 8 points)  */
     int64_t tree_depth;
     size_t workspace_bytes_used;   /* peak workspace use of this call               */
     double max_rel_screen_err;     /* largest |fp32 - fp64| / fp64 between a screened FP32

@@ -8,7 +8,6 @@
 #include <cstring>
 #include <condition_variable>
 #include <deque>
-#include <functional>
 #include <mutex>
 #include <thread>
 #include <unordered_map>
@@ -186,6 +185,7 @@ static size_t estimate_bytes(long long n, int d, int min_pts, const Caps &c)
         b += (size_t)n * 12 + (size_t)n * 8;            // cd64, cd32, node bounds
         b += (size_t)n * kk * 16 * 2;                   // repair edges + sort tmp
         b += (size_t)n * 192;                           // dendrogram / Euler tour scratch
+        b += (size_t)n * (24 * row_floats(d) + 64);     // search tree beside the traversals' tree
     }
     return b + (8u << 20) + (size_t)n * 64 + (size_t)c.extra_bytes;
 }
@@ -265,6 +265,18 @@ __global__ void init_uf_kernel(int *uf, unsigned long long *R, int n)
         R[n + i] = ~0ull;
         R[2LL * n + i] = ~0ull;
         R[3LL * n + i] = ~0ull;
+    }
+}
+
+// core distances from one tree order into another (pid: ids of the new positions, pos: old positions)
+__global__ void reorder_core_kernel(int n, const int *__restrict__ pid, const int *__restrict__ pos,
+                                    const double *__restrict__ cd64, const float *__restrict__ cd32, double *__restrict__ out64,
+                                    float *__restrict__ out32)
+{
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const int j = pos[pid[i]];
+        out64[i] = cd64[j];
+        out32[i] = cd32[j];
     }
 }
 
@@ -455,12 +467,99 @@ static bool nearest_rounds_apply(const Call &C, int n, int d, const HdbState *hd
     return hdb ? C.disjunctive && !C.stats.tie_overflow : d <= 8;
 }
 
-// The spanning tree: nearest-component rounds where they apply, else (or for what they leave) MemoGFK
-// rounds (Algorithm 3).  On return E_out holds the tree edges in K order: n-1 of them, or
+// The spanning tree by nearest-component rounds, as memogfk returns it: its edges in K order, n-1 of them
+// or `target` below rho_cap.
+static int nearest_tree(Call &C, const Points &P, const SearchTree &X, const HdbState *hdb, EdgeK *E_out,
+                        long long target = -1, double rho_cap = INFINITY)
+{
+    const int n = P.n;
+    if (target < 0) target = (long long)n - 1;
+    if (n <= 1) return 0;
+    cudaStream_t st = C.st;
+    Arena &ar = C.ar;
+    const size_t mark = ar.off;
+    Timer tn;
+    unsigned *ovf = ar.get<unsigned>(2);
+    unsigned long long *stat = ar.get<unsigned long long>(16);
+    if (ar.failed) return WM_ENOMEM;
+    WM_CK(cudaMemsetAsync(stat, 0, 16 * sizeof(unsigned long long), st));
+    WM_CK(cudaMemsetAsync(ovf, 0, 2 * sizeof(unsigned), st));
+    TravArgs a;
+    a.n = n; a.d = P.d;
+    a.x64 = P.x64; a.pid = P.pid;
+    a.eta = 2.0 * (double)P.delta * std::sqrt((double)P.d) * (1.0 + 1e-6);
+    a.eta2_f = float_ru(2.0 * a.eta);
+    a.exact32 = a.eta == 0.0;
+    if (hdb) { a.cd32 = hdb->cd32; a.cd64 = hdb->cd64; }
+    a.overflow = ovf;
+    a.stat = stat;
+    // CUDA-event intervals of the search kernel (when C.timing)
+    struct Spans {
+        std::vector<cudaEvent_t> evs;
+        int dev = 0;
+        cudaStream_t st = nullptr;
+        bool on = false;
+        ~Spans() { return_events(dev, evs); }
+    } spans;
+    cudaGetDevice(&spans.dev);
+    spans.st = st;
+    spans.on = C.timing;
+    NcCall N;
+    N.st = st;
+    N.ar = &ar;
+    N.pin = C.pin;
+    N.X = &X;
+    N.pos = P.pos;
+    N.out = E_out;
+    N.target = target;
+    N.cap = rho_cap;
+    N.cap_f = float_ru(rho_cap);
+    N.rep = hdb ? hdb->rep : nullptr;
+    N.nrep = hdb ? hdb->nrep : 0;
+    N.ctx = &spans;
+    N.mark = [](void *p) {   // events in pairs: before and after a search
+        Spans &s = *(Spans *)p;
+        cudaEvent_t e = s.on ? pooled_event(s.dev) : nullptr;
+        if (!e) { s.on = false; return; }
+        cudaEventRecord(e, s.st);
+        s.evs.push_back(e);
+    };
+    WM_TRY(nearest_component_rounds(N, a));
+    if (N.done < target) {
+        set_detail("nearest-component rounds left the forest incomplete%s (%lld edges)", "", N.done);
+        return WM_EINTERNAL;
+    }
+    for (size_t i = 0; i + 1 < spans.evs.size(); i += 2) C.stats.ms_bccp_dual += C.event_ms(spans.evs[i], spans.evs[i + 1]);
+    C.stats.ms_bccp += tn.ms();
+    // every round appended its edges unordered: put the tree in K order
+    Timer ts;
+    EdgeK *tmp = ar.get<EdgeK>(n), *sorted = E_out;
+    if (ar.failed) return WM_ENOMEM;
+    WM_CK(cudaMemcpyAsync(C.pin, stat, 16 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
+    WM_TRY(radix_sort_edges(E_out, tmp, (int)target, st, ar, &sorted, C.pin + 4096));
+    if (sorted != E_out) WM_CK(cudaMemcpyAsync(E_out, sorted, sizeof(EdgeK) * target, cudaMemcpyDeviceToDevice, st));
+    WM_CK(cudaStreamSynchronize(st));
+    unsigned long long hs[16];
+    memcpy(hs, C.pin, sizeof hs);
+    C.stats.ms_kruskal += ts.ms();
+    C.stats.rounds = N.rounds;
+    C.stats.candidate_edges += N.candidates;
+    C.stats.bccp_evals = (int64_t)hs[1];
+    C.stats.bccp_dual_evals = (int64_t)hs[6];
+    C.stats.fp64_rechecks += (int64_t)hs[2];
+    float e;
+    const unsigned eb = (unsigned)hs[12];
+    memcpy(&e, &eb, sizeof e);
+    C.stats.max_rel_screen_err = std::max(C.stats.max_rel_screen_err, (double)e);
+    ar.off = mark;
+    return 0;
+}
+
+// MemoGFK rounds (Algorithm 3).  On return E_out holds the tree edges in K order: n-1 of them, or
 // `target` when the points form several instances that must not be joined (a batch): then every
 // edge weight is below rho_cap, rho_hi never exceeds it, and no pair at or above it is retrieved.
 // hdb: optional HDBSCAN* state (node cd bounds, per-position cd2, repair edges).
-static int memogfk(Call &C, Points &P, Tree &T, SearchTree &X, const HdbState *hdb, const Caps &caps, EdgeK *E_out, int *uf,
+static int memogfk(Call &C, Points &P, Tree &T, const HdbState *hdb, const Caps &caps, EdgeK *E_out, int *uf,
                    unsigned long long *R, unsigned *overflow_bits, long long target = -1, double rho_cap = INFINITY)
 {
     const int n = P.n;
@@ -470,16 +569,52 @@ static int memogfk(Call &C, Points &P, Tree &T, SearchTree &X, const HdbState *h
     *overflow_bits = 0;
     if (n <= 1) return 0;
     size_t mark = ar.off;
+    const int chunk = (int)caps.chunk;
+    const long long fcap = ((long long)T.N / 2 + 2 + (2LL * T.depth + 4) * 2 * chunk) * caps.frontier_scale;
+    if (fcap > 0x7fffffffLL) { set_detail("WSPD stack capacity exceeds 2^31 pairs%s", ""); return WM_ENOMEM; }
+    int2 *stack = ar.get<int2>(fcap);
+    int2 *const xbuf[2] = {ar.get<int2>(4LL * chunk), ar.get<int2>(4LL * chunk)};   // step outputs
+    // pair lists hold kListChunks chunks' worth of retrieved pairs; they are flushed (BCCP) when
+    // one of them could overflow within the next poll interval, and when the traversal ends
+    const int kPoll = 3, kListChunks = 8;
+    const long long lcap = (long long)kListChunks * chunk;
+    int2 *lists[5];
+    float *list_lbs[5];
+    for (int c = 0; c < 5; ++c) {
+        lists[c] = ar.get<int2>(lcap);
+        list_lbs[c] = ar.get<float>(lcap);
+    }
+    EdgeK *huge_best = ar.get<EdgeK>(lcap + 1);
+    unsigned *huge_sbest = ar.get<unsigned>(lcap + 1);
+    long long *huge_items = ar.get<long long>(lcap + 1);
+    const int stack_warps = num_sms() * 8 * 8;   // warps of the dual-tree kernel (grid-stride)
+    int *dual_stack = ar.get<int>((size_t)stack_warps * (T.depth + 4));
     const int dp = P.d <= 4 ? 4 : P.d <= 8 ? 8 : 16;
+    NodeRec *rec = ar.get<NodeRec>(T.N);
+    float *box = ar.get<float>((size_t)T.N * 2 * dp);
+    float4 *x4 = ar.get<float4>((size_t)n * (dp / 4));
+    EdgeK *batch = ar.get<EdgeK>(caps.edges), *filt = ar.get<EdgeK>(caps.edges), *tmp = ar.get<EdgeK>(caps.edges);
     int *cnts = ar.get<int>(64);
     unsigned *rho = ar.get<unsigned>(2);
+    int *split_hist = ar.get<int>(kSplitBins);
+    unsigned long long *split_max = ar.get<unsigned long long>(1);
     unsigned *ovf = ar.get<unsigned>(2);
     unsigned long long *stat = ar.get<unsigned long long>(16);
+    int *comp_scratch = ar.get<int>(2LL * n + 1);
     if (ar.failed) return WM_ENOMEM;
     // counters: [2..6] pair-list counts, [7] edge count, [10..11] counts of the two node lists,
     // [12..13] 64-bit huge-pair item total, [16..17] tile-kernel pair dispensers,
     // [32..32+kTravCounters) traversal state
     int *lcount = cnts + 2, *ecount = cnts + 7, *tcnt = cnts + 32;
+    Tree T2 = T;
+    if (hdb) {
+        T2.cdmin = ar.get<float>(T.N);
+        T2.cdmax = ar.get<float>(T.N);
+        if (ar.failed) return WM_ENOMEM;
+        WM_TRY(node_core_bounds(T, *hdb, T2.cdmin, T2.cdmax, ar, st));
+    }
+    pack_nodes(T2, P.d, dp, rec, box, st);
+    point_major(P.x32, n, P.d, dp, x4, st);
     WM_CK(cudaMemsetAsync(stat, 0, 16 * sizeof(unsigned long long), st));
     WM_CK(cudaMemsetAsync(ovf, 0, 2 * sizeof(unsigned), st));
     WM_CK(cudaMemsetAsync(cnts, 0, 64 * sizeof(int), st));
@@ -488,7 +623,7 @@ static int memogfk(Call &C, Points &P, Tree &T, SearchTree &X, const HdbState *h
     a.N = T.N; a.n = n; a.d = P.d;
     a.lo = T.lo; a.hi = T.hi; a.diam2 = T.diam2;
     a.begin = T.begin; a.end = T.end; a.left = T.left; a.right = T.right; a.comp = T.comp;
-    a.x32 = P.x32; a.x64 = P.x64; a.pid = P.pid;
+    a.x32 = P.x32; a.x4 = x4; a.x64 = P.x64; a.pid = P.pid;
     a.fp64 = C.precision == WM_PREC_FP64;
     a.eta = a.fp64 ? 0.0 : 2.0 * (double)P.delta * std::sqrt((double)P.d) * (1.0 + 1e-6);
     a.eta2_f = float_ru(2.0 * a.eta);
@@ -499,10 +634,28 @@ static int memogfk(Call &C, Points &P, Tree &T, SearchTree &X, const HdbState *h
     a.big_max = C.tune.big_max;
     a.disjunctive = C.disjunctive;
     a.rho_sample = C.tune.getrho_sample > 0 ? C.tune.getrho_sample : 1;
-    if (hdb) { a.cd32 = hdb->cd32; a.cd64 = hdb->cd64; }
-    a.dp = dp;
+    if (hdb) {
+        a.cdmin = T2.cdmin; a.cdmax = T2.cdmax; a.cd32 = hdb->cd32; a.cd64 = hdb->cd64;
+    }
+    a.frontier_cap = (int)fcap;
+    a.rec = rec; a.box = box; a.dp = dp;
+    for (int c = 0; c < 5; ++c) { a.list[c] = lists[c]; a.list_lb[c] = list_lbs[c]; a.list_cap[c] = (int)lcap; }
+    a.list_count = lcount;
+    a.big = lists[3]; a.big_count = lcount + 3;
+    a.huge_best = huge_best; a.huge_sbest = huge_sbest;
+    a.stack = dual_stack; a.stack_cap = T.depth + 4;
+    a.edges = batch; a.edge_count = ecount;
+    a.edge_cap = (int)(caps.edges_soft > 0 && caps.edges_soft < caps.edges ? caps.edges_soft : caps.edges);
     a.overflow = ovf;
     a.stat = stat;
+    a.rho_bits = rho;
+    EdgeK *spare = filt;   // second edge buffer for compaction when rho_hi shrinks
+    int *nodes[2] = {ar.get<int>(T.N / 2 + 1), ar.get<int>(T.N / 2 + 1)};
+    if (ar.failed) return WM_ENOMEM;
+    a.node_in = nullptr;
+    a.node_in_n = nullptr;
+    a.node_out = nodes[0];
+    a.node_out_n = cnts + 10;
 
     // CUDA-event intervals of the round's kernels (when C.timing), summed into the stats per kind
     enum { kSpanGetPairs, kSpanGetRho, kSpanFlush, kSpanGroup, kSpanTile, kSpanDual };
@@ -544,107 +697,7 @@ static int memogfk(Call &C, Points &P, Tree &T, SearchTree &X, const HdbState *h
         spans.clear();
         return 0;
     };
-    int nE = 0, rounds = 0;
-    if (nearest_rounds_apply(C, n, P.d, hdb)) {
-        Timer tn;
-        const size_t xmark = ar.off;
-        if (!X.rows) WM_TRY(build_search_tree(P, T, X, ar, st, C.pin));
-        struct Hooks {
-            std::function<int()> mark;
-            std::function<void(int, int)> span;
-        } hooks{[&] { return mark_event(); }, [&](int i, int j) { add_span(i, j, kSpanDual); }};
-        NcCall N;
-        N.st = st;
-        N.ar = &ar;
-        N.pin = C.pin;
-        N.X = &X;
-        N.pos = P.pos;
-        N.uf = uf;
-        N.out = E_out;
-        N.target = target;
-        N.cap = rho_cap;
-        N.cap_f = float_ru(rho_cap);
-        N.rep = hdb ? hdb->rep : nullptr;
-        N.nrep = hdb ? hdb->nrep : 0;
-        N.ctx = &hooks;
-        N.mark = [](void *h) { return ((Hooks *)h)->mark(); };
-        N.span = [](void *h, int i, int j) { ((Hooks *)h)->span(i, j); };
-        WM_TRY(nearest_component_rounds(N, a));
-        WM_TRY(collect_spans());
-        nE = (int)N.done;
-        rounds = N.rounds;
-        C.stats.candidate_edges += N.candidates;
-        C.stats.ms_bccp += tn.ms();
-        ar.off = xmark;
-        X.rows = nullptr;   // its memory is released, or its labels are used up
-    }
-    // ---- MemoGFK state
-    const int chunk = (int)caps.chunk;
-    const int kPoll = 3, kListChunks = 8;
-    const long long lcap = (long long)kListChunks * chunk;
-    int2 *stack = nullptr, *xbuf[2] = {nullptr, nullptr}, *lists[5] = {};
-    float *list_lbs[5] = {};
-    long long *huge_items = nullptr;
-    const int stack_warps = num_sms() * 8 * 8;   // warps of the dual-tree kernel (grid-stride)
-    EdgeK *batch = nullptr, *filt = nullptr, *tmp = nullptr;
-    int *split_hist = nullptr, *comp_scratch = nullptr, *nodes[2] = {nullptr, nullptr};
-    unsigned long long *split_max = nullptr;
-    NodeRec *rec = nullptr;
-    if (nE < target) {
-        Tree T2 = T;
-        if (hdb) {
-            T2.cdmin = ar.get<float>(T.N);
-            T2.cdmax = ar.get<float>(T.N);
-            if (ar.failed) return WM_ENOMEM;
-            WM_TRY(node_core_bounds(T, *hdb, T2.cdmin, T2.cdmax, ar, st));
-            a.cdmin = T2.cdmin;
-            a.cdmax = T2.cdmax;
-        }
-        rec = ar.get<NodeRec>(T.N);
-        float *box = ar.get<float>((size_t)T.N * 2 * dp);
-        float4 *x4 = ar.get<float4>((size_t)n * (dp / 4));
-        if (ar.failed) return WM_ENOMEM;
-        pack_nodes(T2, P.d, dp, rec, box, st);
-        point_major(P.x32, n, P.d, dp, x4, st);
-        a.rec = rec; a.box = box; a.x4 = x4;
-        const long long fcap = ((long long)T.N / 2 + 2 + (2LL * T.depth + 4) * 2 * chunk) * caps.frontier_scale;
-        if (fcap > 0x7fffffffLL) { set_detail("WSPD stack capacity exceeds 2^31 pairs%s", ""); return WM_ENOMEM; }
-        stack = ar.get<int2>(fcap);
-        for (int i = 0; i < 2; ++i) xbuf[i] = ar.get<int2>(4LL * chunk);   // step outputs
-        // pair lists hold kListChunks chunks' worth of retrieved pairs; they are flushed (BCCP) when
-        // one of them could overflow within the next poll interval, and when the traversal ends
-        for (int c = 0; c < 5; ++c) {
-            lists[c] = ar.get<int2>(lcap);
-            list_lbs[c] = ar.get<float>(lcap);
-        }
-        a.huge_best = ar.get<EdgeK>(lcap + 1);
-        a.huge_sbest = ar.get<unsigned>(lcap + 1);
-        huge_items = ar.get<long long>(lcap + 1);
-        a.stack = ar.get<int>((size_t)stack_warps * (T.depth + 4));
-        batch = ar.get<EdgeK>(caps.edges);
-        filt = ar.get<EdgeK>(caps.edges);
-        tmp = ar.get<EdgeK>(caps.edges);
-        split_hist = ar.get<int>(kSplitBins);
-        split_max = ar.get<unsigned long long>(1);
-        comp_scratch = ar.get<int>(2LL * n + 1);
-        for (int i = 0; i < 2; ++i) nodes[i] = ar.get<int>(T.N / 2 + 1);
-        a.frontier_cap = (int)fcap;
-    } else {
-        tmp = ar.get<EdgeK>(n);   // the final sort's second buffer
-    }
-    if (ar.failed) return WM_ENOMEM;
-    for (int c = 0; c < 5; ++c) { a.list[c] = lists[c]; a.list_lb[c] = list_lbs[c]; a.list_cap[c] = (int)lcap; }
-    a.list_count = lcount;
-    a.big = lists[3]; a.big_count = lcount + 3;
-    a.stack_cap = T.depth + 4;
-    a.edges = batch; a.edge_count = ecount;
-    a.edge_cap = (int)(caps.edges_soft > 0 && caps.edges_soft < caps.edges ? caps.edges_soft : caps.edges);
-    a.rho_bits = rho;
-    EdgeK *spare = filt;   // second edge buffer for compaction when rho_hi shrinks
-    a.node_in = nullptr;
-    a.node_in_n = nullptr;
-    a.node_out = nodes[0];
-    a.node_out_n = cnts + 10;
+    int nE = 0;
     double rho_lo = 0.0;
     long long beta = 2;
     // tuning combined = 2: rounds start as two passes; once, after two rounds or more, the GetRho
@@ -654,6 +707,7 @@ static int memogfk(Call &C, Points &P, Tree &T, SearchTree &X, const HdbState *h
     constexpr double kOnePassRatio = 0.5;
     bool adaptive_one_pass = false;
     const double inf = INFINITY;
+    int rounds = 0;
     while (nE < target) {
         if (++rounds > 4096) { set_detail("MemoGFK made no progress%s (%lld rounds)", "", rounds); return WM_EINTERNAL; }
         Timer tw;
@@ -1145,41 +1199,60 @@ static int gfk_rounds(Call &C, Points &P, Tree &T, const HdbState *hdb, const Ca
 }
 
 // ---------------------------------------------------------------------- shared front half
+// A call's points and tree: the traversals' k-d tree T (single-point leaves, SoA coordinates), or the
+// walks' search tree X.
 struct Prepared {
     Points P;
     Tree T;
-    SearchTree X;   // built where the FP32-screened walks need it (rows is null otherwise)
+    SearchTree X;
+    const void *src = nullptr;   // the input on the device
 };
 
+static int input_on_device(Call &C, const void *pts, int64_t n, int32_t d, int32_t dtype, Prepared &S)
+{
+    S.src = pts;
+    if (!is_device_ptr(pts)) {
+        const size_t bytes = (size_t)n * d * (dtype == WM_F32 ? 4 : 8);
+        void *buf = C.ar.take(bytes);
+        if (!buf) return WM_ENOMEM;
+        WM_CK(cudaMemcpyAsync(buf, pts, bytes, cudaMemcpyHostToDevice, C.st));
+        S.src = buf;
+    }
+    return 0;
+}
+
+static int bad_coordinate(int rc)
+{
+    if (rc == WM_EINVAL) set_detail("non-finite coordinate or |coordinate| > 2^60%s", "");
+    return rc;
+}
+
+// for the traversals
 static int prepare(Call &C, const void *pts, int64_t n, int32_t d, int32_t dtype, int32_t layout, Prepared &S)
 {
     cudaStream_t st = C.st;
-    const void *dsrc = pts;
-    size_t bytes = (size_t)n * d * (dtype == WM_F32 ? 4 : 8);
-    if (!is_device_ptr(pts)) {
-        void *buf = C.ar.take(bytes);
-        if (!buf) return WM_ENOMEM;
-        WM_CK(cudaMemcpyAsync(buf, pts, bytes, cudaMemcpyHostToDevice, st));
-        dsrc = buf;
-    }
+    WM_TRY(input_on_device(C, pts, n, d, dtype, S));
     Timer ti;
-    int rc = ingest_points(dsrc, (int)n, d, dtype, layout, S.P, C.ar, st, (unsigned *)C.pin);
-    if (rc == WM_EINVAL) { set_detail("non-finite coordinate or |coordinate| > 2^60%s", ""); return rc; }
-    if (rc) return rc;
+    WM_TRY(bad_coordinate(ingest_points(S.src, (int)n, d, dtype, layout, S.P, C.ar, st, (unsigned *)C.pin)));
     C.stats.ms_ingest = ti.ms();
     Timer tt;
     WM_TRY(build_tree(S.P, S.T, C.ar, st, C.pin, C.tune.tight_diameters != 0));
-    C.stats.ms_build_tree = tt.ms();
+    C.stats.ms_build_tree += tt.ms();
     C.stats.tree_nodes = S.T.N;
     C.stats.tree_depth = S.T.depth;
     return 0;
 }
 
-// the k-NN pass of the FP32 screen walks the search tree (positions of 28 bits)
-static int search_tree_for_knn(Call &C, Prepared &S)
+// for the walks (n < 2^28)
+static int prepare_walk(Call &C, const void *pts, int64_t n, int32_t d, int32_t dtype, int32_t layout, Prepared &S)
 {
-    if (C.precision == WM_PREC_FP64 || S.P.n >= 1 << 28) return 0;
-    return build_search_tree(S.P, S.T, S.X, C.ar, C.st, C.pin);
+    WM_TRY(input_on_device(C, pts, n, d, dtype, S));
+    Timer tt;
+    WM_TRY(bad_coordinate(build_search_tree(S.src, (int)n, d, dtype, layout, S.P, S.X, C.ar, C.st, C.pin)));
+    C.stats.ms_build_tree += tt.ms();
+    C.stats.tree_nodes = 2 * n - 1;   // down to single points; X stores those above its buckets
+    C.stats.tree_depth = S.X.depth;
+    return 0;
 }
 
 static int write_edges(Call &C, const EdgeK *E, int m, wm_edge *out, double *total)
@@ -1330,23 +1403,55 @@ struct EmstCtx {
     double *total;
 };
 
+// EdgeK tree of an EMST or, with min_pts >= 1, of HDBSCAN* (core distances in H, by position of S.P)
+static int spanning_tree(Call &C, const void *pts, int64_t n64, int d, int dtype, int layout, int min_pts, const Caps &caps,
+                         Prepared &S, HdbState &H, EdgeK *&E, unsigned *ovf, long long target = -1, double cap = INFINITY)
+{
+    const int n = (int)n64;
+    const bool hdb = min_pts >= 1, wspd_form = C.method == WM_METHOD_GFK || C.method == WM_METHOD_NAIVE;
+    // the FP32-screened k-NN pass and the nearest-component rounds walk the search tree
+    const bool walk = hdb ? C.precision != WM_PREC_FP64 && n < 1 << 28 : !wspd_form && nearest_rounds_apply(C, n, d, nullptr);
+    if (walk) WM_TRY(prepare_walk(C, pts, n64, d, dtype, layout, S));
+    else WM_TRY(prepare(C, pts, n64, d, dtype, layout, S));
+    if (hdb) {
+        Timer tc;
+        WM_TRY(core_distances(S.P, &S.T, walk ? &S.X : nullptr, min_pts, H, C.ar, C.st, C.pin, &C.stats));
+        C.stats.ms_core_dist = tc.ms();
+    }
+    E = C.ar.get<EdgeK>(n);
+    if (C.ar.failed) return WM_ENOMEM;
+    if (walk && !wspd_form && nearest_rounds_apply(C, n, d, hdb ? &H : nullptr))
+        return nearest_tree(C, S.P, S.X, hdb ? &H : nullptr, E, target, cap);
+    // the traversals: with their own tree, and the core distances in its order
+    Prepared Q;
+    HdbState HQ = H;
+    if (walk) {
+        WM_TRY(prepare(C, S.src, n64, d, dtype, layout, Q));
+        HQ.cd64 = C.ar.get<double>(n);
+        HQ.cd32 = C.ar.get<float>(n);
+        if (C.ar.failed) return WM_ENOMEM;
+        launch(reorder_core_kernel, grid_for(n, 256), 256, 0, C.st, n, Q.P.pid, S.P.pos, H.cd64, H.cd32, HQ.cd64, HQ.cd32);
+    } else {
+        Q = S;
+    }
+    int *uf = C.ar.get<int>(n);
+    unsigned long long *R = C.ar.get<unsigned long long>(4LL * n);
+    if (C.ar.failed) return WM_ENOMEM;
+    launch(init_uf_kernel, grid_for(n, 256), 256, 0, C.st, uf, R, n);
+    if (wspd_form)
+        return gfk_rounds(C, Q.P, Q.T, hdb ? &HQ : nullptr, caps, E, uf, R, ovf, C.method == WM_METHOD_NAIVE);
+    return memogfk(C, Q.P, Q.T, hdb ? &HQ : nullptr, caps, E, uf, R, ovf, target, cap);
+}
+
 static int emst_body(Call &C, void *vctx, const Caps &caps, unsigned *ovf)
 {
     EmstCtx &x = *(EmstCtx *)vctx;
     Prepared S;
-    WM_TRY(prepare(C, x.pts, x.n, x.d, x.dtype, x.layout, S));
-    const int n = (int)x.n;
-    int *uf = C.ar.get<int>(n);
-    unsigned long long *R = C.ar.get<unsigned long long>(4LL * n);
-    EdgeK *E = C.ar.get<EdgeK>(n);
-    if (C.ar.failed) return WM_ENOMEM;
-    launch(init_uf_kernel, grid_for(n, 256), 256, 0, C.st, uf, R, n);
-    if (C.method == WM_METHOD_GFK || C.method == WM_METHOD_NAIVE)
-        WM_TRY(gfk_rounds(C, S.P, S.T, nullptr, caps, E, uf, R, ovf, C.method == WM_METHOD_NAIVE));
-    else
-        WM_TRY(memogfk(C, S.P, S.T, S.X, nullptr, caps, E, uf, R, ovf));
+    HdbState H;
+    EdgeK *E = nullptr;
+    WM_TRY(spanning_tree(C, x.pts, x.n, x.d, x.dtype, x.layout, 0, caps, S, H, E, ovf));
     if (*ovf) return 0;
-    return write_edges(C, E, n - 1, x.out, x.total);
+    return write_edges(C, E, (int)x.n - 1, x.out, x.total);
 }
 
 struct HdbCtx {
@@ -1364,23 +1469,11 @@ static int hdbscan_body(Call &C, void *vctx, const Caps &caps, unsigned *ovf)
 {
     HdbCtx &x = *(HdbCtx *)vctx;
     Prepared S;
-    WM_TRY(prepare(C, x.pts, x.n, x.d, x.dtype, x.layout, S));
-    const int n = (int)x.n;
     HdbState H;
-    Timer tc;
-    WM_TRY(search_tree_for_knn(C, S));
-    WM_TRY(core_distances(S.P, S.T, &S.X, x.min_pts, C.precision == WM_PREC_FP64, H, C.ar, C.st, C.pin, &C.stats));
-    C.stats.ms_core_dist = tc.ms();
-    int *uf = C.ar.get<int>(n);
-    unsigned long long *R = C.ar.get<unsigned long long>(4LL * n);
-    EdgeK *E = C.ar.get<EdgeK>(n);
-    if (C.ar.failed) return WM_ENOMEM;
-    launch(init_uf_kernel, grid_for(n, 256), 256, 0, C.st, uf, R, n);
-    if (C.method == WM_METHOD_GFK || C.method == WM_METHOD_NAIVE)
-        WM_TRY(gfk_rounds(C, S.P, S.T, &H, caps, E, uf, R, ovf, C.method == WM_METHOD_NAIVE));
-    else
-        WM_TRY(memogfk(C, S.P, S.T, S.X, &H, caps, E, uf, R, ovf));
+    EdgeK *E = nullptr;
+    WM_TRY(spanning_tree(C, x.pts, x.n, x.d, x.dtype, x.layout, x.min_pts, caps, S, H, E, ovf));
     if (*ovf) return 0;
+    const int n = (int)x.n;
     WM_TRY(write_core_distances(S.P, H, x.cd, C.ar, C.st));
     WM_TRY(write_edges(C, E, n - 1, x.mst, nullptr));
     Timer td;
@@ -1541,20 +1634,9 @@ static int batch_body(Call &C, void *vctx, const Caps &caps, unsigned *ovf)
     batch_scale(raw + (size_t)d * total, total, L, st);
     // ---- the joint problem
     Prepared S;
-    WM_TRY(prepare(C, raw, total, D, WM_F64, WM_SOA, S));
     HdbState H;
-    if (hdb) {
-        Timer tc;
-        WM_TRY(search_tree_for_knn(C, S));
-        WM_TRY(core_distances(S.P, S.T, &S.X, x.min_pts, C.precision == WM_PREC_FP64, H, ar, st, C.pin, &C.stats));
-        C.stats.ms_core_dist = tc.ms();
-    }
-    int *uf = ar.get<int>(n);
-    unsigned long long *R = ar.get<unsigned long long>(4LL * n);
-    EdgeK *E = ar.get<EdgeK>(n);
-    if (ar.failed) return WM_ENOMEM;
-    launch(init_uf_kernel, grid_for(n, 256), 256, 0, st, uf, R, n);
-    WM_TRY(memogfk(C, S.P, S.T, S.X, hdb ? &H : nullptr, caps, E, uf, R, ovf, m, L * L / 4));
+    EdgeK *E = nullptr;
+    WM_TRY(spanning_tree(C, raw, total, D, WM_F64, WM_SOA, hdb ? x.min_pts : 0, caps, S, H, E, ovf, m, L * L / 4));
     if (*ovf) return 0;
     // ---- tree edges grouped by instance, K order inside each
     EdgeK *keys = ar.get<EdgeK>(m + 1), *ktmp = ar.get<EdgeK>(m + 1);

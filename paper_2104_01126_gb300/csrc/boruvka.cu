@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(kWalkThreads) nc_search_kernel(TravArgs a, NcA
             for (int r = 1; r < kBucket; ++r) v = r == p ? w[r] : v;
             if (EXACT) {
                 const int j = j0 + p;
-                double x2 = dist64(a.x64, n, a.d, i, j);
+                double x2 = walk_dist64<D, S>(a.x64, n, a.d, X.rows, i, j);
                 if (HDB) x2 = pos_dmax(x2, pos_dmax(a.cd64[i], a.cd64[j]));
                 note_err(v, x2, err);
                 kmin_update(best, x2, a.pid[i], a.pid[j]);
@@ -378,9 +378,10 @@ __global__ void nc_active_kernel(TravArgs a, NcArgs b)
 }
 
 // K-minimum of a point's list entries inside the band of its component's screened minimum
-template <bool HDB>
+template <int D, bool HDB>
 __global__ void nc_pick_kernel(TravArgs a, NcArgs b)
 {
+    constexpr int S = row_floats(D);
     __shared__ int sh[32];
     const int n = a.n;
     unsigned long long n_re = 0;
@@ -401,7 +402,7 @@ __global__ void nc_pick_kernel(TravArgs a, NcArgs b)
                     if (s > T) break;
                     const int j = b.lj[(size_t)h * n + i];
                     if (j < 0 || b.lab[j] == c) continue;
-                    double w = dist64(a.x64, n, a.d, i, j);
+                    double w = walk_dist64<D, S>(a.x64, n, a.d, b.rows, i, j);
                     if (HDB) w = pos_dmax(w, pos_dmax(a.cd64[i], a.cd64[j]));
                     note_err(s, w, err);
                     kmin_update(best, w, a.pid[i], a.pid[j]);
@@ -527,12 +528,6 @@ __global__ void nc_node_labels_kernel(int Ns, int S, const int2 *__restrict__ ra
     }
 }
 
-// the union-find over input ids that the MemoGFK rounds continue from
-__global__ void nc_export_kernel(const int *__restrict__ lab, const int *__restrict__ pid, int n, int *__restrict__ uf)
-{
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) uf[pid[i]] = pid[lab[i]];
-}
-
 template <int D, bool HDB>
 int rounds(NcCall &C, TravArgs &a, NcArgs &b)
 {
@@ -576,12 +571,11 @@ int rounds(NcCall &C, TravArgs &a, NcArgs &b)
             launch(nc_refresh_kernel<D, HDB>, g, 256, 0, st, a, b);
             launch(nc_active_kernel<HDB>, g, 256, 0, st, a, b);
         }
-        const int e0 = C.mark(C.ctx);
+        C.mark(C.ctx);
         launch(nc_search_kernel<D, HDB, false>, gs, kWalkThreads, 0, st, a, b, X, n);
-        const int e1 = C.mark(C.ctx);
-        C.span(C.ctx, e0, e1);
+        C.mark(C.ctx);
         if (b.first) launch(nc_refresh_kernel<D, HDB>, g, 256, 0, st, a, b);   // the lists' minima into S
-        launch(nc_pick_kernel<HDB>, g, 256, 0, st, a, b);
+        launch(nc_pick_kernel<D, HDB>, g, 256, 0, st, a, b);
         launch(nc_search_kernel<D, HDB, true>, gs, kWalkThreads, 0, st, a, b, X, n);
         launch(nc_low_kernel, g, 256, 0, st, b);
         if (HDB) launch(nc_low_repair_kernel, grid_for(C.nrep, 256), 256, 0, st, b, rnow, rn);
@@ -600,11 +594,10 @@ int rounds(NcCall &C, TravArgs &a, NcArgs &b)
             set_error_detail("nearest-component rounds: an internal check failed");
             return WM_EINTERNAL;
         }
-        if (C.pin[5] <= done) break;   // no progress: the caller's other path takes over
+        if (C.pin[5] <= done) break;   // cannot happen while an edge is missing; the caller checks
         done = C.pin[5];
     }
     C.done = done;
-    launch(nc_export_kernel, g, 256, 0, st, b.lab, a.pid, n, C.uf);
     return 0;
 }
 

@@ -14,7 +14,6 @@ struct NcCall {
     int *pin = nullptr;             // pinned host scratch
     const SearchTree *X = nullptr;
     const int *pos = nullptr;       // input id -> tree position
-    int *uf = nullptr;              // union-find over input ids, left flat on return
     EdgeK *out = nullptr;           // tree edges, in no particular order
     long long target = 0;           // edges to find
     double cap = INFINITY;          // no edge at or above this weight is taken (batches)
@@ -24,13 +23,12 @@ struct NcCall {
     EdgeK *rep_tmp0 = nullptr, *rep_tmp1 = nullptr;
     int *E = nullptr;
     // results
-    long long done = 0;             // tree edges found (< target: the caller finishes the forest)
+    long long done = 0;             // tree edges found
     int rounds = 0;
     long long candidates = 0;
-    // timing hooks around the search kernel
+    // called before and after every search
     void *ctx = nullptr;
-    int (*mark)(void *ctx) = nullptr;
-    void (*span)(void *ctx, int from, int to) = nullptr;
+    void (*mark)(void *ctx) = nullptr;
 };
 
 // Boruvka rounds on the search tree (whose labels they overwrite).  Returns 0 or an error code; C.done tells

@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(kWalkThreads) knn_walk_kernel(KnnArgs a, Searc
         for (int h = 0; h < k; ++h) {
             const int j = (int)heap[h * T].y;
             if (j == i) continue;
-            const double w = dist64(a.x64, n, a.d, i, j);
+            const double w = walk_dist64<D, S>(a.x64, n, a.d, X.rows, i, j);
             cd = max(cd, (unsigned long long)__double_as_longlong(w));
             if (r < a.rq) {
                 a.rep_q[(size_t)r * n + i] = j;
@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(32 * kTieWarps) knn_tie_kernel(KnnArgs a, Sear
             if (lane == 0) slow2[atomicAdd(slow2_cnt, 1)] = i;
             continue;
         }
-        for (int e = lane; e < c; e += 32) cw[e] = cj[e] == i ? 0.0 : dist64(a.x64, n, a.d, i, cj[e]);
+        for (int e = lane; e < c; e += 32) cw[e] = cj[e] == i ? 0.0 : walk_dist64<D, S>(a.x64, n, a.d, X.rows, i, cj[e]);
         n_re += (unsigned long long)(lane == 0 ? c : 0);
         __syncwarp();
         // the k-th smallest: the value with fewer than k values below it and at least k at or below it
@@ -497,10 +497,24 @@ __global__ void __launch_bounds__(32 * kTieWarps) knn_tie_kernel(KnnArgs a, Sear
     if (lane == 0 && n_re) atomicAdd(a.stat + 1, n_re);
 }
 
+// exact squared distance from the FP64 coordinates, or (x64 null) from rows of S floats
+__device__ inline double any_dist64(const double *__restrict__ x64, const float *__restrict__ rows, int S, int n, int d, int i,
+                                    int j)
+{
+    if (x64) return dist64(x64, n, d, i, j);
+    double s = 0.0;
+    for (int k = 0; k < d; ++k) {
+        const double t = __dsub_rn((double)rows[(size_t)i * S + k], (double)rows[(size_t)j * S + k]);
+        s = __dadd_rn(s, __dmul_rn(t, t));
+    }
+    return s;
+}
+
 // Exact FP64 answer for one query per warp (ties or duplicates overflowed the list): each lane
 // keeps the k smallest w2 of its strided share, the warp merges the 32 lists, then a second
 // scan collects every q with w2 <= cd2 as repair edges.
-__global__ void __launch_bounds__(32) knn_slow_kernel(KnnArgs a, const int *__restrict__ slow, int nslow,
+__global__ void __launch_bounds__(32) knn_slow_kernel(KnnArgs a, const float *__restrict__ rows, int S,
+                                                      const int *__restrict__ slow, int nslow,
                                                       int *extra_q, int *extra_p, double *extra_d, int *extra_cnt,
                                                       int extra_cap, int *tie_overflow)
 {
@@ -514,7 +528,7 @@ __global__ void __launch_bounds__(32) knn_slow_kernel(KnnArgs a, const int *__re
         const int i = slow[t];
         int cnt = 0;
         for (int j = lane; j < n; j += 32) {
-            double w = j == i ? 0.0 : dist64(a.x64, n, d, i, j);
+            double w = j == i ? 0.0 : any_dist64(a.x64, rows, S, n, d, i, j);
             if (cnt < k || w < lw[(k - 1) * 32 + lane]) {
                 int pos = cnt < k ? cnt : k - 1;
                 while (pos > 0 && lw[(pos - 1) * 32 + lane] > w) { lw[pos * 32 + lane] = lw[(pos - 1) * 32 + lane]; --pos; }
@@ -541,7 +555,7 @@ __global__ void __launch_bounds__(32) knn_slow_kernel(KnnArgs a, const int *__re
         }
         for (int j = lane; j < n; j += 32) {
             if (j == i) continue;
-            double w = dist64(a.x64, n, d, i, j);
+            double w = any_dist64(a.x64, rows, S, n, d, i, j);
             if (w <= kth) {
                 int s = atomicAdd(extra_cnt, 1);
                 if (s < extra_cap) { extra_p[s] = i; extra_q[s] = j; extra_d[s] = w; }
@@ -656,11 +670,11 @@ constexpr int kKnn64SmemMax = 128 << 10;   // lists of minPts + 8 entries and a 
 static_assert((kWalkStack + kMaxMinPts) * 32 * 8 <= kWalkSmemMax && (kMaxMinPts + 8) * 32 * 12 + 3800 * 4 <= kKnn64SmemMax,
               "shared memory limits of the k-NN kernels");
 
-// core distances and repair edges; X: the search tree (without it, or in the FP64 form, all in FP64)
-int core_distances(Points &P, Tree &T, const SearchTree *X, int min_pts, bool fp64, HdbState &H, Arena &ar,
-                   cudaStream_t st, int *pin, wm_stats *stats)
+// core distances and repair edges: by the walk on the search tree X, or (the plain FP64 form) on the tree T
+int core_distances(const Points &P, const Tree *T, const SearchTree *X, int min_pts, HdbState &H, Arena &ar, cudaStream_t st,
+                    int *pin, wm_stats *stats)
 {
-    const int n = P.n, d = P.d, N = T.N;
+    const int n = P.n, d = P.d;
     if (min_pts > kMaxMinPts) return WM_EINVAL;
     const int KL = std::min(min_pts + 8, n);
     H.cd64 = ar.get<double>(n);
@@ -674,9 +688,8 @@ int core_distances(Points &P, Tree &T, const SearchTree *X, int min_pts, bool fp
     size_t mark = ar.off;
     KnnArgs a;
     memset(&a, 0, sizeof a);
-    a.N = N; a.n = n; a.d = d; a.k = min_pts; a.KL = KL;
+    a.n = n; a.d = d; a.k = min_pts; a.KL = KL;
     a.x32 = P.x32; a.x64 = P.x64;
-    a.stack_cap = T.depth + 4;
     a.cd64 = H.cd64; a.cd32 = H.cd32;
     a.rq = RQ;
     a.rep_q = ar.get<int>((size_t)n * RQ);
@@ -700,7 +713,10 @@ int core_distances(Points &P, Tree &T, const SearchTree *X, int min_pts, bool fp
     cudaEvent_t k0, k1;
     cudaEventCreate(&k0);
     cudaEventCreate(&k1);
-    if (fp64 || !X->rows) {
+    if (!X) {
+        const int N = T->N;
+        a.N = N;
+        a.stack_cap = T->depth + 4;
         // launch shape: warps per block limited by shared memory; the grid fills the SMs
         const int dmp = d <= 3 ? 4 : d <= 7 ? 8 : 16;   // = knn_dmp<DM> of the instantiation used
         const size_t per_warp = knn_warp_smem(KL, a.stack_cap);
@@ -711,7 +727,7 @@ int core_distances(Points &P, Tree &T, const SearchTree *X, int min_pts, bool fp
         NodeRec *rec = ar.get<NodeRec>(N);
         float *box = ar.get<float>((size_t)N * 2 * dmp);
         if (!rec || !box) { cudaEventDestroy(k0); cudaEventDestroy(k1); return WM_ENOMEM; }
-        pack_nodes(T, d, dmp, rec, box, st);
+        pack_nodes(*T, d, dmp, rec, box, st);
         a.rec = rec;
         a.box = box;
         cudaEventRecord(k0, st);
@@ -800,7 +816,7 @@ int core_distances(Points &P, Tree &T, const SearchTree *X, int min_pts, bool fp
     if (nslow > 0) {
         size_t sm2 = (size_t)min_pts * 32 * 8 + 32 * 4;
         cudaFuncSetAttribute(knn_slow_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxMinPts * 32 * 8 + 32 * 4);
-        launch(knn_slow_kernel, std::min(nslow, num_sms() * 8), 32, sm2, st, a, slow2, nslow, ex_q, ex_p, ex_d, cnts + 1,
+        launch(knn_slow_kernel, std::min(nslow, num_sms() * 8), 32, sm2, st, a, X ? X->rows : nullptr, X ? X->S : 0, slow2, nslow, ex_q, ex_p, ex_d, cnts + 1,
                                                                      extra_cap, cnts + 2);
     }
     // repair edges: one copy of each, weighted, in no particular order (each round takes those it needs)

@@ -1,9 +1,9 @@
 // stree.cuh -- the search tree that the k-NN pass (knn.cu) and the nearest-component search
 // (boruvka.cu) walk with one thread per query point.
 //
-// It holds the nodes of the k-d tree down to the subtrees of at most kBucket points, siblings adjacent
-// in breadth-first order: about 0.4 nodes per point instead of 2, so that the levels a walk visits most
-// stay in L2.  A node row holds its box in groups of four dimensions (lo then hi, box_lo / box_hi, each
+// It is a spatial-median k-d tree down to buckets of at most kBucket points, siblings adjacent: about
+// 0.4 nodes per point instead of the 2 of a tree with single-point leaves, so that the levels a walk
+// visits most stay in L2.  A node row holds its box in groups of four dimensions (lo then hi, box_lo / box_hi, each
 // group one 256-bit load) and, in the last padded dimension, a reference (lo slot) and a component
 // label or -1 (hi slot): a visit reads the two child rows and nothing else.  A reference is the row of
 // the left child, or for a bucket kBucketBit | (size - 1) << 28 | first point.  A point row holds the
@@ -31,6 +31,7 @@ struct SearchTree {
     int deep_levels = 0;
     int walk_blocks = 0;          // the largest grid the stacks are sized for
     int stack_cap = 0;            // entries of a thread's stack: one per tree level
+    int depth = 0;                // levels
 };
 
 // rows of d coordinates and one more slot
@@ -42,7 +43,10 @@ __host__ __device__ constexpr int walk_dim(int d) { return d <= 2 ? 2 : d <= 8 ?
 constexpr bool walk_dims_fit(int d) { return d > 16 || (walk_dim(d) >= d && row_floats(walk_dim(d)) == row_floats(d) && walk_dims_fit(d + 1)); }
 static_assert(walk_dims_fit(1), "a walk's rows must be as wide as the search tree's");
 
-int build_search_tree(const Points &P, const Tree &T, SearchTree &X, Arena &ar, cudaStream_t st, int *pin);
+int build_search_tree(const void *src, int n, int d, int dtype, int layout, Points &P, SearchTree &X, Arena &ar,
+                      cudaStream_t st, int *pin);
+
+__host__ __device__ inline unsigned bucket_ref(int first, int size) { return kBucketBit | (unsigned)(size - 1) << 28 | (unsigned)first; }
 
 #ifdef __CUDACC__
 __device__ __forceinline__ float next_up(float x) { return x < INFINITY ? __uint_as_float(__float_as_uint(x) + 1u) : x; }
@@ -88,6 +92,30 @@ __device__ __forceinline__ float row_dist(const float (&q)[S], const float (&x)[
     for (int k = 0; k < D; ++k) {
         const float t = q[k] - x[k];
         s = fmaf(t, t, s);
+    }
+    return s;
+}
+
+// exact FP64 squared distance of positions i and j: from the FP64 coordinates where the rows are rounded
+// copies (x64 not null), else from the rows, which then hold the coordinates themselves
+template <int D, int S>
+__device__ inline double walk_dist64(const double *__restrict__ x64, int n, int d, const float *__restrict__ rows, int i, int j)
+{
+    double s = 0.0;
+    if (x64) {
+        for (int k = 0; k < d; ++k) {
+            const double t = __dsub_rn(x64[(size_t)k * n + i], x64[(size_t)k * n + j]);
+            s = __dadd_rn(s, __dmul_rn(t, t));
+        }
+    } else {
+        float x[S], y[S];
+        load_row<S>(rows, i, x);
+        load_row<S>(rows, j, y);
+#pragma unroll
+        for (int k = 0; k < D; ++k) {   // a padded coordinate is 0 on both sides and adds exactly 0
+            const double t = __dsub_rn((double)x[k], (double)y[k]);
+            s = __dadd_rn(s, __dmul_rn(t, t));
+        }
     }
     return s;
 }
