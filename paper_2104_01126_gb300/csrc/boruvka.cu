@@ -16,11 +16,15 @@
 //             those that could still hold a lighter edge than the lists show;
 //   search  : a thread per active point walks the k-d tree, the nearer child first, skipping nodes of
 //             its own component and nodes beyond its bound, and rebuilds the point's list;
-//   pick    : FP64 evaluation of the list entries within T(S[c]); the K-minimum per component by
-//             two 64-bit WriteMins; a point whose list may have dropped a tie (R[i] <= T(S[c])
-//             still) is answered by a walk that evaluates everything within T(S[c]) in FP64;
-//   merge   : every component's root links to the other endpoint's component; of a mutual choice
-//             the smaller root stays and the edge is emitted once.
+//   pick    : collects the points with a list entry within T(S[c]); FP64 evaluation of those entries
+//             and the K-minimum per component by two 64-bit WriteMins; a point whose list may have
+//             dropped a tie (R[i] <= T(S[c]) still) is answered by a walk that evaluates everything
+//             within T(S[c]) in FP64;
+//   merge   : every root links to the other endpoint's component; of a mutual choice the smaller root
+//             stays and the edge is emitted once.  Then the roots left are collected and the points
+//             and nodes relabelled.
+// (Asking only the components of up to 1, 2 or 4 times the average size in a round was no faster on any
+// of the 10^7-point sets: the others cost little to ask, and more rounds are needed.)
 // The lists of the first search (all points, nothing pruned) serve the first few rounds.
 //
 // HDBSCAN*: the weights are mutual reachability distances.  All edges with D <= max(cd2 p, cd2 q)
@@ -45,6 +49,15 @@ namespace {
 // from 8.0 to 7.7 in 2-D, left it in 5-D (31 ms) and cost 13 % in 7-D; 2 entries were slower everywhere.
 __host__ __device__ constexpr int list_len(int D) { return D <= 3 ? 6 : 4; }
 
+// counters: the first kCntRound are zeroed every round
+enum {
+    kCntActive, kCntSearch, kCntCand, kCntExact, kCntExactNext, kCntPicked, kCntRound,
+    kCntEdges = kCntRound,            // tree edges so far
+    kCntRep,                          // [2] repair edges left, by round parity
+    kCntRoots = kCntRep + 2,          // [2] roots, by round parity
+    kCntAll = kCntRoots + 2
+};
+
 struct NcArgs {
     int *lab;                  // component of a tree position (a tree position: the root)
     int *par;                  // links between roots
@@ -54,11 +67,12 @@ struct NcArgs {
     int *lj;                   // [list_len][n] list positions (-1: none)
     float *R;                  // every point outside the component and the list screens at >= R
     unsigned char *hd;         // first list entry that may lie outside the component
-    int *act, *amb;            // active points; points that need the exact scan
+    int *roots[2];             // the roots of this round and the next
+    int *act, *amb, *picked;   // active points; points that need the exact scan; points with a candidate
+    int *nlab;                 // labels in the node rows
     EdgeK *cand;               // candidate edges of the round and the component each serves
     int *cand_c;
-    int *cnt;                  // [0] active, [1] search dispenser, [2] candidates, [3] exact scans,
-                               // [4] their dispenser, [5] tree edges, [6] repair edges left
+    int *cnt;                  // counters, see kCnt*
     int K;                     // list_len
     const int *pos;            // input id -> tree position
     unsigned cap_bits;         // no edge at or above this weight (float bits; +inf: none)
@@ -66,6 +80,7 @@ struct NcArgs {
     float *rows;               // the search tree's point rows
     const float *ncd;          // HDBSCAN*: smallest core distance of a node (rounded down)
     int first;                 // first search: components are single points, nothing is pruned by S
+    int n;
 };
 
 // HDBSCAN*: true when the FP32 squared distance d32 proves D <= c for a core distance c (FP32 copy)
@@ -95,7 +110,7 @@ __global__ void __launch_bounds__(kWalkThreads) nc_search_kernel(TravArgs a, NcA
     constexpr bool kStream = S > 4 && !HDB;
     const int lane = threadIdx.x & 31;
     const int n = a.n;
-    const int m = EXACT ? b.cnt[3] : b.first ? m_all : b.cnt[0];
+    const int m = EXACT ? b.cnt[kCntExact] : b.first ? m_all : b.cnt[kCntActive];
     unsigned long long n_ev = 0, n_re = 0;
     float err = 0.f;
     // the lane's query
@@ -203,7 +218,7 @@ __global__ void __launch_bounds__(kWalkThreads) nc_search_kernel(TravArgs a, NcA
         n_ev += ev;
         if (EXACT) {
             if (best.hi < b.cap64) {
-                const int slot = atomicAdd(b.cnt + 2, 1);   // at most one candidate per point: within n
+                const int slot = atomicAdd(b.cnt + kCntCand, 1);   // at most one candidate per point: within n
                 EdgeK e;
                 e.hi = best.hi;
                 e.lo = best.lo;
@@ -221,7 +236,7 @@ __global__ void __launch_bounds__(kWalkThreads) nc_search_kernel(TravArgs a, NcA
             b.hd[i] = 0;
         }
     };
-    walk_queries<D, S, kStream>(X, m, b.cnt + (EXACT ? 4 : 1), &sst[0][threadIdx.x], kWalkThreads,
+    walk_queries<D, S, kStream>(X, m, b.cnt + (EXACT ? kCntExactNext : kCntSearch), &sst[0][threadIdx.x], kWalkThreads,
                                 X.deep + (size_t)blockIdx.x * kWalkThreads + threadIdx.x,
                                 (size_t)gridDim.x * kWalkThreads, (int *)a.overflow, 8, q, begin, bound, need, pending,
                                 scan, finish);
@@ -270,6 +285,7 @@ __global__ void nc_init_kernel(TravArgs a, NcArgs b, bool hdb)
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += gridDim.x * blockDim.x) {
         b.lab[i] = i;
         b.par[i] = i;
+        b.roots[0][i] = i;
         b.S[i] = b.cap_bits;
         b.bhi[i] = ~0ull;
         b.blo[i] = ~0ull;
@@ -278,6 +294,7 @@ __global__ void nc_init_kernel(TravArgs a, NcArgs b, bool hdb)
             b.R[i] = __double2float_rd(a.cd64[i]);
         }
     }
+    if (blockIdx.x == 0 && threadIdx.x == 0) b.cnt[kCntRoots] = a.n;
 }
 
 // WriteMin of a weight into a component's slot; a value that cannot lower it is not issued
@@ -341,10 +358,12 @@ __global__ void nc_repair_kernel(NcArgs b, const EdgeK *__restrict__ in, const i
             keep = cu != cv;
             if (keep && e.hi < b.cap64) {
                 const float s = __double2float_ru(edge_w2(e));
-                s_min(b.S, cu, s);
-                s_min(b.S, cv, s);
-                if (e.hi < *(volatile unsigned long long *)(b.bhi + cu)) atomicMin(b.bhi + cu, e.hi);
-                if (e.hi < *(volatile unsigned long long *)(b.bhi + cv)) atomicMin(b.bhi + cv, e.hi);
+#pragma unroll
+                for (int side = 0; side < 2; ++side) {
+                    const int c = side ? cv : cu;
+                    s_min(b.S, c, s);
+                    if (e.hi < *(volatile unsigned long long *)(b.bhi + c)) atomicMin(b.bhi + c, e.hi);
+                }
             }
         }
         const int slot = block_append(out_n, keep ? 1 : 0, sh);
@@ -372,46 +391,70 @@ __global__ void nc_active_kernel(TravArgs a, NcArgs b)
             on = b.R[i] <= screen_threshold(__uint_as_float(b.S[c]), a);
             if (HDB && on) on = !settled(a, b, i, c);
         }
-        const int slot = block_append(b.cnt + 0, on ? 1 : 0, sh);
+        if (!__syncthreads_or(on)) continue;
+        const int slot = block_append(b.cnt + kCntActive, on ? 1 : 0, sh);
         if (on) b.act[slot] = i;
     }
 }
 
-// K-minimum of a point's list entries inside the band of its component's screened minimum
-template <int D, bool HDB>
+// Points with a list entry inside the band of their component's screened minimum, and points whose list
+// may have dropped one
+template <bool HDB>
 __global__ void nc_pick_kernel(TravArgs a, NcArgs b)
 {
-    constexpr int S = row_floats(D);
     __shared__ int sh[32];
     const int n = a.n;
-    unsigned long long n_re = 0;
-    float err = 0.f;
     for (int b0 = blockIdx.x * blockDim.x; b0 < n; b0 += gridDim.x * blockDim.x) {
         const int i = b0 + threadIdx.x;
-        bool exact = false;
-        int c = -1;
-        KMin best{~0ull, ~0ull};
+        bool exact = false, has = false;
         if (i < n) {
-            c = b.lab[i];
+            const int c = b.lab[i];
             const float T = screen_threshold(__uint_as_float(b.S[c]), a);
             exact = b.R[i] <= T;
             if (HDB && exact) exact = !settled(a, b, i, c);
-            if (!exact) {
-                for (int h = b.hd[i]; h < b.K; ++h) {
-                    const float s = b.ls[(size_t)h * n + i];
-                    if (s > T) break;
-                    const int j = b.lj[(size_t)h * n + i];
-                    if (j < 0 || b.lab[j] == c) continue;
-                    double w = walk_dist64<D, S>(a.x64, n, a.d, b.rows, i, j);
-                    if (HDB) w = pos_dmax(w, pos_dmax(a.cd64[i], a.cd64[j]));
-                    note_err(s, w, err);
-                    kmin_update(best, w, a.pid[i], a.pid[j]);
-                    ++n_re;
-                }
+            const int h = b.hd[i];
+            has = !exact && h < b.K && b.ls[(size_t)h * n + i] <= T;
+        }
+        if (__syncthreads_or(has)) {
+            const int slot = block_append(b.cnt + kCntPicked, has ? 1 : 0, sh);
+            if (has) b.picked[slot] = i;
+        }
+        if (exact) b.amb[atomicAdd(b.cnt + kCntExact, 1)] = i;
+    }
+}
+
+// K-minimum of a picked point's list entries inside the band, in FP64 (on a dense list: an FP64
+// instruction costs a warp the same however few of its lanes need it)
+template <int D, bool HDB>
+__global__ void nc_cand_kernel(TravArgs a, NcArgs b)
+{
+    constexpr int S = row_floats(D);
+    __shared__ int sh[32];
+    const int n = a.n, m = b.cnt[kCntPicked];
+    unsigned long long n_re = 0;
+    float err = 0.f;
+    for (int b0 = blockIdx.x * blockDim.x; b0 < m; b0 += gridDim.x * blockDim.x) {
+        const int t = b0 + threadIdx.x;
+        int c = -1;
+        KMin best{~0ull, ~0ull};
+        if (t < m) {
+            const int i = b.picked[t];
+            c = b.lab[i];
+            const float T = screen_threshold(__uint_as_float(b.S[c]), a);
+            for (int h = b.hd[i]; h < b.K; ++h) {
+                const float s = b.ls[(size_t)h * n + i];
+                if (s > T) break;
+                const int j = b.lj[(size_t)h * n + i];
+                if (j < 0 || b.lab[j] == c) continue;
+                double w = walk_dist64<D, S>(a.x64, n, a.d, b.rows, i, j);
+                if (HDB) w = pos_dmax(w, pos_dmax(a.cd64[i], a.cd64[j]));
+                note_err(s, w, err);
+                kmin_update(best, w, a.pid[i], a.pid[j]);
+                ++n_re;
             }
         }
         const bool has = best.hi < b.cap64;
-        int slot = block_append(b.cnt + 2, has ? 1 : 0, sh);
+        const int slot = block_append(b.cnt + kCntCand, has ? 1 : 0, sh);
         if (has) {
             EdgeK e;
             e.hi = best.hi;
@@ -420,8 +463,6 @@ __global__ void nc_pick_kernel(TravArgs a, NcArgs b)
             b.cand_c[slot] = c;
             if (best.hi < *(volatile unsigned long long *)(b.bhi + c)) atomicMin(b.bhi + c, best.hi);
         }
-        slot = block_append(b.cnt + 3, exact ? 1 : 0, sh);
-        if (exact) b.amb[slot] = i;
     }
     err_flush(a, err);
     n_re = warp_sum_u64(n_re);
@@ -431,7 +472,7 @@ __global__ void nc_pick_kernel(TravArgs a, NcArgs b)
 // Among the candidates with their component's smallest weight: WriteMin of the id pair
 __global__ void nc_low_kernel(NcArgs b)
 {
-    const int m = b.cnt[2];
+    const int m = b.cnt[kCntCand];
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < m; t += gridDim.x * blockDim.x) {
         const EdgeK e = b.cand[t];
         const int c = b.cand_c[t];
@@ -453,17 +494,18 @@ __global__ void nc_low_repair_kernel(NcArgs b, const EdgeK *__restrict__ rep, co
 // Every root with an edge links to the component at its other end; of two roots that chose the same
 // edge the smaller stays a root.  (The keys along a chain of choices strictly fall, so there is no
 // longer cycle.)
-__global__ void nc_merge_kernel(TravArgs a, NcArgs b, EdgeK *__restrict__ out, int out_cap)
+__global__ void nc_merge_kernel(TravArgs a, NcArgs b, int cur, EdgeK *__restrict__ out, int out_cap)
 {
     __shared__ int sh[32];
-    const int n = a.n;
-    for (int b0 = blockIdx.x * blockDim.x; b0 < n; b0 += gridDim.x * blockDim.x) {
-        const int i = b0 + threadIdx.x;
+    const int m = b.cnt[kCntRoots + cur];
+    for (int b0 = blockIdx.x * blockDim.x; b0 < m; b0 += gridDim.x * blockDim.x) {
+        const int t = b0 + threadIdx.x;
         bool emit = false;
         EdgeK e;
         e.hi = 0;
         e.lo = 0;
-        if (i < n && b.lab[i] == i) {
+        if (t < m) {
+            const int i = b.roots[cur][t];
             e.hi = b.bhi[i];
             e.lo = b.blo[i];
             if (e.hi != ~0ull) {
@@ -474,12 +516,11 @@ __global__ void nc_merge_kernel(TravArgs a, NcArgs b, EdgeK *__restrict__ out, i
                 } else {
                     const bool mutual = b.bhi[o] == e.hi && b.blo[o] == e.lo;
                     emit = !mutual || i < o;
-                    if (emit && mutual) b.par[i] = i;
-                    else b.par[i] = o;
+                    if (!(emit && mutual)) b.par[i] = o;
                 }
             }
         }
-        const int slot = block_append(b.cnt + 5, emit ? 1 : 0, sh);
+        const int slot = block_append(b.cnt + kCntEdges, emit ? 1 : 0, sh);
         if (emit) {
             if (slot < out_cap) out[slot] = e;
             else atomicOr(a.overflow, 16u);
@@ -487,44 +528,135 @@ __global__ void nc_merge_kernel(TravArgs a, NcArgs b, EdgeK *__restrict__ out, i
     }
 }
 
-// New labels; the per-round slots are reset on the way
-__global__ void nc_relabel_kernel(NcArgs b, int n, int S)
+// After the links: every root of the round is brought close to its component's root; the roots left are
+// collected and their slots reset for the next round.
+__global__ void nc_roots_kernel(NcArgs b, int cur)
 {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int c = b.lab[i];
-        int x = c;
-        for (int it = 0; it < n; ++it) {
-            const int p = *(volatile int *)(b.par + x);
-            if (p == x) break;
-            const int g = *(volatile int *)(b.par + p);
-            if (g != p) *(volatile int *)(b.par + x) = g;   // path halving (the forest is static)
-            x = p;
+    __shared__ int sh[32];
+    const int m = b.cnt[kCntRoots + cur];
+    for (int b0 = blockIdx.x * blockDim.x; b0 < m; b0 += gridDim.x * blockDim.x) {
+        const int t = b0 + threadIdx.x;
+        bool stays = false;
+        int i = 0;
+        if (t < m) {
+            i = b.roots[cur][t];
+            int x = i;
+            for (int it = 0; it < b.n; ++it) {
+                const int p = *(volatile int *)(b.par + x);
+                if (p == x) break;
+                const int g = *(volatile int *)(b.par + p);
+                if (g != p) *(volatile int *)(b.par + x) = g;   // path halving (the forest is static)
+                x = p;
+            }
+            stays = x == i;
+            if (stays) {
+                b.S[i] = b.cap_bits;
+                b.bhi[i] = ~0ull;
+                b.blo[i] = ~0ull;
+            } else {
+                *(volatile int *)(b.par + i) = x;
+            }
         }
-        if (x != c) {
-            b.lab[i] = x;
-            b.rows[(size_t)i * S + S - 1] = __int_as_float(x);
-        }
-        if (x == i) {   // only roots' slots are read
-            b.S[i] = b.cap_bits;
-            b.bhi[i] = ~0ull;
-            b.blo[i] = ~0ull;
-        }
+        const int slot = block_append(b.cnt + kCntRoots + (cur ^ 1), stays ? 1 : 0, sh);
+        if (stays) b.roots[cur ^ 1][slot] = i;
     }
 }
 
-__global__ void nc_change_kernel(const int *__restrict__ lab, int n, int *__restrict__ chg)
+// The root above x.  nc_roots_kernel leaves every root of the round pointing at its new root or, where a
+// concurrent walk halved the path once more, at an ancestor below it.
+__device__ __forceinline__ int root_of(const int *__restrict__ par, int x, int n)
 {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        chg[i] = i > 0 && lab[i] != lab[i - 1];
+    for (int it = 0; it < n; ++it) {
+        const int p = par[x];
+        if (p == x) break;
+        x = p;
+    }
+    return x;
+}
+
+// New labels, and per tile of positions the number of label changes along tree order (a node is in one
+// component when none falls inside its range).
+constexpr int kTileItems = 8, kTile = 256 * kTileItems;
+
+__global__ void __launch_bounds__(256) nc_relabel_kernel(NcArgs b, int S, int *__restrict__ sums)
+{
+    __shared__ int s_chg;
+    const int n = b.n;
+    const int *par = b.par;
+    for (int tile = blockIdx.x; tile * (long long)kTile < n; tile += gridDim.x) {
+        if (threadIdx.x == 0) s_chg = 0;
+        __syncthreads();
+        const int i0 = tile * kTile + threadIdx.x * kTileItems;
+        // (a neighbour's label may be replaced already: a root points at itself)
+        int prev = i0 > 0 && i0 < n ? root_of(par, *(volatile int *)(b.lab + i0 - 1), n) : -1;
+        int chg = 0;
+#pragma unroll
+        for (int t = 0; t < kTileItems; ++t) {
+            const int i = i0 + t;
+            if (i >= n) break;
+            const int c = b.lab[i], x = root_of(par, c, n);
+            if (x != c) {
+                *(volatile int *)(b.lab + i) = x;
+                b.rows[(size_t)i * S + S - 1] = __int_as_float(x);
+            }
+            chg += i > 0 && x != prev;
+            prev = x;
+        }
+        chg = __reduce_add_sync(0xffffffffu, chg);
+        if ((threadIdx.x & 31) == 0 && chg) atomicAdd(&s_chg, chg);
+        __syncthreads();
+        if (threadIdx.x == 0) sums[tile] = s_chg;
+    }
+}
+
+// E[i] = label changes in (0, i), from the tiles' prefixes; E[n] all of them
+__global__ void __launch_bounds__(256) nc_prefix_kernel(int n, const int *__restrict__ lab, const int *__restrict__ sums,
+                                                        int *__restrict__ E)
+{
+    __shared__ int sw[8];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int tile = blockIdx.x; tile * (long long)kTile < n; tile += gridDim.x) {
+        const int i0 = tile * kTile + threadIdx.x * kTileItems;
+        int prev = i0 > 0 && i0 < n ? lab[i0 - 1] : -1;
+        int chg[kTileItems], s = 0;
+#pragma unroll
+        for (int t = 0; t < kTileItems; ++t) {
+            const int i = i0 + t;
+            const int x = i < n ? lab[i] : prev;
+            chg[t] = i > 0 && x != prev;
+            prev = x;
+            s += chg[t];
+        }
+        int x = s;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) sw[wid] = x;
+        __syncthreads();
+        int base = sums[tile];
+        for (int w = 0; w < wid; ++w) base += sw[w];
+        x += base - s;
+#pragma unroll
+        for (int t = 0; t < kTileItems; ++t) {
+            if (i0 + t < n) E[i0 + t] = x;
+            x += chg[t];
+            if (i0 + t == n - 1) E[n] = x;
+        }
+        __syncthreads();
+    }
 }
 
 __global__ void nc_node_labels_kernel(int Ns, int S, const int2 *__restrict__ range, float *__restrict__ nodes,
-                                      const int *__restrict__ lab, const int *__restrict__ E)
+                                      int *__restrict__ nlab, const int *__restrict__ lab, const int *__restrict__ E)
 {
     for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < Ns; x += gridDim.x * blockDim.x) {
         const int2 r = range[x];
         if (E[r.y] != E[r.x + 1]) continue;   // mixed: the label is -1 from the start
-        nodes[(size_t)x * 2 * S + box_hi(S - 1)] = __int_as_float(lab[r.x]);
+        const int c = lab[r.x];
+        if (nlab[x] == c) continue;
+        nlab[x] = c;
+        nodes[(size_t)x * 2 * S + box_hi(S - 1)] = __int_as_float(c);
     }
 }
 
@@ -533,20 +665,24 @@ int rounds(NcCall &C, TravArgs &a, NcArgs &b)
 {
     cudaStream_t st = C.st;
     const int n = a.n;
-    const int g = grid_for(n, 256);
+    const int g = grid_for(n, 256), gt = grid_for(n, kTile);
     constexpr int S = row_floats(D);
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, nc_search_kernel<D, HDB, false>, kWalkThreads, 0) != cudaSuccess ||
-        per_sm < 1) {
-        cudaGetLastError();
-        return 0;
-    }
+        per_sm < 1)
+        return WM_ECUDA;
     const int gs = std::min(num_sms() * per_sm, C.X->walk_blocks);
     const SearchTree &X = *C.X;
+    Arena &ar = *C.ar;
+    b.nlab = ar.get<int>(X.Ns);
+    const int tiles = (n + kTile - 1) / kTile;
+    int *sums = ar.get<int>(tiles), *E = ar.get<int>((size_t)n + 1);
+    if (ar.failed) return WM_ENOMEM;
+    cudaMemsetAsync(b.nlab, 0xff, sizeof(int) * X.Ns, st);
     if (HDB) {
-        float *ncd = C.ar->get<float>(X.Ns);
-        int *arrive = C.ar->get<int>(X.Ns);
-        if (C.ar->failed) return WM_ENOMEM;
+        float *ncd = ar.get<float>(X.Ns);
+        int *arrive = ar.get<int>(X.Ns);
+        if (ar.failed) return WM_ENOMEM;
         cudaMemsetAsync(arrive, 0, sizeof(int) * X.Ns, st);
         launch(nc_core_min_kernel, grid_for(X.Ns, 256), 256, 0, st, X.Ns, X.range, X.parent, a.cd64, ncd, arrive);
         b.ncd = ncd;
@@ -554,17 +690,20 @@ int rounds(NcCall &C, TravArgs &a, NcArgs &b)
     launch(nc_init_kernel, g, 256, 0, st, a, b, HDB);
     const EdgeK *rin = C.rep;
     EdgeK *rbuf[2] = {C.rep_tmp0, C.rep_tmp1};
-    long long done = 0;
-    for (int r = 0; r < 64 && done < C.target; ++r) {
-        cudaMemsetAsync(b.cnt, 0, 5 * sizeof(int), st);
-        cudaMemsetAsync(b.cnt + 6 + (r & 1), 0, sizeof(int), st);
+    long long edges = 0;
+    // every component that can still grow links in a round: their number at least halves
+    for (int r = 0; r < 64 && edges < C.target; ++r) {
+        const int cur = r & 1;
+        cudaMemsetAsync(b.cnt, 0, kCntRound * sizeof(int), st);
+        cudaMemsetAsync(b.cnt + kCntRoots + (cur ^ 1), 0, sizeof(int), st);
         const EdgeK *rnow = nullptr;
         const int *rn = nullptr;
         if (HDB) {
-            launch(nc_repair_kernel, grid_for(C.nrep, 256), 256, 0, st, b, rin, r ? b.cnt + 6 + ((r & 1) ^ 1) : (const int *)nullptr,
-                   C.nrep, rbuf[r & 1], b.cnt + 6 + (r & 1));
-            rin = rnow = rbuf[r & 1];
-            rn = b.cnt + 6 + (r & 1);
+            cudaMemsetAsync(b.cnt + kCntRep + cur, 0, sizeof(int), st);
+            launch(nc_repair_kernel, grid_for(C.nrep, 256), 256, 0, st, b, rin, r ? b.cnt + kCntRep + (cur ^ 1) : (const int *)nullptr,
+                   C.nrep, rbuf[cur], b.cnt + kCntRep + cur);
+            rin = rnow = rbuf[cur];
+            rn = b.cnt + kCntRep + cur;
         }
         b.first = !HDB && r == 0;
         if (!b.first) {
@@ -575,29 +714,32 @@ int rounds(NcCall &C, TravArgs &a, NcArgs &b)
         launch(nc_search_kernel<D, HDB, false>, gs, kWalkThreads, 0, st, a, b, X, n);
         C.mark(C.ctx);
         if (b.first) launch(nc_refresh_kernel<D, HDB>, g, 256, 0, st, a, b);   // the lists' minima into S
-        launch(nc_pick_kernel<D, HDB>, g, 256, 0, st, a, b);
+        launch(nc_pick_kernel<HDB>, g, 256, 0, st, a, b);
+        launch(nc_cand_kernel<D, HDB>, g, 256, 0, st, a, b);
         launch(nc_search_kernel<D, HDB, true>, gs, kWalkThreads, 0, st, a, b, X, n);
         launch(nc_low_kernel, g, 256, 0, st, b);
         if (HDB) launch(nc_low_repair_kernel, grid_for(C.nrep, 256), 256, 0, st, b, rnow, rn);
-        launch(nc_merge_kernel, g, 256, 0, st, a, b, C.out, n - 1);
-        launch(nc_relabel_kernel, g, 256, 0, st, b, n, S);
-        launch(nc_change_kernel, g, 256, 0, st, b.lab, n, C.E);
-        int rc = scan_exclusive_i32(C.E, C.E, n, C.E + n, st, *C.ar);
+        launch(nc_merge_kernel, g, 256, 0, st, a, b, cur, C.out, n - 1);
+        launch(nc_roots_kernel, g, 256, 0, st, b, cur);
+        launch(nc_relabel_kernel, gt, 256, 0, st, b, S, sums);
+        int rc = scan_exclusive_i32(sums, sums, tiles, nullptr, st, ar);
         if (rc) return rc;
-        launch(nc_node_labels_kernel, grid_for(X.Ns, 256), 256, 0, st, X.Ns, S, X.range, X.nodes, b.lab, C.E);
-        cudaMemcpyAsync(C.pin, b.cnt, 8 * sizeof(int), cudaMemcpyDeviceToHost, st);
-        cudaMemcpyAsync(C.pin + 8, a.overflow, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
+        launch(nc_prefix_kernel, gt, 256, 0, st, n, b.lab, sums, E);
+        launch(nc_node_labels_kernel, grid_for(X.Ns, 256), 256, 0, st, X.Ns, S, X.range, X.nodes, b.nlab, b.lab, E);
+        cudaMemcpyAsync(C.pin, b.cnt, kCntAll * sizeof(int), cudaMemcpyDeviceToHost, st);
+        cudaMemcpyAsync(C.pin + 32, a.overflow, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
         if (cudaStreamSynchronize(st) != cudaSuccess) return WM_ECUDA;
         ++C.rounds;
-        C.candidates += C.pin[2] + (HDB ? C.pin[6 + (r & 1)] : 0);
-        if (C.pin[8]) {
+        C.candidates += C.pin[kCntCand] + (HDB ? C.pin[kCntRep + cur] : 0);
+        // (every edge takes one root)
+        if (C.pin[32] || C.pin[kCntRoots + (cur ^ 1)] != n - C.pin[kCntEdges]) {
             set_error_detail("nearest-component rounds: an internal check failed");
             return WM_EINTERNAL;
         }
-        if (C.pin[5] <= done) break;   // cannot happen while an edge is missing; the caller checks
-        done = C.pin[5];
+        if (C.pin[kCntEdges] == edges) break;   // cannot happen while an edge is missing; the caller checks
+        edges = C.pin[kCntEdges];
     }
-    C.done = done;
+    C.done = edges;
     return 0;
 }
 
@@ -624,14 +766,17 @@ int nearest_component_rounds(NcCall &C, TravArgs &a)
     b.amb = ar.get<int>(n);
     b.cand = ar.get<EdgeK>(n);
     b.cand_c = ar.get<int>(n);
-    b.cnt = ar.get<int>(16);
-    C.E = ar.get<int>((size_t)n + 1);
+    b.cnt = ar.get<int>(kCntAll);
+    b.roots[0] = ar.get<int>(n);
+    b.roots[1] = ar.get<int>(n);
+    b.picked = ar.get<int>(n);
+    b.n = n;
     if (C.rep) {
         C.rep_tmp0 = ar.get<EdgeK>(C.nrep);
         C.rep_tmp1 = ar.get<EdgeK>(C.nrep);
     }
     if (ar.failed) return WM_ENOMEM;
-    cudaMemsetAsync(b.cnt, 0, 16 * sizeof(int), C.st);
+    cudaMemsetAsync(b.cnt, 0, kCntAll * sizeof(int), C.st);
     b.pos = C.pos;
     b.rows = C.X->rows;
     const float cf = C.cap < INFINITY ? C.cap_f : INFINITY;

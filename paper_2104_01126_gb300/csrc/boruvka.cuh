@@ -21,7 +21,6 @@ struct NcCall {
     const EdgeK *rep = nullptr;     // HDBSCAN*: the complete list of edges with D <= max(cd2, cd2)
     int nrep = 0;
     EdgeK *rep_tmp0 = nullptr, *rep_tmp1 = nullptr;
-    int *E = nullptr;
     // results
     long long done = 0;             // tree edges found
     int rounds = 0;
