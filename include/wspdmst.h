@@ -13,8 +13,8 @@
  * computations, and batched Kruskal over a union-find shared across rounds.  By default the forest
  * is first built by nearest-component rounds on the same tree (Boruvka's algorithm, the single-tree
  * form of the dual-tree method that Sec. 5 compares with), which return the same tree faster; MemoGFK
- * rounds build what they leave, and everything in the FP64 form, under wm_set_tuning, for EMSTs above
- * 8 dimensions, and for HDBSCAN* under the geometric separation or with overflowing ties.  The dendrogram and
+ * rounds build the tree under wm_set_tuning, for EMSTs above 8 dimensions, and for HDBSCAN* under the
+ * geometric separation or with overflowing ties.  The dendrogram and
  * plot come from a top-down heavy/light construction after Sec. 4.2 (the heavy set of a
  * subproblem is the upper half of its rank interval, light components come from a union-find,
  * and the output equals the sequential definition exactly).

@@ -454,7 +454,6 @@ static void set_rho(TravArgs &a, double lo, double hi)
 // size measured up to 8 dimensions (GB300, ms: EMST uniform 3-D / 5-D and variable-density 7-D points at
 // 10^7: 35 / 72 / 212 against 58 / 130 / 890; uniform 2-D at 3x10^6, FP64: 10.3 against 11.3; 10^3
 // points in 3-D: 1.6 against 3.5; HDBSCAN* of 10^6 points in 3-D: 14 against 31).  MemoGFK keeps
-//   - the plain FP64 form, whose distances are all FP64 (the lists here are screened in FP32);
 //   - calls under wm_set_tuning, whose parameters are those of the traversals, and the geometric
 //     separation of the GanTao baseline, which is a property of the WSPD;
 //   - HDBSCAN* inputs whose repair list overflowed: the rounds here need it complete;
@@ -463,7 +462,7 @@ static void set_rho(TravArgs &a, double lo, double hi)
 //   - 2^28 points and more (references hold 28-bit positions).
 static bool nearest_rounds_apply(const Call &C, int n, int d, const HdbState *hdb)
 {
-    if (C.precision == WM_PREC_FP64 || C.tune_override || n >= 1 << 28) return false;
+    if (C.tune_override || n >= 1 << 28) return false;
     return hdb ? C.disjunctive && !C.stats.tie_overflow : d <= 8;
 }
 
@@ -487,9 +486,11 @@ static int nearest_tree(Call &C, const Points &P, const SearchTree &X, const Hdb
     TravArgs a;
     a.n = n; a.d = P.d;
     a.x64 = P.x64; a.pid = P.pid;
-    a.eta = 2.0 * (double)P.delta * std::sqrt((double)P.d) * (1.0 + 1e-6);
+    a.fp64 = C.precision == WM_PREC_FP64;
+    a.eta = a.fp64 ? 0.0 : 2.0 * (double)P.delta * std::sqrt((double)P.d) * (1.0 + 1e-6);
     a.eta2_f = float_ru(2.0 * a.eta);
     a.exact32 = a.eta == 0.0;
+    a.delta32 = P.delta;
     if (hdb) { a.cd32 = hdb->cd32; a.cd64 = hdb->cd64; }
     a.overflow = ovf;
     a.stat = stat;
@@ -1248,7 +1249,8 @@ static int prepare_walk(Call &C, const void *pts, int64_t n, int32_t d, int32_t 
 {
     WM_TRY(input_on_device(C, pts, n, d, dtype, S));
     Timer tt;
-    WM_TRY(bad_coordinate(build_search_tree(S.src, (int)n, d, dtype, layout, S.P, S.X, C.ar, C.st, C.pin)));
+    WM_TRY(bad_coordinate(build_search_tree(S.src, (int)n, d, dtype, layout, C.precision == WM_PREC_FP64 ? 2 : 1, S.P, S.X, C.ar,
+                                            C.st, C.pin)));
     C.stats.ms_build_tree += tt.ms();
     C.stats.tree_nodes = 2 * n - 1;   // down to single points; X stores those above its buckets
     C.stats.tree_depth = S.X.depth;
@@ -1409,13 +1411,17 @@ static int spanning_tree(Call &C, const void *pts, int64_t n64, int d, int dtype
 {
     const int n = (int)n64;
     const bool hdb = min_pts >= 1, wspd_form = C.method == WM_METHOD_GFK || C.method == WM_METHOD_NAIVE;
-    // the FP32-screened k-NN pass and the nearest-component rounds walk the search tree
-    const bool walk = hdb ? C.precision != WM_PREC_FP64 && n < 1 << 28 : !wspd_form && nearest_rounds_apply(C, n, d, nullptr);
+    if (hdb && n >= 1 << 28) {   // (its workspace alone would exceed the device)
+        set_detail("HDBSCAN* of 2^28 points or more does not fit the device%s (n=%lld)", "", n64);
+        return WM_ENOMEM;
+    }
+    // the k-NN pass and the nearest-component rounds walk the search tree
+    const bool walk = hdb || (!wspd_form && nearest_rounds_apply(C, n, d, nullptr));
     if (walk) WM_TRY(prepare_walk(C, pts, n64, d, dtype, layout, S));
     else WM_TRY(prepare(C, pts, n64, d, dtype, layout, S));
     if (hdb) {
         Timer tc;
-        WM_TRY(core_distances(S.P, &S.T, walk ? &S.X : nullptr, min_pts, H, C.ar, C.st, C.pin, &C.stats));
+        WM_TRY(core_distances(S.P, S.X, min_pts, C.precision == WM_PREC_FP64, H, C.ar, C.st, C.pin, &C.stats));
         C.stats.ms_core_dist = tc.ms();
     }
     E = C.ar.get<EdgeK>(n);

@@ -27,6 +27,9 @@
 // of the 10^7-point sets: the others cost little to ask, and more rounds are needed.)
 // The lists of the first search (all points, nothing pruned) serve the first few rounds.
 //
+// The plain form (WM_PREC_FP64) runs the same rounds with every point distance evaluated in FP64: a list
+// holds the FP64 distances rounded to FP32, whose band then only covers that rounding.
+//
 // HDBSCAN*: the weights are mutual reachability distances.  All edges with D <= max(cd2 p, cd2 q)
 // (the only ones that tie in general position) are in the k-NN pass's repair list, which a round
 // scans edge by edge; the search only has to find lighter edges with D above both core distances,
@@ -102,8 +105,13 @@ __device__ inline void note_err(float s, double w, float &err)
 // EXACT = false rebuilds the lists of the active points.  EXACT = true answers the points whose list may
 // have dropped a tie: every point within T(S[c]) is evaluated in FP64 and the K-minimum becomes the
 // point's candidate edge.
-template <int D, bool HDB, bool EXACT>
-__global__ void __launch_bounds__(kWalkThreads) nc_search_kernel(TravArgs a, NcArgs b, SearchTree X, int m_all)
+// Blocks per SM to compile for: 8 (64 registers) for the searches that run long; with 10 or 12 the EMST
+// searches spill (7-D, 10^7 points: 91 ms at 8, 94 at will, 121 and 152 at 10 and 12), and the short HDBSCAN*
+// searches above 3 dimensions are faster with all the registers they ask for.
+constexpr int search_blocks(int D, bool HDB, bool F64, bool EXACT) { return EXACT || F64 || (HDB && D > 3) ? 1 : 8; }
+
+template <int D, bool HDB, bool F64, bool EXACT>
+__global__ void __launch_bounds__(kWalkThreads, search_blocks(D, HDB, F64, EXACT)) nc_search_kernel(TravArgs a, NcArgs b, SearchTree X, int m_all)
 {
     __shared__ uint2 sst[kWalkStack][kWalkThreads];
     constexpr int S = row_floats(D), K = list_len(D);
@@ -160,30 +168,49 @@ __global__ void __launch_bounds__(kWalkThreads) nc_search_kernel(TravArgs a, NcA
                 const int j = j0 + min(p, sz - 1);
                 float x[S];
                 load_row<S, kStream>(X.rows, j, x);
-                const float s = row_dist<D>(q, x);
                 bool take = p < sz && __float_as_int(x[S - 1]) != c;
-                w[p] = s;
-                if (HDB) {
-                    const float cdm = fmaxf(qcd, a.cd32[j]);
-                    w[p] = fmaxf(s, cdm);
-                    take = take && w[p] < lim && !proven_repair(a, s, cdm);
+                if (F64) {
+                    // (FP64 is slow enough that even a point is first tried against the bound)
+                    take = take && point_bound<D>(q, x, 2.f * a.delta32) <= pb;
+                    ev += take;
+                } else {
+                    w[p] = row_dist<D>(q, x);
+                    if (HDB) {
+                        const float cdm = fmaxf(qcd, a.cd32[j]);
+                        take = take && !proven_repair(a, w[p], cdm);
+                        w[p] = fmaxf(w[p], cdm);
+                    }
+                    take = take && w[p] < lim;
                 }
-                if (take && w[p] < lim) todo |= 1u << p;
+                if (take) todo |= 1u << p;
             }
         }
-        ev += (unsigned)sz;
+        if (!F64) ev += (unsigned)sz;
         const float was = sl[0];
         while (todo) {
             const int p = __ffs(todo) - 1;
             todo &= todo - 1;
-            float v = w[0];
+            float v;
+            if (F64) {
+                float x[S];
+                load_row<S, kStream>(X.rows, j0 + p, x);
+                v = screen_dist<D, S, F64>(a.x64, n, a.d, X.rows, i, j0 + p, q, x);
+                if (HDB) {
+                    const float cdm = fmaxf(qcd, a.cd32[j0 + p]);
+                    if (proven_repair(a, v, cdm)) continue;
+                    v = fmaxf(v, cdm);
+                }
+                if (!(v < lim)) continue;
+            } else {
+                v = w[0];
 #pragma unroll
-            for (int r = 1; r < kBucket; ++r) v = r == p ? w[r] : v;
+                for (int r = 1; r < kBucket; ++r) v = r == p ? w[r] : v;
+            }
             if (EXACT) {
                 const int j = j0 + p;
                 double x2 = walk_dist64<D, S>(a.x64, n, a.d, X.rows, i, j);
                 if (HDB) x2 = pos_dmax(x2, pos_dmax(a.cd64[i], a.cd64[j]));
-                note_err(v, x2, err);
+                if (!F64) note_err(v, x2, err);
                 kmin_update(best, x2, a.pid[i], a.pid[j]);
                 ++n_re;
             } else if (v < lim) {
@@ -306,7 +333,7 @@ __device__ __forceinline__ void s_min(unsigned *S, int c, float v)
 
 // Advances the list heads past entries that joined the component; the first entry left bounds the
 // component's minimum.  A point without one offers its neighbours in tree order.
-template <int D, bool HDB>
+template <int D, bool HDB, bool F64>
 __global__ void nc_refresh_kernel(TravArgs a, NcArgs b)
 {
     constexpr int S = row_floats(D);
@@ -332,7 +359,7 @@ __global__ void nc_refresh_kernel(TravArgs a, NcArgs b)
                 float x[S], y[S];
                 load_row<S>(b.rows, i, x);
                 load_row<S>(b.rows, j, y);
-                float acc = row_dist<D>(x, y);
+                float acc = screen_dist<D, S, F64>(a.x64, n, a.d, b.rows, i, j, x, y);
                 if (HDB) acc = fmaxf(acc, fmaxf(a.cd32[i], a.cd32[j]));
                 s_min(b.S, c, acc);
             }
@@ -425,7 +452,7 @@ __global__ void nc_pick_kernel(TravArgs a, NcArgs b)
 
 // K-minimum of a picked point's list entries inside the band, in FP64 (on a dense list: an FP64
 // instruction costs a warp the same however few of its lanes need it)
-template <int D, bool HDB>
+template <int D, bool HDB, bool F64>
 __global__ void nc_cand_kernel(TravArgs a, NcArgs b)
 {
     constexpr int S = row_floats(D);
@@ -448,7 +475,7 @@ __global__ void nc_cand_kernel(TravArgs a, NcArgs b)
                 if (j < 0 || b.lab[j] == c) continue;
                 double w = walk_dist64<D, S>(a.x64, n, a.d, b.rows, i, j);
                 if (HDB) w = pos_dmax(w, pos_dmax(a.cd64[i], a.cd64[j]));
-                note_err(s, w, err);
+                if (!F64) note_err(s, w, err);
                 kmin_update(best, w, a.pid[i], a.pid[j]);
                 ++n_re;
             }
@@ -660,7 +687,7 @@ __global__ void nc_node_labels_kernel(int Ns, int S, const int2 *__restrict__ ra
     }
 }
 
-template <int D, bool HDB>
+template <int D, bool HDB, bool F64>
 int rounds(NcCall &C, TravArgs &a, NcArgs &b)
 {
     cudaStream_t st = C.st;
@@ -668,7 +695,7 @@ int rounds(NcCall &C, TravArgs &a, NcArgs &b)
     const int g = grid_for(n, 256), gt = grid_for(n, kTile);
     constexpr int S = row_floats(D);
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, nc_search_kernel<D, HDB, false>, kWalkThreads, 0) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, nc_search_kernel<D, HDB, F64, false>, kWalkThreads, 0) != cudaSuccess ||
         per_sm < 1)
         return WM_ECUDA;
     const int gs = std::min(num_sms() * per_sm, C.X->walk_blocks);
@@ -707,16 +734,16 @@ int rounds(NcCall &C, TravArgs &a, NcArgs &b)
         }
         b.first = !HDB && r == 0;
         if (!b.first) {
-            launch(nc_refresh_kernel<D, HDB>, g, 256, 0, st, a, b);
+            launch(nc_refresh_kernel<D, HDB, F64>, g, 256, 0, st, a, b);
             launch(nc_active_kernel<HDB>, g, 256, 0, st, a, b);
         }
         C.mark(C.ctx);
-        launch(nc_search_kernel<D, HDB, false>, gs, kWalkThreads, 0, st, a, b, X, n);
+        launch(nc_search_kernel<D, HDB, F64, false>, gs, kWalkThreads, 0, st, a, b, X, n);
         C.mark(C.ctx);
-        if (b.first) launch(nc_refresh_kernel<D, HDB>, g, 256, 0, st, a, b);   // the lists' minima into S
+        if (b.first) launch(nc_refresh_kernel<D, HDB, F64>, g, 256, 0, st, a, b);   // the lists' minima into S
         launch(nc_pick_kernel<HDB>, g, 256, 0, st, a, b);
-        launch(nc_cand_kernel<D, HDB>, g, 256, 0, st, a, b);
-        launch(nc_search_kernel<D, HDB, true>, gs, kWalkThreads, 0, st, a, b, X, n);
+        launch(nc_cand_kernel<D, HDB, F64>, g, 256, 0, st, a, b);
+        launch(nc_search_kernel<D, HDB, F64, true>, gs, kWalkThreads, 0, st, a, b, X, n);
         launch(nc_low_kernel, g, 256, 0, st, b);
         if (HDB) launch(nc_low_repair_kernel, grid_for(C.nrep, 256), 256, 0, st, b, rnow, rn);
         launch(nc_merge_kernel, g, 256, 0, st, a, b, cur, C.out, n - 1);
@@ -785,7 +812,9 @@ int nearest_component_rounds(NcCall &C, TravArgs &a)
     if (!(C.cap < INFINITY)) b.cap64 = ~0ull;
     int rc;
     const bool hdb = a.cd64 != nullptr;
-#define WM_NC(DV) rc = hdb ? rounds<DV, true>(C, a, b) : rounds<DV, false>(C, a, b)
+#define WM_NC(DV)                                                                          \
+    rc = a.fp64 ? (hdb ? rounds<DV, true, true>(C, a, b) : rounds<DV, false, true>(C, a, b)) \
+                : (hdb ? rounds<DV, true, false>(C, a, b) : rounds<DV, false, false>(C, a, b))
     const int wd = walk_dim(a.d);
     if (row_floats(wd) != C.X->S) { ar.off = mark; return WM_EINTERNAL; }
     switch (wd) {

@@ -15,7 +15,7 @@ struct HdbState {
     int nrep = 0;             //   weights, each pair once, in no particular order
 };
 
-int core_distances(const Points &P, const Tree *T, const SearchTree *X, int min_pts, HdbState &H, Arena &ar, cudaStream_t st,
+int core_distances(const Points &P, const SearchTree &X, int min_pts, bool fp64, HdbState &H, Arena &ar, cudaStream_t st,
                    int *pin, wm_stats *stats);
 // per node: min cd2 rounded down, max cd2 rounded up (for the WSPD traversals)
 int node_core_bounds(const Tree &T, const HdbState &H, float *cdmin, float *cdmax, Arena &ar, cudaStream_t st);

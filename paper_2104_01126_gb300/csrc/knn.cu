@@ -3,8 +3,8 @@
 // per-node cd_min / cd_max bounds (Table 1) and the repair edges that make the returned MST the
 // canonical one under the key K.
 //
-// k-NN, FP32 screen: one thread per query walks the search tree (stree.cuh), the nearer child first, and
-// keeps the minPts smallest screened values in a max-heap in shared memory (slot-major, one bank per
+// k-NN: one thread per query walks the search tree (stree.cuh), the nearer child first, and
+// keeps the minPts smallest screened (FP32) values in a 4-ary max-heap in shared memory (slot-major, one bank per
 // lane).  A node is skipped when its box is provably beyond the band threshold T of the heap's top, so
 // every point that the walk does not evaluate screens above T.  The smallest value that the heap
 // turned away or gave up (out) then tells whether the heap holds exactly the points screened within
@@ -13,8 +13,8 @@
 // collects every point within T(s_k), evaluates them in FP64 and selects the k-th; a band of more than
 // kTieCap points (heavy duplicates) is answered by an exact FP64 scan of all points.
 //
-// k-NN, plain FP64 form: one warp answers 32 consecutive tree positions with a shared depth-first
-// traversal of the k-d tree; each lane keeps the KL = minPts + 8 smallest values in a sorted list.
+// The plain FP64 form is the same walk with every point distance evaluated in FP64: the heap holds them
+// rounded to FP32.
 //
 // Repair edges: R = {(p,q), q != p : w2(p,q) <= cd2(p)}, weighted by the mutual reachability
 // distance.  Under general position every edge of the K-minimum spanning tree of G_MR either has
@@ -35,13 +35,8 @@ namespace wm {
 namespace {
 
 struct KnnArgs {
-    int N, n, d, k, KL;
-    const NodeRec *rec;  // FP64 form: packed node records (right child = left + 1)
-    const float *box;    // packed boxes, 2 DMP floats per node (DMP = d rounded up to 4, 8, 16) in groups of
-                         // four dimensions: lo[4c..4c+3], hi[4c..4c+3]
-    const float *x32;
-    const double *x64;
-    int stack_cap;       // FP64 form: entries of a warp's traversal stack (in shared memory): depth + 4
+    int n, d, k;
+    const double *x64;   // FP64 coordinates where the rows are rounded copies, else null
     double *cd64;
     float *cd32;
     int rq;              // slots of a repair row
@@ -57,185 +52,11 @@ struct KnnArgs {
                                 //     error of a screened k-th value against the exact one
 };
 
-// stride of the packed boxes: d rounded up to 4, 8 or 16
-template <int DM> constexpr int knn_dmp() { return DM <= 4 ? 4 : DM <= 8 ? 8 : 16; }
-
-// shared memory of one warp of the FP64 kernel: values, indices, stack
-__host__ __device__ inline size_t knn_warp_smem(int KL, int stack_cap)
-{
-    const size_t b = (size_t)KL * 32 * (sizeof(double) + sizeof(int)) + (size_t)stack_cap * sizeof(int);
-    return (b + 15) & ~(size_t)15;
-}
-
-template <int DM>
-__global__ void __launch_bounds__(256) knn64_kernel(KnnArgs a)
-{
-    extern __shared__ unsigned char smem_raw[];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int KL = a.KL;
-    // per-warp shared region: double sv[KL][32]; int sj[KL][32] (slot-major, one bank per lane);
-    // int stk[stack_cap] (the warp's traversal stack)
-    constexpr int DMP = knn_dmp<DM>(), DQ = DMP / 4;
-    size_t per_warp = knn_warp_smem(KL, a.stack_cap);
-    unsigned char *base = smem_raw + per_warp * wib;
-    double *sv = (double *)base;
-    int *sj = (int *)(sv + (size_t)KL * 32);
-    int *stk = sj + (size_t)KL * 32;
-    const int n = a.n, d = a.d;
-    unsigned long long n_ev = 0;
-    // 32-query groups handed out dynamically: their costs differ too much for a static deal
-    while (true) {
-        int q0 = 0;
-        if (lane == 0) q0 = atomicAdd(a.next_group, 32);
-        q0 = __shfl_sync(0xffffffffu, q0, 0);
-        if (q0 >= n) break;
-        const int i = q0 + lane;
-        const bool valid = i < n;
-        float qx[DMP];
-        double qx64[DM];
-#pragma unroll
-        for (int k = 0; k < DMP; ++k) qx[k] = k < d && valid ? a.x32[(size_t)k * n + i] : 0.f;
-#pragma unroll
-        for (int k = 0; k < DM; ++k)
-            if (k < d) qx64[k] = valid ? a.x64[(size_t)k * n + i] : 0.0;
-        // the group's centroid orders the children of a visited node (nearer first) without a
-        // reduction over the lanes at every node
-        float cent[DMP];
-        {
-            const float nv = (float)__popc(__ballot_sync(0xffffffffu, valid));
-#pragma unroll
-            for (int k = 0; k < DMP; ++k) {
-                float v = valid ? qx[k] : 0.f;
-                for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                cent[k] = v / nv;
-            }
-        }
-        int cnt = 0;
-        double thr = INFINITY;   // KL-th kept value (list full) or +inf
-        double cut = INFINITY;   // the current k-th value: a point above it can never be a candidate
-        int sp = 0;
-        if (lane == 0) stk[0] = 0;
-        sp = 1;
-        __syncwarp();
-        for (int guard = 0; sp > 0 && guard < 2 * a.N + 2; ++guard) {
-            int node = stk[sp - 1];
-            __syncwarp();
-            --sp;
-            const int4 L = a.rec[node].l;
-            const int b = L.x, e = L.y;
-            // prune test for each lane (packed box: groups of four dimensions, lo then hi, padding 0)
-            float lb = 0.f;
-            {
-                const float4 *bx = (const float4 *)(a.box + (size_t)node * 2 * DMP);
-#pragma unroll
-                for (int c = 0; c < DQ; ++c) {
-                    const float4 l4 = bx[2 * c], h4 = bx[2 * c + 1];
-                    const float lv[4] = {l4.x, l4.y, l4.z, l4.w}, hv[4] = {h4.x, h4.y, h4.z, h4.w};
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        const float g = fmaxf(fmaxf(lv[r] - qx[4 * c + r], qx[4 * c + r] - hv[r]), 0.f);
-                        lb = fmaf(g, g, lb);
-                    }
-                }
-            }
-            const double lw = lower_w2(lb);
-            const bool need = valid && lw <= cut * (1.0 + 1.0 / 131072.0) && (cnt < KL || lw <= thr);
-            if (!__any_sync(0xffffffffu, need)) continue;
-            if (e - b <= 32) {
-                // scan the subtree's points
-                const int m = e - b;
-                double px64[DM];
-#pragma unroll
-                for (int k = 0; k < DM; ++k)
-                    if (k < d) px64[k] = lane < m ? a.x64[(size_t)k * n + b + lane] : 0.0;
-                for (int p = 0; p < m; ++p) {
-                    double s = 0.0;
-#pragma unroll
-                    for (int k = 0; k < DM; ++k) {
-                        if (k < d) {
-                            double t = __dsub_rn(qx64[k], __shfl_sync(0xffffffffu, px64[k], p));
-                            s = __dadd_rn(s, __dmul_rn(t, t));
-                        }
-                    }
-                    if (valid && s <= cut && (cnt < KL || s < thr)) {
-                        int pos = cnt < KL ? cnt : KL - 1;
-                        while (pos > 0 && sv[(pos - 1) * 32 + lane] > s) {
-                            sv[pos * 32 + lane] = sv[(pos - 1) * 32 + lane];
-                            sj[pos * 32 + lane] = sj[(pos - 1) * 32 + lane];
-                            --pos;
-                        }
-                        sv[pos * 32 + lane] = s;
-                        sj[pos * 32 + lane] = b + p;
-                        if (cnt < KL) ++cnt;
-                        if (cnt >= a.k && pos < a.k) {
-                            cut = sv[(a.k - 1) * 32 + lane];
-                            // entries above the cut can never be candidates again: drop them
-                            while (cnt > a.k && sv[(cnt - 1) * 32 + lane] > cut) --cnt;
-                        }
-                        thr = cnt == KL ? sv[(KL - 1) * 32 + lane] : INFINITY;
-                    }
-                }
-                n_ev += (unsigned long long)m;
-            } else {
-                // push the farther child (from the group's centroid) first so the nearer one is
-                // visited next
-                const int c0 = L.z, c1 = L.z + 1;
-                const float4 *b0 = (const float4 *)(a.box + (size_t)c0 * 2 * DMP);
-                const float4 *b1 = (const float4 *)(a.box + (size_t)c1 * 2 * DMP);
-                float l0 = 0.f, l1 = 0.f;
-#pragma unroll
-                for (int c = 0; c < DQ; ++c) {
-                    const float4 lo0 = b0[2 * c], hi0 = b0[2 * c + 1], lo1 = b1[2 * c], hi1 = b1[2 * c + 1];
-                    const float a0[4] = {lo0.x, lo0.y, lo0.z, lo0.w}, z0[4] = {hi0.x, hi0.y, hi0.z, hi0.w};
-                    const float a1[4] = {lo1.x, lo1.y, lo1.z, lo1.w}, z1[4] = {hi1.x, hi1.y, hi1.z, hi1.w};
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        const float g0 = fmaxf(fmaxf(a0[r] - cent[4 * c + r], cent[4 * c + r] - z0[r]), 0.f);
-                        const float g1 = fmaxf(fmaxf(a1[r] - cent[4 * c + r], cent[4 * c + r] - z1[r]), 0.f);
-                        l0 = fmaf(g0, g0, l0);
-                        l1 = fmaf(g1, g1, l1);
-                    }
-                }
-                int first = l0 <= l1 ? c1 : c0, second = l0 <= l1 ? c0 : c1;
-                if (sp + 2 > a.stack_cap) {   // cannot happen: cap = depth + 4; reported, not ignored
-                    if (lane == 0) atomicOr(a.err, 1);
-                    sp = 0;
-                    break;
-                }
-                if (lane == 0) { stk[sp] = first; stk[sp + 1] = second; }
-                __syncwarp();
-                sp += 2;
-            }
-        }
-        if (!valid) continue;
-        const double cd2 = sv[(a.k - 1) * 32 + lane];
-        if (cnt == KL && !(sv[(KL - 1) * 32 + lane] > cd2)) {   // ties may have been dropped
-            a.slow[atomicAdd(a.slow_cnt, 1)] = i;
-            continue;
-        }
-        a.cd64[i] = cd2;
-        a.cd32[i] = __double2float_rn(cd2);
-        int r = 0;
-        for (int c = 0; c < cnt && r < a.rq; ++c) {
-            const double w = sv[c * 32 + lane];
-            if (!(w <= cd2)) break;
-            const int j = sj[c * 32 + lane];
-            if (j == i) continue;
-            a.rep_q[(size_t)r * n + i] = j;
-            a.rep_d[(size_t)r * n + i] = w;
-            ++r;
-        }
-        a.rep_cnt[i] = r;
-    }
-    for (int o = 16; o; o >>= 1) n_ev += __shfl_xor_sync(0xffffffffu, n_ev, o);
-    if (lane == 0) atomicAdd(a.stat + 0, n_ev);
-}
-
-// ------------------------------------------------------------------- FP32 screen, thread per query
+// -------------------------------------------------------------------------- thread per query
 // Shared memory of a block of T threads: uint2 stk[kWalkStack][T], uint2 heap[k][T] (value bits,
 // position), both slot-major: a lane's slots lie in its own banks, whatever slots its neighbours use.
-template <int D>
-__global__ void __launch_bounds__(kWalkThreads) knn_walk_kernel(KnnArgs a, SearchTree X, TravArgs band)
+template <int D, bool F64>
+__global__ void __launch_bounds__(kWalkThreads, F64 ? 1 : D <= 3 ? 8 : 6) knn_walk_kernel(KnnArgs a, SearchTree X, TravArgs band)
 {
     extern __shared__ uint2 walk_smem[];
     constexpr int S = row_floats(D);
@@ -273,26 +94,39 @@ __global__ void __launch_bounds__(kWalkThreads) knn_walk_kernel(KnnArgs a, Searc
 #pragma unroll
             for (int p = h; p < h + 4; ++p) {
                 float x[S];
-                load_row<S, kStream>(X.rows, j0 + min(p, sz - 1), x);
-                s[p] = row_dist<D>(q, x);
-                if (p < sz) {
-                    if (s[p] < top) todo |= 1u << p;
-                    else out = fminf(out, s[p]);
+                const int j = j0 + min(p, sz - 1);
+                load_row<S, kStream>(X.rows, j, x);
+                if (F64) {
+                    // (FP64 is slow enough that even a point is first tried against the bound)
+                    if (p < sz && point_bound<D>(q, x, 2.f * band.delta32) <= pb) todo |= 1u << p;
+                } else {
+                    s[p] = row_dist<D>(q, x);
+                    if (p < sz) {
+                        if (s[p] < top) todo |= 1u << p;
+                        else out = fminf(out, s[p]);
+                    }
                 }
             }
         }
-        ev += (unsigned)sz;
+        ev += F64 ? __popc(todo) : (unsigned)sz;
         while (todo) {
             const int p = __ffs(todo) - 1;
             todo &= todo - 1;
-            float v = s[0];
+            float v;
+            if (F64) {
+                float x[S];
+                load_row<S, kStream>(X.rows, j0 + p, x);
+                v = screen_dist<D, S, F64>(a.x64, n, a.d, X.rows, i, j0 + p, q, x);
+            } else {
+                v = s[0];
 #pragma unroll
-            for (int r = 1; r < kBucket; ++r) v = r == p ? s[r] : v;
+                for (int r = 1; r < kBucket; ++r) v = r == p ? s[r] : v;
+            }
             const uint2 mine = make_uint2(__float_as_uint(v), (unsigned)(j0 + p));
             if (cnt < k) {   // fill: sift up
                 int h = cnt++;
                 while (h > 0) {
-                    const int u = (h - 1) >> 1;
+                    const int u = (h - 1) >> 2;
                     const uint2 e = heap[u * T];
                     if (__uint_as_float(e.x) >= v) break;
                     heap[h * T] = e;
@@ -304,12 +138,15 @@ __global__ void __launch_bounds__(kWalkThreads) knn_walk_kernel(KnnArgs a, Searc
                 out = fminf(out, top);
                 int h = 0;
                 while (true) {
-                    int u = 2 * h + 1;
-                    if (u >= k) break;
-                    uint2 e = heap[u * T];
-                    if (u + 1 < k) {
-                        const uint2 f = heap[(u + 1) * T];
-                        if (__uint_as_float(f.x) > __uint_as_float(e.x)) { e = f; ++u; }
+                    const int u0 = 4 * h + 1;
+                    if (u0 >= k) break;
+                    int u = u0;
+                    uint2 e = heap[u0 * T];
+#pragma unroll
+                    for (int c = 1; c < 4; ++c) {
+                        const int uc = min(u0 + c, k - 1);
+                        const uint2 f = heap[uc * T];
+                        if (__uint_as_float(f.x) > __uint_as_float(e.x)) { e = f; u = uc; }
                     }
                     if (__uint_as_float(e.x) <= v) break;
                     heap[h * T] = e;
@@ -350,7 +187,7 @@ __global__ void __launch_bounds__(kWalkThreads) knn_walk_kernel(KnnArgs a, Searc
         a.cd64[i] = cd2;
         a.cd32[i] = __double2float_rn(cd2);
         a.rep_cnt[i] = r;
-        if (cd2 > 0.0)
+        if (!F64 && cd2 > 0.0)
             kerr = fmaxf(kerr, __fdiv_ru(__double2float_ru(fabs((double)top - cd2)), __double2float_rd(cd2)));
     };
     walk_queries<D, S, kStream>(X, n, a.next_group, walk_smem + threadIdx.x, T, X.deep + (size_t)blockIdx.x * T + threadIdx.x,
@@ -369,7 +206,7 @@ __global__ void __launch_bounds__(kWalkThreads) knn_walk_kernel(KnnArgs a, Searc
 // k-th value, evaluates them in FP64 and takes the k-th smallest.
 constexpr int kTieCap = 512, kTieWarps = 4;
 
-template <int D>
+template <int D, bool F64>
 __global__ void __launch_bounds__(32 * kTieWarps) knn_tie_kernel(KnnArgs a, SearchTree X, TravArgs band,
                                                                  const int *__restrict__ m_dev, int *next, int *slow2,
                                                                  int *slow2_cnt, int *extra_q, int *extra_p,
@@ -412,7 +249,7 @@ __global__ void __launch_bounds__(32 * kTieWarps) knn_tie_kernel(KnnArgs a, Sear
                     j = (int)(ref & 0x0fffffffu) + lane;
                     float x[S];
                     load_row<S>(X.rows, j, x);
-                    take = row_dist<D>(q, x) <= Tk;
+                    take = screen_dist<D, S, F64>(a.x64, n, a.d, X.rows, i, j, q, x) <= Tk;
                 }
                 const unsigned b = __ballot_sync(0xffffffffu, take);
                 const int slot = c + __popc(b & lanemask_lt());
@@ -666,17 +503,15 @@ __global__ void core_out_kernel(const double *__restrict__ cd64, const int *__re
 constexpr int kWalkSmemMax = 100 << 10;    // (kWalkStack + minPts) entries for at least 32 threads
 constexpr int kTieSmemMax = 64 << 10;      // stacks of kTieWarps warps in the deepest tree (FP32 exponents
                                            // and mantissas allow about 3800 levels in 16 dimensions)
-constexpr int kKnn64SmemMax = 128 << 10;   // lists of minPts + 8 entries and a stack for one warp
-static_assert((kWalkStack + kMaxMinPts) * 32 * 8 <= kWalkSmemMax && (kMaxMinPts + 8) * 32 * 12 + 3800 * 4 <= kKnn64SmemMax,
-              "shared memory limits of the k-NN kernels");
+static_assert((kWalkStack + kMaxMinPts) * 32 * 8 <= kWalkSmemMax, "shared memory limit of the k-NN walk");
 
-// core distances and repair edges: by the walk on the search tree X, or (the plain FP64 form) on the tree T
-int core_distances(const Points &P, const Tree *T, const SearchTree *X, int min_pts, HdbState &H, Arena &ar, cudaStream_t st,
-                    int *pin, wm_stats *stats)
+// core distances and repair edges (fp64: the plain form)
+int core_distances(const Points &P, const SearchTree &X, int min_pts, bool fp64, HdbState &H, Arena &ar, cudaStream_t st,
+                   int *pin, wm_stats *stats)
 {
     const int n = P.n, d = P.d;
     if (min_pts > kMaxMinPts) return WM_EINVAL;
-    const int KL = std::min(min_pts + 8, n);
+    const int KL = std::min(min_pts + 8, n);   // a point's repair edges: itself left out, up to 8 more by ties
     H.cd64 = ar.get<double>(n);
     H.cd32 = ar.get<float>(n);
     if (ar.failed) return WM_ENOMEM;
@@ -688,8 +523,8 @@ int core_distances(const Points &P, const Tree *T, const SearchTree *X, int min_
     size_t mark = ar.off;
     KnnArgs a;
     memset(&a, 0, sizeof a);
-    a.n = n; a.d = d; a.k = min_pts; a.KL = KL;
-    a.x32 = P.x32; a.x64 = P.x64;
+    a.n = n; a.d = d; a.k = min_pts;
+    a.x64 = P.x64;
     a.cd64 = H.cd64; a.cd32 = H.cd32;
     a.rq = RQ;
     a.rep_q = ar.get<int>((size_t)n * RQ);
@@ -713,42 +548,11 @@ int core_distances(const Points &P, const Tree *T, const SearchTree *X, int min_
     cudaEvent_t k0, k1;
     cudaEventCreate(&k0);
     cudaEventCreate(&k1);
-    if (!X) {
-        const int N = T->N;
-        a.N = N;
-        a.stack_cap = T->depth + 4;
-        // launch shape: warps per block limited by shared memory; the grid fills the SMs
-        const int dmp = d <= 3 ? 4 : d <= 7 ? 8 : 16;   // = knn_dmp<DM> of the instantiation used
-        const size_t per_warp = knn_warp_smem(KL, a.stack_cap);
-        const int wpb = (int)std::min<size_t>(8, std::max<size_t>(1, (48u << 10) / per_warp));
-        const size_t smem = per_warp * wpb;
-        const int blocks = num_sms() * std::max(1, 32 / wpb);
-        // packed node records and boxes (the traversal reads a node with two or three vector loads)
-        NodeRec *rec = ar.get<NodeRec>(N);
-        float *box = ar.get<float>((size_t)N * 2 * dmp);
-        if (!rec || !box) { cudaEventDestroy(k0); cudaEventDestroy(k1); return WM_ENOMEM; }
-        pack_nodes(*T, d, dmp, rec, box, st);
-        a.rec = rec;
-        a.box = box;
-        cudaEventRecord(k0, st);
-#define WM_KNN(DM)                                                                                            \
-    do {                                                                                                      \
-        cudaFuncSetAttribute(knn64_kernel<DM>, cudaFuncAttributeMaxDynamicSharedMemorySize, kKnn64SmemMax);   \
-        launch(knn64_kernel<DM>, blocks, 32 * wpb, smem, st, a);                                              \
-    } while (0)
-        if (d <= 2) WM_KNN(2);
-        else if (d <= 3) WM_KNN(3);
-        else if (d <= 5) WM_KNN(5);
-        else if (d <= 7) WM_KNN(7);
-        else WM_KNN(16);
-#undef WM_KNN
-        cudaEventRecord(k1, st);
-        cudaMemcpyAsync(cnts + 7, cnts, sizeof(int), cudaMemcpyDeviceToDevice, st);   // all ties: the full scan
-        slow2 = a.slow;
-    } else {
+    {
         TravArgs band;
-        band.eta = 2.0 * (double)P.delta * sqrt((double)d) * (1.0 + 1e-6);
+        band.eta = fp64 ? 0.0 : 2.0 * (double)P.delta * sqrt((double)d) * (1.0 + 1e-6);
         band.exact32 = band.eta == 0.0;
+        band.delta32 = P.delta;
         band.eta2_f = (float)(2.0 * band.eta);
         if ((double)band.eta2_f < 2.0 * band.eta) band.eta2_f = std::nextafter(band.eta2_f, INFINITY);
         // threads per block: four warps while two blocks of them fit an SM's shared memory
@@ -756,29 +560,32 @@ int core_distances(const Points &P, const Tree *T, const SearchTree *X, int min_
         int threads = kWalkThreads;
         while (threads > 32 && per_thread * threads > (size_t)kWalkSmemMax) threads >>= 1;
         const size_t smem = per_thread * threads;
-        const size_t smem_tie = (size_t)kTieWarps * (X->stack_cap + 2) * sizeof(unsigned);
+        const size_t smem_tie = (size_t)kTieWarps * (X.stack_cap + 2) * sizeof(unsigned);
         int rc = 0;
-#define WM_KNN(DM)                                                                                            \
+#define WM_KNN_(DM, F)                                                                                            \
     do {                                                                                                      \
         int per_sm = 0;                                                                                       \
-        if (cudaFuncSetAttribute(knn_walk_kernel<DM>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWalkSmemMax) != cudaSuccess || \
-            cudaFuncSetAttribute(knn_tie_kernel<DM>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTieSmemMax) != cudaSuccess || \
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, knn_walk_kernel<DM>, threads, smem) != cudaSuccess || \
+        if (cudaFuncSetAttribute(knn_walk_kernel<DM, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWalkSmemMax) != cudaSuccess || \
+            cudaFuncSetAttribute(knn_tie_kernel<DM, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTieSmemMax) != cudaSuccess || \
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, knn_walk_kernel<DM, F>, threads, smem) != cudaSuccess || \
             per_sm < 1) {                                                                                     \
             rc = WM_ECUDA;                                                                                    \
             break;                                                                                            \
         }                                                                                                     \
         const int blocks = (int)std::min<long long>(std::min<long long>((long long)num_sms() * per_sm,        \
-                                                    (long long)X->walk_blocks * (kWalkThreads / threads)),    \
+                                                    (long long)X.walk_blocks * (kWalkThreads / threads)),    \
                                                     ((long long)n + threads - 1) / threads);                  \
         cudaEventRecord(k0, st);                                                                              \
-        launch(knn_walk_kernel<DM>, blocks, threads, smem, st, a, *X, band);                                  \
-        launch(knn_tie_kernel<DM>, num_sms() * 4, 32 * kTieWarps, smem_tie, st, a, *X, band, cnts, cnts + 4, slow2,   \
+        launch(knn_walk_kernel<DM, F>, blocks, threads, smem, st, a, X, band);                                  \
+        launch(knn_tie_kernel<DM, F>, num_sms() * 4, 32 * kTieWarps, smem_tie, st, a, X, band, cnts, cnts + 4, slow2,   \
                cnts + 7, ex_q, ex_p, ex_d, cnts + 1, extra_cap, cnts + 2);                                    \
         cudaEventRecord(k1, st);                                                                              \
     } while (0)
+#define WM_KNN(DM)                 \
+    if (fp64) WM_KNN_(DM, true);   \
+    else WM_KNN_(DM, false)
         const int wd = walk_dim(d);
-        if (row_floats(wd) != X->S) rc = WM_EINTERNAL;
+        if (row_floats(wd) != X.S) rc = WM_EINTERNAL;
         else switch (wd) {
             case 2: WM_KNN(2); break;
             case 3: WM_KNN(3); break;
@@ -791,6 +598,7 @@ int core_distances(const Points &P, const Tree *T, const SearchTree *X, int min_
             default: WM_KNN(16); break;
             }
 #undef WM_KNN
+#undef WM_KNN_
         if (rc) {
             cudaGetLastError();
             cudaEventDestroy(k0);
@@ -816,7 +624,7 @@ int core_distances(const Points &P, const Tree *T, const SearchTree *X, int min_
     if (nslow > 0) {
         size_t sm2 = (size_t)min_pts * 32 * 8 + 32 * 4;
         cudaFuncSetAttribute(knn_slow_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxMinPts * 32 * 8 + 32 * 4);
-        launch(knn_slow_kernel, std::min(nslow, num_sms() * 8), 32, sm2, st, a, X ? X->rows : nullptr, X ? X->S : 0, slow2, nslow, ex_q, ex_p, ex_d, cnts + 1,
+        launch(knn_slow_kernel, std::min(nslow, num_sms() * 8), 32, sm2, st, a, X.rows, X.S, slow2, nslow, ex_q, ex_p, ex_d, cnts + 1,
                                                                      extra_cap, cnts + 2);
     }
     // repair edges: one copy of each, weighted, in no particular order (each round takes those it needs)

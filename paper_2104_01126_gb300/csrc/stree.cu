@@ -52,7 +52,7 @@ struct LNode {
 };
 
 struct StArgs {
-    int n, d, dtype, layout;
+    int n, d, dtype, layout, widen;
     const void *src;
     float *buf[2];           // point rows, ping-pong; buf[0] becomes the final array
     float *nodes;
@@ -144,7 +144,7 @@ __device__ inline void choose_split(const unsigned *acc, int d, int &dim, float 
     }
 }
 
-// box of a node row, widened by delta so that it holds the FP64 points
+// box of a node row, widened by delta (see build_search_tree)
 template <int S>
 __device__ inline void write_box(float *row, const unsigned *acc, int d, float delta)
 {
@@ -169,7 +169,7 @@ template <int S>
 __global__ void st_root_kernel(StArgs a)
 {
     BuildState &s = *a.state;
-    write_box<S>(a.nodes, a.root_acc, a.d, __uint_as_float(s.delta));
+    write_box<S>(a.nodes, a.root_acc, a.d, a.widen * __uint_as_float(s.delta));
     a.range[0] = make_int2(0, a.n);
     a.parent[0] = -1;
     int dim;
@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(1024) st_level_kernel(StArgs a, int level)
     __shared__ int sh[32];
     __shared__ int s_act, s_units;
     const int A = a.state->active, id0 = a.state->next_id, d = a.d, cur = level & 1;
-    const float delta = __uint_as_float(a.state->delta);
+    const float delta = a.widen * __uint_as_float(a.state->delta);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (threadIdx.x == 0) { s_act = 0; s_units = 0; }
     __syncthreads();
@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(kStThreads) st_block_kernel(StArgs a)
     float *sval = (float *)(seg + 2 * (M / 8));      // [2][M / 8]
     __shared__ int s_entry, s_next, s_base;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, d = a.d;
-    const float delta = __uint_as_float(a.state->delta);
+    const float delta = a.widen * __uint_as_float(a.state->delta);
     const int nsub = a.state->subs;
     while (true) {
         if (threadIdx.x == 0) s_entry = atomicAdd(&a.state->sub_next, 1);
@@ -596,7 +596,7 @@ int build(StArgs &a, SearchTree &X, Points &P, Arena &ar, cudaStream_t st, int *
 
 // Search tree and tree-order points of the input (device memory); n < 2^28 (28-bit positions in a
 // bucket's reference).  P.x64 is set when the FP32 copy is inexact (FP64 input); P.x32 is not.
-int build_search_tree(const void *src, int n, int d, int dtype, int layout, Points &P, SearchTree &X, Arena &ar,
+int build_search_tree(const void *src, int n, int d, int dtype, int layout, int widen, Points &P, SearchTree &X, Arena &ar,
                       cudaStream_t st, int *pin)
 {
     P.n = n;
@@ -608,6 +608,7 @@ int build_search_tree(const void *src, int n, int d, int dtype, int layout, Poin
     a.d = d;
     a.dtype = dtype;
     a.layout = layout;
+    a.widen = widen;
     a.src = src;
     X.rows = a.buf[0] = ar.get<float>((size_t)n * X.S);
     X.nodes = a.nodes = ar.get<float>((size_t)(2LL * n) * 2 * X.S);

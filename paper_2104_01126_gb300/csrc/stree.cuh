@@ -43,7 +43,9 @@ __host__ __device__ constexpr int walk_dim(int d) { return d <= 2 ? 2 : d <= 8 ?
 constexpr bool walk_dims_fit(int d) { return d > 16 || (walk_dim(d) >= d && row_floats(walk_dim(d)) == row_floats(d) && walk_dims_fit(d + 1)); }
 static_assert(walk_dims_fit(1), "a walk's rows must be as wide as the search tree's");
 
-int build_search_tree(const void *src, int n, int d, int dtype, int layout, Points &P, SearchTree &X, Arena &ar,
+// widen: the boxes are widened by this multiple of the FP32 copy's error: 1 when distances are screened
+// in FP32 (both points rounded alike), 2 when they are exact but the walk bounds them from the rounded query
+int build_search_tree(const void *src, int n, int d, int dtype, int layout, int widen, Points &P, SearchTree &X, Arena &ar,
                       cudaStream_t st, int *pin);
 
 __host__ __device__ inline unsigned bucket_ref(int first, int size) { return kBucketBit | (unsigned)(size - 1) << 28 | (unsigned)first; }
@@ -118,6 +120,29 @@ __device__ inline double walk_dist64(const double *__restrict__ x64, int n, int 
         }
     }
     return s;
+}
+
+// screened distance of positions i (row q) and j (row x): the FP32 distance of the rows, or in the plain
+// form the FP64 distance rounded to FP32 (which only orders lists and bounds; decisions compare FP64)
+template <int D, int S, bool F64>
+__device__ inline float screen_dist(const double *__restrict__ x64, int n, int d, const float *__restrict__ rows, int i, int j,
+                                    const float (&q)[S], const float (&x)[S])
+{
+    return F64 ? __double2float_rn(walk_dist64<D, S>(x64, n, d, rows, i, j)) : row_dist<D>(q, x);
+}
+
+// rigorous lower bound of the FP64 squared distance from two rows whose coordinates err by at most
+// delta2 together: the node bound of visit_children for a single point
+template <int D, int S>
+__device__ __forceinline__ float point_bound(const float (&q)[S], const float (&x)[S], float delta2)
+{
+    float g = 0.f;
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+        const float t = fmaxf(fabsf(q[k] - x[k]) - delta2, 0.f);
+        g = fmaf(t, t, g);
+    }
+    return lower_w2(g);
 }
 
 // One visit: rigorous lower bounds of the FP64 squared distance from q to the boxes of the children

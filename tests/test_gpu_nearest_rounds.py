@@ -92,3 +92,18 @@ def test_batch_instances_stay_apart():
         ref = oracle.emst(x) if mp <= 1 else oracle.hdbscan(x, mp, s=s)
         for k in ("u", "v", "w") + (HDB_KEYS if mp > 1 else ()):
             assert np.array_equal(to_np(r[k]), ref[k]), k
+
+
+@pytest.mark.parametrize("name", ["grid2", "coarse5", "copies40", "offset", "offset5", "gaps", "deep"])
+def test_plain_form(name):
+    # every distance in FP64: no screen error, the same trees, with rounded and exact FP32 rows
+    x = np.ascontiguousarray(SETS[name])
+    got = wm.emst(x, precision="fp64", return_stats=True)
+    assert got["stats"].max_rel_screen_err == 0.0 and got["stats"].getpairs_visits == 0
+    assert_same_tree({k: to_np(got[k]) for k in ("u", "v", "w")}, oracle.emst_at_scale(x))
+    if name in ("offset5", "gaps"):
+        h = wm.hdbscan(x, min_pts=5, precision="fp64", return_stats=True)
+        ref = oracle.hdbscan_at_scale(x, 5, 0)
+        assert h["stats"].max_rel_screen_err == 0.0
+        for k in ("u", "v", "w") + HDB_KEYS:
+            assert np.array_equal(to_np(h[k]), ref[k]), k
