@@ -1,16 +1,16 @@
 // dendro.cu -- ordered dendrogram and reachability plot of a weighted spanning tree (Sec. 4).
 //
 // Input: the n-1 tree edges sorted by K (rank i = position).  Dendrogram node n+i is the merge
-// of edge i; leaves are the points.  The construction follows the top-down heavy/light scheme
-// of Sec. 4.2 with the heavy set of a subproblem taken as the edges in the upper half of its
-// rank interval (interval halves are global bit positions of the rank, so there are
-// ceil(log2(n-1)) levels).  At each level, per subproblem:
-//   light components  = connected components of the light edges over the current supervertices
-//                       (union-find over supervertex ids);
-//   a light component's dendrogram root (its heaviest light edge) hangs below the lightest
-//   heavy edge incident to the component (a WriteMin), which is the first merge touching it;
-//   heavy edges are relabelled to the light components' roots and form the next subproblem.
-// Every leaf hangs below its lightest incident edge.
+// of edge i; leaves are the points.  The parents come from contracting the tree bottom-up (after
+// Sao, Prokopenko and Lebrun-Grandie, PANDORA, 2024; the output is that of Sec. 4): a level contracts the
+// lightest edge P(v) of every vertex v, as a Boruvka round does, and the contracted components are the
+// vertices of the next level, at most half as many.  An edge that is the lightest at one of its ends has
+// a vertex below it, so it does not branch, and contracting it only shortens a chain of the dendrogram.
+// Let V be the vertex that an edge e is contracted into.  While P(V) is lighter than e, e lies above P(V)
+// and V is replaced by the next level's vertex that contains it; the V at which this stops names the
+// chain of e: the edges that stop at V, in rank order, hang below one another, and the last of them
+// below P(V).  Every leaf hangs below its lightest incident edge.  (The heavy/light recursion of Sec. 4.2
+// passes over all edges once per bit of the rank; here level l has at most n / 2^l vertices.)
 //
 // Order (Sec. 4.2, ordering theorem): with the tree rooted at s, the child of merge (u,v) that
 // contains the endpoint nearer s is the left child.  The tree is rooted by an Euler tour and list
@@ -153,196 +153,196 @@ __global__ void rooting_kernel(const EdgeK *__restrict__ E, int m, const int *__
     }
 }
 
-// ------------------------------------------------------------------ heavy/light recursion
-__global__ void leaf_parent_kernel(const EdgeK *__restrict__ E, int m, int *pmin)
+// ---------------------------------------------------------------------- contraction levels
+// Vertices of all levels share one index space: level l holds [off[l], off[l] + nv[l]), level 0 the n
+// points.  Per vertex: P (rank of its lightest edge, kNoRank: none left), hook (link to the other end of
+// that edge, or itself at the root of its component) and next (the next level's vertex).
+constexpr int kNoRank = 0x7f7f7f7f;   // above every rank; a byte pattern that cudaMemset can write
+constexpr int kLevelsMax = 40;
+
+struct Contract {
+    int *cu, *cv;            // ends of an edge in the current level, by rank
+    int *list[2];            // ranks of the edges left
+    int *P, *hook, *next;
+    int *sup;                // vertex an edge was contracted into
+    int *off, *nv, *ne;      // per level
+    int cap;                 // vertices of all levels
+};
+
+__global__ void ct_init_kernel(const EdgeK *__restrict__ E, int m, int n, Contract c)
 {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
-        atomicMin(&pmin[edge_u(E[i])], i);
-        atomicMin(&pmin[edge_v(E[i])], i);
+        c.cu[i] = edge_u(E[i]);
+        c.cv[i] = edge_v(E[i]);
+        c.list[0][i] = i;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        c.off[0] = 0;
+        c.nv[0] = n;
+        c.ne[0] = m;
     }
 }
 
-__global__ void leaf_parent_set_kernel(const int *__restrict__ pmin, int n, int *__restrict__ par)
+// the steps of a level, for one edge or vertex
+__device__ __forceinline__ void ct_lightest(const Contract &c, int r)
 {
-    for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < n; x += gridDim.x * blockDim.x)
-        par[x] = pmin[x] == 0x7fffffff ? -1 : n + pmin[x];
+    const int u = __ldcg(c.cu + r), v = __ldcg(c.cv + r);
+    if (r < __ldcg(c.P + u)) atomicMin(c.P + u, r);
+    if (r < __ldcg(c.P + v)) atomicMin(c.P + v, r);
 }
 
-__global__ void endpoints_init_kernel(const EdgeK *__restrict__ E, int m, int *__restrict__ ex, int *__restrict__ ey)
+// links v along its lightest edge; true at the root of a component (of a mutual choice, the smaller one)
+__device__ __forceinline__ bool ct_hook(const Contract &c, int v)
 {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
-        ex[i] = edge_u(E[i]);
-        ey[i] = edge_v(E[i]);
+    const int r = __ldcg(c.P + v);
+    c.next[v] = -1;
+    if (r == kNoRank) {   // nothing left to join
+        c.hook[v] = v;
+        return false;
     }
+    const int a = __ldcg(c.cu + r), o = a == v ? __ldcg(c.cv + r) : a;
+    const bool root = __ldcg(c.P + o) == r && v <= o;
+    c.hook[v] = root ? v : o;
+    return root;
 }
 
-__device__ inline int uf_find(int *uf, int x)
+__device__ __forceinline__ int ct_root(const Contract &c, int v, int limit)
 {
-    for (int it = 0; it < (1 << 30); ++it) {
-        int p = uf[x];
-        if (p == x) return x;
-        int g = uf[p];
-        if (g != p) uf[x] = g;
+    int x = v;
+    for (int it = 0; it < limit; ++it) {
+        const int p = *(volatile int *)(c.hook + x);
+        if (p == x) break;
+        const int g = *(volatile int *)(c.hook + p);
+        if (g != p) *(volatile int *)(c.hook + x) = g;   // path halving (the forest is static)
         x = p;
     }
     return x;
 }
 
-__global__ void level_init_kernel(const int *__restrict__ ex, const int *__restrict__ ey, int m, int *uf, int *rootrank,
-                                  int *minheavy)
+// a contracted edge notes its component; another one moves to the next level
+__device__ __forceinline__ bool ct_edge(const Contract &c, int r)
 {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
-        int a = ex[i], b = ey[i];
-        uf[a] = a; uf[b] = b;
-        rootrank[a] = -1; rootrank[b] = -1;
-        minheavy[a] = 0x7fffffff; minheavy[b] = 0x7fffffff;
+    const int u = __ldcg(c.cu + r), v = __ldcg(c.cv + r);
+    const int nu = __ldcg(c.next + u);
+    if (u == v || __ldcg(c.P + u) == r || __ldcg(c.P + v) == r) {
+        c.sup[r] = nu;
+        return false;
     }
+    c.cu[r] = nu;
+    c.cv[r] = __ldcg(c.next + v);
+    return true;
 }
 
-__global__ void level_union_kernel(const int *__restrict__ ex, const int *__restrict__ ey, int m, int bit, int *uf)
+__global__ void ct_lightest_kernel(Contract c, int level)
 {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
-        if ((i >> bit) & 1) continue;   // heavy at this level
-        int x = ex[i], y = ey[i];
-        for (int it = 0; it < (1 << 24); ++it) {
-            int a = uf_find(uf, x), b = uf_find(uf, y);
-            if (a == b) break;
-            if (a > b) { int t = a; a = b; b = t; }
-            if (atomicCAS(&uf[b], b, a) == b) break;
+    const int m = c.ne[level];
+    const int *list = c.list[level & 1];
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < m; t += gridDim.x * blockDim.x) ct_lightest(c, list[t]);
+}
+
+__global__ void ct_hook_kernel(Contract c, int level, int *bad)
+{
+    __shared__ int sh[32];
+    const int m = c.nv[level], off = c.off[level], to = off + m;
+    if (blockIdx.x == 0 && threadIdx.x == 0) c.off[level + 1] = to;
+    for (int b0 = blockIdx.x * blockDim.x; b0 < m; b0 += gridDim.x * blockDim.x) {
+        const int t = b0 + threadIdx.x;
+        const bool root = t < m && ct_hook(c, off + t);
+        const int slot = to + block_append(c.nv + level + 1, root ? 1 : 0, sh);
+        if (root) {
+            if (slot < c.cap) c.next[off + t] = slot;
+            else atomicOr(bad, 16);
         }
     }
 }
 
-// Component roots of every edge's endpoints (rx, ry; ry for heavy edges only), rootrank (largest
-// light edge of a component) and minheavy (smallest heavy edge touching it).  The updates are
-// aggregated per warp: edges of one warp often share a component (a large one at the top levels),
-// so each group of equal roots issues one atomic.
-__global__ void level_mark_kernel(const int *__restrict__ ex, const int *__restrict__ ey, int m, int bit, int *uf,
-                                  int *rootrank, int *minheavy, int *__restrict__ rx, int *__restrict__ ry)
+__global__ void ct_next_kernel(Contract c, int level)
 {
-    const int lane = threadIdx.x & 31;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i - lane < m; i += gridDim.x * blockDim.x) {
-        const bool ok = i < m;
-        const bool light = ok && ((i >> bit) & 1) == 0, heavy = ok && !light;
-        const int kx = ok ? uf_find(uf, ex[i]) : -1;
-        const int ky = heavy ? uf_find(uf, ey[i]) : -1;
-        if (ok) { rx[i] = kx; ry[i] = ky; }
-        int key = light ? kx : -1;
-        unsigned grp = __match_any_sync(0xffffffffu, key);
-        int v = __reduce_max_sync(grp, light ? i : -1);
-        if (key >= 0 && lane == __ffs(grp) - 1) atomicMax(&rootrank[key], v);
-        key = heavy ? kx : -1;
-        grp = __match_any_sync(0xffffffffu, key);
-        v = __reduce_min_sync(grp, heavy ? i : 0x7fffffff);
-        if (key >= 0 && lane == __ffs(grp) - 1) atomicMin(&minheavy[key], v);
-        grp = __match_any_sync(0xffffffffu, ky);
-        v = __reduce_min_sync(grp, heavy ? i : 0x7fffffff);
-        if (ky >= 0 && lane == __ffs(grp) - 1) atomicMin(&minheavy[ky], v);
+    const int m = c.nv[level], off = c.off[level];
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < m; t += gridDim.x * blockDim.x) {
+        const int x = ct_root(c, off + t, m);
+        if (x != off + t) c.next[off + t] = *(volatile int *)(c.next + x);
     }
 }
 
-// Parents of the light components' top merges; heavy endpoints relabelled to their component's
-// top merge.  The next level's union-find entries and its (other) rootrank / minheavy set are
-// initialised here for the endpoints each edge has from now on: this level reads neither.
-__global__ void level_link_kernel(int *ex, int *ey, int m, int bit, int n, const int *__restrict__ rx,
-                                  const int *__restrict__ ry, const int *__restrict__ rootrank,
-                                  const int *__restrict__ minheavy, int *__restrict__ par, int *uf, int *rr_next,
-                                  int *mh_next)
+__global__ void ct_edge_kernel(Contract c, int level)
 {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
-        int x = ex[i], y = ey[i];
-        if (((i >> bit) & 1) == 0) {
-            const int c = rx[i];
-            if (rootrank[c] == i && minheavy[c] != 0x7fffffff) par[n + i] = n + minheavy[c];
-        } else {
-            const int cx = rx[i], cy = ry[i];
-            x = rootrank[cx] >= 0 ? n + rootrank[cx] : cx;
-            y = rootrank[cy] >= 0 ? n + rootrank[cy] : cy;
-            ex[i] = x;
-            ey[i] = y;
-        }
-        uf[x] = x; uf[y] = y;
-        rr_next[x] = -1; rr_next[y] = -1;
-        mh_next[x] = 0x7fffffff; mh_next[y] = 0x7fffffff;
+    __shared__ int sh[32];
+    const int m = c.ne[level];
+    const int *list = c.list[level & 1];
+    int *out = c.list[(level & 1) ^ 1];
+    for (int b0 = blockIdx.x * blockDim.x; b0 < m; b0 += gridDim.x * blockDim.x) {
+        const int t = b0 + threadIdx.x;
+        const int r = t < m ? list[t] : -1;
+        const bool keep = r >= 0 && ct_edge(c, r);
+        const int slot = block_append(c.ne + level + 1, keep ? 1 : 0, sh);
+        if (keep) out[slot] = r;
     }
 }
 
-// The lowest kLeafLevels levels: the subproblems are aligned blocks of at most kLeafChunk edges
-// that share no vertex (after the relabelling of the levels above, every vertex and merge node
-// occurs in one subproblem of a level), so one CTA runs all of them for its block in shared
-// memory.  Vertices get local ids on entry (the first occurrence claims map[v]); the merge node
-// of local edge r is 2 * kLeafChunk + r.  The steps of a level are those of the global kernels.
-constexpr int kLeafLevels = 11;
-constexpr int kLeafChunk = 1 << kLeafLevels;
-constexpr int kLeafThreads = 1024;
-constexpr int kLeafSmem = (3 * 3 * kLeafChunk + 2 * kLeafChunk) * (int)sizeof(int);   // uf, rr, mh; lx, ly
-
-__device__ inline int sm_find(int *uf, int x)
+// The levels left, by one block (their vertices and edges are few after the levels above): the same steps
+// with barriers between them.
+__global__ void __launch_bounds__(1024) ct_tail_kernel(Contract c, int level, int *bad)
 {
-    for (int it = 0; it < 3 * kLeafChunk; ++it) {
-        int p = uf[x];
-        if (p == x) return x;
-        int g = uf[p];
-        if (g != p) uf[x] = g;
-        x = p;
-    }
-    return x;
-}
-
-__global__ void __launch_bounds__(kLeafThreads) level_leaf_kernel(const int *__restrict__ ex, const int *__restrict__ ey,
-                                                                  int m, int n, int top, int *map,
-                                                                  int *__restrict__ par)
-{
-    extern __shared__ int leaf_smem[];
-    int *uf = leaf_smem, *rr = uf + 3 * kLeafChunk, *mh = rr + 3 * kLeafChunk;
-    int *lx = mh + 3 * kLeafChunk, *ly = lx + kLeafChunk;
-    const int b = blockIdx.x * kLeafChunk;
-    const int cnt = min(kLeafChunk, m - b);
-    for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
-        const int me = 2 * t;
-        int prev = atomicCAS(&map[ex[b + t]], -1, me);
-        lx[t] = prev < 0 ? me : prev;
-        prev = atomicCAS(&map[ey[b + t]], -1, me + 1);
-        ly[t] = prev < 0 ? me + 1 : prev;
-    }
-    for (int bit = top - 1; bit >= 0; --bit) {
-        for (int v = threadIdx.x; v < 3 * kLeafChunk; v += blockDim.x) {
-            uf[v] = v;
-            rr[v] = -1;
-            mh[v] = 0x7fffffff;
-        }
+    __shared__ int sh[32];
+    for (; level + 1 < kLevelsMax; ++level) {
+        const int m = __ldcg(c.ne + level), nv = __ldcg(c.nv + level), off = __ldcg(c.off + level), to = off + nv;
+        if (m == 0) return;   // the same for every thread
+        const int *list = c.list[level & 1];
+        int *out = c.list[(level & 1) ^ 1];
+        for (int t = threadIdx.x; t < m; t += 1024) ct_lightest(c, __ldcg(list + t));
+        if (threadIdx.x == 0) c.off[level + 1] = to;
         __syncthreads();
-        for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
-            if ((t >> bit) & 1) continue;
-            const int x = lx[t], y = ly[t];
-            for (int it = 0; it < 3 * kLeafChunk; ++it) {
-                int a = sm_find(uf, x), c = sm_find(uf, y);
-                if (a == c) break;
-                if (a > c) { int q = a; a = c; c = q; }
-                if (atomicCAS(&uf[c], c, a) == c) break;
+        for (int b0 = 0; b0 < nv; b0 += 1024) {
+            const int t = b0 + threadIdx.x;
+            const bool root = t < nv && ct_hook(c, off + t);
+            const int slot = to + block_append(c.nv + level + 1, root ? 1 : 0, sh);
+            if (root) {
+                if (slot < c.cap) c.next[off + t] = slot;
+                else atomicOr(bad, 16);
             }
         }
         __syncthreads();
-        for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
-            if (((t >> bit) & 1) == 0) {
-                atomicMax(&rr[sm_find(uf, lx[t])], t);
-            } else {
-                atomicMin(&mh[sm_find(uf, lx[t])], t);
-                atomicMin(&mh[sm_find(uf, ly[t])], t);
-            }
+        for (int t = threadIdx.x; t < nv; t += 1024) {
+            const int x = ct_root(c, off + t, nv);
+            if (x != off + t) c.next[off + t] = *(volatile int *)(c.next + x);
         }
         __syncthreads();
-        for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
-            if (((t >> bit) & 1) == 0) {
-                const int c = sm_find(uf, lx[t]);
-                if (rr[c] == t && mh[c] != 0x7fffffff) par[n + b + t] = n + b + mh[c];
-            } else {
-                const int cx = sm_find(uf, lx[t]), cy = sm_find(uf, ly[t]);
-                lx[t] = rr[cx] >= 0 ? 2 * kLeafChunk + rr[cx] : cx;
-                ly[t] = rr[cy] >= 0 ? 2 * kLeafChunk + rr[cy] : cy;
-            }
+        for (int b0 = 0; b0 < m; b0 += 1024) {
+            const int t = b0 + threadIdx.x;
+            const int r = t < m ? __ldcg(list + t) : -1;
+            const bool keep = r >= 0 && ct_edge(c, r);
+            const int slot = block_append(c.ne + level + 1, keep ? 1 : 0, sh);
+            if (keep) out[slot] = r;
         }
         __syncthreads();
+    }
+}
+
+// the chain of every edge, as a sort key (the edges are in rank order already)
+__global__ void ct_chain_kernel(Contract c, int m, EdgeK *__restrict__ key)
+{
+    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < m; r += gridDim.x * blockDim.x) {
+        int g = c.sup[r];
+        for (int it = 0; it < kLevelsMax && c.P[g] < r; ++it) g = c.next[g];
+        EdgeK k;
+        k.hi = (unsigned long long)g;
+        k.lo = (unsigned long long)r;
+        key[r] = k;
+    }
+}
+
+// parents of the merges from the sorted chains, and of the leaves
+__global__ void ct_parent_kernel(Contract c, const EdgeK *__restrict__ key, int m, int n, int *__restrict__ par)
+{
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
+        par[t] = c.P[t] == kNoRank ? -1 : n + c.P[t];   // (-1: not a spanning tree)
+        if (t >= m) continue;
+        const EdgeK k = key[t];
+        int p;
+        if (t + 1 < m && key[t + 1].hi == k.hi) p = (int)key[t + 1].lo;
+        else p = c.P[k.hi];
+        par[n + (int)k.lo] = p == kNoRank ? -1 : n + p;
     }
 }
 
@@ -368,6 +368,7 @@ __global__ void order_children_kernel(const EdgeK *__restrict__ E, int m, int n,
                                       int *__restrict__ lc, int *__restrict__ rc, int *bad)
 {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
+        lc[i] = rc[i] = 0;
         if (nch[i] != 2) { atomicOr(bad, 4); continue; }
         int c = child[i];
         int a = ch[2 * i], b = ch[2 * i + 1];
@@ -416,7 +417,8 @@ __global__ void dendro_out_kernel(const EdgeK *__restrict__ E, int m, int n, con
             o.reserved = 0;
             out_d[i] = o;
         }
-        if (reach) reach[n - S[2 * rc[i]]] = h;
+        const int at = n - S[2 * rc[i]];
+        if (reach && at >= 0 && at < n) reach[at] = h;   // (outside only when the edges are no tree: reported)
     }
 }
 
@@ -424,7 +426,7 @@ __global__ void order_out_kernel(int n, const int *__restrict__ S, int *__restri
 {
     for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < n; x += gridDim.x * blockDim.x) {
         int idx = n - S[2 * x];
-        if (order) order[idx] = x;
+        if (order && idx >= 0 && idx < n) order[idx] = x;
         if (reach && idx == 0) reach[0] = INFINITY;
     }
 }
@@ -530,9 +532,20 @@ int dendrogram_impl(const EdgeK *E, int n, int start, int key_squared, wm_dnode 
     int *deg = ar.get<int>(n + 1), *cur = ar.get<int>(n), *adj = ar.get<int>(L), *slot = ar.get<int>(L);
     int *succ = ar.get<int>(2 * total), *w = ar.get<int>(2 * total), *S = ar.get<int>(2 * total);
     int *child = ar.get<int>(m), *tin = ar.get<int>(n), *tout = ar.get<int>(n);
-    int *par = ar.get<int>(total), *pmin = ar.get<int>(n), *ex = ar.get<int>(m), *ey = ar.get<int>(m);
-    int *uf = ar.get<int>(total), *rootrank = ar.get<int>(total), *minheavy = ar.get<int>(total);
-    int *rootrank2 = ar.get<int>(total), *minheavy2 = ar.get<int>(total), *rxa = ar.get<int>(m), *rya = ar.get<int>(m);
+    int *par = ar.get<int>(total);
+    Contract c;
+    c.cap = 2 * n + 64;
+    c.cu = ar.get<int>(m);
+    c.cv = ar.get<int>(m);
+    c.list[0] = ar.get<int>(m);
+    c.list[1] = ar.get<int>(m);
+    c.P = ar.get<int>(c.cap);
+    c.hook = ar.get<int>(c.cap);
+    c.next = ar.get<int>(c.cap);
+    c.sup = ar.get<int>(m);
+    c.off = ar.get<int>(3 * kLevelsMax);
+    c.nv = c.off + kLevelsMax;
+    c.ne = c.nv + kLevelsMax;
     int *nch = ar.get<int>(m), *ch = ar.get<int>(2 * m), *lc = ar.get<int>(m), *rc = ar.get<int>(m);
     int *bad = ar.get<int>(1);
     if (ar.failed) return WM_ENOMEM;
@@ -558,27 +571,29 @@ int dendrogram_impl(const EdgeK *E, int n, int start, int key_squared, wm_dnode 
         int neg = -1;
         cudaMemcpyAsync(tin + start, &neg, sizeof(int), cudaMemcpyHostToDevice, st);
     }
-    // ---- merge parents (heavy/light levels)
-    fill_i32(pmin, 0x7fffffff, n, st);
-    fill_i32(par, -1, total, st);
-    launch(leaf_parent_kernel, g, 256, 0, st, E, m, pmin);
-    launch(leaf_parent_set_kernel, g, 256, 0, st, pmin, n, par);
-    launch(endpoints_init_kernel, g, 256, 0, st, E, m, ex, ey);
-    int levels = 0;
-    while ((1LL << levels) < (long long)m) ++levels;
-    if (levels > kLeafLevels) launch(level_init_kernel, g, 256, 0, st, ex, ey, m, uf, rootrank, minheavy);
-    for (int k = levels, set = 0; k > kLeafLevels; --k, set ^= 1) {
-        const int bit = k - 1;
-        int *rr = set ? rootrank2 : rootrank, *mh = set ? minheavy2 : minheavy;
-        int *rrn = set ? rootrank : rootrank2, *mhn = set ? minheavy : minheavy2;
-        launch(level_union_kernel, g, 256, 0, st, ex, ey, m, bit, uf);
-        launch(level_mark_kernel, g, 256, 0, st, ex, ey, m, bit, uf, rr, mh, rxa, rya);
-        launch(level_link_kernel, g, 256, 0, st, ex, ey, m, bit, n, rxa, rya, rr, mh, par, uf, rrn, mhn);
+    // ---- merge parents (contraction levels)
+    cudaMemsetAsync(c.P, 0x7f, sizeof(int) * (size_t)c.cap, st);
+    cudaMemsetAsync(c.off, 0, sizeof(int) * 3 * kLevelsMax, st);
+    launch(ct_init_kernel, g, 256, 0, st, E, m, n, c);
+    // Grid-wide levels until about a thousand vertices are left: a level keeps a third of them on the
+    // trees measured (at most half in any case), and the block that finishes takes whatever is left.
+    int level = 0;
+    for (double v = n; v > 2048.0 && level < 24; v /= 2.7, ++level) {
+        const int gl = grid_for(std::max(1, n >> level), 256);
+        launch(ct_lightest_kernel, gl, 256, 0, st, c, level);
+        launch(ct_hook_kernel, gl, 256, 0, st, c, level, bad);
+        launch(ct_next_kernel, gl, 256, 0, st, c, level);
+        launch(ct_edge_kernel, gl, 256, 0, st, c, level);
     }
-    fill_i32(uf, -1, total, st);
-    cudaFuncSetAttribute(level_leaf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kLeafSmem);
-    launch(level_leaf_kernel, (m + kLeafChunk - 1) / kLeafChunk, kLeafThreads, kLeafSmem, st, ex, ey, m, n,
-           std::min(levels, kLeafLevels), uf, par);
+    launch(ct_tail_kernel, 1, 1024, 0, st, c, level, bad);
+    {
+        // (the Euler tour's arrays are free here and hold the keys: 2 total ints are at least m keys)
+        EdgeK *keys = (EdgeK *)succ, *sorted = keys;
+        launch(ct_chain_kernel, g, 256, 0, st, c, m, keys);
+        rc0 = radix_sort_edges(keys, (EdgeK *)w, m, st, ar, &sorted, pin + 4096, true);
+        if (rc0) return rc0;
+        launch(ct_parent_kernel, g, 256, 0, st, c, sorted, m, n, par);
+    }
     // ---- children, left/right, in-order
     cudaMemsetAsync(nch, 0, sizeof(int) * m, st);
     launch(children_kernel, g, 256, 0, st, par, total, n, nch, ch, bad);

@@ -231,8 +231,10 @@ __global__ void __launch_bounds__(kRsBlock) rs_pass_scatter(const EdgeK *__restr
 }  // namespace
 
 // Sorts m keys ascending as 128-bit unsigned integers (stable LSD, 8-bit digits, byte
-// positions on which all keys agree are skipped).  The result is in *result (keys or tmp).
-int radix_sort_edges(EdgeK *keys, EdgeK *tmp, int m, cudaStream_t st, Arena &ar, EdgeK **result, void *host_scratch)
+// positions on which all keys agree are skipped; hi_only: by the hi words alone).  The result is in
+// *result (keys or tmp).
+int radix_sort_edges(EdgeK *keys, EdgeK *tmp, int m, cudaStream_t st, Arena &ar, EdgeK **result, void *host_scratch,
+                     bool hi_only)
 {
     *result = keys;
     if (m <= 1) return 0;
@@ -247,7 +249,7 @@ int radix_sort_edges(EdgeK *keys, EdgeK *tmp, int m, cudaStream_t st, Arena &ar,
     if (ce != cudaSuccess) { ar.off = mark; return WM_ECUDA; }
     bool need[16];
     for (int b = 0; b < 16; ++b) {
-        need[b] = true;
+        need[b] = !(hi_only && b < 8);
         for (int g = 0; g < 256; ++g)
             if (hhist[b * 256 + g] == (unsigned)m) { need[b] = false; break; }
     }

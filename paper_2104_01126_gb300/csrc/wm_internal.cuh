@@ -200,7 +200,8 @@ int scan_exclusive_i64_dev(const long long *in, long long *out, const int *n_dev
 // message for the last failure on this thread (read by wm_last_error_detail)
 void set_error_detail(const char *msg);
 // host_scratch: at least 16 KiB of host memory (pinned preferred) for the digit histogram readback
-int radix_sort_edges(EdgeK *keys, EdgeK *tmp, int m, cudaStream_t st, Arena &ar, EdgeK **result, void *host_scratch);
+int radix_sort_edges(EdgeK *keys, EdgeK *tmp, int m, cudaStream_t st, Arena &ar, EdgeK **result, void *host_scratch,
+                     bool hi_only = false);
 void fill_i32(int *p, int v, size_t n, cudaStream_t st);
 
 // Every kernel launch of the library goes through launch(), which counts it.
