@@ -15,9 +15,8 @@
  * form of the dual-tree method that Sec. 5 compares with), which return the same tree faster; MemoGFK
  * rounds build the tree under wm_set_tuning, for EMSTs above 8 dimensions, and for HDBSCAN* under the
  * geometric separation or with overflowing ties.  The dendrogram and
- * plot come from a top-down heavy/light construction after Sec. 4.2 (the heavy set of a
- * subproblem is the upper half of its rank interval, light components come from a union-find,
- * and the output equals the sequential definition exactly).
+ * plot come from levels that each contract every vertex's lightest edge, in place of the heavy/light
+ * construction of Sec. 4.2 (the output equals the sequential definition exactly).
  *
  * Canonical result.  Every edge comparison uses the strict total key
  *     K(u,v) = (w2, min(u,v), max(u,v))   (lexicographic),
@@ -247,6 +246,26 @@ typedef struct {
 } wm_instance;
 
 int wm_batch(const wm_instance *inst, int32_t count, int32_t dtype, int32_t layout, const wm_opts *opts);
+
+/*
+ * wm_split_records -- the fields of interleaved device records as arrays of their own, on the
+ * device, without a synchronisation.
+ *   r          count descriptors (host memory): m edges and, unless dendro is NULL, m merges, and
+ *              a device array of m items for each of their fields
+ *   stream     cudaStream_t to issue the work on; NULL = legacy default stream
+ */
+typedef struct {
+    const wm_edge *edges;
+    const wm_dnode *dendro;
+    int64_t m;
+    int32_t *u, *v;
+    double *w;
+    int32_t *left, *right;
+    double *height;
+    int32_t *size;
+} wm_records;
+
+int wm_split_records(const wm_records *r, int32_t count, void *stream);
 
 /*
  * wm_single_linkage -- ordered dendrogram and reachability plot of any weighted spanning tree

@@ -1930,6 +1930,23 @@ int wm_batch(const wm_instance *inst, int32_t count, int32_t dtype, int32_t layo
     return rc;
 }
 
+int wm_split_records(const wm_records *r, int32_t count, void *stream)
+{
+    g_detail.clear();
+    bool ok = count >= 0 && (r || count == 0);
+    for (int j = 0; ok && j < count; ++j) {
+        const wm_records &q = r[j];
+        ok = q.m >= 0 && (q.m == 0 || (q.edges && q.u && q.v && q.w &&
+                                       (!q.dendro || (q.left && q.right && q.height && q.size))));
+    }
+    if (!ok) {
+        set_detail("invalid argument to wm_split_records%s (count=%lld)", "", (long long)count);
+        return WM_EINVAL;
+    }
+    WM_CK(split_records(r, count, (cudaStream_t)stream));
+    return WM_OK;
+}
+
 int wm_get_tuning(int64_t n, int32_t d, int32_t min_pts, wm_tuning *out)
 {
     if (!out || n < 0 || d < 1 || d > kMaxDim || min_pts < 0) return WM_EINVAL;

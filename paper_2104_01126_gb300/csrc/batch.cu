@@ -181,7 +181,52 @@ __global__ void scatter_out_kernel(const T *__restrict__ stage, long long cnt, c
     }
 }
 
+// The fields of wm_edge and wm_dnode records as arrays of their own: blockIdx.y is an instance, a
+// thread a record.  A copy: 16 + 24 bytes read and 36 written per record, reads of neighbouring
+// threads side by side in L1.  The descriptors travel as the kernel's parameter, so there is no upload
+// to wait for; 48 of 80 bytes are what 4 KB hold.
+constexpr int kSplitMax = 48;
+struct SplitArgs {
+    wm_records r[kSplitMax];
+};
+
+__global__ void split_kernel(const __grid_constant__ SplitArgs A)
+{
+    const wm_records &r = A.r[blockIdx.y];
+    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < r.m; t += (long long)gridDim.x * blockDim.x) {
+        const wm_edge e = r.edges[t];
+        r.u[t] = e.u;
+        r.v[t] = e.v;
+        r.w[t] = e.w;
+        if (r.dendro) {
+            const wm_dnode d = r.dendro[t];
+            r.left[t] = d.left;
+            r.right[t] = d.right;
+            r.height[t] = d.height;
+            r.size[t] = d.size;
+        }
+    }
+}
+
 }  // namespace
+
+cudaError_t split_records(const wm_records *r, int count, cudaStream_t st)
+{
+    for (int b = 0; b < count; b += kSplitMax) {
+        SplitArgs A{};
+        const int k = std::min(count - b, kSplitMax);
+        long long m = 0;
+        for (int j = 0; j < k; ++j) {
+            A.r[j] = r[b + j];
+            m = std::max<long long>(m, A.r[j].m);
+        }
+        if (m == 0) continue;
+        launch(split_kernel, dim3(grid_for(m, 256), k), 256, 0, st, A);
+        const cudaError_t e = cudaPeekAtLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
 
 void batch_gather(const void *const *src, const int *dims, const long long *base, int k, long long total, int d,
                   int dtype, int layout, double *raw, unsigned *maxabs, cudaStream_t st)

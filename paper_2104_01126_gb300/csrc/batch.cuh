@@ -23,6 +23,8 @@ void batch_dendro(const wm_dnode *dn, const EdgeK *E, int m, long long total, co
                   const int *local, wm_dnode *stage, int *bad, cudaStream_t st);
 void batch_order(const int *order, const double *reach, long long total, const long long *base, int k, int *ostage,
                  double *rstage, int *bad, cudaStream_t st);
+// wm_split_records on checked descriptors
+cudaError_t split_records(const wm_records *r, int count, cudaStream_t st);
 // dst[j][t - off[j]] = stage[t] for t in [off[j], off[j+1]) where dst[j] is not null
 template <typename T>
 void batch_scatter(const T *stage, long long cnt, const long long *off, int k, T *const *dst, cudaStream_t st);
