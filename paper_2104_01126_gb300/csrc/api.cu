@@ -177,7 +177,7 @@ static size_t estimate_bytes(long long n, int d, int min_pts, const Caps &c)
     b += (size_t)8 * (c.chunk + 1) * (5 * 12 + 16 + 4 + 8);  // pair lists with bounds (8 chunks each), huge-pair slots
     b += (size_t)num_sms() * 64 * (depth + 4) * 4;                                                           // dual stacks
     b += (size_t)c.edges * 16 * 3 + (size_t)c.edges * 24;   // batch, filtered, sort tmp, kruskal
-    b += (size_t)n * 16 * 2;                // output tree + conversion
+    b += (size_t)n * 16 * 5;                // output tree + conversion, sort
     if (c.wspd_pairs > 0)                   // GFK / EMST-Naive: pairs and bounds (x2), pool (x2), batch, sort
         b += (size_t)c.wspd_pairs * (12 * 2 + 16 * 2 + 16 + 16) + (size_t)n * 16;
     if (min_pts > 0) {
@@ -511,7 +511,9 @@ static int nearest_tree(Call &C, const Points &P, const SearchTree &X, const Hdb
     N.pin = C.pin;
     N.X = &X;
     N.pos = P.pos;
-    N.out = E_out;
+    EdgeK *raw = ar.get<EdgeK>(n);
+    if (ar.failed) return WM_ENOMEM;
+    N.out = raw;
     N.target = target;
     N.cap = rho_cap;
     N.cap_f = float_ru(rho_cap);
@@ -534,11 +536,8 @@ static int nearest_tree(Call &C, const Points &P, const SearchTree &X, const Hdb
     C.stats.ms_bccp += tn.ms();
     // every round appended its edges unordered: put the tree in K order
     Timer ts;
-    EdgeK *tmp = ar.get<EdgeK>(n), *sorted = E_out;
-    if (ar.failed) return WM_ENOMEM;
     WM_CK(cudaMemcpyAsync(C.pin, stat, 16 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
-    WM_TRY(radix_sort_edges(E_out, tmp, (int)target, st, ar, &sorted, C.pin + 4096));
-    if (sorted != E_out) WM_CK(cudaMemcpyAsync(E_out, sorted, sizeof(EdgeK) * target, cudaMemcpyDeviceToDevice, st));
+    WM_TRY(sort_edges(raw, E_out, (int)target, st, ar, C.pin + 4096));
     WM_CK(cudaStreamSynchronize(st));
     unsigned long long hs[16];
     memcpy(hs, C.pin, sizeof hs);
@@ -944,9 +943,8 @@ static int memogfk(Call &C, Points &P, Tree &T, const HdbState *hdb, const Caps 
     {
         // every round appended its tree edges unordered: put the tree in K order
         Timer ts;
-        EdgeK *sorted = E_out;
-        WM_TRY(radix_sort_edges(E_out, tmp, (int)target, st, ar, &sorted, C.pin + 4096));
-        if (sorted != E_out) WM_CK(cudaMemcpyAsync(E_out, sorted, sizeof(EdgeK) * target, cudaMemcpyDeviceToDevice, st));
+        WM_TRY(sort_edges(E_out, tmp, (int)target, st, ar, C.pin + 4096));
+        WM_CK(cudaMemcpyAsync(E_out, tmp, sizeof(EdgeK) * target, cudaMemcpyDeviceToDevice, st));
         WM_CK(cudaStreamSynchronize(st));
         C.stats.ms_kruskal += ts.ms();
     }
@@ -1178,9 +1176,8 @@ static int gfk_rounds(Call &C, Points &P, Tree &T, const HdbState *hdb, const Ca
     }
     {
         Timer ts;
-        EdgeK *sorted = E_out;
-        WM_TRY(radix_sort_edges(E_out, tmp, (int)target, st, ar, &sorted, C.pin + 4096));
-        if (sorted != E_out) WM_CK(cudaMemcpyAsync(E_out, sorted, sizeof(EdgeK) * target, cudaMemcpyDeviceToDevice, st));
+        WM_TRY(sort_edges(E_out, tmp, (int)target, st, ar, C.pin + 4096));
+        WM_CK(cudaMemcpyAsync(E_out, tmp, sizeof(EdgeK) * target, cudaMemcpyDeviceToDevice, st));
         WM_CK(cudaStreamSynchronize(st));
         C.stats.ms_kruskal += ts.ms();
     }
@@ -1515,13 +1512,12 @@ static int sl_body(Call &C, void *vctx, const Caps &, unsigned *ovf)
         int *bad = C.ar.get<int>(1);
         if (!bad) return WM_ENOMEM;
         WM_TRY(edges_from_wm(src, n, E, bad, C.st));
-        EdgeK *sorted = E;
-        WM_TRY(radix_sort_edges(E, tmp, n - 1, C.st, C.ar, &sorted, C.pin + 4096));
+        WM_TRY(sort_edges(E, tmp, n - 1, C.st, C.ar, C.pin + 4096));
         WM_CK(cudaMemcpyAsync(C.pin, bad, sizeof(int), cudaMemcpyDeviceToHost, C.st));
         WM_CK(cudaStreamSynchronize(C.st));
         if (C.pin[0]) { set_detail("tree edge with an endpoint outside [0, n) or a bad weight%s", ""); return WM_EINVAL; }
         Timer td;
-        WM_TRY(dendrogram_impl(sorted, n, x.start, 0, x.dendro, x.order, x.reach, C.ar, C.st, C.pin));
+        WM_TRY(dendrogram_impl(tmp, n, x.start, 0, x.dendro, x.order, x.reach, C.ar, C.st, C.pin));
         C.stats.ms_dendrogram = td.ms();
     } else {
         WM_TRY(dendrogram_impl(E, n, x.start, 0, x.dendro, x.order, x.reach, C.ar, C.st, C.pin));
@@ -1645,14 +1641,16 @@ static int batch_body(Call &C, void *vctx, const Caps &caps, unsigned *ovf)
     WM_TRY(spanning_tree(C, raw, total, D, WM_F64, WM_SOA, hdb ? x.min_pts : 0, caps, S, H, E, ovf, m, L * L / 4));
     if (*ovf) return 0;
     // ---- tree edges grouped by instance, K order inside each
-    EdgeK *keys = ar.get<EdgeK>(m + 1), *ktmp = ar.get<EdgeK>(m + 1);
+    SortPairs sp;
     int *local = ar.get<int>(m + 1);
     wm_edge *se = ar.get<wm_edge>(m + 1);
     if (ar.failed) return WM_ENOMEM;
-    batch_edge_inst(E, (int)m, base_d, k, keys, st);
-    EdgeK *grouped = keys;
-    WM_TRY(radix_sort_edges(keys, ktmp, (int)m, st, ar, &grouped, C.pin + 4096));
-    batch_edge_place(grouped, E, (int)m, base_d, local, se, bad, st);
+    if (m > 0) {
+        WM_TRY(sort_pairs_begin(sp, (int)m, ar));
+        batch_edge_inst(E, (int)m, base_d, k, sp.key[0], sp.idx[0], st);
+        sort_pairs(sp, (unsigned)(k - 1), st);
+        batch_edge_place(sp.key[sp.cur], sp.idx[sp.cur], E, (int)m, base_d, local, se, bad, st);
+    }
     {
         std::vector<wm_edge *> dst(k);
         for (int j = 0; j < k; ++j) dst[j] = I(j).out_edges;

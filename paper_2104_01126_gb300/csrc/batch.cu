@@ -64,23 +64,21 @@ __global__ void scale_kernel(double *__restrict__ x, long long total, double L)
 
 // keys[g] = {hi = instance of tree edge g, lo = g}: sorted, they group the edges by instance in K order
 __global__ void edge_inst_kernel(const EdgeK *__restrict__ E, int m, const long long *__restrict__ base, int k,
-                                 EdgeK *__restrict__ keys)
+                                 unsigned *__restrict__ inst, int *__restrict__ idx)
 {
     for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < m; g += gridDim.x * blockDim.x) {
-        EdgeK key;
-        key.hi = (unsigned long long)inst_of(base, k, edge_u(E[g]));
-        key.lo = (unsigned long long)g;
-        keys[g] = key;
+        inst[g] = (unsigned)inst_of(base, k, edge_u(E[g]));
+        idx[g] = g;
     }
 }
 
 // position t of the grouped list: instance j, local index t - eoff[j]; stage the instance-local edge
-__global__ void edge_place_kernel(const EdgeK *__restrict__ keys, const EdgeK *__restrict__ E, int m,
+__global__ void edge_place_kernel(const unsigned *__restrict__ inst, const int *__restrict__ idx, const EdgeK *__restrict__ E, int m,
                                   const long long *__restrict__ base, int *__restrict__ local,
                                   wm_edge *__restrict__ stage, int *bad)
 {
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < m; t += gridDim.x * blockDim.x) {
-        const int g = (int)keys[t].lo, j = (int)keys[t].hi;
+        const int g = idx[t], j = (int)inst[t];
         const long long eo = base[j] - j;   // edges of the instances before j
         local[g] = (int)(t - eo);
         const EdgeK x = E[g];
@@ -239,15 +237,15 @@ void batch_scale(double *x, long long total, double L, cudaStream_t st)
     launch(scale_kernel, grid_for(total, 256), 256, 0, st, x, total, L);
 }
 
-void batch_edge_inst(const EdgeK *E, int m, const long long *base, int k, EdgeK *keys, cudaStream_t st)
+void batch_edge_inst(const EdgeK *E, int m, const long long *base, int k, unsigned *inst, int *idx, cudaStream_t st)
 {
-    if (m > 0) launch(edge_inst_kernel, grid_for(m, 256), 256, 0, st, E, m, base, k, keys);
+    if (m > 0) launch(edge_inst_kernel, grid_for(m, 256), 256, 0, st, E, m, base, k, inst, idx);
 }
 
-void batch_edge_place(const EdgeK *keys, const EdgeK *E, int m, const long long *base, int *local, wm_edge *stage,
+void batch_edge_place(const unsigned *inst, const int *idx, const EdgeK *E, int m, const long long *base, int *local, wm_edge *stage,
                       int *bad, cudaStream_t st)
 {
-    if (m > 0) launch(edge_place_kernel, grid_for(m, 256), 256, 0, st, keys, E, m, base, local, stage, bad);
+    if (m > 0) launch(edge_place_kernel, grid_for(m, 256), 256, 0, st, inst, idx, E, m, base, local, stage, bad);
 }
 
 void batch_totals(const wm_edge *stage, const long long *base, int k, double *tot, cudaStream_t st)

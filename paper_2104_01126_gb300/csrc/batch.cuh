@@ -13,8 +13,8 @@ namespace wm {
 void batch_gather(const void *const *src, const int *dims, const long long *base, int k, long long total, int d,
                   int dtype, int layout, double *raw, unsigned *maxabs, cudaStream_t st);
 void batch_scale(double *x, long long total, double L, cudaStream_t st);
-void batch_edge_inst(const EdgeK *E, int m, const long long *base, int k, EdgeK *keys, cudaStream_t st);
-void batch_edge_place(const EdgeK *keys, const EdgeK *E, int m, const long long *base, int *local, wm_edge *stage,
+void batch_edge_inst(const EdgeK *E, int m, const long long *base, int k, unsigned *inst, int *idx, cudaStream_t st);
+void batch_edge_place(const unsigned *inst, const int *idx, const EdgeK *E, int m, const long long *base, int *local, wm_edge *stage,
                       int *bad, cudaStream_t st);
 void batch_totals(const wm_edge *stage, const long long *base, int k, double *tot, cudaStream_t st);
 void batch_cd(const double *cd64, const int *pid, int total, double *stage, cudaStream_t st);

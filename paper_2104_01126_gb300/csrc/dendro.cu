@@ -319,30 +319,27 @@ __global__ void __launch_bounds__(1024) ct_tail_kernel(Contract c, int level, in
     }
 }
 
-// the chain of every edge, as a sort key (the edges are in rank order already)
-__global__ void ct_chain_kernel(Contract c, int m, EdgeK *__restrict__ key)
+// the chain of every edge (the edges are in rank order already)
+__global__ void ct_chain_kernel(Contract c, int m, unsigned *__restrict__ key, int *__restrict__ rank)
 {
     for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < m; r += gridDim.x * blockDim.x) {
         int g = c.sup[r];
         for (int it = 0; it < kLevelsMax && c.P[g] < r; ++it) g = c.next[g];
-        EdgeK k;
-        k.hi = (unsigned long long)g;
-        k.lo = (unsigned long long)r;
-        key[r] = k;
+        key[r] = (unsigned)g;
+        rank[r] = r;
     }
 }
 
 // parents of the merges from the sorted chains, and of the leaves
-__global__ void ct_parent_kernel(Contract c, const EdgeK *__restrict__ key, int m, int n, int *__restrict__ par)
+__global__ void ct_parent_kernel(Contract c, const unsigned *__restrict__ key, const int *__restrict__ rank, int m, int n,
+                                 int *__restrict__ par)
 {
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
         par[t] = c.P[t] == kNoRank ? -1 : n + c.P[t];   // (-1: not a spanning tree)
         if (t >= m) continue;
-        const EdgeK k = key[t];
-        int p;
-        if (t + 1 < m && key[t + 1].hi == k.hi) p = (int)key[t + 1].lo;
-        else p = c.P[k.hi];
-        par[n + (int)k.lo] = p == kNoRank ? -1 : n + p;
+        const unsigned k = key[t];
+        const int p = t + 1 < m && key[t + 1] == k ? rank[t + 1] : c.P[k];
+        par[n + rank[t]] = p == kNoRank ? -1 : n + p;
     }
 }
 
@@ -587,12 +584,14 @@ int dendrogram_impl(const EdgeK *E, int n, int start, int key_squared, wm_dnode 
     }
     launch(ct_tail_kernel, 1, 1024, 0, st, c, level, bad);
     {
-        // (the Euler tour's arrays are free here and hold the keys: 2 total ints are at least m keys)
-        EdgeK *keys = (EdgeK *)succ, *sorted = keys;
-        launch(ct_chain_kernel, g, 256, 0, st, c, m, keys);
-        rc0 = radix_sort_edges(keys, (EdgeK *)w, m, st, ar, &sorted, pin + 4096, true);
+        const size_t at = ar.off;
+        SortPairs sp;
+        rc0 = sort_pairs_begin(sp, m, ar, succ);   // (free here: 4 n - 2 ints)
         if (rc0) return rc0;
-        launch(ct_parent_kernel, g, 256, 0, st, c, sorted, m, n, par);
+        launch(ct_chain_kernel, g, 256, 0, st, c, m, sp.key[0], sp.idx[0]);
+        sort_pairs(sp, (unsigned)c.cap, st);   // (a chain is named by a vertex)
+        launch(ct_parent_kernel, g, 256, 0, st, c, sp.key[sp.cur], sp.idx[sp.cur], m, n, par);
+        ar.off = at;
     }
     // ---- children, left/right, in-order
     cudaMemsetAsync(nch, 0, sizeof(int) * m, st);

@@ -199,9 +199,19 @@ int scan_exclusive_i64_dev(const long long *in, long long *out, const int *n_dev
                            cudaStream_t st, Arena &ar);
 // message for the last failure on this thread (read by wm_last_error_detail)
 void set_error_detail(const char *msg);
-// host_scratch: at least 16 KiB of host memory (pinned preferred) for the digit histogram readback
-int radix_sort_edges(EdgeK *keys, EdgeK *tmp, int m, cudaStream_t st, Arena &ar, EdgeK **result, void *host_scratch,
-                     bool hi_only = false);
+// Stable sort of pairs of a key and an index: the caller fills key[0] and idx[0] (m >= 1 of them) after
+// sort_pairs_begin and finds the result in key[cur], idx[cur].  room: 4 m ints for the pairs, or null.
+struct SortPairs {
+    int m = 0, cur = 0, G = 0, chunk = 0;
+    unsigned *key[2] = {nullptr, nullptr};
+    int *idx[2] = {nullptr, nullptr};
+    int *bh = nullptr, *total = nullptr;
+};
+int sort_pairs_begin(SortPairs &P, int m, Arena &ar, int *room = nullptr);
+void sort_pairs_pass(SortPairs &P, int bit, cudaStream_t st);        // by the 8 bits from `bit` up
+void sort_pairs(SortPairs &P, unsigned max_key, cudaStream_t st);    // no key above max_key
+// m edges in K order into out (not the same array); pin: pinned host scratch
+int sort_edges(const EdgeK *in, EdgeK *out, int m, cudaStream_t st, Arena &ar, void *pin);
 void fill_i32(int *p, int v, size_t n, cudaStream_t st);
 
 // Every kernel launch of the library goes through launch(), which counts it.
