@@ -129,7 +129,9 @@ typedef struct {
     double max_rel_screen_err;     /* largest |fp32 - fp64| / fp64 between a screened FP32
                                       value and its exact FP64 value, over every BCCP
                                       candidate re-evaluated in FP64 (every winner among
-                                      them) and every core distance; 0 in the FP64 form.
+                                      them) and every core distance; 0 in the FP64 form
+                                      (also taken where the FP32 copy of FP64 coordinates
+                                      errs by more than a 128th of the points' spacing).
                                       A priori bound: 2^-19 for FP32-exact coordinates  */
     int32_t tie_overflow;          /* HDBSCAN*: 1 when the pairs within some point's core
                                       distance (the tie-repair edges) exceeded their

@@ -468,7 +468,7 @@ static bool nearest_rounds_apply(const Call &C, int n, int d, const HdbState *hd
 
 // The spanning tree by nearest-component rounds, as memogfk returns it: its edges in K order, n-1 of them
 // or `target` below rho_cap.
-static int nearest_tree(Call &C, const Points &P, const SearchTree &X, const HdbState *hdb, EdgeK *E_out,
+static int nearest_tree(Call &C, const Points &P, const SearchTree &X, bool fp64, const HdbState *hdb, EdgeK *E_out,
                         long long target = -1, double rho_cap = INFINITY)
 {
     const int n = P.n;
@@ -486,7 +486,7 @@ static int nearest_tree(Call &C, const Points &P, const SearchTree &X, const Hdb
     TravArgs a;
     a.n = n; a.d = P.d;
     a.x64 = P.x64; a.pid = P.pid;
-    a.fp64 = C.precision == WM_PREC_FP64;
+    a.fp64 = fp64;
     a.eta = a.fp64 ? 0.0 : 2.0 * (double)P.delta * std::sqrt((double)P.d) * (1.0 + 1e-6);
     a.eta2_f = float_ru(2.0 * a.eta);
     a.exact32 = a.eta == 0.0;
@@ -1204,6 +1204,7 @@ struct Prepared {
     Tree T;
     SearchTree X;
     const void *src = nullptr;   // the input on the device
+    bool fp64 = false;           // the walks evaluate every distance in FP64
 };
 
 static int input_on_device(Call &C, const void *pts, int64_t n, int32_t d, int32_t dtype, Prepared &S)
@@ -1246,8 +1247,12 @@ static int prepare_walk(Call &C, const void *pts, int64_t n, int32_t d, int32_t 
 {
     WM_TRY(input_on_device(C, pts, n, d, dtype, S));
     Timer tt;
-    WM_TRY(bad_coordinate(build_search_tree(S.src, (int)n, d, dtype, layout, C.precision == WM_PREC_FP64 ? 2 : 1, S.P, S.X, C.ar,
-                                            C.st, C.pin)));
+    WM_TRY(bad_coordinate(build_search_tree(S.src, (int)n, d, dtype, layout, S.P, S.X, C.ar, C.st, C.pin)));
+    // Where the FP32 copy of FP64 coordinates errs by more than a 128th of the points' spacing, most distances
+    // fall into one band of the screen and are evaluated twice: the plain FP64 walks answer such a call.
+    // (Uniform points in 3-D at an offset, FP32 screen / FP64 walks, ms: EMST of 10^5 at 10^3, error
+    // 0.0014 of the spacing, 2.0 / 2.2; of 5x10^4 at 10^5, 0.15 of it, 4.8 / 2.3; HDBSCAN* there 12.0 / 3.2.)
+    S.fp64 = C.precision == WM_PREC_FP64 || (double)S.P.delta * 128.0 > S.X.spacing;
     C.stats.ms_build_tree += tt.ms();
     C.stats.tree_nodes = 2 * n - 1;   // down to single points; X stores those above its buckets
     C.stats.tree_depth = S.X.depth;
@@ -1418,13 +1423,13 @@ static int spanning_tree(Call &C, const void *pts, int64_t n64, int d, int dtype
     else WM_TRY(prepare(C, pts, n64, d, dtype, layout, S));
     if (hdb) {
         Timer tc;
-        WM_TRY(core_distances(S.P, S.X, min_pts, C.precision == WM_PREC_FP64, H, C.ar, C.st, C.pin, &C.stats));
+        WM_TRY(core_distances(S.P, S.X, min_pts, S.fp64, H, C.ar, C.st, C.pin, &C.stats));
         C.stats.ms_core_dist = tc.ms();
     }
     E = C.ar.get<EdgeK>(n);
     if (C.ar.failed) return WM_ENOMEM;
     if (walk && !wspd_form && nearest_rounds_apply(C, n, d, hdb ? &H : nullptr))
-        return nearest_tree(C, S.P, S.X, hdb ? &H : nullptr, E, target, cap);
+        return nearest_tree(C, S.P, S.X, S.fp64, hdb ? &H : nullptr, E, target, cap);
     // the traversals: with their own tree, and the core distances in its order
     Prepared Q;
     HdbState HQ = H;

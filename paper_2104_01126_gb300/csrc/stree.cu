@@ -28,7 +28,13 @@ __device__ inline unsigned f2key(float f)
     const unsigned u = __float_as_uint(f);
     return (u & 0x80000000u) ? ~u : u | 0x80000000u;
 }
-__device__ inline float key2f(unsigned k) { return __uint_as_float((k & 0x80000000u) ? k & 0x7fffffffu : ~k); }
+__host__ __device__ inline float key2f(unsigned k)
+{
+    const unsigned u = (k & 0x80000000u) ? k & 0x7fffffffu : ~k;
+    float f;
+    memcpy(&f, &u, sizeof f);
+    return f;
+}
 
 constexpr int kStThreads = 256;
 template <int S> constexpr int rows_per_thread() { return S == 4 ? 8 : S == 8 ? 4 : 2; }
@@ -46,13 +52,17 @@ struct BuildState {
     unsigned delta;   // bits of max |x64 - x32|
 };
 
+// The boxes are widened by this multiple of the FP32 copy's error: the walks bound exact distances from the
+// rounded query (screened ones, of two points rounded alike, would need 1).
+constexpr float kWiden = 2.f;
+
 struct LNode {
     int node, b, e, dim;
     float val;
 };
 
 struct StArgs {
-    int n, d, dtype, layout, widen;
+    int n, d, dtype, layout;
     const void *src;
     float *buf[2];           // point rows, ping-pong; buf[0] becomes the final array
     float *nodes;
@@ -144,7 +154,7 @@ __device__ inline void choose_split(const unsigned *acc, int d, int &dim, float 
     }
 }
 
-// box of a node row, widened by delta (see build_search_tree)
+// box of a node row, widened by delta (see kWiden)
 template <int S>
 __device__ inline void write_box(float *row, const unsigned *acc, int d, float delta)
 {
@@ -169,7 +179,7 @@ template <int S>
 __global__ void st_root_kernel(StArgs a)
 {
     BuildState &s = *a.state;
-    write_box<S>(a.nodes, a.root_acc, a.d, a.widen * __uint_as_float(s.delta));
+    write_box<S>(a.nodes, a.root_acc, a.d, kWiden * __uint_as_float(s.delta));
     a.range[0] = make_int2(0, a.n);
     a.parent[0] = -1;
     int dim;
@@ -311,7 +321,7 @@ __global__ void __launch_bounds__(1024) st_level_kernel(StArgs a, int level)
     __shared__ int sh[32];
     __shared__ int s_act, s_units;
     const int A = a.state->active, id0 = a.state->next_id, d = a.d, cur = level & 1;
-    const float delta = a.widen * __uint_as_float(a.state->delta);
+    const float delta = kWiden * __uint_as_float(a.state->delta);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (threadIdx.x == 0) { s_act = 0; s_units = 0; }
     __syncthreads();
@@ -399,7 +409,7 @@ __global__ void __launch_bounds__(kStThreads) st_block_kernel(StArgs a)
     float *sval = (float *)(seg + 2 * (M / 8));      // [2][M / 8]
     __shared__ int s_entry, s_next, s_base;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, d = a.d;
-    const float delta = a.widen * __uint_as_float(a.state->delta);
+    const float delta = kWiden * __uint_as_float(a.state->delta);
     const int nsub = a.state->subs;
     while (true) {
         if (threadIdx.x == 0) s_entry = atomicAdd(&a.state->sub_next, 1);
@@ -580,6 +590,7 @@ int build(StArgs &a, SearchTree &X, Points &P, Arena &ar, cudaStream_t st, int *
     launch(st_block_kernel<S>, n > M ? num_sms() * per_sm : 1, kStThreads, smem, st, a);
     launch(st_finish_kernel<S>, grid_for(n, 256), 256, 0, st, a);
     cudaMemcpyAsync(pin, a.state, sizeof(BuildState), cudaMemcpyDeviceToHost, st);
+    cudaMemcpyAsync(pin + 64, a.root_acc, sizeof(unsigned) * 2 * a.d, cudaMemcpyDeviceToHost, st);
     if (cudaPeekAtLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) return WM_ECUDA;
     BuildState h;
     memcpy(&h, pin, sizeof h);
@@ -587,6 +598,16 @@ int build(StArgs &a, SearchTree &X, Points &P, Arena &ar, cudaStream_t st, int *
     float delta;
     memcpy(&delta, &h.delta, sizeof delta);
     P.delta = delta;
+    // side of the cube that a point would have to itself if all filled their box evenly
+    double log_vol = 0.0;
+    int dims = 0;
+    for (int k = 0; k < a.d; ++k) {
+        const double ext = (double)key2f((unsigned)pin[64 + 2 * k + 1]) - (double)key2f(~(unsigned)pin[64 + 2 * k]);
+        if (!(ext > 0.0)) continue;
+        log_vol += std::log(ext);
+        ++dims;
+    }
+    X.spacing = dims ? std::exp((log_vol - std::log((double)n)) / dims) : 0.0;
     X.Ns = h.next_id;
     X.depth = level + h.depth + 1;
     return 0;
@@ -596,7 +617,7 @@ int build(StArgs &a, SearchTree &X, Points &P, Arena &ar, cudaStream_t st, int *
 
 // Search tree and tree-order points of the input (device memory); n < 2^28 (28-bit positions in a
 // bucket's reference).  P.x64 is set when the FP32 copy is inexact (FP64 input); P.x32 is not.
-int build_search_tree(const void *src, int n, int d, int dtype, int layout, int widen, Points &P, SearchTree &X, Arena &ar,
+int build_search_tree(const void *src, int n, int d, int dtype, int layout, Points &P, SearchTree &X, Arena &ar,
                       cudaStream_t st, int *pin)
 {
     P.n = n;
@@ -608,7 +629,6 @@ int build_search_tree(const void *src, int n, int d, int dtype, int layout, int 
     a.d = d;
     a.dtype = dtype;
     a.layout = layout;
-    a.widen = widen;
     a.src = src;
     X.rows = a.buf[0] = ar.get<float>((size_t)n * X.S);
     X.nodes = a.nodes = ar.get<float>((size_t)(2LL * n) * 2 * X.S);

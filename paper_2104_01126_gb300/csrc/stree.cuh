@@ -32,6 +32,7 @@ struct SearchTree {
     int walk_blocks = 0;          // the largest grid the stacks are sized for
     int stack_cap = 0;            // entries of a thread's stack: one per tree level
     int depth = 0;                // levels
+    double spacing = 0.0;         // (volume of the points' box / n)^(1/d), over the dimensions with an extent
 };
 
 // rows of d coordinates and one more slot
@@ -43,9 +44,7 @@ __host__ __device__ constexpr int walk_dim(int d) { return d <= 2 ? 2 : d <= 8 ?
 constexpr bool walk_dims_fit(int d) { return d > 16 || (walk_dim(d) >= d && row_floats(walk_dim(d)) == row_floats(d) && walk_dims_fit(d + 1)); }
 static_assert(walk_dims_fit(1), "a walk's rows must be as wide as the search tree's");
 
-// widen: the boxes are widened by this multiple of the FP32 copy's error: 1 when distances are screened
-// in FP32 (both points rounded alike), 2 when they are exact but the walk bounds them from the rounded query
-int build_search_tree(const void *src, int n, int d, int dtype, int layout, int widen, Points &P, SearchTree &X, Arena &ar,
+int build_search_tree(const void *src, int n, int d, int dtype, int layout, Points &P, SearchTree &X, Arena &ar,
                       cudaStream_t st, int *pin);
 
 __host__ __device__ inline unsigned bucket_ref(int first, int size) { return kBucketBit | (unsigned)(size - 1) << 28 | (unsigned)first; }
