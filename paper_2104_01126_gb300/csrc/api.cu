@@ -478,11 +478,9 @@ static int nearest_tree(Call &C, const Points &P, const SearchTree &X, bool fp64
     Arena &ar = C.ar;
     const size_t mark = ar.off;
     Timer tn;
-    unsigned *ovf = ar.get<unsigned>(2);
     unsigned long long *stat = ar.get<unsigned long long>(16);
     if (ar.failed) return WM_ENOMEM;
     WM_CK(cudaMemsetAsync(stat, 0, 16 * sizeof(unsigned long long), st));
-    WM_CK(cudaMemsetAsync(ovf, 0, 2 * sizeof(unsigned), st));
     TravArgs a;
     a.n = n; a.d = P.d;
     a.x64 = P.x64; a.pid = P.pid;
@@ -492,7 +490,6 @@ static int nearest_tree(Call &C, const Points &P, const SearchTree &X, bool fp64
     a.exact32 = a.eta == 0.0;
     a.delta32 = P.delta;
     if (hdb) { a.cd32 = hdb->cd32; a.cd64 = hdb->cd64; }
-    a.overflow = ovf;
     a.stat = stat;
     // CUDA-event intervals of the search kernel (when C.timing)
     struct Spans {

@@ -13,10 +13,11 @@
 //   refresh : drops the list heads that have joined i's component and WriteMins the first remaining
 //             weight into S[c], the component's screened minimum;
 //   active  : collects the points with R[i] <= T(S[c]) (T: the band threshold of the screen), i.e.
-//             those that could still hold a lighter edge than the lists show;
+//             those that could still hold a lighter edge than the lists show, and those with a list
+//             entry within T(S[c]);
 //   search  : a thread per active point walks the k-d tree, the nearer child first, skipping nodes of
 //             its own component and nodes beyond its bound, and rebuilds the point's list;
-//   pick    : collects the points with a list entry within T(S[c]); FP64 evaluation of those entries
+//   pick    : of these, the points with a list entry still within T(S[c]); FP64 evaluation of those entries
 //             and the K-minimum per component by two 64-bit WriteMins; a point whose list may have
 //             dropped a tie (R[i] <= T(S[c]) still) is answered by a walk that evaluates everything
 //             within T(S[c]) in FP64;
@@ -52,14 +53,32 @@ namespace {
 // from 8.0 to 7.7 in 2-D, left it in 5-D (31 ms) and cost 13 % in 7-D; 2 entries were slower everywhere.
 __host__ __device__ constexpr int list_len(int D) { return D <= 3 ? 6 : 4; }
 
-// counters: the first kCntRound are zeroed every round
+// A query that has evaluated kLongEvals points (above 2x10^6 points: a 1024th of them) and is still walking is
+// handed to warps that share a scan of all points: the centre of a sphere of points is as far from all of
+// them, and its walk visits every node on one lane while the GPU waits (50,000 points and their centre: 83 ms
+// a call, of which 81 on that lane; 5.0 now, 3.3 with a limit of 1024, which 7-D sets reach in ordinary
+// walks: 2 % slower).  A round scans at most kLongMax queries and about kLongWork points in all: where such
+// queries are many, there are lanes enough for them.  They are rare, so the scan is launched when the host has
+// seen one (launched every time it cost 10^4 points 6 %); until then the kernels behind the search hold back
+// (held).
+constexpr int kLongEvals = 2048, kLongMax = 512, kLongChunk = 2048, kLongChunks = 1024, kLongMinPoints = 8192;
+constexpr long long kLongWork = 1 << 26;
+
+// Counters.  Those that a round starts from zero lie side by side: an even one's are [kCntEven, kCntEdges), an
+// odd one's [0, kCntOddEnd).
 enum {
-    kCntActive, kCntSearch, kCntCand, kCntExact, kCntExactNext, kCntPicked, kCntRound,
-    kCntEdges = kCntRound,            // tree edges so far
-    kCntRep,                          // [2] repair edges left, by round parity
-    kCntRoots = kCntRep + 2,          // [2] roots, by round parity
-    kCntAll = kCntRoots + 2
+    kCntRootsEven, kCntRepOdd,        // roots that even rounds start from; repair edges that odd rounds leave
+    kCntEven,
+    kCntActive = kCntEven, kCntNear, kCntSearch, kCntCand, kCntExact, kCntExactNext, kCntPicked,
+    kCntLong, kCntLongExact,          // queries handed to the scan of all points
+    kCntOddEnd,
+    kCntRepEven = kCntOddEnd, kCntRootsOdd,
+    kCntEdges,                        // tree edges so far
+    kCntError,                        // error bits of the kernels
+    kCntAll
 };
+__host__ __device__ constexpr int cnt_roots(int parity) { return parity ? kCntRootsOdd : kCntRootsEven; }
+__host__ __device__ constexpr int cnt_rep(int parity) { return parity ? kCntRepOdd : kCntRepEven; }
 
 struct NcArgs {
     int *lab;                  // component of a tree position (a tree position: the root)
@@ -70,8 +89,10 @@ struct NcArgs {
     int *lj;                   // [list_len][n] list positions (-1: none)
     float *R;                  // every point outside the component and the list screens at >= R
     unsigned char *hd;         // first list entry that may lie outside the component
+    float *low;                // smaller of the head's weight (no head: +inf) and R
     int *roots[2];             // the roots of this round and the next
     int *act, *amb, *picked;   // active points; points that need the exact scan; points with a candidate
+    int *near;                 // points that may come to need the scan or have a candidate
     int *nlab;                 // labels in the node rows
     EdgeK *cand;               // candidate edges of the round and the component each serves
     int *cand_c;
@@ -82,9 +103,24 @@ struct NcArgs {
     unsigned long long cap64;  // the same in FP64 bits
     float *rows;               // the search tree's point rows
     const float *ncd;          // HDBSCAN*: smallest core distance of a node (rounded down)
+    // queries handed to the scan of all points (chunks: parts of the points; 0: no hand-over)
+    int chunks, long_max;
+    unsigned long_evals;
+    int guard;                 // 1: hold back while queries of the search wait for the scan, 2: of the exact one
+    int *longq;                // [long_max] positions
+    int *long_done;            // [long_max] parts finished
+    float *long_s;             // [long_max][chunks][K] a part's list
+    int *long_j;
+    KMin *long_k;              // [long_max][chunks] a part's K-minimum
     int first;                 // first search: components are single points, nothing is pruned by S
     int n;
 };
+
+// true while queries that were handed over wait for the scan of all points
+__device__ __forceinline__ bool held(const NcArgs &b, int what)
+{
+    return (b.guard & what & 1 && b.cnt[kCntLong] > 0) || (b.guard & what & 2 && b.cnt[kCntLongExact] > 0);
+}
 
 // HDBSCAN*: true when the FP32 squared distance d32 proves D <= c for a core distance c (FP32 copy)
 __device__ inline bool proven_repair(const TravArgs &a, float d32, float c)
@@ -98,6 +134,22 @@ __device__ inline bool proven_repair(const TravArgs &a, float d32, float c)
 __device__ inline void note_err(float s, double w, float &err)
 {
     if (w > 0.0) err = fmaxf(err, __fdiv_ru(__double2float_ru(fabs((double)s - w)), __double2float_rd(w)));
+}
+
+// v into an ascending list (its largest entry drops out)
+template <int K>
+__device__ __forceinline__ void list_insert(float (&sl)[K], int (&sj)[K], float v, int j)
+{
+#pragma unroll
+    for (int k = K - 1; k >= 0; --k) {
+        if (k > 0 && v < sl[k - 1]) {
+            sl[k] = sl[k - 1];
+            sj[k] = sj[k - 1];
+        } else if (v < sl[k]) {
+            sl[k] = v;
+            sj[k] = j;
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------------- search
@@ -119,7 +171,7 @@ __global__ void __launch_bounds__(kWalkThreads, search_blocks(D, HDB, F64, EXACT
     const int lane = threadIdx.x & 31;
     const int n = a.n;
     const int m = EXACT ? b.cnt[kCntExact] : b.first ? m_all : b.cnt[kCntActive];
-    unsigned long long n_ev = 0, n_re = 0;
+    unsigned n_ev = 0, n_re = 0;   // (a lane's share)
     float err = 0.f;
     // the lane's query
     float q[S];
@@ -214,16 +266,7 @@ __global__ void __launch_bounds__(kWalkThreads, search_blocks(D, HDB, F64, EXACT
                 kmin_update(best, x2, a.pid[i], a.pid[j]);
                 ++n_re;
             } else if (v < lim) {
-#pragma unroll
-                for (int k = K - 1; k >= 0; --k) {
-                    if (k > 0 && v < sl[k - 1]) {
-                        sl[k] = sl[k - 1];
-                        sj[k] = sj[k - 1];
-                    } else if (v < sl[k]) {
-                        sl[k] = v;
-                        sj[k] = j0 + p;
-                    }
-                }
+                list_insert<K>(sl, sj, v, j0 + p);
                 lim = fminf(lim, sl[K - 1]);
             }
         }
@@ -240,9 +283,19 @@ __global__ void __launch_bounds__(kWalkThreads, search_blocks(D, HDB, F64, EXACT
             }
         }
         pb = lim * (1.0f + 1.0f / 131072.0f);
+        if (ev >= b.long_evals) {
+            n_ev += ev;
+            ev = 0;
+            const int slot = atomicAdd(b.cnt + (EXACT ? kCntLongExact : kCntLong), 1);
+            if (slot < b.long_max) {
+                b.longq[slot] = i;
+                pb = -1.f;   // nothing left to visit
+            }
+        }
     };
     auto finish = [&] {
         n_ev += ev;
+        if (pb < 0.f) return;   // handed over
         if (EXACT) {
             if (best.hi < b.cap64) {
                 const int slot = atomicAdd(b.cnt + kCntCand, 1);   // at most one candidate per point: within n
@@ -260,6 +313,7 @@ __global__ void __launch_bounds__(kWalkThreads, search_blocks(D, HDB, F64, EXACT
                 b.lj[(size_t)k * n + i] = sj[k];
             }
             b.R[i] = lim;
+            b.low[i] = fminf(sl[0], lim);
             b.hd[i] = 0;
         }
     };
@@ -267,6 +321,155 @@ __global__ void __launch_bounds__(kWalkThreads, search_blocks(D, HDB, F64, EXACT
                                 X.deep + (size_t)blockIdx.x * kWalkThreads + threadIdx.x,
                                 (size_t)gridDim.x * kWalkThreads, (int *)a.overflow, 8, q, begin, bound, need, pending,
                                 scan, finish);
+    const unsigned long long all_ev = warp_sum_u64(n_ev);
+    if (lane == 0 && all_ev) {
+        atomicAdd(a.stat + 1, all_ev);
+        atomicAdd(a.stat + 6, all_ev);
+    }
+    if (EXACT) {
+        err_flush(a, err);
+        const unsigned long long all_re = warp_sum_u64(n_re);
+        if (lane == 0 && all_re) atomicAdd(a.stat + 2, all_re);
+    }
+}
+
+// the smallest K entries of the lanes' ascending lists, to every lane
+template <int K>
+__device__ __forceinline__ void warp_lists(float (&sl)[K], int (&sj)[K], float (&ol)[K], int (&oj)[K])
+{
+#pragma unroll
+    for (int r = 0; r < K; ++r) {
+        const unsigned u = __float_as_uint(sl[0]), m = __reduce_min_sync(0xffffffffu, u);
+        const int src = __ffs(__ballot_sync(0xffffffffu, u == m)) - 1;
+        ol[r] = __uint_as_float(m);
+        oj[r] = __shfl_sync(0xffffffffu, sj[0], src);
+        if ((threadIdx.x & 31) == src) {
+#pragma unroll
+            for (int k = 0; k + 1 < K; ++k) { sl[k] = sl[k + 1]; sj[k] = sj[k + 1]; }
+            sl[K - 1] = INFINITY;
+            sj[K - 1] = -1;
+        }
+    }
+}
+
+__device__ __forceinline__ void warp_kmin(KMin &m)
+{
+    for (int o = 16; o; o >>= 1) {
+        const unsigned long long h = __shfl_xor_sync(0xffffffffu, m.hi, o), l = __shfl_xor_sync(0xffffffffu, m.lo, o);
+        if (h < m.hi || (h == m.hi && l < m.lo)) { m.hi = h; m.lo = l; }
+    }
+}
+
+// The queries that the search handed over: a warp per query and part of the points; the warp that
+// finishes a query's last part puts the parts together.
+template <int D, bool HDB, bool F64, bool EXACT>
+__global__ void __launch_bounds__(kWalkThreads) nc_long_kernel(TravArgs a, NcArgs b)
+{
+    constexpr int S = row_floats(D), K = list_len(D);
+    const int lane = threadIdx.x & 31, n = a.n;
+    const int m = min(b.cnt[EXACT ? kCntLongExact : kCntLong], b.long_max) * b.chunks;   // at most 2^19
+    const int part = (n + b.chunks - 1) / b.chunks;
+    unsigned long long n_ev = 0, n_re = 0;
+    float err = 0.f;
+    for (int it = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < m; it += (gridDim.x * blockDim.x) >> 5) {
+        const int l = it / b.chunks, ch = it % b.chunks, i = b.longq[l], c = b.lab[i];
+        const int j1 = (int)min((long long)n, (long long)(ch + 1) * part);
+        float q[S];
+        load_row<S>(b.rows, i, q);
+        const float qcd = HDB ? a.cd32[i] : 0.f;
+        const float lim = EXACT ? next_up(screen_threshold(__uint_as_float(*(volatile unsigned *)(b.S + c)), a)) : INFINITY;
+        float sl[K], ol[K];
+        int sj[K], oj[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) { sl[k] = INFINITY; sj[k] = -1; }
+        KMin best{~0ull, ~0ull};
+        for (long long j0 = (long long)ch * part + lane; j0 < j1; j0 += 32) {
+            const int j = (int)j0;
+            float x[S];
+            load_row<S>(b.rows, j, x);
+            if (__float_as_int(x[S - 1]) == c) continue;
+            const float now = EXACT ? lim : sl[K - 1];
+            if (F64 && point_bound<D>(q, x, 2.f * a.delta32) > now * (1.0f + 1.0f / 131072.0f)) continue;
+            float v = screen_dist<D, S, F64>(a.x64, n, a.d, b.rows, i, j, q, x);
+            ++n_ev;
+            if (HDB) {
+                const float cdm = fmaxf(qcd, a.cd32[j]);
+                if (proven_repair(a, v, cdm)) continue;
+                v = fmaxf(v, cdm);
+            }
+            if (!(v < now)) continue;
+            if (EXACT) {
+                double x2 = walk_dist64<D, S>(a.x64, n, a.d, b.rows, i, j);
+                if (HDB) x2 = pos_dmax(x2, pos_dmax(a.cd64[i], a.cd64[j]));
+                if (!F64) note_err(v, x2, err);
+                kmin_update(best, x2, a.pid[i], a.pid[j]);
+                ++n_re;
+            } else {
+                list_insert<K>(sl, sj, v, j);
+            }
+        }
+        __syncwarp();
+        if (EXACT) {
+            warp_kmin(best);
+            if (lane == 0) b.long_k[it] = best;
+        } else {
+            warp_lists<K>(sl, sj, ol, oj);
+            if (lane == 0) {
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    b.long_s[(size_t)it * K + k] = ol[k];
+                    b.long_j[(size_t)it * K + k] = oj[k];
+                }
+            }
+        }
+        int done = 0;
+        if (lane == 0) {
+            __threadfence();
+            done = atomicAdd(b.long_done + l, 1);
+            __threadfence();
+        }
+        if (__shfl_sync(0xffffffffu, done, 0) != b.chunks - 1) continue;
+        const size_t at = (size_t)l * b.chunks;
+        if (EXACT) {
+            best = KMin{~0ull, ~0ull};
+            for (int p = lane; p < b.chunks; p += 32) {
+                const unsigned long long h = __ldcg(&b.long_k[at + p].hi), w = __ldcg(&b.long_k[at + p].lo);
+                if (h < best.hi || (h == best.hi && w < best.lo)) { best.hi = h; best.lo = w; }
+            }
+            __syncwarp();
+            warp_kmin(best);
+            if (lane == 0 && best.hi < b.cap64) {
+                const int slot = atomicAdd(b.cnt + kCntCand, 1);   // at most one candidate per point: within n
+                EdgeK e;
+                e.hi = best.hi;
+                e.lo = best.lo;
+                b.cand[slot] = e;
+                b.cand_c[slot] = c;
+                if (best.hi < *(volatile unsigned long long *)(b.bhi + c)) atomicMin(b.bhi + c, best.hi);
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < K; ++k) { sl[k] = INFINITY; sj[k] = -1; }
+            for (int p = lane; p < b.chunks * K; p += 32) {
+                const float v = __ldcg(b.long_s + at * K + p);
+                if (v < sl[K - 1]) list_insert<K>(sl, sj, v, __ldcg(b.long_j + at * K + p));
+            }
+            __syncwarp();
+            warp_lists<K>(sl, sj, ol, oj);
+            if (lane == 0) {
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    b.ls[(size_t)k * n + i] = ol[k];
+                    b.lj[(size_t)k * n + i] = oj[k];
+                }
+                b.R[i] = ol[K - 1];
+                b.low[i] = ol[0];
+                b.hd[i] = 0;
+                if (!b.first && ol[0] < INFINITY) atomicMin(b.S + c, __float_as_uint(ol[0]));
+            }
+        }
+        if (lane == 0) b.long_done[l] = 0;
+    }
     n_ev = warp_sum_u64(n_ev);
     if (lane == 0 && n_ev) {
         atomicAdd(a.stat + 1, n_ev);
@@ -318,10 +521,10 @@ __global__ void nc_init_kernel(TravArgs a, NcArgs b, bool hdb)
         b.blo[i] = ~0ull;
         if (hdb) {   // no list yet: an edge outside the repair list is longer than the core distance
             b.hd[i] = (unsigned char)b.K;
-            b.R[i] = __double2float_rd(a.cd64[i]);
+            b.R[i] = b.low[i] = __double2float_rd(a.cd64[i]);
         }
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) b.cnt[kCntRoots] = a.n;
+    if (blockIdx.x == 0 && threadIdx.x == 0) b.cnt[cnt_roots(0)] = a.n;
 }
 
 // WriteMin of a weight into a component's slot; a value that cannot lower it is not issued
@@ -332,14 +535,20 @@ __device__ __forceinline__ void s_min(unsigned *S, int c, float v)
 }
 
 // Advances the list heads past entries that joined the component; the first entry left bounds the
-// component's minimum.  A point without one offers its neighbours in tree order.
+// component's minimum.  A point without one offers its neighbours in tree order.  Nothing is looked up where
+// neither the head's weight nor the radius beyond the list can lower the minimum as it stands: such a head
+// may lie inside the component (it is looked at again once it matters).  In the late rounds most points stop
+// there; in the early ones a component's points are read together, before its minimum has come down (10^7
+// points in 3-D: 200 us in the second round, 80 in the tenth, bound by the gather of the heads' labels).
 template <int D, bool HDB, bool F64>
-__global__ void nc_refresh_kernel(TravArgs a, NcArgs b)
+__device__ __forceinline__ void refresh_points(const TravArgs &a, const NcArgs &b)
 {
+    if (b.first && held(b, 1)) return;   // (lists are missing)
     constexpr int S = row_floats(D);
     const int n = a.n;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int c = b.lab[i];
+        if (__float_as_uint(b.low[i]) >= *(volatile unsigned *)(b.S + c)) continue;
         int h = b.hd[i];
         if (h < b.K) {
             const int h0 = h;
@@ -348,8 +557,12 @@ __global__ void nc_refresh_kernel(TravArgs a, NcArgs b)
                 j = b.lj[(size_t)h * n + i];
                 if (j >= 0 && b.lab[j] != c) break;
             }
-            if (h != h0) b.hd[i] = (unsigned char)h;
-            if (h < b.K) s_min(b.S, c, b.ls[(size_t)h * n + i]);
+            const float s = h < b.K ? b.ls[(size_t)h * n + i] : INFINITY;
+            if (h != h0) {
+                b.hd[i] = (unsigned char)h;
+                b.low[i] = fminf(s, b.R[i]);
+            }
+            if (h < b.K) s_min(b.S, c, s);
         }
         if (h >= b.K) {
 #pragma unroll
@@ -405,36 +618,59 @@ __device__ __forceinline__ bool settled(const TravArgs &a, const NcArgs &b, int 
     return *(volatile unsigned long long *)(b.bhi + c) <= (unsigned long long)__double_as_longlong(a.cd64[i]);
 }
 
+// The active points, and those that pick_points has to look at: S only falls until then, and T with it.
+// (Eight points per thread between two appends: an append per 256 points, which most of those have a point
+// for, made the pass wait for one counter, 120 us for 10^7 points against 37 now.  With the list, this pass
+// and the one that picks take 0.67 ms a call where two passes over all points took 1.40.)
 template <bool HDB>
-__global__ void nc_active_kernel(TravArgs a, NcArgs b)
+__device__ __forceinline__ void active_points(const TravArgs &a, const NcArgs &b, int *sh)
 {
-    __shared__ int sh[32];
-    const int n = a.n;
-    for (int b0 = blockIdx.x * blockDim.x; b0 < n; b0 += gridDim.x * blockDim.x) {
-        const int i = b0 + threadIdx.x;
-        bool on = false;
-        if (i < n) {
-            const int c = b.lab[i];
-            on = b.R[i] <= screen_threshold(__uint_as_float(b.S[c]), a);
-            if (HDB && on) on = !settled(a, b, i, c);
+    const int n = a.n, items = 8 * blockDim.x;
+    for (long long b0 = (long long)blockIdx.x * items; b0 < n; b0 += (long long)gridDim.x * items) {
+        unsigned on = 0, near = 0;
+        int c[8];
+        float low[8], T[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            const long long at = b0 + t * blockDim.x + threadIdx.x;
+            c[t] = at < n ? b.lab[at] : -1;
+            low[t] = at < n ? b.low[at] : 0.f;
         }
+#pragma unroll
+        for (int t = 0; t < 8; ++t) T[t] = c[t] >= 0 ? __uint_as_float(b.S[c[t]]) : 0.f;
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            T[t] = screen_threshold(T[t], a);
+            if (c[t] >= 0 && low[t] <= T[t]) near |= 1u << t;
+        }
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            if (!((near >> t) & 1u)) continue;
+            const int i = (int)(b0 + t * blockDim.x + threadIdx.x);
+            if (b.R[i] <= T[t] && !(HDB && settled(a, b, i, c[t]))) on |= 1u << t;
+        }
+        if (!__syncthreads_or(near)) continue;
+        int slot = block_append(b.cnt + kCntNear, __popc(near), sh);
+        for (unsigned m = near; m; m &= m - 1) b.near[slot++] = (int)(b0 + (__ffs(m) - 1) * blockDim.x + threadIdx.x);
         if (!__syncthreads_or(on)) continue;
-        const int slot = block_append(b.cnt + kCntActive, on ? 1 : 0, sh);
-        if (on) b.act[slot] = i;
+        slot = block_append(b.cnt + kCntActive, __popc(on), sh);
+        for (unsigned m = on; m; m &= m - 1) b.act[slot++] = (int)(b0 + (__ffs(m) - 1) * blockDim.x + threadIdx.x);
     }
 }
 
 // Points with a list entry inside the band of their component's screened minimum, and points whose list
 // may have dropped one
 template <bool HDB>
-__global__ void nc_pick_kernel(TravArgs a, NcArgs b)
+__device__ __forceinline__ void pick_points(const TravArgs &a, const NcArgs &b, int *sh)
 {
-    __shared__ int sh[32];
-    const int n = a.n;
-    for (int b0 = blockIdx.x * blockDim.x; b0 < n; b0 += gridDim.x * blockDim.x) {
-        const int i = b0 + threadIdx.x;
+    if (held(b, 1)) return;
+    const int n = a.n, m = b.first ? n : b.cnt[kCntNear];
+    for (int b0 = blockIdx.x * blockDim.x; b0 < m; b0 += gridDim.x * blockDim.x) {
+        const int t = b0 + threadIdx.x;
         bool exact = false, has = false;
-        if (i < n) {
+        int i = 0;
+        if (t < m) {
+            i = b.first ? t : b.near[t];
             const int c = b.lab[i];
             const float T = screen_threshold(__uint_as_float(b.S[c]), a);
             exact = b.R[i] <= T;
@@ -453,10 +689,9 @@ __global__ void nc_pick_kernel(TravArgs a, NcArgs b)
 // K-minimum of a picked point's list entries inside the band, in FP64 (on a dense list: an FP64
 // instruction costs a warp the same however few of its lanes need it)
 template <int D, bool HDB, bool F64>
-__global__ void nc_cand_kernel(TravArgs a, NcArgs b)
+__device__ __forceinline__ void candidates(const TravArgs &a, const NcArgs &b, int *sh)
 {
     constexpr int S = row_floats(D);
-    __shared__ int sh[32];
     const int n = a.n, m = b.cnt[kCntPicked];
     unsigned long long n_re = 0;
     float err = 0.f;
@@ -497,8 +732,9 @@ __global__ void nc_cand_kernel(TravArgs a, NcArgs b)
 }
 
 // Among the candidates with their component's smallest weight: WriteMin of the id pair
-__global__ void nc_low_kernel(NcArgs b)
+__device__ __forceinline__ void low_ids(const NcArgs &b)
 {
+    if (held(b, 3)) return;
     const int m = b.cnt[kCntCand];
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < m; t += gridDim.x * blockDim.x) {
         const EdgeK e = b.cand[t];
@@ -509,6 +745,7 @@ __global__ void nc_low_kernel(NcArgs b)
 
 __global__ void nc_low_repair_kernel(NcArgs b, const EdgeK *__restrict__ rep, const int *__restrict__ m_dev)
 {
+    if (held(b, 3)) return;
     const int m = *m_dev;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < m; t += gridDim.x * blockDim.x) {
         const EdgeK e = rep[t];
@@ -521,10 +758,10 @@ __global__ void nc_low_repair_kernel(NcArgs b, const EdgeK *__restrict__ rep, co
 // Every root with an edge links to the component at its other end; of two roots that chose the same
 // edge the smaller stays a root.  (The keys along a chain of choices strictly fall, so there is no
 // longer cycle.)
-__global__ void nc_merge_kernel(TravArgs a, NcArgs b, int cur, EdgeK *__restrict__ out, int out_cap)
+__device__ __forceinline__ void merge_roots(const TravArgs &a, const NcArgs &b, int cur, EdgeK *out, int out_cap, int *sh)
 {
-    __shared__ int sh[32];
-    const int m = b.cnt[kCntRoots + cur];
+    if (held(b, 3)) return;
+    const int m = b.cnt[cnt_roots(cur)];
     for (int b0 = blockIdx.x * blockDim.x; b0 < m; b0 += gridDim.x * blockDim.x) {
         const int t = b0 + threadIdx.x;
         bool emit = false;
@@ -557,10 +794,10 @@ __global__ void nc_merge_kernel(TravArgs a, NcArgs b, int cur, EdgeK *__restrict
 
 // After the links: every root of the round is brought close to its component's root; the roots left are
 // collected and their slots reset for the next round.
-__global__ void nc_roots_kernel(NcArgs b, int cur)
+__device__ __forceinline__ void collect_roots(const NcArgs &b, int cur, int *sh)
 {
-    __shared__ int sh[32];
-    const int m = b.cnt[kCntRoots + cur];
+    if (held(b, 3)) return;
+    const int m = b.cnt[cnt_roots(cur)];
     for (int b0 = blockIdx.x * blockDim.x; b0 < m; b0 += gridDim.x * blockDim.x) {
         const int t = b0 + threadIdx.x;
         bool stays = false;
@@ -584,12 +821,12 @@ __global__ void nc_roots_kernel(NcArgs b, int cur)
                 *(volatile int *)(b.par + i) = x;
             }
         }
-        const int slot = block_append(b.cnt + kCntRoots + (cur ^ 1), stays ? 1 : 0, sh);
+        const int slot = block_append(b.cnt + cnt_roots(cur ^ 1), stays ? 1 : 0, sh);
         if (stays) b.roots[cur ^ 1][slot] = i;
     }
 }
 
-// The root above x.  nc_roots_kernel leaves every root of the round pointing at its new root or, where a
+// The root above x.  collect_roots leaves every root of the round pointing at its new root or, where a
 // concurrent walk halved the path once more, at an ancestor below it.
 __device__ __forceinline__ int root_of(const int *__restrict__ par, int x, int n)
 {
@@ -602,81 +839,95 @@ __device__ __forceinline__ int root_of(const int *__restrict__ par, int x, int n
 }
 
 // New labels, and per tile of positions the number of label changes along tree order (a node is in one
-// component when none falls inside its range).
+// component when none falls inside its range).  A warp takes kTileItems times 32 consecutive positions, so that
+// labels and rows are read and written by neighbouring lanes (10^7 points in 3-D: 52 us a round, where eight
+// consecutive positions per thread took 130, and 15 for the prefixes instead of 40).
 constexpr int kTileItems = 8, kTile = 256 * kTileItems;
 
-__global__ void __launch_bounds__(256) nc_relabel_kernel(NcArgs b, int S, int *__restrict__ sums)
+// Up to this many points the steps between the searches are run by one block each, see nc_small_back_kernel
+constexpr int kSmallThreads = 512, kSmallPoints = kSmallThreads * kTileItems;
+
+// Once a single component is left nobody reads a label again, and the steps below return at once.
+__device__ __forceinline__ void relabel_points(const NcArgs &b, int S, const int *roots, int *sums)
 {
     __shared__ int s_chg;
-    const int n = b.n;
+    const int n = b.n, lane = threadIdx.x & 31, tile_items = blockDim.x * kTileItems;
+    if (*roots == 1) return;
     const int *par = b.par;
-    for (int tile = blockIdx.x; tile * (long long)kTile < n; tile += gridDim.x) {
+    for (int tile = blockIdx.x; tile * (long long)tile_items < n; tile += gridDim.x) {
         if (threadIdx.x == 0) s_chg = 0;
         __syncthreads();
-        const int i0 = tile * kTile + threadIdx.x * kTileItems;
-        // (a neighbour's label may be replaced already: a root points at itself)
-        int prev = i0 > 0 && i0 < n ? root_of(par, *(volatile int *)(b.lab + i0 - 1), n) : -1;
-        int chg = 0;
+        const int i0 = tile * tile_items + (threadIdx.x >> 5) * (32 * kTileItems) + lane;
+        // (the label before may be replaced already: a root points at itself)
+        int last = lane == 0 && i0 > 0 && i0 < n ? root_of(par, *(volatile int *)(b.lab + i0 - 1), n) : -1;
+        int chg = 0, c[kTileItems], x[kTileItems];
+        // (the loads of all positions first: most roots are two links away)
+#pragma unroll
+        for (int t = 0; t < kTileItems; ++t) c[t] = i0 + 32 * t < n ? b.lab[i0 + 32 * t] : -1;
+#pragma unroll
+        for (int t = 0; t < kTileItems; ++t) x[t] = c[t] >= 0 ? par[c[t]] : -1;
 #pragma unroll
         for (int t = 0; t < kTileItems; ++t) {
-            const int i = i0 + t;
-            if (i >= n) break;
-            const int c = b.lab[i], x = root_of(par, c, n);
-            if (x != c) {
-                *(volatile int *)(b.lab + i) = x;
-                b.rows[(size_t)i * S + S - 1] = __int_as_float(x);
+            const int up = x[t] >= 0 ? par[x[t]] : -1;
+            if (up != x[t]) x[t] = root_of(par, up, n);
+        }
+#pragma unroll
+        for (int t = 0; t < kTileItems; ++t) {
+            const int i = i0 + 32 * t;
+            if (x[t] != c[t]) {
+                *(volatile int *)(b.lab + i) = x[t];
+                b.rows[(size_t)i * S + S - 1] = __int_as_float(x[t]);
             }
-            chg += i > 0 && x != prev;
-            prev = x;
+            const int before = __shfl_up_sync(0xffffffffu, x[t], 1);
+            chg += i > 0 && i < n && x[t] != (lane ? before : last);
+            last = __shfl_sync(0xffffffffu, x[t], 31);
         }
         chg = __reduce_add_sync(0xffffffffu, chg);
-        if ((threadIdx.x & 31) == 0 && chg) atomicAdd(&s_chg, chg);
+        if (lane == 0 && chg) atomicAdd(&s_chg, chg);
         __syncthreads();
         if (threadIdx.x == 0) sums[tile] = s_chg;
     }
 }
 
-// E[i] = label changes in (0, i), from the tiles' prefixes; E[n] all of them
-__global__ void __launch_bounds__(256) nc_prefix_kernel(int n, const int *__restrict__ lab, const int *__restrict__ sums,
-                                                        int *__restrict__ E)
+// E[i] = label changes in (0, i), from the tiles' prefixes (null: there is one tile); E[n] all of them
+__device__ __forceinline__ void change_prefixes(int n, const int *lab, const int *sums, const int *roots, int *E)
 {
-    __shared__ int sw[8];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int tile = blockIdx.x; tile * (long long)kTile < n; tile += gridDim.x) {
-        const int i0 = tile * kTile + threadIdx.x * kTileItems;
-        int prev = i0 > 0 && i0 < n ? lab[i0 - 1] : -1;
-        int chg[kTileItems], s = 0;
+    if (*roots == 1) return;
+    __shared__ int sw[kSmallThreads / 32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, tile_items = blockDim.x * kTileItems;
+    for (int tile = blockIdx.x; tile * (long long)tile_items < n; tile += gridDim.x) {
+        const int i0 = tile * tile_items + wid * (32 * kTileItems) + lane;
+        int last = lane == 0 && i0 > 0 && i0 < n ? lab[i0 - 1] : -1;
+        unsigned chg[kTileItems];
+        int s = 0;
 #pragma unroll
         for (int t = 0; t < kTileItems; ++t) {
-            const int i = i0 + t;
-            const int x = i < n ? lab[i] : prev;
-            chg[t] = i > 0 && x != prev;
-            prev = x;
-            s += chg[t];
+            const int i = i0 + 32 * t;
+            const int x = i < n ? lab[i] : -1;
+            const int before = __shfl_up_sync(0xffffffffu, x, 1);
+            chg[t] = __ballot_sync(0xffffffffu, i > 0 && i < n && x != (lane ? before : last));
+            last = __shfl_sync(0xffffffffu, x, 31);
+            s += __popc(chg[t]);
         }
-        int x = s;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) sw[wid] = x;
+        if (lane == 0) sw[wid] = s;
         __syncthreads();
-        int base = sums[tile];
-        for (int w = 0; w < wid; ++w) base += sw[w];
-        x += base - s;
+        int at = sums ? sums[tile] : 0;
+        for (int w = 0; w < wid; ++w) at += sw[w];
 #pragma unroll
         for (int t = 0; t < kTileItems; ++t) {
-            if (i0 + t < n) E[i0 + t] = x;
-            x += chg[t];
-            if (i0 + t == n - 1) E[n] = x;
+            const int i = i0 + 32 * t, e = at + __popc(chg[t] & lanemask_lt());
+            if (i < n) E[i] = e;
+            if (i == n - 1) E[n] = e + (int)((chg[t] >> lane) & 1u);
+            at += __popc(chg[t]);
         }
         __syncthreads();
     }
 }
 
-__global__ void nc_node_labels_kernel(int Ns, int S, const int2 *__restrict__ range, float *__restrict__ nodes,
-                                      int *__restrict__ nlab, const int *__restrict__ lab, const int *__restrict__ E)
+__device__ __forceinline__ void node_labels(int Ns, int S, const int2 *__restrict__ range, float *nodes, int *nlab, const int *lab,
+                                            const int *E, const int *roots)
 {
+    if (*roots == 1) return;
     for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < Ns; x += gridDim.x * blockDim.x) {
         const int2 r = range[x];
         if (E[r.y] != E[r.x + 1]) continue;   // mixed: the label is -1 from the start
@@ -685,6 +936,103 @@ __global__ void nc_node_labels_kernel(int Ns, int S, const int2 *__restrict__ ra
         nlab[x] = c;
         nodes[(size_t)x * 2 * S + box_hi(S - 1)] = __int_as_float(c);
     }
+}
+
+template <int D, bool HDB, bool F64>
+__global__ void nc_refresh_kernel(TravArgs a, NcArgs b) { refresh_points<D, HDB, F64>(a, b); }
+
+template <bool HDB>
+__global__ void nc_active_kernel(TravArgs a, NcArgs b)
+{
+    __shared__ int sh[32];
+    active_points<HDB>(a, b, sh);
+}
+
+template <bool HDB>
+__global__ void nc_pick_kernel(TravArgs a, NcArgs b)
+{
+    __shared__ int sh[32];
+    pick_points<HDB>(a, b, sh);
+}
+
+template <int D, bool HDB, bool F64>
+__global__ void nc_cand_kernel(TravArgs a, NcArgs b)
+{
+    __shared__ int sh[32];
+    candidates<D, HDB, F64>(a, b, sh);
+}
+
+__global__ void nc_low_kernel(NcArgs b) { low_ids(b); }
+
+__global__ void nc_merge_kernel(TravArgs a, NcArgs b, int cur, EdgeK *out, int out_cap)
+{
+    __shared__ int sh[32];
+    merge_roots(a, b, cur, out, out_cap, sh);
+}
+
+__global__ void nc_roots_kernel(NcArgs b, int cur)
+{
+    __shared__ int sh[32];
+    collect_roots(b, cur, sh);
+}
+
+__global__ void __launch_bounds__(256) nc_relabel_kernel(NcArgs b, int S, const int *roots, int *sums)
+{
+    relabel_points(b, S, roots, sums);
+}
+
+__global__ void __launch_bounds__(256) nc_prefix_kernel(int n, const int *lab, const int *sums, const int *roots, int *E)
+{
+    change_prefixes(n, lab, sums, roots, E);
+}
+
+__global__ void nc_node_labels_kernel(int Ns, int S, const int2 *range, float *nodes, int *nlab, const int *lab, const int *E,
+                                      const int *roots)
+{
+    node_labels(Ns, S, range, nodes, nlab, lab, E, roots);
+}
+
+// Few points: the steps before, between and after the searches by one block, with barriers for the ends of the
+// kernels.  Each of them is then shorter than the gap between two launches (EMST of 10^3 points 790 -> 686 us;
+// the launches win again where one block takes longer than they do).
+template <int D, bool HDB, bool F64>
+__global__ void __launch_bounds__(kSmallThreads) nc_small_front_kernel(TravArgs a, NcArgs b)
+{
+    __shared__ int sh[32];
+    refresh_points<D, HDB, F64>(a, b);
+    __syncthreads();
+    active_points<HDB>(a, b, sh);
+}
+
+template <int D, bool HDB, bool F64>
+__global__ void __launch_bounds__(kSmallThreads) nc_small_mid_kernel(TravArgs a, NcArgs b)
+{
+    __shared__ int sh[32];
+    if (b.first) {
+        refresh_points<D, HDB, F64>(a, b);
+        __syncthreads();
+    }
+    pick_points<HDB>(a, b, sh);
+    __syncthreads();
+    candidates<D, HDB, F64>(a, b, sh);
+}
+
+__global__ void __launch_bounds__(kSmallThreads) nc_small_back_kernel(TravArgs a, NcArgs b, int cur, EdgeK *out, int out_cap, int Ns,
+                                                                      int S, const int2 *range, float *nodes, int *sums, int *E)
+{
+    __shared__ int sh[32];
+    const int *roots = b.cnt + cnt_roots(cur ^ 1);
+    low_ids(b);
+    __syncthreads();
+    merge_roots(a, b, cur, out, out_cap, sh);
+    __syncthreads();
+    collect_roots(b, cur, sh);
+    __syncthreads();
+    relabel_points(b, S, roots, sums);
+    __syncthreads();
+    change_prefixes(b.n, b.lab, nullptr, roots, E);
+    __syncthreads();
+    node_labels(Ns, S, range, nodes, b.nlab, b.lab, E, roots);
 }
 
 template <int D, bool HDB, bool F64>
@@ -715,51 +1063,84 @@ int rounds(NcCall &C, TravArgs &a, NcArgs &b)
         b.ncd = ncd;
     }
     launch(nc_init_kernel, g, 256, 0, st, a, b, HDB);
+    const bool small = n <= kSmallPoints;
     const EdgeK *rin = C.rep;
     EdgeK *rbuf[2] = {C.rep_tmp0, C.rep_tmp1};
     long long edges = 0;
     // every component that can still grow links in a round: their number at least halves
     for (int r = 0; r < 64 && edges < C.target; ++r) {
         const int cur = r & 1;
-        cudaMemsetAsync(b.cnt, 0, kCntRound * sizeof(int), st);
-        cudaMemsetAsync(b.cnt + kCntRoots + (cur ^ 1), 0, sizeof(int), st);
+        cudaMemsetAsync(b.cnt + (cur ? 0 : kCntEven), 0, (cur ? kCntOddEnd : kCntEdges - kCntEven) * sizeof(int), st);
+        const int *roots = b.cnt + cnt_roots(cur ^ 1);
         const EdgeK *rnow = nullptr;
         const int *rn = nullptr;
         if (HDB) {
-            cudaMemsetAsync(b.cnt + kCntRep + cur, 0, sizeof(int), st);
-            launch(nc_repair_kernel, grid_for(C.nrep, 256), 256, 0, st, b, rin, r ? b.cnt + kCntRep + (cur ^ 1) : (const int *)nullptr,
-                   C.nrep, rbuf[cur], b.cnt + kCntRep + cur);
+            launch(nc_repair_kernel, grid_for(C.nrep, 256), 256, 0, st, b, rin, r ? b.cnt + cnt_rep(cur ^ 1) : (const int *)nullptr,
+                   C.nrep, rbuf[cur], b.cnt + cnt_rep(cur));
             rin = rnow = rbuf[cur];
-            rn = b.cnt + kCntRep + cur;
+            rn = b.cnt + cnt_rep(cur);
         }
         b.first = !HDB && r == 0;
         if (!b.first) {
-            launch(nc_refresh_kernel<D, HDB, F64>, g, 256, 0, st, a, b);
-            launch(nc_active_kernel<HDB>, g, 256, 0, st, a, b);
+            if (small) {
+                launch(nc_small_front_kernel<D, HDB, F64>, 1, kSmallThreads, 0, st, a, b);
+            } else {
+                launch(nc_refresh_kernel<D, HDB, F64>, g, 256, 0, st, a, b);
+                launch(nc_active_kernel<HDB>, gt, 256, 0, st, a, b);
+            }
         }
+        auto middle = [&] {
+            if (small) {
+                launch(nc_small_mid_kernel<D, HDB, F64>, 1, kSmallThreads, 0, st, a, b);
+            } else {
+                if (b.first) launch(nc_refresh_kernel<D, HDB, F64>, g, 256, 0, st, a, b);   // the lists' minima into S
+                launch(nc_pick_kernel<HDB>, g, 256, 0, st, a, b);
+                launch(nc_cand_kernel<D, HDB, F64>, g, 256, 0, st, a, b);
+            }
+            launch(nc_search_kernel<D, HDB, F64, true>, gs, kWalkThreads, 0, st, a, b, X, n);
+        };
+        auto back = [&]() -> int {
+            if (HDB) launch(nc_low_repair_kernel, grid_for(C.nrep, 256), 256, 0, st, b, rnow, rn);
+            if (small) {
+                launch(nc_small_back_kernel, 1, kSmallThreads, 0, st, a, b, cur, C.out, n - 1, X.Ns, S, X.range, X.nodes, sums, E);
+            } else {
+                launch(nc_low_kernel, g, 256, 0, st, b);
+                launch(nc_merge_kernel, g, 256, 0, st, a, b, cur, C.out, n - 1);
+                launch(nc_roots_kernel, g, 256, 0, st, b, cur);
+                launch(nc_relabel_kernel, gt, 256, 0, st, b, S, roots, sums);
+                const int rc = scan_exclusive_i32(sums, sums, tiles, nullptr, st, ar);
+                if (rc) return rc;
+                launch(nc_prefix_kernel, gt, 256, 0, st, n, b.lab, sums, roots, E);
+                launch(nc_node_labels_kernel, grid_for(X.Ns, 256), 256, 0, st, X.Ns, S, X.range, X.nodes, b.nlab, b.lab, E, roots);
+            }
+            cudaMemcpyAsync(C.pin, b.cnt, kCntAll * sizeof(int), cudaMemcpyDeviceToHost, st);
+            return cudaStreamSynchronize(st) == cudaSuccess ? 0 : WM_ECUDA;
+        };
+        b.guard = 3;
         C.mark(C.ctx);
         launch(nc_search_kernel<D, HDB, F64, false>, gs, kWalkThreads, 0, st, a, b, X, n);
         C.mark(C.ctx);
-        if (b.first) launch(nc_refresh_kernel<D, HDB, F64>, g, 256, 0, st, a, b);   // the lists' minima into S
-        launch(nc_pick_kernel<HDB>, g, 256, 0, st, a, b);
-        launch(nc_cand_kernel<D, HDB, F64>, g, 256, 0, st, a, b);
-        launch(nc_search_kernel<D, HDB, F64, true>, gs, kWalkThreads, 0, st, a, b, X, n);
-        launch(nc_low_kernel, g, 256, 0, st, b);
-        if (HDB) launch(nc_low_repair_kernel, grid_for(C.nrep, 256), 256, 0, st, b, rnow, rn);
-        launch(nc_merge_kernel, g, 256, 0, st, a, b, cur, C.out, n - 1);
-        launch(nc_roots_kernel, g, 256, 0, st, b, cur);
-        launch(nc_relabel_kernel, gt, 256, 0, st, b, S, sums);
-        int rc = scan_exclusive_i32(sums, sums, tiles, nullptr, st, ar);
+        middle();
+        int rc = back();
+        if (rc == 0 && C.pin[kCntLong] > 0) {
+            b.guard = 2;
+            C.mark(C.ctx);
+            launch(nc_long_kernel<D, HDB, F64, false>, num_sms() * 8, kWalkThreads, 0, st, a, b);
+            C.mark(C.ctx);
+            cudaMemsetAsync(b.cnt + kCntExactNext, 0, sizeof(int), st);   // (the search with nothing to do drew from it)
+            middle();
+            rc = back();
+        }
+        if (rc == 0 && C.pin[kCntLongExact] > 0) {
+            b.guard = 0;
+            launch(nc_long_kernel<D, HDB, F64, true>, num_sms() * 8, kWalkThreads, 0, st, a, b);
+            rc = back();
+        }
         if (rc) return rc;
-        launch(nc_prefix_kernel, gt, 256, 0, st, n, b.lab, sums, E);
-        launch(nc_node_labels_kernel, grid_for(X.Ns, 256), 256, 0, st, X.Ns, S, X.range, X.nodes, b.nlab, b.lab, E);
-        cudaMemcpyAsync(C.pin, b.cnt, kCntAll * sizeof(int), cudaMemcpyDeviceToHost, st);
-        cudaMemcpyAsync(C.pin + 32, a.overflow, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
-        if (cudaStreamSynchronize(st) != cudaSuccess) return WM_ECUDA;
         ++C.rounds;
-        C.candidates += C.pin[kCntCand] + (HDB ? C.pin[kCntRep + cur] : 0);
+        C.candidates += C.pin[kCntCand] + (HDB ? C.pin[cnt_rep(cur)] : 0);
         // (every edge takes one root)
-        if (C.pin[32] || C.pin[kCntRoots + (cur ^ 1)] != n - C.pin[kCntEdges]) {
+        if (C.pin[kCntError] || C.pin[cnt_roots(cur ^ 1)] != n - C.pin[kCntEdges]) {
             set_error_detail("nearest-component rounds: an internal check failed");
             return WM_EINTERNAL;
         }
@@ -789,6 +1170,7 @@ int nearest_component_rounds(NcCall &C, TravArgs &a)
     b.lj = ar.get<int>((size_t)b.K * n);
     b.R = ar.get<float>(n);
     b.hd = ar.get<unsigned char>(n);
+    b.low = ar.get<float>(n);
     b.act = ar.get<int>(n);
     b.amb = ar.get<int>(n);
     b.cand = ar.get<EdgeK>(n);
@@ -797,13 +1179,27 @@ int nearest_component_rounds(NcCall &C, TravArgs &a)
     b.roots[0] = ar.get<int>(n);
     b.roots[1] = ar.get<int>(n);
     b.picked = ar.get<int>(n);
+    b.near = b.cand_c;   // (read before the candidates are written)
+    a.overflow = (unsigned *)b.cnt + kCntError;
     b.n = n;
+    b.long_evals = ~0u;          // (of few points even a walk of all is short)
+    if (n >= kLongMinPoints) {
+        b.long_evals = (unsigned)std::max(kLongEvals, n / 1024);
+        b.chunks = std::min(kLongChunks, n / kLongChunk);
+        b.long_max = (int)std::min<long long>(kLongMax, std::max<long long>(4, kLongWork / n));
+        b.longq = ar.get<int>(b.long_max);
+        b.long_done = ar.get<int>(b.long_max);
+        b.long_s = ar.get<float>((size_t)b.long_max * b.chunks * b.K);
+        b.long_j = ar.get<int>((size_t)b.long_max * b.chunks * b.K);
+        b.long_k = ar.get<KMin>((size_t)b.long_max * b.chunks);
+    }
     if (C.rep) {
         C.rep_tmp0 = ar.get<EdgeK>(C.nrep);
         C.rep_tmp1 = ar.get<EdgeK>(C.nrep);
     }
     if (ar.failed) return WM_ENOMEM;
     cudaMemsetAsync(b.cnt, 0, kCntAll * sizeof(int), C.st);
+    if (b.chunks) cudaMemsetAsync(b.long_done, 0, b.long_max * sizeof(int), C.st);
     b.pos = C.pos;
     b.rows = C.X->rows;
     const float cf = C.cap < INFINITY ? C.cap_f : INFINITY;
