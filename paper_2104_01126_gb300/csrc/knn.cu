@@ -46,11 +46,23 @@ struct KnnArgs {
     int *slow;           // queries with ties around the k-th value
     float *slow_s;       // their screened k-th values
     int *slow_cnt;
+    int *slow2;          // queries left for the full scan
+    int *slow2_cnt;
+    unsigned long_evals; // a walk that has evaluated more points than this is handed to the full scan,
+    int *long_cnt;       // kKnnLongMax of them at most
     int *next_group;     // dispenser of 32-query groups
     int *err;            // set when a traversal stack would overflow (an internal error)
     unsigned long long *stat;   // [0] evals, [1] fp64 rechecks, [2] bits of the largest relative
                                 //     error of a screened k-th value against the exact one
 };
+
+// FP64 form: a walk that has evaluated a 32nd of all points (16384 at least) is an outlier, such as the
+// centre of a sphere of points, which visits every node on one lane while the GPU waits: it goes to the full
+// scan's blocks.  Where that is what every walk does (high dimension), the first four per SM are scanned.
+// (HDBSCAN* of 50,000 points on a sphere and their centre 68 -> 24 ms, with the searches' own hand-over.  The
+// FP32 walk is four times as fast per point, and the test cost every call 2 %.)
+constexpr unsigned kKnnLongEvals = 16384;
+constexpr int kKnnLongMax = 608;
 
 // -------------------------------------------------------------------------- thread per query
 // Shared memory of a block of T threads: uint2 stk[kWalkStack][T], uint2 heap[k][T] (value bits,
@@ -159,9 +171,18 @@ __global__ void __launch_bounds__(kWalkThreads, F64 ? 1 : D <= 3 ? 8 : 6) knn_wa
             }
         }
         pb = screen_threshold(top, band) * (1.0f + 1.0f / 131072.0f);
+        if (F64 && ev > a.long_evals) {
+            n_ev += ev;
+            ev = 0;
+            if (atomicAdd(a.long_cnt, 1) < kKnnLongMax) {
+                a.slow2[atomicAdd(a.slow2_cnt, 1)] = i;
+                pb = -1.f;   // nothing left to visit
+            }
+        }
     };
     auto finish = [&] {
         n_ev += ev;
+        if (F64 && pb < 0.f) return;   // handed over
         if (cnt < k || !(out > screen_threshold(top, band))) {
             const int t = atomicAdd(a.slow_cnt, 1);
             a.slow[t] = i;
@@ -347,59 +368,78 @@ __device__ inline double any_dist64(const double *__restrict__ x64, const float 
     return s;
 }
 
-// Exact FP64 answer for one query per warp (ties or duplicates overflowed the list): each lane
-// keeps the k smallest w2 of its strided share, the warp merges the 32 lists, then a second
-// scan collects every q with w2 <= cd2 as repair edges.
-__global__ void __launch_bounds__(32) knn_slow_kernel(KnnArgs a, const float *__restrict__ rows, int S,
-                                                      const int *__restrict__ slow, int nslow,
-                                                      int *extra_q, int *extra_p, double *extra_d, int *extra_cnt,
-                                                      int extra_cap, int *tie_overflow)
+// rigorous lower bound of any_dist64 from the rows, whose coordinates err by at most delta2 together
+__device__ inline float any_bound(const float *__restrict__ rows, int S, int d, int i, int j, float delta2)
 {
-    extern __shared__ unsigned char smem_raw[];
-    const int lane = threadIdx.x;
+    float g = 0.f;
+    for (int k = 0; k < d; ++k) {
+        const float t = fmaxf(fabsf(rows[(size_t)i * S + k] - rows[(size_t)j * S + k]) - delta2, 0.f);
+        g = fmaf(t, t, g);
+    }
+    return lower_w2(g);
+}
+
+// Exact FP64 answer for one query per block (ties or duplicates overflowed the list, or a walk that does not
+// end): each thread keeps the k smallest w2 of its strided share, the block merges the lists, then a
+// second scan collects every q with w2 <= cd2 as repair edges.  A point whose FP32 bound is beyond the
+// list costs no FP64 (whose rate is 1/64).
+__global__ void __launch_bounds__(256) knn_slow_kernel(KnnArgs a, const float *__restrict__ rows, int S, float delta2,
+                                                       const int *__restrict__ slow, int nslow,
+                                                       int *extra_q, int *extra_p, double *extra_d, int *extra_cnt,
+                                                       int extra_cap, int *tie_overflow)
+{
+    extern __shared__ double slow_lists[];   // [k][T]
+    __shared__ double s_min[8];
+    __shared__ int s_who;
+    const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31;
     const int k = a.k, n = a.n, d = a.d;
-    double *lw = (double *)smem_raw;            // [k][32]
-    int *head = (int *)(lw + (size_t)k * 32);   // [32]
+    double *lw = slow_lists + tid;
     for (int t = blockIdx.x; t < nslow; t += gridDim.x) {
-        __syncwarp();
         const int i = slow[t];
         int cnt = 0;
-        for (int j = lane; j < n; j += 32) {
-            double w = j == i ? 0.0 : any_dist64(a.x64, rows, S, n, d, i, j);
-            if (cnt < k || w < lw[(k - 1) * 32 + lane]) {
+        float far = INFINITY;   // the list's largest value, rounded up, once it is full
+        for (int j = tid; j < n; j += T) {
+            if (any_bound(rows, S, d, i, j, delta2) > far) continue;
+            const double w = j == i ? 0.0 : any_dist64(a.x64, rows, S, n, d, i, j);
+            if (cnt < k || w < lw[(k - 1) * T]) {
                 int pos = cnt < k ? cnt : k - 1;
-                while (pos > 0 && lw[(pos - 1) * 32 + lane] > w) { lw[pos * 32 + lane] = lw[(pos - 1) * 32 + lane]; --pos; }
-                lw[pos * 32 + lane] = w;
+                while (pos > 0 && lw[(pos - 1) * T] > w) { lw[pos * T] = lw[(pos - 1) * T]; --pos; }
+                lw[pos * T] = w;
                 if (cnt < k) ++cnt;
+                if (cnt == k) far = __double2float_ru(lw[(k - 1) * T]);
             }
         }
-        head[lane] = 0;
-        __syncwarp();
+        int head = 0;
         double kth = 0.0;
-        for (int r = 0; r < k; ++r) {
-            double mine = head[lane] < cnt ? lw[head[lane] * 32 + lane] : INFINITY;
+        for (int r = 0; r < k; ++r) {   // (n >= k points are in the lists)
+            const double mine = head < cnt ? lw[head * T] : INFINITY;
             double mn = mine;
             for (int o = 16; o; o >>= 1) mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-            unsigned who = __ballot_sync(0xffffffffu, mine == mn);
-            if (lane == __ffs(who) - 1) head[lane]++;
-            __syncwarp();
+            if (lane == 0) s_min[tid >> 5] = mn;
+            if (tid == 0) s_who = T;
+            __syncthreads();
+            for (int w = 0; w < T / 32; ++w) mn = fmin(mn, s_min[w]);
+            if (mine == mn && head < cnt) atomicMin(&s_who, tid);
+            __syncthreads();
+            if (tid == s_who) ++head;
             kth = mn;
+            __syncthreads();
         }
-        if (lane == 0) {
+        if (tid == 0) {
             a.cd64[i] = kth;
             a.cd32[i] = __double2float_rn(kth);
             a.rep_cnt[i] = 0;
         }
-        for (int j = lane; j < n; j += 32) {
-            if (j == i) continue;
-            double w = any_dist64(a.x64, rows, S, n, d, i, j);
+        far = __double2float_ru(kth);
+        for (int j = tid; j < n; j += T) {
+            if (j == i || any_bound(rows, S, d, i, j, delta2) > far) continue;
+            const double w = any_dist64(a.x64, rows, S, n, d, i, j);
             if (w <= kth) {
-                int s = atomicAdd(extra_cnt, 1);
+                const int s = atomicAdd(extra_cnt, 1);
                 if (s < extra_cap) { extra_p[s] = i; extra_q[s] = j; extra_d[s] = w; }
                 else atomicOr(tie_overflow, 1);
             }
         }
-        __syncwarp();
     }
 }
 
@@ -503,6 +543,8 @@ __global__ void core_out_kernel(const double *__restrict__ cd64, const int *__re
 constexpr int kWalkSmemMax = 100 << 10;    // (kWalkStack + minPts) entries for at least 32 threads
 constexpr int kTieSmemMax = 64 << 10;      // stacks of kTieWarps warps in the deepest tree (FP32 exponents
                                            // and mantissas allow about 3800 levels in 16 dimensions)
+constexpr int kSlowSmemMax = 100 << 10;    // minPts values for at least 32 threads
+static_assert(kMaxMinPts * 32 * 8 <= kSlowSmemMax, "shared memory limit of the full scan");
 static_assert((kWalkStack + kMaxMinPts) * 32 * 8 <= kWalkSmemMax, "shared memory limit of the k-NN walk");
 
 // core distances and repair edges (fp64: the plain form)
@@ -532,19 +574,23 @@ int core_distances(const Points &P, const SearchTree &X, int min_pts, bool fp64,
     a.rep_cnt = ar.get<int>(n + 1);
     a.slow = ar.get<int>(n);
     a.slow_s = ar.get<float>(n);
-    int *slow2 = ar.get<int>(n);
+    int *slow2 = a.slow2 = ar.get<int>(n);
     // [0] queries with ties, [1] overflow edges, [2] overflow flag, [3] repair edges, [4] dispenser of
-    // the tie kernel, [5] error, [6] dispenser of the walk, [7] queries left for the full scan
-    int *cnts = ar.get<int>(8);
+    // the tie kernel, [5] error, [6] dispenser of the walk, [7] queries left for the full scan, [8] walks
+    // handed to it
+    int *cnts = ar.get<int>(9);
     a.slow_cnt = cnts;
     a.stat = ar.get<unsigned long long>(4);
     int *ex_p = ar.get<int>(extra_cap), *ex_q = ar.get<int>(extra_cap);
     double *ex_d = ar.get<double>(extra_cap);
     if (ar.failed) return WM_ENOMEM;
-    cudaMemsetAsync(cnts, 0, 8 * sizeof(int), st);
+    cudaMemsetAsync(cnts, 0, 9 * sizeof(int), st);
     cudaMemsetAsync(a.stat, 0, 4 * sizeof(unsigned long long), st);
     a.next_group = cnts + 6;
     a.err = cnts + 5;
+    a.slow2_cnt = cnts + 7;
+    a.long_cnt = cnts + 8;
+    a.long_evals = std::max(kKnnLongEvals, (unsigned)n / 32);
     cudaEvent_t k0, k1;
     cudaEventCreate(&k0);
     cudaEventCreate(&k1);
@@ -622,10 +668,11 @@ int core_distances(const Points &P, const SearchTree &X, int min_pts, bool fp64,
     cudaEventDestroy(k1);
     const int nslow = pin[7];
     if (nslow > 0) {
-        size_t sm2 = (size_t)min_pts * 32 * 8 + 32 * 4;
-        cudaFuncSetAttribute(knn_slow_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxMinPts * 32 * 8 + 32 * 4);
-        launch(knn_slow_kernel, std::min(nslow, num_sms() * 8), 32, sm2, st, a, X.rows, X.S, slow2, nslow, ex_q, ex_p, ex_d, cnts + 1,
-                                                                     extra_cap, cnts + 2);
+        int threads = 256;
+        while (threads > 32 && (size_t)min_pts * threads * 8 > (size_t)kSlowSmemMax) threads >>= 1;
+        cudaFuncSetAttribute(knn_slow_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSlowSmemMax);
+        launch(knn_slow_kernel, std::min(nslow, num_sms() * 8), threads, (size_t)min_pts * threads * 8, st, a, X.rows, X.S,
+               2.f * P.delta, slow2, nslow, ex_q, ex_p, ex_d, cnts + 1, extra_cap, cnts + 2);
     }
     // repair edges: one copy of each, weighted, in no particular order (each round takes those it needs)
     launch(rep_emit_kernel, grid_for(n, 256), 256, 0, st, a.rep_q, a.rep_d, a.rep_cnt, n, H.cd64, P.pid, rep, cnts + 3);
