@@ -418,9 +418,11 @@ def kernel_rooflines(runs, peaks, fp32_peak, fp32_basis, hdb=False):
         lambda s: s.bccp_evals - s.bccp_tile_evals - s.bccp_dual_evals, tot(lambda d, s: s.ms_bccp_group), None, x)
     alu("bccp_pair_tile_kernel (medium and big pairs)", lambda s: s.bccp_tile_evals,
         tot(lambda d, s: s.ms_tile_kernel), None, x)
-    alu("bccp_dual_kernel (huge pairs, pruned dual-tree)", lambda s: s.bccp_dual_evals,
+    # calls without traversals run the nearest-component rounds, whose search reports under the same fields
+    alu("bccp_dual_kernel (huge pairs, pruned dual-tree)" if tot(lambda d, s: s.getpairs_visits) > 0
+        else "nc_search_kernel (nearest-component search)", lambda s: s.bccp_dual_evals,
         tot(lambda d, s: s.ms_bccp_dual), None, x)
-    alu("knn_fast_kernel (core distances)", lambda s: s.knn_evals, tot(lambda d, s: s.ms_knn_kernel),
+    alu("knn_walk_kernel (core distances)", lambda s: s.knn_evals, tot(lambda d, s: s.ms_knn_kernel),
         len(runs))
     if not ks:
         return None
