@@ -210,7 +210,7 @@ def run_batched(wm, torch, count, seed):
                        "batched_ms": ms_sub, "speedup": ms_single / ms_sub},
             "mix": "n log-uniform [64, 65536], d in {2,3,5}, half EMST and half HDBSCAN* (minPts in {5,10,50}), "
                    "uniform or gmm points; instances with equal minPts share one k-d forest and one set of "
-                   "MemoGFK rounds (split by d where a dimension holds >= 2^20 points)"}
+                   "rounds (split by d where a dimension holds >= 2^20 points)"}
 
 
 def run_serving(wm, jobs, workers, budget, rate_hz=None, seed=1, precision="fp32"):
