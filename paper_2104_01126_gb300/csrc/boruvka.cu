@@ -57,11 +57,13 @@ __host__ __device__ constexpr int list_len(int D) { return D <= 3 ? 6 : 4; }
 // handed to warps that share a scan of all points: the centre of a sphere of points is as far from all of
 // them, and its walk visits every node on one lane while the GPU waits (50,000 points and their centre: 83 ms
 // a call, of which 81 on that lane; 5.0 now, 3.3 with a limit of 1024, which 7-D sets reach in ordinary
-// walks: 2 % slower).  A round scans at most kLongMax queries and about kLongWork points in all: where such
-// queries are many, there are lanes enough for them.  They are rare, so the scan is launched when the host has
-// seen one (launched every time it cost 10^4 points 6 %); until then the kernels behind the search hold back
-// (held).
-constexpr int kLongEvals = 2048, kLongMax = 512, kLongChunk = 2048, kLongChunks = 1024, kLongMinPoints = 8192;
+// walks: 2 % slower).  While at most kLongMax queries and about kLongWork points' evaluations are waiting, such
+// a query is handed over at once; one that comes later walks on, and is handed over all the same when it has
+// evaluated a kLongPart-th of all points, since it will hardly stop before the rest.  A query is handed over
+// at most once a search, and the list has a place for every query of the search: its counter cannot pass n.
+// Such queries are rare, so the scan is launched when the host has seen one (launched every time it cost 10^4
+// points 6 %), for kLongMax of them at a time; until then the kernels behind the search hold back (held).
+constexpr int kLongEvals = 2048, kLongMax = 512, kLongPart = 16, kLongChunk = 2048, kLongChunks = 1024, kLongMinPoints = 8192;
 constexpr long long kLongWork = 1 << 26;
 
 // Counters.  Those that a round starts from zero lie side by side: an even one's are [kCntEven, kCntEdges), an
@@ -103,15 +105,16 @@ struct NcArgs {
     unsigned long long cap64;  // the same in FP64 bits
     float *rows;               // the search tree's point rows
     const float *ncd;          // HDBSCAN*: smallest core distance of a node (rounded down)
-    // queries handed to the scan of all points (chunks: parts of the points; 0: no hand-over)
+    // queries handed to the scan of all points (chunks: parts of the points; 0: no hand-over): positions in
+    // amb, which the search leaves alone, or of the exact search in act
     int chunks, long_max;
-    unsigned long_evals;
+    unsigned long_evals, long_most;   // evaluations after which a query is handed over: while fewer than
+                                      // long_max are waiting, in any case
     int guard;                 // 1: hold back while queries of the search wait for the scan, 2: of the exact one
-    int *longq;                // [long_max] positions
-    int *long_done;            // [long_max] parts finished
-    float *long_s;             // [long_max][chunks][K] a part's list
+    int *long_done;            // [kLongMax] parts finished
+    float *long_s;             // [kLongMax][chunks][K] a part's list
     int *long_j;
-    KMin *long_k;              // [long_max][chunks] a part's K-minimum
+    KMin *long_k;              // [kLongMax][chunks] a part's K-minimum
     int first;                 // first search: components are single points, nothing is pruned by S
     int n;
 };
@@ -283,13 +286,11 @@ __global__ void __launch_bounds__(kWalkThreads, search_blocks(D, HDB, F64, EXACT
             }
         }
         pb = lim * (1.0f + 1.0f / 131072.0f);
-        if (ev >= b.long_evals) {
-            n_ev += ev;
-            ev = 0;
-            const int slot = atomicAdd(b.cnt + (EXACT ? kCntLongExact : kCntLong), 1);
-            if (slot < b.long_max) {
-                b.longq[slot] = i;
-                pb = -1.f;   // nothing left to visit
+        if (ev >= b.long_evals && (ev & 255u) < 8u) {   // (a bucket adds at most 8)
+            int *waiting = b.cnt + (EXACT ? kCntLongExact : kCntLong);
+            if (ev >= b.long_most || *(volatile int *)waiting < b.long_max) {
+                (EXACT ? b.act : b.amb)[atomicAdd(waiting, 1)] = i;
+                pb = -1.f;   // nothing left to visit: the query ends here
             }
         }
     };
@@ -360,19 +361,20 @@ __device__ __forceinline__ void warp_kmin(KMin &m)
     }
 }
 
-// The queries that the search handed over: a warp per query and part of the points; the warp that
-// finishes a query's last part puts the parts together.
+// The queries [first, first + kLongMax) that the search handed over: a warp per query and part of the points;
+// the warp that finishes a query's last part puts the parts together.
 template <int D, bool HDB, bool F64, bool EXACT>
-__global__ void __launch_bounds__(kWalkThreads) nc_long_kernel(TravArgs a, NcArgs b)
+__global__ void __launch_bounds__(kWalkThreads) nc_long_kernel(TravArgs a, NcArgs b, int first)
 {
     constexpr int S = row_floats(D), K = list_len(D);
     const int lane = threadIdx.x & 31, n = a.n;
-    const int m = min(b.cnt[EXACT ? kCntLongExact : kCntLong], b.long_max) * b.chunks;   // at most 2^19
+    const int *longq = (EXACT ? b.act : b.amb) + first;
+    const int m = min(b.cnt[EXACT ? kCntLongExact : kCntLong] - first, kLongMax) * b.chunks;   // at most 2^19
     const int part = (n + b.chunks - 1) / b.chunks;
     unsigned long long n_ev = 0, n_re = 0;
     float err = 0.f;
     for (int it = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < m; it += (gridDim.x * blockDim.x) >> 5) {
-        const int l = it / b.chunks, ch = it % b.chunks, i = b.longq[l], c = b.lab[i];
+        const int l = it / b.chunks, ch = it % b.chunks, i = longq[l], c = b.lab[i];
         const int j1 = (int)min((long long)n, (long long)(ch + 1) * part);
         float q[S];
         load_row<S>(b.rows, i, q);
@@ -1125,7 +1127,8 @@ int rounds(NcCall &C, TravArgs &a, NcArgs &b)
         if (rc == 0 && C.pin[kCntLong] > 0) {
             b.guard = 2;
             C.mark(C.ctx);
-            launch(nc_long_kernel<D, HDB, F64, false>, num_sms() * 8, kWalkThreads, 0, st, a, b);
+            for (int f = 0; f < C.pin[kCntLong]; f += kLongMax)
+                launch(nc_long_kernel<D, HDB, F64, false>, num_sms() * 8, kWalkThreads, 0, st, a, b, f);
             C.mark(C.ctx);
             cudaMemsetAsync(b.cnt + kCntExactNext, 0, sizeof(int), st);   // (the search with nothing to do drew from it)
             middle();
@@ -1133,7 +1136,8 @@ int rounds(NcCall &C, TravArgs &a, NcArgs &b)
         }
         if (rc == 0 && C.pin[kCntLongExact] > 0) {
             b.guard = 0;
-            launch(nc_long_kernel<D, HDB, F64, true>, num_sms() * 8, kWalkThreads, 0, st, a, b);
+            for (int f = 0; f < C.pin[kCntLongExact]; f += kLongMax)
+                launch(nc_long_kernel<D, HDB, F64, true>, num_sms() * 8, kWalkThreads, 0, st, a, b, f);
             rc = back();
         }
         if (rc) return rc;
@@ -1185,13 +1189,13 @@ int nearest_component_rounds(NcCall &C, TravArgs &a)
     b.long_evals = ~0u;          // (of few points even a walk of all is short)
     if (n >= kLongMinPoints) {
         b.long_evals = (unsigned)std::max(kLongEvals, n / 1024);
+        b.long_most = std::max(b.long_evals, (unsigned)n / kLongPart);
         b.chunks = std::min(kLongChunks, n / kLongChunk);
         b.long_max = (int)std::min<long long>(kLongMax, std::max<long long>(4, kLongWork / n));
-        b.longq = ar.get<int>(b.long_max);
-        b.long_done = ar.get<int>(b.long_max);
-        b.long_s = ar.get<float>((size_t)b.long_max * b.chunks * b.K);
-        b.long_j = ar.get<int>((size_t)b.long_max * b.chunks * b.K);
-        b.long_k = ar.get<KMin>((size_t)b.long_max * b.chunks);
+        b.long_done = ar.get<int>(kLongMax);
+        b.long_s = ar.get<float>((size_t)kLongMax * b.chunks * b.K);
+        b.long_j = ar.get<int>((size_t)kLongMax * b.chunks * b.K);
+        b.long_k = ar.get<KMin>((size_t)kLongMax * b.chunks);
     }
     if (C.rep) {
         C.rep_tmp0 = ar.get<EdgeK>(C.nrep);
@@ -1199,7 +1203,7 @@ int nearest_component_rounds(NcCall &C, TravArgs &a)
     }
     if (ar.failed) return WM_ENOMEM;
     cudaMemsetAsync(b.cnt, 0, kCntAll * sizeof(int), C.st);
-    if (b.chunks) cudaMemsetAsync(b.long_done, 0, b.long_max * sizeof(int), C.st);
+    if (b.chunks) cudaMemsetAsync(b.long_done, 0, kLongMax * sizeof(int), C.st);
     b.pos = C.pos;
     b.rows = C.X->rows;
     const float cf = C.cap < INFINITY ? C.cap_f : INFINITY;
