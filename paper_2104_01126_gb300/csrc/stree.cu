@@ -107,8 +107,9 @@ __global__ void __launch_bounds__(kStThreads) st_ingest_kernel(StArgs a)
                 const double x = src_coord(a, i, k);
                 v[k] = __double2float_rn(x);
                 if (a.dtype != WM_F32) {
-                    // the error bound rounded up
-                    dmax = fmaxf(dmax, __fmul_ru((float)fabs(x - (double)v[k]), 1.0f + 1.0f / 8388608.0f));
+                    // the error rounded up: above 0 wherever the copy is inexact, however small (the FP64
+                    // coordinates are kept only then)
+                    dmax = fmaxf(dmax, __double2float_ru(fabs(x - (double)v[k])));
                 }
                 bad = bad || !(fabsf(v[k]) <= 1152921504606846976.0f) || fabs(x) > 1152921504606846976.0;
                 mn[k] = fminf(mn[k], v[k]);

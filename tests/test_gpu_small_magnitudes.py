@@ -36,5 +36,5 @@ def test_fp64_coordinates_below_the_fp32_range(scale, min_pts, precision):
 def test_one_cluster_below_the_fp32_range(min_pts):
     # exact FP32 coordinates but for a cluster about the origin that the copies collapse to one point
     g = np.random.default_rng(2)
-    x = np.concatenate([1 + g.random((900, 2)).astype(np.float32).astype(np.float64), 1e-46 * g.random((40, 2))])
+    x = np.concatenate([(1 + g.random((900, 2))).astype(np.float32), 1e-46 * g.random((40, 2))])   # FP64
     _check(g.permutation(x), min_pts)
