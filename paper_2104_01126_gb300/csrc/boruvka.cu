@@ -128,9 +128,9 @@ __device__ __forceinline__ bool held(const NcArgs &b, int what)
 // HDBSCAN*: true when the FP32 squared distance d32 proves D <= c for a core distance c (FP32 copy)
 __device__ inline bool proven_repair(const TravArgs &a, float d32, float c)
 {
-    if (a.exact32) return d32 * (1.0f + 1.0f / 131072.0f) < c * (1.0f - 1.0f / 4194304.0f);
-    const double r = sqrt((double)d32 * (1.0 + 1.0 / 131072.0)) + a.eta;
-    return r * r * (1.0 + 1.0 / 131072.0) < (double)c * (1.0 - 1.0 / 4194304.0);
+    if (a.exact32) return proven_within(d32, c);
+    const double r = sqrt((double)d32 * (1.0 + 1.0 / 131072.0) + kAbsTiny) + a.eta;
+    return r * r * (1.0 + 1.0 / 131072.0) < (double)c * (1.0 - 1.0 / 4194304.0) - kAbsTiny;
 }
 
 // relative error of a screened weight against the exact one (an upper bound, FP32)

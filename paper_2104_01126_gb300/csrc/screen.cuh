@@ -92,15 +92,23 @@ __device__ inline double pos_dmax(double x, double y)
     return __double_as_longlong(x) >= __double_as_longlong(y) ? x : y;
 }
 
+// True when the FP32 squared distance d32 of exact rows proves D <= cd2 for a core distance whose FP32 copy
+// is c.  d32 is within 2^-19 of D and c within 2^-24 of cd2, and each besides within kAbsTiny (2^-140), which
+// bounds what subnormal rounding takes: up to 2^-150 for each of 16 products, so that d32 can be 0 where D is
+// above a cd2 that FP32 still holds.
+__device__ inline bool proven_within(float d32, float c)
+{
+    return __fmaf_ru(d32, 1.0f + 1.0f / 131072.0f, 2.f * kAbsTiny) < __fmul_rd(c, 1.0f - 1.0f / 4194304.0f);
+}
+
 // exact FP64 weight of positions (i,j).  d32: the FP32 squared distance alone; c32: the larger
-// FP32 core distance (HDBSCAN*).  When d32 is provably below the larger core distance (d32 is
-// within 2^-19 of the true distance, a stored cd32 within 2^-24 of its FP64 value), the weight
-// is that core distance and the FP64 distance is skipped.
+// FP32 core distance (HDBSCAN*).  When the distance is provably within the larger core distance, the
+// weight is that core distance and the FP64 distance is skipped.
 __device__ inline double exact_w2(const TravArgs &a, int i, int j, float d32, float c32)
 {
     if (a.cd64) {
         double c = pos_dmax(a.cd64[i], a.cd64[j]);
-        if (a.exact32 && d32 * (1.0f + 1.0f / 131072.0f) < c32 * (1.0f - 1.0f / 4194304.0f)) return c;
+        if (a.exact32 && proven_within(d32, c32)) return c;
         return pos_dmax(c, dist64(a.x64, a.n, a.d, i, j));
     }
     return dist64(a.x64, a.n, a.d, i, j);

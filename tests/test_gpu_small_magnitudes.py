@@ -38,3 +38,26 @@ def test_one_cluster_below_the_fp32_range(min_pts):
     g = np.random.default_rng(2)
     x = np.concatenate([(1 + g.random((900, 2))).astype(np.float32), 1e-46 * g.random((40, 2))])   # FP64
     _check(g.permutation(x), min_pts)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("min_pts", [2, 5, 12])
+@pytest.mark.parametrize("d,scale", [(2, 1e-21), (3, 3e-22), (3, 1e-22), (7, 1e-22), (7, 3e-23), (7, 1e-23), (16, 3e-23)])
+def test_fp32_distances_that_underflow(d, scale, min_pts):
+    # FP32 squared differences vanish beside core distances that do not
+    _check((scale * np.random.default_rng(d).random((700, d))).astype(np.float32), min_pts)
+
+
+@pytest.mark.gpu
+def test_inexact_copies_of_distances_that_underflow():
+    # the same with rounded copies: the cluster's FP64 coordinates lie 1e-30 beside FP32 ones
+    x = (1e-22 * np.random.default_rng(4).random((700, 7))).astype(np.float32).astype(np.float64)
+    _check(x + 1e-30 * np.random.default_rng(5).random(x.shape), 5)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("d,scale", [(3, 3e-22), (7, 1e-22)])
+def test_distances_that_underflow_in_the_pair_traversals(d, scale):
+    require_gpu()
+    with wm.tuning():   # an override: the pair traversals
+        _check((scale * np.random.default_rng(d).random((700, d))).astype(np.float32), 5)
