@@ -1409,7 +1409,8 @@ static int spanning_tree(Call &C, const void *pts, int64_t n64, int d, int dtype
                          Prepared &S, HdbState &H, EdgeK *&E, unsigned *ovf, long long target = -1, double cap = INFINITY)
 {
     const int n = (int)n64;
-    const bool hdb = min_pts >= 1, wspd_form = C.method == WM_METHOD_GFK || C.method == WM_METHOD_NAIVE;
+    // (a batch has no such form: the full WSPD would pair its instances with one another)
+    const bool hdb = min_pts >= 1, wspd_form = target < 0 && (C.method == WM_METHOD_GFK || C.method == WM_METHOD_NAIVE);
     if (hdb && n >= 1 << 28) {   // (its workspace alone would exceed the device)
         set_detail("HDBSCAN* of 2^28 points or more does not fit the device%s (n=%lld)", "", n64);
         return WM_ENOMEM;
