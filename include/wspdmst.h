@@ -152,8 +152,9 @@ typedef struct {
     int64_t getpairs_launches;     /* number of GetPairs step launches                  */
     int64_t getpairs_visits;       /* node pairs examined by the GetPairs traversals     */
     int64_t getrho_visits;         /* node pairs examined by the GetRho traversals       */
-    int64_t bccp_dual_evals;       /* distance evaluations in the nearest-component search and
-                                      in the pruned dual-tree BCCP                        */
+    int64_t bccp_dual_evals;       /* distance evaluations of the kernels that ms_bccp_dual
+                                      times (bccp_evals also counts the nearest-component
+                                      rounds' exact searches among ties)                  */
     int64_t rho_shrinks;           /* times a round lowered rho_hi to fit its edge batch  */
     int64_t max_pending_pairs;     /* peak node pairs pending in a WSPD traversal         */
     int64_t bccp_pairs_below;      /* retrieved pairs whose BCCP lay below the round's

@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(kWalkThreads, search_blocks(D, HDB, F64, EXACT
     const unsigned long long all_ev = warp_sum_u64(n_ev);
     if (lane == 0 && all_ev) {
         atomicAdd(a.stat + 1, all_ev);
-        atomicAdd(a.stat + 6, all_ev);
+        if (!EXACT) atomicAdd(a.stat + 6, all_ev);   // (the searches that are timed)
     }
     if (EXACT) {
         err_flush(a, err);
@@ -475,7 +475,7 @@ __global__ void __launch_bounds__(kWalkThreads) nc_long_kernel(TravArgs a, NcArg
     n_ev = warp_sum_u64(n_ev);
     if (lane == 0 && n_ev) {
         atomicAdd(a.stat + 1, n_ev);
-        atomicAdd(a.stat + 6, n_ev);
+        if (!EXACT) atomicAdd(a.stat + 6, n_ev);
     }
     if (EXACT) {
         err_flush(a, err);
