@@ -18,6 +18,7 @@
 // it lies in the Euler interval of the deeper endpoint.  The reachability plot is the in-order
 // sequence of leaves, obtained by list ranking an Euler tour of the ordered dendrogram; the bar
 // of leaf i is the height of the in-order internal node before it.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -206,17 +207,14 @@ __device__ __forceinline__ bool ct_hook(const Contract &c, int v)
     return root;
 }
 
-__device__ __forceinline__ int ct_root(const Contract &c, int v, int limit)
+// the next level's vertices of those that hook below a root
+__device__ __forceinline__ void ct_next(const Contract &c, int off, int nv)
 {
-    int x = v;
-    for (int it = 0; it < limit; ++it) {
-        const int p = *(volatile int *)(c.hook + x);
-        if (p == x) break;
-        const int g = *(volatile int *)(c.hook + p);
-        if (g != p) *(volatile int *)(c.hook + x) = g;   // path halving (the forest is static)
-        x = p;
+    link_to_roots(c.hook, nv, [off](int t) { return off + t; });
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nv; t += gridDim.x * blockDim.x) {
+        const int x = *(volatile int *)(c.hook + off + t);
+        if (x != off + t) c.next[off + t] = *(volatile int *)(c.next + x);
     }
-    return x;
 }
 
 // a contracted edge notes its component; another one moves to the next level
@@ -256,14 +254,7 @@ __global__ void ct_hook_kernel(Contract c, int level, int *bad)
     }
 }
 
-__global__ void ct_next_kernel(Contract c, int level)
-{
-    const int m = c.nv[level], off = c.off[level];
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < m; t += gridDim.x * blockDim.x) {
-        const int x = ct_root(c, off + t, m);
-        if (x != off + t) c.next[off + t] = *(volatile int *)(c.next + x);
-    }
-}
+__global__ void __launch_bounds__(256) ct_next_kernel(Contract c, int level) { ct_next(c, c.off[level], c.nv[level]); }
 
 __global__ void ct_edge_kernel(Contract c, int level)
 {
@@ -303,10 +294,7 @@ __global__ void __launch_bounds__(1024) ct_tail_kernel(Contract c, int level, in
             }
         }
         __syncthreads();
-        for (int t = threadIdx.x; t < nv; t += 1024) {
-            const int x = ct_root(c, off + t, nv);
-            if (x != off + t) c.next[off + t] = *(volatile int *)(c.next + x);
-        }
+        ct_next(c, off, nv);
         __syncthreads();
         for (int b0 = 0; b0 < m; b0 += 1024) {
             const int t = b0 + threadIdx.x;
@@ -579,7 +567,7 @@ int dendrogram_impl(const EdgeK *E, int n, int start, int key_squared, wm_dnode 
         const int gl = grid_for(std::max(1, n >> level), 256);
         launch(ct_lightest_kernel, gl, 256, 0, st, c, level);
         launch(ct_hook_kernel, gl, 256, 0, st, c, level, bad);
-        launch(ct_next_kernel, gl, 256, 0, st, c, level);
+        launch(ct_next_kernel, std::min(gl, num_sms() * kLinkBlocks), 256, 0, st, c, level);
         launch(ct_edge_kernel, gl, 256, 0, st, c, level);
     }
     launch(ct_tail_kernel, 1, 1024, 0, st, c, level, bad);
