@@ -794,33 +794,25 @@ __device__ __forceinline__ void merge_roots(const TravArgs &a, const NcArgs &b, 
     }
 }
 
-// After the links: every root of the round is brought close to its component's root; the roots left are
-// collected and their slots reset for the next round.
+// After the links: every root of the round is linked to its component's root; the roots left are collected and
+// their slots reset for the next round.
 __device__ __forceinline__ void collect_roots(const NcArgs &b, int cur, int *sh)
 {
     if (held(b, 3)) return;
     const int m = b.cnt[cnt_roots(cur)];
+    const int *roots = b.roots[cur];
+    link_to_roots(b.par, m, [roots](int t) { return roots[t]; });
     for (int b0 = blockIdx.x * blockDim.x; b0 < m; b0 += gridDim.x * blockDim.x) {
         const int t = b0 + threadIdx.x;
         bool stays = false;
         int i = 0;
         if (t < m) {
-            i = b.roots[cur][t];
-            int x = i;
-            for (int it = 0; it < b.n; ++it) {
-                const int p = *(volatile int *)(b.par + x);
-                if (p == x) break;
-                const int g = *(volatile int *)(b.par + p);
-                if (g != p) *(volatile int *)(b.par + x) = g;   // path halving (the forest is static)
-                x = p;
-            }
-            stays = x == i;
+            i = roots[t];
+            stays = *(volatile int *)(b.par + i) == i;
             if (stays) {
                 b.S[i] = b.cap_bits;
                 b.bhi[i] = ~0ull;
                 b.blo[i] = ~0ull;
-            } else {
-                *(volatile int *)(b.par + i) = x;
             }
         }
         const int slot = block_append(b.cnt + cnt_roots(cur ^ 1), stays ? 1 : 0, sh);
@@ -828,8 +820,7 @@ __device__ __forceinline__ void collect_roots(const NcArgs &b, int cur, int *sh)
     }
 }
 
-// The root above x.  collect_roots leaves every root of the round pointing at its new root or, where a
-// concurrent walk halved the path once more, at an ancestor below it.
+// The root above x: x itself or, for a root that linked in this round, where collect_roots has linked it.
 __device__ __forceinline__ int root_of(const int *__restrict__ par, int x, int n)
 {
     for (int it = 0; it < n; ++it) {
@@ -972,7 +963,7 @@ __global__ void nc_merge_kernel(TravArgs a, NcArgs b, int cur, EdgeK *out, int o
     merge_roots(a, b, cur, out, out_cap, sh);
 }
 
-__global__ void nc_roots_kernel(NcArgs b, int cur)
+__global__ void __launch_bounds__(256) nc_roots_kernel(NcArgs b, int cur)
 {
     __shared__ int sh[32];
     collect_roots(b, cur, sh);
@@ -1108,7 +1099,7 @@ int rounds(NcCall &C, TravArgs &a, NcArgs &b)
             } else {
                 launch(nc_low_kernel, g, 256, 0, st, b);
                 launch(nc_merge_kernel, g, 256, 0, st, a, b, cur, C.out, n - 1);
-                launch(nc_roots_kernel, g, 256, 0, st, b, cur);
+                launch(nc_roots_kernel, std::min(g, num_sms() * kLinkBlocks), 256, 0, st, b, cur);
                 launch(nc_relabel_kernel, gt, 256, 0, st, b, S, roots, sums);
                 const int rc = scan_exclusive_i32(sums, sums, tiles, nullptr, st, ar);
                 if (rc) return rc;

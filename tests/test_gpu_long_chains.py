@@ -7,7 +7,7 @@ import numpy as np
 import pytest
 
 import paper_2104_01126_gb300 as wm
-from gpu_common import require_gpu, torch
+from gpu_common import require_gpu, to_np, torch
 
 N = 1_000_000
 
@@ -35,4 +35,29 @@ def test_single_linkage_of_a_path(weights):
     first, rest = (r["left"], r["right"]) if weights != "falling" else (r["right"], r["left"])
     assert np.array_equal(first[1:], N + i[:-1])                        # each merge holds the one before
     assert np.array_equal(rest, i + 1 if weights != "falling" else (N - 2) - i)
+    assert took < 20 * usual
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("min_pts", [1, 4])
+def test_points_whose_gaps_grow(min_pts):
+    # every point's nearest neighbour is the one before it: the first round links all of them
+    require_gpu()
+    x = np.zeros((N, 2))
+    x[:, 0] = np.cumsum(np.arange(N))   # gaps 1, 2, ..., N - 1
+    p = np.random.default_rng(2).permutation(N)
+    t, u = torch.from_numpy(x[p]).cuda(), torch.from_numpy(np.random.default_rng(3).random((N, 2))).cuda()
+    run = wm.emst if min_pts == 1 else lambda y, **kw: wm.hdbscan(y, min_pts=min_pts, **kw)
+    usual, _ = _seconds(lambda: run(u, precision="fp64"))
+    took, r = _seconds(lambda: run(t, precision="fp64"))
+    at = np.argsort(p)   # the row of each point along the line
+    if min_pts == 1:
+        assert np.array_equal(to_np(r["u"]), np.minimum(at[:-1], at[1:]))
+        assert np.array_equal(to_np(r["v"]), np.maximum(at[:-1], at[1:]))
+        assert np.array_equal(to_np(r["w"]), np.arange(1.0, N))
+    else:
+        pad = np.concatenate([np.full(3, -np.inf), x[:, 0], np.full(3, np.inf)])
+        near = np.abs(np.lib.stride_tricks.sliding_window_view(pad, 7) - x[:, :1])   # three points on either side
+        cd = np.partition(near, min_pts - 1, axis=1)[:, min_pts - 1]
+        assert np.array_equal(to_np(r["cd"])[at], cd)
     assert took < 20 * usual
