@@ -53,17 +53,20 @@ namespace {
 // from 8.0 to 7.7 in 2-D, left it in 5-D (31 ms) and cost 13 % in 7-D; 2 entries were slower everywhere.
 __host__ __device__ constexpr int list_len(int D) { return D <= 3 ? 6 : 4; }
 
-// A query that has evaluated kLongEvals points (above 2x10^6 points: a 1024th of them) and is still walking is
-// handed to warps that share a scan of all points: the centre of a sphere of points is as far from all of
-// them, and its walk visits every node on one lane while the GPU waits (50,000 points and their centre: 83 ms
-// a call, of which 81 on that lane; 5.0 now, 3.3 with a limit of 1024, which 7-D sets reach in ordinary
-// walks: 2 % slower).  While at most kLongMax queries and about kLongWork points' evaluations are waiting, such
-// a query is handed over at once; one that comes later walks on, and is handed over all the same when it has
-// evaluated a kLongPart-th of all points, since it will hardly stop before the rest.  A query is handed over
-// at most once a search, and the list has a place for every query of the search: its counter cannot pass n.
-// Such queries are rare, so the scan is launched when the host has seen one (launched every time it cost 10^4
-// points 6 %), for kLongMax of them at a time; until then the kernels behind the search hold back (held).
-constexpr int kLongEvals = 2048, kLongMax = 512, kLongPart = 16, kLongChunk = 2048, kLongChunks = 1024, kLongMinPoints = 8192;
+// A query that has looked at long_points points (above 10^6 or two: a 1024th of all) and is still walking is handed
+// to warps that share a scan of all points: the centre of a sphere of points is as far from all of them, and
+// its walk visits every node on one lane while the GPU waits (EMST of 50,000 points and their centre: 83 ms, of
+// which 81 on that lane; 3.2 now, FP64 form 142 and 4.5; with a limit of 2048 5.0 and 7.6.  7-D sets reach 1024 in
+// ordinary walks, and were 2 % slower with it).  Points count whether they are evaluated or only bounded: in the
+// FP64 form a walk that bounded most of 10^6 points went unnoticed (36 -> 16 ms).  While at most kLongMax
+// queries and about kLongWork points' evaluations are waiting, such a query is handed over at once; one that
+// comes later walks on, and is handed over all the same when it has looked at a kLongPart-th of all points
+// (twice the limit at least), since it will hardly stop before the rest.  A query is handed over at most once a
+// search, and the list has a place for every query of the search: its counter cannot pass n.  Such queries are
+// rare, so the scan is launched when the host has seen one (launched every time it cost 10^4 points 6 %), for
+// kLongMax of them at a time; until then the kernels behind the search hold back (held).
+constexpr int kLongMax = 512, kLongPart = 16, kLongChunk = 512, kLongChunks = 1024;
+constexpr int long_points(int D) { return D <= 5 ? 1024 : 2048; }
 constexpr long long kLongWork = 1 << 26;
 
 // Counters.  Those that a round starts from zero lie side by side: an even one's are [kCntEven, kCntEdges), an
@@ -108,8 +111,8 @@ struct NcArgs {
     // queries handed to the scan of all points (chunks: parts of the points; 0: no hand-over): positions in
     // amb, which the search leaves alone, or of the exact search in act
     int chunks, long_max;
-    unsigned long_evals, long_most;   // evaluations after which a query is handed over: while fewer than
-                                      // long_max are waiting, in any case
+    unsigned long_few, long_most;   // points after which a query is handed over: while fewer than long_max
+                                    // are waiting, in any case
     int guard;                 // 1: hold back while queries of the search wait for the scan, 2: of the exact one
     int *long_done;            // [kLongMax] parts finished
     float *long_s;             // [kLongMax][chunks][K] a part's list
@@ -185,7 +188,7 @@ __global__ void __launch_bounds__(kWalkThreads, search_blocks(D, HDB, F64, EXACT
     KMin best{~0ull, ~0ull};
     float lim = 0.f, pb = 0.f;   // a candidate screens below lim; a node is skipped when its lower bound
                                  // exceeds pb (it bounds the exact weight, within 2^-19 of the screened one)
-    unsigned ev = 0;
+    unsigned ev = 0;   // points of the buckets scanned
     auto begin = [&](int t) {
         i = EXACT ? b.amb[t] : b.first ? t : b.act[t];
         load_row<S>(X.rows, i, q);
@@ -227,7 +230,7 @@ __global__ void __launch_bounds__(kWalkThreads, search_blocks(D, HDB, F64, EXACT
                 if (F64) {
                     // (FP64 is slow enough that even a point is first tried against the bound)
                     take = take && point_bound<D>(q, x, 2.f * a.delta32) <= pb;
-                    ev += take;
+                    n_ev += take;
                 } else {
                     w[p] = row_dist<D>(q, x);
                     if (HDB) {
@@ -240,7 +243,7 @@ __global__ void __launch_bounds__(kWalkThreads, search_blocks(D, HDB, F64, EXACT
                 if (take) todo |= 1u << p;
             }
         }
-        if (!F64) ev += (unsigned)sz;
+        ev += (unsigned)sz;
         const float was = sl[0];
         while (todo) {
             const int p = __ffs(todo) - 1;
@@ -286,7 +289,7 @@ __global__ void __launch_bounds__(kWalkThreads, search_blocks(D, HDB, F64, EXACT
             }
         }
         pb = lim * (1.0f + 1.0f / 131072.0f);
-        if (ev >= b.long_evals && (ev & 255u) < 8u) {   // (a bucket adds at most 8)
+        if (ev >= b.long_few && (ev & 255u) < 8u) {   // (a bucket adds at most 8)
             int *waiting = b.cnt + (EXACT ? kCntLongExact : kCntLong);
             if (ev >= b.long_most || *(volatile int *)waiting < b.long_max) {
                 (EXACT ? b.act : b.amb)[atomicAdd(waiting, 1)] = i;
@@ -295,7 +298,7 @@ __global__ void __launch_bounds__(kWalkThreads, search_blocks(D, HDB, F64, EXACT
         }
     };
     auto finish = [&] {
-        n_ev += ev;
+        if (!F64) n_ev += ev;
         if (pb < 0.f) return;   // handed over
         if (EXACT) {
             if (best.hi < b.cap64) {
@@ -1177,10 +1180,11 @@ int nearest_component_rounds(NcCall &C, TravArgs &a)
     b.near = b.cand_c;   // (read before the candidates are written)
     a.overflow = (unsigned *)b.cnt + kCntError;
     b.n = n;
-    b.long_evals = ~0u;          // (of few points even a walk of all is short)
-    if (n >= kLongMinPoints) {
-        b.long_evals = (unsigned)std::max(kLongEvals, n / 1024);
-        b.long_most = std::max(b.long_evals, (unsigned)n / kLongPart);
+    b.long_few = ~0u;            // (of few points even a walk of all is short)
+    const int few = long_points(walk_dim(a.d));
+    if (n >= 2 * few) {
+        b.long_few = (unsigned)std::max(few, n / 1024);
+        b.long_most = std::max(2 * b.long_few, (unsigned)n / kLongPart);
         b.chunks = std::min(kLongChunks, n / kLongChunk);
         b.long_max = (int)std::min<long long>(kLongMax, std::max<long long>(4, kLongWork / n));
         b.long_done = ar.get<int>(kLongMax);

@@ -44,3 +44,19 @@ def test_limit_that_follows_the_number_of_points(n, inner):
         ref = wm.emst(x, return_stats=True)
     assert ref["stats"].getpairs_visits > 0
     assert_same_tree({k: to_np(got[k]) for k in "uvw"}, {k: to_np(ref[k]) for k in "uvw"})
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("min_pts", [1, 10])
+@pytest.mark.parametrize("n,d", [(2_047, 3), (2_048, 3), (3_001, 5), (4_096, 8), (4_097, 8)])
+def test_smallest_sizes_that_hand_over(n, d, min_pts, precision):
+    # up to 4096 points the steps behind the search are one block's: they hold back in the same way
+    require_gpu()
+    x = _ball_in_sphere(n, 40, d, 1e-6, n + d, "f8")
+    if min_pts == 1:
+        got, ref = wm.emst(x, precision=precision), oracle.emst_at_scale(x)
+    else:
+        got, ref = wm.hdbscan(x, min_pts=min_pts, precision=precision), oracle.hdbscan_at_scale(x, min_pts, 0)
+        assert np.array_equal(to_np(got["cd"]), ref["cd"])
+    assert_same_tree({k: to_np(got[k]) for k in "uvw"}, ref)
