@@ -53,6 +53,13 @@ namespace {
 // from 8.0 to 7.7 in 2-D, left it in 5-D (31 ms) and cost 13 % in 7-D; 2 entries were slower everywhere.
 __host__ __device__ constexpr int list_len(int D) { return D <= 3 ? 6 : 4; }
 
+// A point with R >= S cannot lower S.  Where its list is full and all of one band besides, the next list would be too,
+// and the point is left to the exact search at once: such are lattice points, whose 2 D nearest neighbours a list
+// of list_len(D) does not hold above 3 dimensions.  (EMST of a 7-D lattice of 280,000 points 6.3 -> 4.9 ms, FP64 form
+// 8.6 -> 6.1; of a 5-D one of 100,000 2.4 -> 2.1 and 2.7 -> 2.3.  In 3-D lists get room as neighbours join the component,
+// and the same rule took 2.0 -> 2.6 ms.)
+__host__ __device__ constexpr bool marks_ties(int D) { return list_len(D) < 2 * D; }
+
 // A query that has looked at long_points points (above 10^6 or two: a 1024th of all) and is still walking is handed
 // to warps that share a scan of all points: the centre of a sphere of points is as far from all of them, and
 // its walk visits every node on one lane while the GPU waits (EMST of 50,000 points and their centre: 83 ms, of
@@ -92,7 +99,8 @@ struct NcArgs {
     unsigned long long *bhi, *blo;   // per root: K-minimum outgoing edge
     float *ls;                 // [list_len][n] list weights, ascending
     int *lj;                   // [list_len][n] list positions (-1: none)
-    float *R;                  // every point outside the component and the list screens at >= R
+    float *R;                  // every point outside the component and the list screens at >= |R|; the sign marks
+                               // a full list of one band (see marks_ties)
     unsigned char *hd;         // first list entry that may lie outside the component
     float *low;                // smaller of the head's weight (no head: +inf) and R
     int *roots[2];             // the roots of this round and the next
@@ -121,6 +129,8 @@ struct NcArgs {
     int first;                 // first search: components are single points, nothing is pruned by S
     int n;
 };
+
+__device__ __forceinline__ bool all_tied(float R) { return __float_as_int(R) < 0; }
 
 // true while queries that were handed over wait for the scan of all points
 __device__ __forceinline__ bool held(const NcArgs &b, int what)
@@ -249,10 +259,11 @@ __global__ void __launch_bounds__(kWalkThreads, search_blocks(D, HDB, F64, EXACT
             const int p = __ffs(todo) - 1;
             todo &= todo - 1;
             float v;
+            double x2 = 0.0;
             if (F64) {
-                float x[S];
-                load_row<S, kStream>(X.rows, j0 + p, x);
-                v = screen_dist<D, S, F64>(a.x64, n, a.d, X.rows, i, j0 + p, q, x);
+                x2 = EXACT ? tie_dist64<D, S>(a.x64, n, a.d, X.rows, i, j0 + p)
+                           : walk_dist64<D, S>(a.x64, n, a.d, X.rows, i, j0 + p);
+                v = __double2float_rn(x2);
                 if (HDB) {
                     const float cdm = fmaxf(qcd, a.cd32[j0 + p]);
                     if (proven_repair(a, v, cdm)) continue;
@@ -266,7 +277,7 @@ __global__ void __launch_bounds__(kWalkThreads, search_blocks(D, HDB, F64, EXACT
             }
             if (EXACT) {
                 const int j = j0 + p;
-                double x2 = walk_dist64<D, S>(a.x64, n, a.d, X.rows, i, j);
+                if (!F64) x2 = tie_dist64<D, S>(a.x64, n, a.d, X.rows, i, j);
                 if (HDB) x2 = pos_dmax(x2, pos_dmax(a.cd64[i], a.cd64[j]));
                 if (!F64) note_err(v, x2, err);
                 kmin_update(best, x2, a.pid[i], a.pid[j]);
@@ -316,7 +327,9 @@ __global__ void __launch_bounds__(kWalkThreads, search_blocks(D, HDB, F64, EXACT
                 b.ls[(size_t)k * n + i] = sl[k];
                 b.lj[(size_t)k * n + i] = sj[k];
             }
-            b.R[i] = lim;
+            // (one band, and more of it may have been turned away)
+            const bool tied = marks_ties(D) && sl[K - 1] < INFINITY && sl[K - 1] <= screen_threshold(sl[0], a);
+            b.R[i] = tied ? -lim : lim;
             b.low[i] = fminf(sl[0], lim);
             b.hd[i] = 0;
         }
@@ -404,7 +417,7 @@ __global__ void __launch_bounds__(kWalkThreads) nc_long_kernel(TravArgs a, NcArg
             }
             if (!(v < now)) continue;
             if (EXACT) {
-                double x2 = walk_dist64<D, S>(a.x64, n, a.d, b.rows, i, j);
+                double x2 = tie_dist64<D, S>(a.x64, n, a.d, b.rows, i, j);
                 if (HDB) x2 = pos_dmax(x2, pos_dmax(a.cd64[i], a.cd64[j]));
                 if (!F64) note_err(v, x2, err);
                 kmin_update(best, x2, a.pid[i], a.pid[j]);
@@ -565,7 +578,7 @@ __device__ __forceinline__ void refresh_points(const TravArgs &a, const NcArgs &
             const float s = h < b.K ? b.ls[(size_t)h * n + i] : INFINITY;
             if (h != h0) {
                 b.hd[i] = (unsigned char)h;
-                b.low[i] = fminf(s, b.R[i]);
+                b.low[i] = fminf(s, fabsf(b.R[i]));
             }
             if (h < b.K) s_min(b.S, c, s);
         }
@@ -627,7 +640,7 @@ __device__ __forceinline__ bool settled(const TravArgs &a, const NcArgs &b, int 
 // (Eight points per thread between two appends: an append per 256 points, which most of those have a point
 // for, made the pass wait for one counter, 120 us for 10^7 points against 37 now.  With the list, this pass
 // and the one that picks take 0.67 ms a call where two passes over all points took 1.40.)
-template <bool HDB>
+template <bool HDB, bool MARK>
 __device__ __forceinline__ void active_points(const TravArgs &a, const NcArgs &b, int *sh)
 {
     const int n = a.n, items = 8 * blockDim.x;
@@ -652,7 +665,10 @@ __device__ __forceinline__ void active_points(const TravArgs &a, const NcArgs &b
         for (int t = 0; t < 8; ++t) {
             if (!((near >> t) & 1u)) continue;
             const int i = (int)(b0 + t * blockDim.x + threadIdx.x);
-            if (b.R[i] <= T[t] && !(HDB && settled(a, b, i, c[t]))) on |= 1u << t;
+            const float R = b.R[i];
+            if (fabsf(R) <= T[t] && !(MARK && all_tied(R) && fabsf(R) >= __uint_as_float(b.S[c[t]])) &&
+                !(HDB && settled(a, b, i, c[t])))
+                on |= 1u << t;
         }
         if (!__syncthreads_or(near)) continue;
         int slot = block_append(b.cnt + kCntNear, __popc(near), sh);
@@ -678,7 +694,7 @@ __device__ __forceinline__ void pick_points(const TravArgs &a, const NcArgs &b, 
             i = b.first ? t : b.near[t];
             const int c = b.lab[i];
             const float T = screen_threshold(__uint_as_float(b.S[c]), a);
-            exact = b.R[i] <= T;
+            exact = fabsf(b.R[i]) <= T;
             if (HDB && exact) exact = !settled(a, b, i, c);
             const int h = b.hd[i];
             has = !exact && h < b.K && b.ls[(size_t)h * n + i] <= T;
@@ -937,11 +953,11 @@ __device__ __forceinline__ void node_labels(int Ns, int S, const int2 *__restric
 template <int D, bool HDB, bool F64>
 __global__ void nc_refresh_kernel(TravArgs a, NcArgs b) { refresh_points<D, HDB, F64>(a, b); }
 
-template <bool HDB>
+template <bool HDB, bool MARK>
 __global__ void nc_active_kernel(TravArgs a, NcArgs b)
 {
     __shared__ int sh[32];
-    active_points<HDB>(a, b, sh);
+    active_points<HDB, MARK>(a, b, sh);
 }
 
 template <bool HDB>
@@ -997,7 +1013,7 @@ __global__ void __launch_bounds__(kSmallThreads) nc_small_front_kernel(TravArgs 
     __shared__ int sh[32];
     refresh_points<D, HDB, F64>(a, b);
     __syncthreads();
-    active_points<HDB>(a, b, sh);
+    active_points<HDB, marks_ties(D)>(a, b, sh);
 }
 
 template <int D, bool HDB, bool F64>
@@ -1082,7 +1098,7 @@ int rounds(NcCall &C, TravArgs &a, NcArgs &b)
                 launch(nc_small_front_kernel<D, HDB, F64>, 1, kSmallThreads, 0, st, a, b);
             } else {
                 launch(nc_refresh_kernel<D, HDB, F64>, g, 256, 0, st, a, b);
-                launch(nc_active_kernel<HDB>, gt, 256, 0, st, a, b);
+                launch(nc_active_kernel<HDB, marks_ties(D)>, gt, 256, 0, st, a, b);
             }
         }
         auto middle = [&] {
