@@ -48,20 +48,22 @@ struct KnnArgs {
     int *slow_cnt;
     int *slow2;          // queries left for the full scan
     int *slow2_cnt;
-    unsigned long_points; // a walk that has looked at more points than this is handed to the full scan,
-    int *long_cnt;        // kKnnLongMax of them at most
+    unsigned long_evals; // a walk that has evaluated more points than this is handed to the full scan,
+    int *long_cnt;       // kKnnLongMax of them at most
     int *next_group;     // dispenser of 32-query groups
     int *err;            // set when a traversal stack would overflow (an internal error)
     unsigned long long *stat;   // [0] evals, [1] fp64 rechecks, [2] bits of the largest relative
                                 //     error of a screened k-th value against the exact one
 };
 
-// FP64 form: a walk that has looked at a 16th of all points (knn_long_points at least) is an outlier, such as the
+// FP64 form: a walk that has evaluated a 32nd of all points (and knn_long_evals) is an outlier, such as the
 // centre of a sphere of points, which visits every node on one lane while the GPU waits: it goes to the full
-// scan's blocks.  Where that is what every walk does (high dimension), the first four per SM are scanned.
-// (HDBSCAN* of 50,000 points on a sphere and their centre 68 -> 6.9 ms, of 10,000 14.6 -> 4.5, with the searches' own
+// scan's blocks.  Where that is what every walk does (high dimension), the first four per SM are scanned.  Up to 5
+// dimensions ordinary walks stay far below 2048 evaluations at minPts 10; above, and with long lists, they do not
+// (with 4096 in 7-D, 60,000 points at minPts 256 took 89 ms instead of 60).
+// (HDBSCAN* of 50,000 points on a sphere and their centre 68 -> 5.5 ms, of 10,000 14.6 -> 4.5, with the searches' own
 // hand-over.  The FP32 walk is four times as fast per point, and the test cost every call 2 %.)
-constexpr unsigned knn_long_points(int D) { return D <= 3 ? 2048 : 4096; }
+inline unsigned knn_long_evals(int D, int n, int k) { return std::max(D <= 5 ? std::min(2048 * (1 + k / 32), 16384) : 16384, n / 32); }
 constexpr int kKnnLongMax = 608;
 
 // -------------------------------------------------------------------------- thread per query
@@ -120,8 +122,7 @@ __global__ void __launch_bounds__(kWalkThreads, F64 ? 1 : D <= 3 ? 8 : 6) knn_wa
                 }
             }
         }
-        ev += (unsigned)sz;
-        n_ev += F64 ? __popc(todo) : sz;
+        ev += F64 ? __popc(todo) : (unsigned)sz;
         while (todo) {
             const int p = __ffs(todo) - 1;
             todo &= todo - 1;
@@ -172,16 +173,17 @@ __global__ void __launch_bounds__(kWalkThreads, F64 ? 1 : D <= 3 ? 8 : 6) knn_wa
             }
         }
         pb = screen_threshold(top, band) * (1.0f + 1.0f / 131072.0f);
-        if (F64 && ev > a.long_points) {
+        if (F64 && ev > a.long_evals) {
+            n_ev += ev;
+            ev = 0;
             if (*(volatile int *)a.long_cnt < kKnnLongMax && atomicAdd(a.long_cnt, 1) < kKnnLongMax) {
                 a.slow2[atomicAdd(a.slow2_cnt, 1)] = i;
                 pb = -1.f;   // nothing left to visit
-            } else {
-                ev = 0;
             }
         }
     };
     auto finish = [&] {
+        n_ev += ev;
         if (F64 && pb < 0.f) return;   // handed over
         if (cnt < k || !(out > screen_threshold(top, band))) {
             const int t = atomicAdd(a.slow_cnt, 1);
@@ -590,7 +592,7 @@ int core_distances(const Points &P, const SearchTree &X, int min_pts, bool fp64,
     a.err = cnts + 5;
     a.slow2_cnt = cnts + 7;
     a.long_cnt = cnts + 8;
-    a.long_points = std::max(knn_long_points(walk_dim(d)), (unsigned)n / 16);
+    a.long_evals = knn_long_evals(walk_dim(d), n, min_pts);
     cudaEvent_t k0, k1;
     cudaEventCreate(&k0);
     cudaEventCreate(&k1);
