@@ -1239,17 +1239,21 @@ static int prepare(Call &C, const void *pts, int64_t n, int32_t d, int32_t dtype
     return 0;
 }
 
+// share of the buckets that the FP32 copy blurs (SearchTree::coarse) above which the walks are FP64 ones
+constexpr double kCoarseShare = 1.0 / 16;
+
 // for the walks (n < 2^28)
 static int prepare_walk(Call &C, const void *pts, int64_t n, int32_t d, int32_t dtype, int32_t layout, Prepared &S)
 {
     WM_TRY(input_on_device(C, pts, n, d, dtype, S));
     Timer tt;
     WM_TRY(bad_coordinate(build_search_tree(S.src, (int)n, d, dtype, layout, S.P, S.X, C.ar, C.st, C.pin)));
-    // Where the FP32 copy of FP64 coordinates errs by more than a 128th of the points' spacing, most distances
-    // fall into one band of the screen and are evaluated twice: the plain FP64 walks answer such a call.
-    // (Uniform points in 3-D at an offset, FP32 screen / FP64 walks, ms: EMST of 10^5 at 10^3, error
-    // 0.0014 of the spacing, 2.0 / 2.2; of 5x10^4 at 10^5, 0.15 of it, 4.8 / 2.3; HDBSCAN* there 12.0 / 3.2.)
-    S.fp64 = C.precision == WM_PREC_FP64 || (double)S.P.delta * 128.0 > S.X.spacing;
+    // Where the FP32 copy of FP64 coordinates errs by more than a tenth or so of the points' spacing, most distances
+    // fall into one band of the screen and are evaluated twice; the plain FP64 walks answer a call with a share of such
+    // points.  (EMST of 3x10^5 Cauchy-distributed points in 5-D, whose farthest coordinates blur all others: FP32 screen
+    // 6100 ms, FP64 walks 8.2.  Of 5x10^6 variable-density points in 2-D, 1 in 30 of them in blobs below the copy's
+    // resolution: 11.4 and 17.8, so a few such points do not decide.)
+    S.fp64 = C.precision == WM_PREC_FP64 || S.X.coarse > kCoarseShare;
     C.stats.ms_build_tree += tt.ms();
     C.stats.tree_nodes = 2 * n - 1;   // down to single points; X stores those above its buckets
     C.stats.tree_depth = S.X.depth;

@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(kWalkThreads, search_blocks(D, HDB, F64, EXACT
                 bool take = p < sz && __float_as_int(x[S - 1]) != c;
                 if (F64) {
                     // (FP64 is slow enough that even a point is first tried against the bound)
-                    take = take && point_bound<D>(q, x, 2.f * a.delta32) <= pb;
+                    take = take && point_bound<D>(q, x, row_error(a.delta32)) <= pb;
                     n_ev += take;
                 } else {
                     w[p] = row_dist<D>(q, x);
@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(kWalkThreads) nc_long_kernel(TravArgs a, NcArg
             load_row<S>(b.rows, j, x);
             if (__float_as_int(x[S - 1]) == c) continue;
             const float now = EXACT ? lim : sl[K - 1];
-            if (F64 && point_bound<D>(q, x, 2.f * a.delta32) > now * (1.0f + 1.0f / 131072.0f)) continue;
+            if (F64 && point_bound<D>(q, x, row_error(a.delta32)) > now * (1.0f + 1.0f / 131072.0f)) continue;
             float v = screen_dist<D, S, F64>(a.x64, n, a.d, b.rows, i, j, q, x);
             ++n_ev;
             if (HDB) {

@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(kWalkThreads, F64 ? 1 : D <= 3 ? 8 : 6) knn_wa
                 load_row<S, kStream>(X.rows, j, x);
                 if (F64) {
                     // (FP64 is slow enough that even a point is first tried against the bound)
-                    if (p < sz && point_bound<D>(q, x, 2.f * band.delta32) <= pb) todo |= 1u << p;
+                    if (p < sz && point_bound<D>(q, x, row_error(band.delta32)) <= pb) todo |= 1u << p;
                 } else {
                     s[p] = row_dist<D>(q, x);
                     if (p < sz) {
@@ -370,12 +370,13 @@ __device__ inline double any_dist64(const double *__restrict__ x64, const float 
     return s;
 }
 
-// rigorous lower bound of any_dist64 from the rows, whose coordinates err by at most delta2 together
-__device__ inline float any_bound(const float *__restrict__ rows, int S, int d, int i, int j, float delta2)
+// rigorous lower bound of any_dist64 from the rows (point_bound at run time)
+__device__ inline float any_bound(const float *__restrict__ rows, int S, int d, int i, int j, float rel)
 {
     float g = 0.f;
     for (int k = 0; k < d; ++k) {
-        const float t = fmaxf(fabsf(rows[(size_t)i * S + k] - rows[(size_t)j * S + k]) - delta2, 0.f);
+        const float q = rows[(size_t)i * S + k], x = rows[(size_t)j * S + k];
+        const float t = fmaxf(fmaf(-rel, fmaxf(fabsf(q), fabsf(x)), fabsf(q - x)), 0.f);
         g = fmaf(t, t, g);
     }
     return lower_w2(g);
@@ -385,7 +386,7 @@ __device__ inline float any_bound(const float *__restrict__ rows, int S, int d, 
 // end): each thread keeps the k smallest w2 of its strided share, the block merges the lists, then a
 // second scan collects every q with w2 <= cd2 as repair edges.  A point whose FP32 bound is beyond the
 // list costs no FP64 (whose rate is 1/64).
-__global__ void __launch_bounds__(256) knn_slow_kernel(KnnArgs a, const float *__restrict__ rows, int S, float delta2,
+__global__ void __launch_bounds__(256) knn_slow_kernel(KnnArgs a, const float *__restrict__ rows, int S, float rel,
                                                        const int *__restrict__ slow, int nslow,
                                                        int *extra_q, int *extra_p, double *extra_d, int *extra_cnt,
                                                        int extra_cap, int *tie_overflow)
@@ -401,7 +402,7 @@ __global__ void __launch_bounds__(256) knn_slow_kernel(KnnArgs a, const float *_
         int cnt = 0;
         float far = INFINITY;   // the list's largest value, rounded up, once it is full
         for (int j = tid; j < n; j += T) {
-            if (any_bound(rows, S, d, i, j, delta2) > far) continue;
+            if (any_bound(rows, S, d, i, j, rel) > far) continue;
             const double w = j == i ? 0.0 : any_dist64(a.x64, rows, S, n, d, i, j);
             if (cnt < k || w < lw[(k - 1) * T]) {
                 int pos = cnt < k ? cnt : k - 1;
@@ -434,7 +435,7 @@ __global__ void __launch_bounds__(256) knn_slow_kernel(KnnArgs a, const float *_
         }
         far = __double2float_ru(kth);
         for (int j = tid; j < n; j += T) {
-            if (j == i || any_bound(rows, S, d, i, j, delta2) > far) continue;
+            if (j == i || any_bound(rows, S, d, i, j, rel) > far) continue;
             const double w = any_dist64(a.x64, rows, S, n, d, i, j);
             if (w <= kth) {
                 const int s = atomicAdd(extra_cnt, 1);
@@ -674,7 +675,7 @@ int core_distances(const Points &P, const SearchTree &X, int min_pts, bool fp64,
         while (threads > 32 && (size_t)min_pts * threads * 8 > (size_t)kSlowSmemMax) threads >>= 1;
         cudaFuncSetAttribute(knn_slow_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSlowSmemMax);
         launch(knn_slow_kernel, std::min(nslow, num_sms() * 8), threads, (size_t)min_pts * threads * 8, st, a, X.rows, X.S,
-               2.f * P.delta, slow2, nslow, ex_q, ex_p, ex_d, cnts + 1, extra_cap, cnts + 2);
+               row_error(P.delta), slow2, nslow, ex_q, ex_p, ex_d, cnts + 1, extra_cap, cnts + 2);
     }
     // repair edges: one copy of each, weighted, in no particular order (each round takes those it needs)
     launch(rep_emit_kernel, grid_for(n, 256), 256, 0, st, a.rep_q, a.rep_d, a.rep_cnt, n, H.cd64, P.pid, rep, cnts + 3);

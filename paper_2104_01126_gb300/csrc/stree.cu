@@ -13,7 +13,6 @@
 // counting pass is needed) and accumulates the children's boxes on the way.  A node of at most M points
 // is finished by one block in shared memory, a warp per segment and level.
 #include <algorithm>
-#include <cmath>
 #include <cstring>
 
 #include "stree.cuh"
@@ -50,11 +49,25 @@ struct BuildState {
     int depth;        // levels below a block's root
     unsigned bad;     // non-finite or too large coordinate
     unsigned delta;   // bits of max |x64 - x32|
+    int buckets;      // of more than kBucket / 2 points, made by the blocks
+    int coarse;       // those whose widest extent is below kCoarse times that
 };
 
-// The boxes are widened by this multiple of the FP32 copy's error: the walks bound exact distances from the
-// rounded query (screened ones, of two points rounded alike, would need 1).
-constexpr float kWiden = 2.f;
+// A bucket's extent of two spacings or so, in units of the FP32 copy's largest error, below which most of its
+// points' distances are in one band of the screen.
+constexpr float kCoarse = 32.f;
+
+// Where the FP32 copy is inexact, a box side is widened so that it bounds exact distances from a rounded query:
+// rounding moves a coordinate of the box by half an ulp of the side's larger magnitude m at most, and the query
+// by as much, by twice that where it lies in the next binade, or, farther out, by 2^-23 of its distance from
+// the box, which the margin of lower_w2 holds.  (The widening follows the side, not the largest error of any
+// point: one coordinate of 10^6 would else blur all points within 0.1.)
+__device__ inline float widening(float lo, float hi)
+{
+    const unsigned e = __float_as_uint(fmaxf(fabsf(lo), fabsf(hi))) >> 23;   // biased exponent of m
+    const float half_ulp = __uint_as_float(e > 24 ? (e - 24) << 23 : 1u << max((int)e - 2, 0));
+    return __fmul_ru(3.f, half_ulp);
+}
 
 struct LNode {
     int node, b, e, dim;
@@ -155,16 +168,20 @@ __device__ inline void choose_split(const unsigned *acc, int d, int &dim, float 
     }
 }
 
-// box of a node row, widened by delta (see kWiden)
+// box of a node row, widened where the copy is inexact
 template <int S>
-__device__ inline void write_box(float *row, const unsigned *acc, int d, float delta)
+__device__ inline void write_box(float *row, const unsigned *acc, int d, bool inexact)
 {
     for (int k = 0; k < S; ++k) {
         float lo = 0.f, hi = 0.f;
         if (k < d) {
             lo = key2f(~acc[2 * k]);
             hi = key2f(acc[2 * k + 1]);
-            if (delta > 0.f) { lo = __fsub_rd(lo, delta); hi = __fadd_ru(hi, delta); }
+            if (inexact) {
+                const float w = widening(lo, hi);
+                lo = __fsub_rd(lo, w);
+                hi = __fadd_ru(hi, w);
+            }
         }
         row[box_lo(k)] = lo;
         row[box_hi(k)] = k == S - 1 ? __int_as_float(-1) : hi;
@@ -180,7 +197,7 @@ template <int S>
 __global__ void st_root_kernel(StArgs a)
 {
     BuildState &s = *a.state;
-    write_box<S>(a.nodes, a.root_acc, a.d, kWiden * __uint_as_float(s.delta));
+    write_box<S>(a.nodes, a.root_acc, a.d, s.delta != 0);
     a.range[0] = make_int2(0, a.n);
     a.parent[0] = -1;
     int dim;
@@ -322,7 +339,7 @@ __global__ void __launch_bounds__(1024) st_level_kernel(StArgs a, int level)
     __shared__ int sh[32];
     __shared__ int s_act, s_units;
     const int A = a.state->active, id0 = a.state->next_id, d = a.d, cur = level & 1;
-    const float delta = kWiden * __uint_as_float(a.state->delta);
+    const bool inexact = a.state->delta != 0;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (threadIdx.x == 0) { s_act = 0; s_units = 0; }
     __syncthreads();
@@ -347,7 +364,7 @@ __global__ void __launch_bounds__(1024) st_level_kernel(StArgs a, int level)
                 c.b = s ? nd.b + L : nd.b;
                 c.e = s ? nd.e : nd.b + L;
                 choose_split(box, d, c.dim, c.val);
-                write_box<S>(a.nodes + (size_t)c.node * 2 * S, box, d, delta);
+                write_box<S>(a.nodes + (size_t)c.node * 2 * S, box, d, inexact);
                 a.range[c.node] = make_int2(c.b, c.e);
                 a.parent[c.node] = nd.node;
                 const int m = c.e - c.b;
@@ -408,15 +425,20 @@ __global__ void __launch_bounds__(kStThreads) st_block_kernel(StArgs a)
     float *buf0 = (float *)st_smem, *buf1 = buf0 + (size_t)M * S;
     int4 *seg = (int4 *)(buf1 + (size_t)M * S);      // [2][M / 8]: first, end, node, dim
     float *sval = (float *)(seg + 2 * (M / 8));      // [2][M / 8]
-    __shared__ int s_entry, s_next, s_base;
+    __shared__ int s_entry, s_next, s_base, s_buckets, s_coarse;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, d = a.d;
-    const float delta = kWiden * __uint_as_float(a.state->delta);
+    const float delta = __uint_as_float(a.state->delta);
+    if (threadIdx.x == 0) s_buckets = s_coarse = 0;
     const int nsub = a.state->subs;
     while (true) {
         if (threadIdx.x == 0) s_entry = atomicAdd(&a.state->sub_next, 1);
         __syncthreads();
         const int entry = s_entry;
-        if (entry >= nsub) return;   // the same for every thread
+        if (entry >= nsub) {   // the same for every thread
+            if (threadIdx.x == 0 && s_coarse) atomicAdd(&a.state->coarse, s_coarse);
+            if (threadIdx.x == 0 && s_buckets) atomicAdd(&a.state->buckets, s_buckets);
+            return;
+        }
         const int4 E = a.sub[entry];
         const int node = E.x, gb = E.y, m = E.z & 0xffff, dim = (E.z >> 16) & 0x7fff;
         const float4 *src = (const float4 *)(a.buf[(unsigned)E.z >> 31] + (size_t)gb * S);
@@ -500,7 +522,11 @@ __global__ void __launch_bounds__(kStThreads) st_block_kernel(StArgs a)
                             cdim = k;
                             cval = lo + (hi - lo) * 0.5f;
                         }
-                        if (delta > 0.f) { lo = __fsub_rd(lo, delta); hi = __fadd_ru(hi, delta); }
+                        if (delta > 0.f) {
+                            const float w = widening(lo, hi);
+                            lo = __fsub_rd(lo, w);
+                            hi = __fadd_ru(hi, w);
+                        }
                         if (lane == (box_lo(k) & 31)) v[box_lo(k) >> 5] = lo;
                         if (lane == (box_hi(k) & 31)) v[box_hi(k) >> 5] = hi;
                     }
@@ -514,6 +540,10 @@ __global__ void __launch_bounds__(kStThreads) st_block_kernel(StArgs a)
                         a.parent[id] = g.z;
                     }
                     if (sz <= kBucket) {
+                        if (delta > 0.f && lane == 0 && sz > kBucket / 2) {   // (a few points have no extent)
+                            atomicAdd(&s_buckets, 1);
+                            if (ext < kCoarse * delta) atomicAdd(&s_coarse, 1);
+                        }
                         for (int t = lane; t < sz * C; t += 32)
                             ((float4 *)(a.buf[0] + (size_t)(gb + cb) * S))[t] = ((const float4 *)db)[cb * C + t];
                     } else if (lane == 0) {
@@ -591,7 +621,6 @@ int build(StArgs &a, SearchTree &X, Points &P, Arena &ar, cudaStream_t st, int *
     launch(st_block_kernel<S>, n > M ? num_sms() * per_sm : 1, kStThreads, smem, st, a);
     launch(st_finish_kernel<S>, grid_for(n, 256), 256, 0, st, a);
     cudaMemcpyAsync(pin, a.state, sizeof(BuildState), cudaMemcpyDeviceToHost, st);
-    cudaMemcpyAsync(pin + 64, a.root_acc, sizeof(unsigned) * 2 * a.d, cudaMemcpyDeviceToHost, st);
     if (cudaPeekAtLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) return WM_ECUDA;
     BuildState h;
     memcpy(&h, pin, sizeof h);
@@ -599,16 +628,7 @@ int build(StArgs &a, SearchTree &X, Points &P, Arena &ar, cudaStream_t st, int *
     float delta;
     memcpy(&delta, &h.delta, sizeof delta);
     P.delta = delta;
-    // side of the cube that a point would have to itself if all filled their box evenly
-    double log_vol = 0.0;
-    int dims = 0;
-    for (int k = 0; k < a.d; ++k) {
-        const double ext = (double)key2f((unsigned)pin[64 + 2 * k + 1]) - (double)key2f(~(unsigned)pin[64 + 2 * k]);
-        if (!(ext > 0.0)) continue;
-        log_vol += std::log(ext);
-        ++dims;
-    }
-    X.spacing = dims ? std::exp((log_vol - std::log((double)n)) / dims) : 0.0;
+    X.coarse = h.buckets > 0 ? (double)h.coarse / h.buckets : 0.0;
     X.Ns = h.next_id;
     X.depth = level + h.depth + 1;
     return 0;

@@ -32,7 +32,7 @@ struct SearchTree {
     int walk_blocks = 0;          // the largest grid the stacks are sized for
     int stack_cap = 0;            // entries of a thread's stack: one per tree level
     int depth = 0;                // levels
-    double spacing = 0.0;         // (volume of the points' box / n)^(1/d), over the dimensions with an extent
+    double coarse = 0.0;          // share of the buckets whose extent the FP32 copy's largest error blurs
 };
 
 // rows of d coordinates and one more slot
@@ -166,15 +166,19 @@ __device__ inline float screen_dist(const double *__restrict__ x64, int n, int d
     return F64 ? __double2float_rn(walk_dist64<D, S>(x64, n, d, rows, i, j)) : row_dist<D>(q, x);
 }
 
-// rigorous lower bound of the FP64 squared distance from two rows whose coordinates err by at most
-// delta2 together: the node bound of visit_children for a single point
+// Relative error of a coordinate difference of two rounded rows, for point_bound (0: exact rows): both round by
+// at most 2^-24 of the larger magnitude.
+__host__ __device__ constexpr float row_error(float delta) { return delta > 0.f ? 1.2e-7f : 0.f; }   // > 2^-23
+
+// rigorous lower bound of the FP64 squared distance from two rows: the node bound of visit_children for a
+// single point
 template <int D, int S>
-__device__ __forceinline__ float point_bound(const float (&q)[S], const float (&x)[S], float delta2)
+__device__ __forceinline__ float point_bound(const float (&q)[S], const float (&x)[S], float rel)
 {
     float g = 0.f;
 #pragma unroll
     for (int k = 0; k < D; ++k) {
-        const float t = fmaxf(fabsf(q[k] - x[k]) - delta2, 0.f);
+        const float t = fmaxf(fmaf(-rel, fmaxf(fabsf(q[k]), fabsf(x[k])), fabsf(q[k] - x[k])), 0.f);
         g = fmaf(t, t, g);
     }
     return lower_w2(g);
