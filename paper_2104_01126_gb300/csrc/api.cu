@@ -1252,7 +1252,8 @@ static int prepare_walk(Call &C, const void *pts, int64_t n, int32_t d, int32_t 
     // fall into one band of the screen and are evaluated twice; the plain FP64 walks answer a call with a share of such
     // points.  (EMST of 3x10^5 Cauchy-distributed points in 5-D, whose farthest coordinates blur all others: FP32 screen
     // 6100 ms, FP64 walks 8.2.  Of 5x10^6 variable-density points in 2-D, 1 in 30 of them in blobs below the copy's
-    // resolution: 11.4 and 17.8, so a few such points do not decide.)
+    // resolution: 11.4 and 17.8, so a few such points do not decide.  Points far from the origin do not come here: their
+    // copy is centred.)
     S.fp64 = C.precision == WM_PREC_FP64 || S.X.coarse > kCoarseShare;
     C.stats.ms_build_tree += tt.ms();
     C.stats.tree_nodes = 2 * n - 1;   // down to single points; X stores those above its buckets

@@ -6,7 +6,7 @@
 // no node below a bucket, so about 0.4 nodes per point are made instead of the 2 of the traversals' tree
 // (kdtree.cu), and each is written once, in the form the walks read.
 //
-// A point travels as one row: its FP32 coordinates and its input id, 16 bytes up to 3 dimensions and 32
+// A point travels as one row: its FP32 coordinates (less a centre, see centre()) and its input id, 16 bytes up to 3 dimensions and 32
 // up to 7, moved by vector loads and stores.  Nodes above M points are split level by level over the
 // whole GPU in one pass per level: a block takes 256 x R rows into registers, splits them with one pair
 // of atomics on the node's two ends (left points fill the range upwards, right points downwards, so no
@@ -49,9 +49,14 @@ struct BuildState {
     int depth;        // levels below a block's root
     unsigned bad;     // non-finite or too large coordinate
     unsigned delta;   // bits of max |x64 - x32|
+    unsigned delta_c; // the same of the centred copy
+    int centred;      // 1: it replaces the other
     int buckets;      // of more than kBucket / 2 points, made by the blocks
     int coarse;       // those whose widest extent is below kCoarse times that
 };
+
+constexpr size_t kStateBytes = 64;   // of a BuildState; root_acc follows, and one fill clears both
+static_assert(sizeof(BuildState) <= kStateBytes, "BuildState has outgrown its place");
 
 // A bucket's extent of two spacings or so, in units of the FP32 copy's largest error, below which most of its
 // points' distances are in one band of the screen.
@@ -66,7 +71,7 @@ __device__ inline float widening(float lo, float hi)
 {
     const unsigned e = __float_as_uint(fmaxf(fabsf(lo), fabsf(hi))) >> 23;   // biased exponent of m
     const float half_ulp = __uint_as_float(e > 24 ? (e - 24) << 23 : 1u << max((int)e - 2, 0));
-    return __fmul_ru(3.f, half_ulp);
+    return __fmul_ru(3.f + 1.0f / 1048576.0f, half_ulp);   // (more than 3, for centred copies)
 }
 
 struct LNode {
@@ -86,7 +91,7 @@ struct StArgs {
     int *unit_off[2];
     int *lr;                 // per active node: points placed left, right
     unsigned *acc;           // per active node: [2][d][2] box keys of the children (max of ~key, key)
-    unsigned *root_acc;      // [d][2] of all points
+    unsigned *root_acc;      // [d][2] of all points; then the same of the centred copy
     int4 *sub;               // block list: node, first point, size | dim << 16 | buffer << 31, split value
     int *pid, *pos;
     double *x64;
@@ -152,6 +157,64 @@ __global__ void __launch_bounds__(kStThreads) st_ingest_kernel(StArgs a)
         atomicMax(a.root_acc + threadIdx.x, sk[threadIdx.x]);
 }
 
+// The centre of a dimension whose FP64 coordinates lie far from 0 beside their range (timestamps, map coordinates),
+// else 0.  The rows then hold coordinates less that, rounded: distances are what the walks need, and the copy of
+// 1.6x10^9 + [0, 10^5] errs by 0.004 instead of 64.  (The FP64 subtraction adds 2^-53 of the result.)
+__device__ inline float centre(const StArgs &a, int k)
+{
+    const float lo = key2f(~a.root_acc[2 * k]), hi = key2f(a.root_acc[2 * k + 1]), mid = lo + (hi - lo) * 0.5f;
+    return fabsf(mid) > 4.f * (hi - lo) ? mid : 0.f;
+}
+
+// The centred copy, its error and box; nothing where no dimension needs it.
+template <int S>
+__global__ void __launch_bounds__(kStThreads) st_centre_kernel(StArgs a)
+{
+    __shared__ unsigned sk[2 * S];
+    const int d = a.d, lane = threadIdx.x & 31;
+    if (threadIdx.x < 2 * S) sk[threadIdx.x] = 0;
+    const bool away = threadIdx.x < d && centre(a, threadIdx.x) != 0.f, inexact = a.state->delta != 0 && !a.state->bad;
+    if (!__syncthreads_or(away && inexact)) return;   // the same for every block
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.state->centred = 1;
+    unsigned *acc = a.root_acc + 2 * S;
+    float dmax = 0.f, mn[S], mx[S], c[S];
+#pragma unroll
+    for (int k = 0; k < S; ++k) {
+        mn[k] = INFINITY;
+        mx[k] = -INFINITY;
+        c[k] = k < d ? centre(a, k) : 0.f;
+    }
+    for (int i = blockIdx.x * kStThreads + threadIdx.x; i < a.n; i += gridDim.x * kStThreads) {
+        float *row = a.buf[0] + (size_t)i * S;
+#pragma unroll
+        for (int k = 0; k < S - 1; ++k) {
+            if (k >= d) break;
+            const double x = __dsub_rn(src_coord(a, i, k), (double)c[k]);
+            const float v = __double2float_rn(x);
+            float e = __double2float_ru(fabs(x - (double)v));
+            if (c[k] != 0.f) e = __fmaf_ru(fabsf(v), 1.0f / 4503599627370496.0f, e);
+            dmax = fmaxf(dmax, e);
+            mn[k] = fminf(mn[k], v);
+            mx[k] = fmaxf(mx[k], v);
+            row[k] = v;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < S - 1; ++k) {
+        if (k >= d) break;
+        const unsigned lo = __reduce_max_sync(0xffffffffu, ~f2key(mn[k]));
+        const unsigned hi = __reduce_max_sync(0xffffffffu, f2key(mx[k]));
+        if (lane == 0) {
+            atomicMax(&sk[2 * k], lo);
+            atomicMax(&sk[2 * k + 1], hi);
+        }
+    }
+    for (int o = 16; o; o >>= 1) dmax = fmaxf(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+    if (lane == 0 && dmax > 0.f) atomicMax(&a.state->delta_c, __float_as_uint(dmax));
+    __syncthreads();
+    if (threadIdx.x < 2 * d && sk[threadIdx.x] > *(volatile unsigned *)(acc + threadIdx.x)) atomicMax(acc + threadIdx.x, sk[threadIdx.x]);
+}
+
 // the split of a box: its widest dimension, at the midpoint
 __device__ inline void choose_split(const unsigned *acc, int d, int &dim, float &val)
 {
@@ -197,6 +260,10 @@ template <int S>
 __global__ void st_root_kernel(StArgs a)
 {
     BuildState &s = *a.state;
+    if (s.centred) {
+        for (int k = 0; k < 2 * a.d; ++k) a.root_acc[k] = a.root_acc[2 * S + k];
+        s.delta = s.delta_c;
+    }
     write_box<S>(a.nodes, a.root_acc, a.d, s.delta != 0);
     a.range[0] = make_int2(0, a.n);
     a.parent[0] = -1;
@@ -593,12 +660,11 @@ int build(StArgs &a, SearchTree &X, Points &P, Arena &ar, cudaStream_t st, int *
     }
     a.lr = ar.get<int>(2 * (size_t)cap);
     a.acc = ar.get<unsigned>((size_t)cap * 4 * a.d);
-    a.root_acc = ar.get<unsigned>(2 * S);
     a.sub = ar.get<int4>(n > M ? n : 1);
     if (ar.failed) return WM_ENOMEM;
-    cudaMemsetAsync(a.state, 0, sizeof(BuildState), st);
-    cudaMemsetAsync(a.root_acc, 0, sizeof(unsigned) * 2 * S, st);
+    cudaMemsetAsync(a.state, 0, kStateBytes + sizeof(unsigned) * 4 * S, st);   // (and root_acc)
     launch(st_ingest_kernel<S>, grid_for(n, kStThreads, num_sms() * 8), kStThreads, 0, st, a);
+    if (a.dtype != WM_F32) launch(st_centre_kernel<S>, grid_for(n, kStThreads, num_sms() * 8), kStThreads, 0, st, a);
     launch(st_root_kernel<S>, 1, 1, 0, st, a);
     // levels: at least log2(n / M) are needed; the host then learns every two levels whether more are
     int level = 0, want = 0;
@@ -661,7 +727,8 @@ int build_search_tree(const void *src, int n, int d, int dtype, int layout, Poin
     if (ar.failed) return WM_ENOMEM;
     const size_t mark = ar.off;
     a.buf[1] = ar.get<float>((size_t)n * X.S);
-    a.state = ar.get<BuildState>(1);
+    a.state = (BuildState *)ar.take(kStateBytes + sizeof(unsigned) * 4 * X.S);
+    a.root_acc = (unsigned *)((char *)a.state + kStateBytes);   // (not used before the check below)
     if (ar.failed) return WM_ENOMEM;
     int rc;
     switch (X.S) {

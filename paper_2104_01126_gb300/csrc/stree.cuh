@@ -7,7 +7,7 @@
 // group one 256-bit load) and, in the last padded dimension, a reference (lo slot) and a component
 // label or -1 (hi slot): a visit reads the two child rows and nothing else.  A reference is the row of
 // the left child, or for a bucket kBucketBit | (size - 1) << 28 | first point.  A point row holds the
-// FP32 coordinates and, in its last slot, the point's component label.
+// FP32 coordinates (of FP64 ones far from 0: less a centre) and, in its last slot, the point's component label.
 #pragma once
 
 #include "wm_internal.cuh"

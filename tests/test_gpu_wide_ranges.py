@@ -62,7 +62,7 @@ def test_batch_far_from_the_origin():
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("min_pts", [1, 10])
-@pytest.mark.parametrize("name", ["cauchy", "lognormal"])
+@pytest.mark.parametrize("name", ["cauchy", "lognormal", "timestamps", "offset"])
 def test_times(name, min_pts):
     require_gpu()
 
