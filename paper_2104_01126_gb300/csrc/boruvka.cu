@@ -856,8 +856,12 @@ __device__ __forceinline__ int root_of(const int *__restrict__ par, int x, int n
 // consecutive positions per thread took 130, and 15 for the prefixes instead of 40).
 constexpr int kTileItems = 8, kTile = 256 * kTileItems;
 
-// Up to this many points the steps between the searches are run by one block each, see nc_small_back_kernel
-constexpr int kSmallThreads = 512, kSmallPoints = kSmallThreads * kTileItems;
+// Up to this many points the steps between the searches are run by one block each, see nc_small_back_kernel.  The line
+// lies where one block takes as long as the launches it saves (ms, one block / launches, EMST in 2-D: 1000 points 0.66 /
+// 0.78, 2000 0.77 / 0.83, 3000 0.92 / 0.93, 4096 1.04 / 0.96; in 7-D 1.27 / 1.33, 2.07 / 2.15, 2.53 / 2.48, 3.21 / 3.05;
+// HDBSCAN* in 2-D 1.09 / 1.18, 1.26 / 1.29, 1.41 / 1.41, 1.66 / 1.59).
+constexpr int kSmallThreads = 512, kSmallPoints = 3072;
+static_assert(kSmallPoints <= kSmallThreads * kTileItems, "one tile (change_prefixes)");
 
 // Once a single component is left nobody reads a label again, and the steps below return at once.
 __device__ __forceinline__ void relabel_points(const NcArgs &b, int S, const int *roots, int *sums)
@@ -1005,8 +1009,7 @@ __global__ void nc_node_labels_kernel(int Ns, int S, const int2 *range, float *n
 }
 
 // Few points: the steps before, between and after the searches by one block, with barriers for the ends of the
-// kernels.  Each of them is then shorter than the gap between two launches (EMST of 10^3 points 790 -> 686 us;
-// the launches win again where one block takes longer than they do).
+// kernels.  Each of them is then shorter than the gap between two launches (figures at kSmallPoints).
 template <int D, bool HDB, bool F64>
 __global__ void __launch_bounds__(kSmallThreads) nc_small_front_kernel(TravArgs a, NcArgs b)
 {

@@ -49,9 +49,9 @@ def test_limit_that_follows_the_number_of_points(n, inner):
 @pytest.mark.gpu
 @pytest.mark.parametrize("precision", ["fp32", "fp64"])
 @pytest.mark.parametrize("min_pts", [1, 10])
-@pytest.mark.parametrize("n,d", [(2_047, 3), (2_048, 3), (3_001, 5), (4_096, 8), (4_097, 8)])
+@pytest.mark.parametrize("n,d", [(2_047, 3), (2_048, 3), (3_001, 5), (3_072, 8), (3_073, 8), (4_097, 8)])
 def test_smallest_sizes_that_hand_over(n, d, min_pts, precision):
-    # up to 4096 points the steps behind the search are one block's: they hold back in the same way
+    # up to 3072 points the steps behind the search are one block's: they hold back in the same way
     require_gpu()
     x = _ball_in_sphere(n, 40, d, 1e-6, n + d, "f8")
     if min_pts == 1:
