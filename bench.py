@@ -287,15 +287,23 @@ def serving_sweep(wm, args, rank):
 
 
 def run_ablation(wm, torch, call, timed_pass, release):
-    """MemoGFK (the default) against GFK (the full WSPD materialised, Algorithm 2) and EMST-Naive
-    on the EMST of 10^7 uniform points in 3-D; and, on the HDBSCAN* workload, the disjunctive
+    """The default's nearest-component rounds ("nearest") against MemoGFK rounds (Algorithm 3, under an
+    override of the tuning by the table's own row), GFK (the full WSPD materialised, Algorithm 2) and
+    EMST-Naive on the EMST of 10^7 uniform points in 3-D; and, on the HDBSCAN* workload, the disjunctive
     separation of Sec. 3.1.2 against the geometric one of the GanTao baseline (the full WSPD of
     each counted by the GFK form).  One warm-up and one timed call per method."""
-    def run(w, x, method):
+    def run(w, x, form):
+        method = "memogfk" if form == "nearest" else form
+        row = wm.get_tuning(w["n"], w["d"], w.get("min_pts", 0)) if form == "memogfk" else None
+
         def fn():
-            if w["problem"] == "hdbscan":
-                return wm.hdbscan(x, min_pts=w["min_pts"], start=0, method=method, return_stats=True)
-            return wm.emst(x, method=method, return_stats=True)
+            wm.set_tuning(row)
+            try:
+                if w["problem"] == "hdbscan":
+                    return wm.hdbscan(x, min_pts=w["min_pts"], start=0, method=method, return_stats=True)
+                return wm.emst(x, method=method, return_stats=True)
+            finally:
+                wm.set_tuning(None)
         fn()
         stream = torch.cuda.current_stream()
         e0 = torch.cuda.Event(enable_timing=True)
@@ -311,12 +319,12 @@ def run_ablation(wm, torch, call, timed_pass, release):
     out = {}
     w = WORKLOADS["emst-uniform-10m-3d"]
     x = torch.from_numpy(make_points(w)).cuda()
-    out["emst-uniform-10m-3d"] = {m: run(w, x, m) for m in ("memogfk", "gfk", "naive")}
+    out["emst-uniform-10m-3d"] = {m: run(w, x, m) for m in ("nearest", "memogfk", "gfk", "naive")}
     del x
     release()
     w = WORKLOADS[CFG2]
     x = torch.from_numpy(make_points(w)).cuda()
-    out[CFG2] = {m: run(w, x, m) for m in ("memogfk", "gantao", "gfk", "gfk-geometric")}
+    out[CFG2] = {m: run(w, x, m) for m in ("nearest", "memogfk", "gantao", "gfk", "gfk-geometric")}
     del x
     release()
     out["note"] = ("every method returns the same tree (tests/test_gpu_methods.py checks it); wspd_pairs: size of the materialised WSPD (GFK forms); "
@@ -373,10 +381,11 @@ def visit_bytes(d):
     return 8 + 32 + 32 + 16 * dp + 16
 
 
-def kernel_rooflines(runs, peaks, fp32_peak, fp32_basis, hdb=False):
+def kernel_rooflines(runs, peaks, fp32_peak, fp32_basis, hdb=False, precision="fp32"):
     """Per-kernel roofline entries summed over runs = [(d, stats), ...]: the traversals against
-    HBM (algorithmic bytes per visited pair), the BCCP and k-NN kernels against the measured FP32
-    FMA peak (3d-1 flop per distance evaluation, +2 under mutual reachability)."""
+    HBM (algorithmic bytes per visited pair), the BCCP, search and k-NN kernels against the measured FP32
+    FMA peak (3d-1 flop per distance evaluation, +2 under mutual reachability); evaluations of the FP64 form are
+    not rated against that peak."""
     def tot(f):
         return sum(f(d, s) for d, s in runs)
 
@@ -396,8 +405,8 @@ def kernel_rooflines(runs, peaks, fp32_peak, fp32_basis, hdb=False):
                            f"(d = {runs[0][0]}; the byte count grows with d)",
                    "peak_basis": peaks["hbm_basis"]})
 
-    def alu(name, evals, ms, launches, extra=0):
-        if ms <= 0:
+    def alu(name, evals, ms, launches, extra=0, limited_by=None):
+        if ms <= 0 or precision != "fp32":
             return
         ev = tot(lambda d, s: evals(s))
         if ev <= 0:
@@ -407,7 +416,7 @@ def kernel_rooflines(runs, peaks, fp32_peak, fp32_basis, hdb=False):
         ks.append({"kernel": name, "bound": "alu", "achieved": tf, "peak": fp32_peak, "unit": "TFLOP/s",
                    "frac": tf / fp32_peak, "ms": ms, "launches": launches, "traffic": None,
                    "work": f"{ev} distance evaluations x (3d-1{'+2' if extra else ''}) flop",
-                   "peak_basis": fp32_basis})
+                   "peak_basis": fp32_basis, **({"limited_by": limited_by} if limited_by else {})})
 
     hbm("findpair_dfs_kernel<1> (GetPairs traversal)", "getpairs", lambda s: s.getpairs_visits,
         tot(lambda d, s: s.ms_getpairs), tot(lambda d, s: s.getpairs_launches))
@@ -419,11 +428,15 @@ def kernel_rooflines(runs, peaks, fp32_peak, fp32_basis, hdb=False):
     alu("bccp_pair_tile_kernel (medium and big pairs)", lambda s: s.bccp_tile_evals,
         tot(lambda d, s: s.ms_tile_kernel), None, x)
     # calls without traversals run the nearest-component rounds, whose search reports under the same fields
-    alu("bccp_dual_kernel (huge pairs, pruned dual-tree)" if tot(lambda d, s: s.getpairs_visits) > 0
-        else "nc_search_kernel (nearest-component search)", lambda s: s.bccp_dual_evals,
-        tot(lambda d, s: s.ms_bccp_dual), None, x)
+    walk = "dependent loads through the L1 data pipe and divergence, not FP32 (counters in profiles/)"
+    if tot(lambda d, s: s.getpairs_visits) > 0:
+        alu("bccp_dual_kernel (huge pairs, pruned dual-tree)", lambda s: s.bccp_dual_evals,
+            tot(lambda d, s: s.ms_bccp_dual), None, x)
+    else:
+        alu("nc_search_kernel (nearest-component search)", lambda s: s.bccp_dual_evals,
+            tot(lambda d, s: s.ms_bccp_dual), None, x, walk)
     alu("knn_walk_kernel (core distances)", lambda s: s.knn_evals, tot(lambda d, s: s.ms_knn_kernel),
-        len(runs))
+        len(runs), limited_by=walk)
     if not ks:
         return None
     roof = dict(max(ks, key=lambda k: k["ms"]))
@@ -650,7 +663,8 @@ def main():
     value = whole_job_value(n_total, ws, ms_max)
     clocks = clk.summary()
     runs = [(w["d"], s) for (w, _), s in zip(dev, st)]
-    roof = kernel_rooflines(runs, peaks, fp32_peak, fp32_basis, hdb=any(w["problem"] == "hdbscan" for w, _ in dev))
+    roof = kernel_rooflines(runs, peaks, fp32_peak, fp32_basis, hdb=any(w["problem"] == "hdbscan" for w, _ in dev),
+                            precision=args.precision)
     screen_err = max(s.max_rel_screen_err for s in st)
     workloads = {}
     for i, ((w, x), s) in enumerate(zip(host, st)):
@@ -721,7 +735,7 @@ def main():
                         "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
                 "plain_form": {"value": whole_job_value(w["n"], ws, pms[0]), "unit": "Mpoints/s",
                                "ms_per_step": pms[0], "precision": "fp64"},
-                "roofline": kernel_rooflines([(w["d"], cst)], peaks, fp32_peak, fp32_basis, hdb=True),
+                "roofline": kernel_rooflines([(w["d"], cst)], peaks, fp32_peak, fp32_basis, hdb=True, precision=args.precision),
                 "max_rel_screen_err": cst.max_rel_screen_err,
                 "phases_ms": {k: round(getattr(cst, k), 3) for k in (
                     "ms_build_tree", "ms_core_dist", "ms_knn_kernel", "ms_wspd", "ms_getrho", "ms_getpairs",

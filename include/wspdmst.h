@@ -131,7 +131,7 @@ typedef struct {
                                       candidate re-evaluated in FP64 (every winner among
                                       them) and every core distance; 0 in the FP64 form
                                       (also taken where the FP32 copy of FP64 coordinates
-                                      errs by more than a 128th of the points' spacing).
+                                      blurs a 16th of the points' neighbourhoods).
                                       A priori bound: 2^-19 for FP32-exact coordinates  */
     int32_t tie_overflow;          /* HDBSCAN*: 1 when the pairs within some point's core
                                       distance (the tie-repair edges) exceeded their
@@ -373,10 +373,13 @@ int wm_wait(wm_server *s, int64_t ticket, double *latency_ms);
 int wm_server_counters(wm_server *s, int64_t *finished, size_t *peak_bytes, int32_t *peak_running);
 
 /*
- * Tuning.  Parameters that change how fast a call runs, never what it returns (every setting
- * yields the same K-minimum tree, dendrogram and plot).  A call takes them from a built-in table
- * chosen by (problem, d, n) and written by the project's autotuner (paper_2104_01126_gb300/
- * autotune.py), unless wm_set_tuning has set an override for the whole process.
+ * Tuning.  Parameters of the pair traversals (MemoGFK rounds and the forms GFK, EMST-Naive and GanTao): they
+ * change how fast such a call runs, never what it returns (every setting yields the same K-minimum tree,
+ * dendrogram and plot).  Nearest-component rounds (see the top) have none.  A call takes them from a built-in
+ * table chosen by (problem, d, n) and written by the project's autotuner (paper_2104_01126_gb300/autotune.py),
+ * unless wm_set_tuning has set an override for the whole process.  Any override, the table's own row included,
+ * also takes calls that would run nearest-component rounds to the MemoGFK rounds, which it tunes: 2 to 8 times
+ * slower on most inputs.
  */
 typedef struct {
     int32_t tight_diameters; /* 1: a node's diameter bound is the smallest of its box diagonal,
@@ -415,10 +418,11 @@ typedef struct {
     int32_t reserved[5];
 } wm_tuning;
 
-/* The parameters a call with these sizes uses (min_pts = 0 for EMST); n = 0 gives the built-in
- * defaults (the values before any table row or override). */
+/* The parameters that the pair traversals of a call with these sizes use (min_pts = 0 for EMST); n = 0 gives the
+ * built-in defaults (the values before any table row or override). */
 int wm_get_tuning(int64_t n, int32_t d, int32_t min_pts, wm_tuning *out);
-/* Overrides the table for every later call of the process (NULL restores it).  WM_EINVAL for
+/* Overrides the table for every later call of the process, and takes it to the pair traversals (NULL restores
+ * both).  WM_EINVAL for
  * out-of-range values.  Not for use while other threads are inside library calls. */
 int wm_set_tuning(const wm_tuning *t);
 

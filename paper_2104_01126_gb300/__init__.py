@@ -529,14 +529,15 @@ def query_footprint(n: int, d: int, min_pts: int = 0) -> int:
 
 
 def get_tuning(n: int, d: int, min_pts: int = 0) -> dict:
-    """The speed parameters a call with these sizes uses (wm_get_tuning)."""
+    """The speed parameters of the pair traversals of a call with these sizes (wm_get_tuning)."""
     t = _Tuning()
     _check(load().wm_get_tuning(int(n), int(d), int(min_pts), ctypes.byref(t)), "wm_get_tuning")
     return {f: getattr(t, f) for f in TUNING_FIELDS}
 
 
 def set_tuning(params=None):
-    """Overrides the built-in tuning table for every later call (wm_set_tuning); None restores it.
+    """Overrides the built-in tuning table for every later call, which then runs the pair traversals
+    (wm_set_tuning); None restores both.
     params: a dict of TUNING_FIELDS (missing fields take the built-in defaults)."""
     lib = load()
     if params is None:

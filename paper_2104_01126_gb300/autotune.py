@@ -11,7 +11,7 @@ and stops on a difference.  The chosen table is written to csrc/tuning_table.inc
 library to use it) and a summary, with each bucket's time under the defaults and tuned, to the
 JSON file named by --report.
 
-    python -m paper_2104_01126_gb300.autotune --report gpurun_out/autotune.json
+    python -m paper_2104_01126_gb300.autotune --report autotune.json
 
 --dims / --sizes retune a subset of the buckets; with --merge OLD_REPORT the rows of OLD_REPORT that
 were not retuned are kept, and the table and report are written for the union.

@@ -158,6 +158,11 @@ static long long wspd_pairs_guess(long long n, int d)
     return std::max<long long>(1 << 16, per * n);
 }
 
+// Workspace of a call by either form.  The terms are those of the traversals, which need the more: nearest-component
+// rounds alone take up to 8 dimensions at most 480 + 8 d bytes a point for the tree (its build included), 240 for the
+// rounds and 70 for the sort, and 256 more where the tree is hundreds of levels deep; the terms below hold 36 d + 16 d +
+// 700 bytes a point at the least.  The smaller figure would not do for a caller's arena: an override of the tuning, or
+// ties that overflow the repair list, take the same call to the traversals.
 static size_t estimate_bytes(long long n, int d, int min_pts, const Caps &c)
 {
     const long long N = 2 * n;
@@ -451,14 +456,18 @@ static void set_rho(TravArgs &a, double lo, double hi)
 // Whether the forest is built by nearest-component rounds (boruvka.cu) rather than MemoGFK rounds.  Both
 // give the K-minimum tree; the nearest-component rounds answer one question per component and round
 // instead of visiting every well-separated pair, and are the faster of the two on every generator and
-// size measured up to 8 dimensions (GB300, ms: EMST uniform 3-D / 5-D and variable-density 7-D points at
-// 10^7: 35 / 72 / 212 against 58 / 130 / 890; uniform 2-D at 3x10^6, FP64: 10.3 against 11.3; 10^3
-// points in 3-D: 1.6 against 3.5; HDBSCAN* of 10^6 points in 3-D: 14 against 31).  MemoGFK keeps
+// size measured up to 8 dimensions (GB300, ms, against MemoGFK rounds under the built-in tuning: EMST uniform 3-D /
+// 5-D and variable-density 7-D points at 10^7: 18.4 / 36.1 / 111 against 56.8 / 131 / 794; uniform 2-D at 3x10^6 in the
+// FP64 form: 10.3 against 10.6; 10^3 points in 3-D: 0.63 against 1.90; HDBSCAN* of 10^6 points in 3-D: 5.8 against
+// 24.3, of 10^5 in 10-D 29.6 against 143, of 3x10^4 in 16-D 30.7 against 163).  Slower than MemoGFK rounds are only
+// sets whose points are all about as far from as many others (EMST of a 7-D lattice of 2.8x10^5 points 4.9 against 3.9, of
+// 10^5 points on a sphere with 5x10^4 in a ball inside 10.3 against 6.7).  MemoGFK keeps
 //   - calls under wm_set_tuning, whose parameters are those of the traversals, and the geometric
 //     separation of the GanTao baseline, which is a property of the WSPD;
 //   - HDBSCAN* inputs whose repair list overflowed: the rounds here need it complete;
-//   - EMSTs above 8 dimensions: on uniform points every search visits much of the tree (10^5 points in
-//     10-D: 71 against 57 ms; 3x10^4 in 16-D: 178 against 96), which the pair traversal shares better;
+//   - EMSTs above 8 dimensions.  That line was drawn when the search was half as fast (10^5 uniform points in
+//     10-D: 71 against 57 ms) and has not been moved since; it now costs time (38 against 59; 3x10^4 in 16-D 39 against
+//     130; 10^6 of a mixture in 16-D 731 against 2890);
 //   - 2^28 points and more (references hold 28-bit positions).
 static bool nearest_rounds_apply(const Call &C, int n, int d, const HdbState *hdb)
 {
