@@ -63,9 +63,9 @@ __host__ __device__ constexpr bool marks_ties(int D) { return list_len(D) < 2 * 
 // A query that has looked at long_points points (above 10^6 or two: a 1024th of all) and is still walking is handed
 // to warps that share a scan of all points: the centre of a sphere of points is as far from all of them, and
 // its walk visits every node on one lane while the GPU waits (EMST of 50,000 points and their centre: 83 ms, of
-// which 81 on that lane; 3.2 now, FP64 form 142 and 4.5; with a limit of 2048 5.0 and 7.6.  7-D sets reach 1024 in
+// which 81 on that lane; 2.7 now, FP64 form 142 and 3.7; with a limit of 2048 5.0 and 7.6.  7-D sets reach 1024 in
 // ordinary walks, and were 2 % slower with it).  Points count whether they are evaluated or only bounded: in the
-// FP64 form a walk that bounded most of 10^6 points went unnoticed (36 -> 16 ms).  While at most kLongMax
+// FP64 form a walk that bounded most of 10^6 points went unnoticed (36 -> 13 ms).  While at most kLongMax
 // queries and about kLongWork points' evaluations are waiting, such a query is handed over at once; one that
 // comes later walks on, and is handed over all the same when it has looked at a kLongPart-th of all points
 // (twice the limit at least), since it will hardly stop before the rest.  A query is handed over at most once a
